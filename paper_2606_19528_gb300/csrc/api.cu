@@ -151,15 +151,16 @@ int make_map(CUtensorMap* m, const void* ptr, uint64_t inner, uint64_t outer, ui
 }
 
 // 2-D tensor map of `dtype` elements over a row-major [outer, inner] matrix
-// with row stride `ld` elements, no swizzle (staging boxes read by threads).
+// with row stride `ld` elements, no swizzle or the 128-byte swizzle (staging boxes read by threads).
 int make_map_plain(CUtensorMap* m, CUtensorMapDataType dtype, int esize, const void* ptr, uint64_t inner,
-                   uint64_t outer, uint64_t ld, uint32_t box_inner, uint32_t box_outer) {
+                   uint64_t outer, uint64_t ld, uint32_t box_inner, uint32_t box_outer, bool swizzle = false) {
   cuuint64_t dims[2] = {inner, outer};
   cuuint64_t strides[1] = {ld * (uint64_t)esize};
   cuuint32_t box[2] = {box_inner, box_outer};
   cuuint32_t estr[2] = {1, 1};
   CUresult r = g_encode(m, dtype, 2, const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? LORA_OK : LORA_ECUDA;
 }
@@ -245,8 +246,9 @@ inline int64_t rup(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 // ------------------------------------------------------------------ fused-contraction problems
 // Output [M, N] over a contraction of Kc base columns plus an r-wide adapter
 // slab; one contraction pass, output written directly (no split).
-// tile_n: the launch's tile width (gemm_tile_n(), or gemm_tile_n_f32() for fp32 output).
-void gemm_shape(GemmProblem& g, int64_t M, int64_t N, int64_t Kc, int64_t r, int tile_n = 0) {
+// tile_n, tile_m: the launch's tile (gemm_tile_n() x gemm_tile_m(), gemm_tile_n_f32() columns for fp32
+// output, gemm_tile_n_q4() x gemm_tile_m_q4() with 4-bit weights).
+void gemm_shape(GemmProblem& g, int64_t M, int64_t N, int64_t Kc, int64_t r, int tile_n = 0, int tile_m = 0) {
   g.ldo = (int)N;
   g.out_f32 = 0;
   g.M = (int)M;
@@ -254,13 +256,14 @@ void gemm_shape(GemmProblem& g, int64_t M, int64_t N, int64_t Kc, int64_t r, int
   g.Kmain = (int)Kc;
   g.r = (int)r;
   g.num_n_tiles = cdiv(N, tile_n > 0 ? tile_n : gemm_tile_n());
-  g.num_m_tiles = cdiv(M, gemm_tile_m());
+  if (tile_m <= 0) tile_m = gemm_tile_m();
+  g.num_m_tiles = cdiv(M, tile_m);
   g.m_fast = N >= M ? 1 : 0;  // the weight operand at least as large as the activation operand
   g.kb_main = cdiv(Kc, gemm_tile_k());
   g.kb_total = g.kb_main + cdiv(r, gemm_tile_k());
   g.splits = 1;
   g.kb_split = g.kb_total;
-  g.m_pad = g.num_m_tiles * gemm_tile_m();
+  g.m_pad = g.num_m_tiles * tile_m;
   g.part = nullptr;
   g.ldp = 0;
   g.lse = nullptr;
@@ -270,6 +273,14 @@ void gemm_shape(GemmProblem& g, int64_t M, int64_t N, int64_t Kc, int64_t r, int
   g.cand = nullptr;
   g.cap = 0;
   g.row_off = g.col_off = g.sym = 0;
+}
+
+// The same for the contraction of one projection, whose tile depends on its weight type.
+void proj_gemm_shape(GemmProblem& g, int64_t M, int64_t N, int64_t Kc, int64_t r, bool q4) {
+  if (q4)
+    gemm_shape(g, M, N, Kc, r, gemm_tile_n_q4(), gemm_tile_m_q4());
+  else
+    gemm_shape(g, M, N, Kc, r);
 }
 
 // Appends the problem just filled in at b.prob[b.num_problems].
@@ -296,6 +307,19 @@ constexpr double kPartEpiBlocks = 1.0;    // per split unit: fp32 partial tile i
 constexpr double kReduceFixBlocks = 6.0;  // the reduce launch
 constexpr double kBytesPerBlock = 5.0e6;  // HBM bytes moved in one block time
 
+// A problem's block in those units: a 4-bit problem's 512 x 256 tile holds as many MMAs, half as many when
+// the problem has one 256-row segment only; so does the 256 x 256 tile of fp32 output.
+double block_cost(const GemmProblem& g) {
+  const bool q4 = g.m_pad == g.num_m_tiles * gemm_tile_m_q4();
+  return g.out_f32 ? 0.6 : q4 && g.M <= gemm_tile_m() ? 0.8 : 1.0;
+}
+
+// Up to two tiles per pair, cutting also evens out tiles of unequal depth (a layer's down projection is
+// 129 blocks deep, the others 49) or a second wave that is nearly empty; beyond, the walk evens out by
+// itself.  A single bf16 contraction of at least one tile per pair is never cut: the forward without a
+// workspace gives the same bits there.
+constexpr int kSplitMaxWaves = 2;
+
 double simulate_splits(const GemmBatch& b, const int* sp, int pairs) {
   std::vector<double> fin(pairs, 0.0);  // min-heap of pair finish times
   std::make_heap(fin.begin(), fin.end(), std::greater<double>());
@@ -307,7 +331,7 @@ double simulate_splits(const GemmBatch& b, const int* sp, int pairs) {
     const int kbs = (g.kb_total + sp[p] - 1) / sp[p];
     for (int ks = 0; ks < sp[p]; ++ks) {
       const int len = std::min(g.kb_total, (ks + 1) * kbs) - ks * kbs;
-      const double d = len + kUnitFixBlocks + (sp[p] > 1 ? kPartEpiBlocks : 0.0);
+      const double d = len * block_cost(g) + kUnitFixBlocks + (sp[p] > 1 ? kPartEpiBlocks : 0.0);
       for (int t = 0; t < per; ++t) {
         std::pop_heap(fin.begin(), fin.end(), std::greater<double>());
         fin.back() += d;
@@ -316,7 +340,8 @@ double simulate_splits(const GemmBatch& b, const int* sp, int pairs) {
     }
     if (sp[p] > 1) {
       any = true;
-      reduce += (double)g.m_pad * g.N * (4.0 * sp[p] + 2.0) / kBytesPerBlock;
+      // the epilogue stores, and the reduce reads, the rows of whole 32-row groups only
+      reduce += (double)rup(g.M, 32) * g.N * (4.0 * sp[p] + 2.0) / kBytesPerBlock;
     }
   }
   return *std::max_element(fin.begin(), fin.end()) + reduce + (any ? kReduceFixBlocks : 0.0);
@@ -329,10 +354,10 @@ void choose_splits(const GemmBatch& b, int* splits, int pairs = kPlanPairs) {
   for (int p = 0; p < b.num_problems; ++p) {
     const GemmProblem& g = b.prob[p];
     tiles += (long long)g.num_m_tiles * g.num_n_tiles;
-    key.insert(key.end(), {g.num_m_tiles, g.num_n_tiles, g.kb_total, g.m_pad, g.N});
+    key.insert(key.end(), {g.num_m_tiles, g.num_n_tiles, g.kb_total, g.m_pad, g.M, g.N, g.out_f32});
     splits[p] = 1;
   }
-  if (tiles == 0 || tiles >= pairs) return;
+  if (tiles == 0 || tiles >= (long long)pairs * (b.num_problems > 1 || b.prob[0].out_f32 ? kSplitMaxWaves : 1)) return;
   static std::mutex mu;
   static std::map<std::vector<long long>, std::vector<int>> cache;
   {
@@ -899,9 +924,9 @@ int add_fwd_problem(GemmBatch& b, const lora_proj& p, const Operands& o) {
   if ((rc = r > 0 ? make_map(&b.tmA2[i], o.s_in, r, T, o.ld_s, 64, 128) : (b.tmA2[i] = b.tmA[i], LORA_OK)) != LORA_OK)
     return rc;
   if (is_q4(p)) {
-    // 4-bit W: a box is 64 rows x 64 codes (32 bytes); (s, b) boxes are 128 rows x 4 groups
-    if ((rc = make_map_plain(&b.tmQ[i], CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, p.Wq.codes, K / 2, N, K / 2, 32, 64)) !=
-        LORA_OK)
+    // 4-bit W: a box is 128 rows x 256 codes (128 bytes, swizzled); (s, b) boxes are 128 rows x 4 groups
+    if ((rc = make_map_plain(&b.tmQ[i], CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, p.Wq.codes, K / 2, N, K / 2, 128, 128,
+                             true)) != LORA_OK)
       return rc;
     if ((rc = make_map_plain(&b.tmP[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, p.Wq.params, K / 32, N, K / 32, 8,
                              128)) != LORA_OK)
@@ -913,7 +938,7 @@ int add_fwd_problem(GemmBatch& b, const lora_proj& p, const Operands& o) {
     return rc;
   if ((rc = make_map(&b.tmOut[i], p.y, N, T, N, 64, 32)) != LORA_OK) return rc;
   GemmProblem& g = b.prob[i];
-  gemm_shape(g, T, N, K, r);
+  proj_gemm_shape(g, T, N, K, r, is_q4(p));
   g.out = mb(p.y);
   add_problem(b);
   return LORA_OK;
@@ -944,7 +969,7 @@ int add_bwd_problem(GemmBatch& b, const lora_proj& p, const Operands& o) {
     return rc;
   if ((rc = make_map(&b.tmOut[i], p.dx, K, T, K, 64, 32)) != LORA_OK) return rc;
   GemmProblem& g = b.prob[i];
-  gemm_shape(g, T, K, N, r);
+  proj_gemm_shape(g, T, K, N, r, is_q4(p));
   g.out = mb(p.dx);
   add_problem(b);
   return LORA_OK;
@@ -1047,7 +1072,7 @@ SideWidths side_widths(int num_sms, const lora_proj* projs, int n) {
   for (int i = 0; i < n; ++i) {
     const lora_shape& sh = projs[i].shape;
     const double T = (double)sh.T, K = (double)sh.d_in, N = (double)sh.d_out, r = (double)sh.rank;
-    flops += 2.0 * T * K * N * (is_q4(projs[i]) ? 1.3 : 1.0);
+    flops += 2.0 * T * K * N;
     if (sh.rank == 0) continue;  // a frozen projection puts no work on the side stream
     const double fr = 1.0 + r / 144.0;
     b1 += 2.0 * T * N * fr + kSideAdapter1 * r * N;
@@ -1432,12 +1457,13 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
     }
   }
   std::vector<size_t> split_need(n, 0);
-  for (int dir = 0; dir < 2; ++dir) {
-    if (!(mode & (dir == 0 ? LORA_FWD : LORA_BWD))) continue;
+  // The splits of direction `dir` on `pairs` pairs with the projections' weights as `kind` says (0 bf16,
+  // 1 4-bit, which has tiles of its own): raises split_need, and keeps the counts when `keep` is given.
+  auto plan_splits = [&](int dir, const std::vector<char>& kind, int pairs, std::vector<int>* keep) {
     for (int q4 = 0; q4 < 2; ++q4) {
       std::vector<int> order;
       for (int i = 0; i < n; ++i)
-        if (is_q4(projs[i]) == (q4 != 0)) order.push_back(i);
+        if (kind[i] == q4) order.push_back(i);
       std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
         return dir == 0 ? projs[a].shape.d_in > projs[b].shape.d_in : projs[a].shape.d_out > projs[b].shape.d_out;
       });
@@ -1447,30 +1473,35 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
         for (size_t i = i0; i < order.size() && i < i0 + kMaxProblems; ++i) {
           const lora_shape& sh = projs[order[i]].shape;
           if (dir == 0)
-            gemm_shape(b.prob[b.num_problems], sh.T, sh.d_out, sh.d_in, sh.rank);
+            proj_gemm_shape(b.prob[b.num_problems], sh.T, sh.d_out, sh.d_in, sh.rank, q4 != 0);
           else
-            gemm_shape(b.prob[b.num_problems], sh.T, sh.d_in, sh.d_out, sh.rank);
+            proj_gemm_shape(b.prob[b.num_problems], sh.T, sh.d_in, sh.d_out, sh.rank, q4 != 0);
           add_problem(b);
         }
-        // the splits for the pairs this call's contraction gets, and the partials sized for the
-        // largest of those splits and the ones for the other pair counts above: a forward-and-backward
-        // call's workspace, whose side stream may leave few pairs to a contraction, must also hold a
-        // forward or backward call of the same shapes
-        for (size_t pass = 0; pass <= pairs_alt[dir].size(); ++pass) {
-          const int pairs = pass == 0 ? pairs_dir[dir] : pairs_alt[dir][pass - 1];
-          if (pass > 0 && pairs == pairs_dir[dir]) continue;
-          int sp[kMaxProblems];
-          choose_splits(b, sp, pairs);
-          if (!allow_split)
-            for (int q = 0; q < b.num_problems; ++q) sp[q] = 1;
-          for (int q = 0; q < b.num_problems; ++q) {
-            const int pi = order[i0 + q];
-            if (pass == 0) (dir == 0 ? pl->split_f : pl->split_b)[pi] = sp[q];
-            split_need[pi] = std::max(split_need[pi], split_floats(b.prob[q], sp[q]));
-          }
+        int sp[kMaxProblems];
+        choose_splits(b, sp, pairs);
+        if (!allow_split)
+          for (int q = 0; q < b.num_problems; ++q) sp[q] = 1;
+        for (int q = 0; q < b.num_problems; ++q) {
+          const int pi = order[i0 + q];
+          if (keep) (*keep)[pi] = sp[q];
+          split_need[pi] = std::max(split_need[pi], split_floats(b.prob[q], sp[q]));
         }
       }
     }
+  };
+  // The splits for the weights and the pairs of this call, and the partials sized for the largest of those
+  // splits and the ones of either weight kind on the other pair counts above: a forward-and-backward call's
+  // workspace, whose side stream may leave few pairs to a contraction, must also hold a forward or backward
+  // call of the same shapes.
+  std::vector<char> kind(n);
+  for (int i = 0; i < n; ++i) kind[i] = is_q4(projs[i]) ? 1 : 0;
+  for (int dir = 0; dir < 2; ++dir) {
+    if (!(mode & (dir == 0 ? LORA_FWD : LORA_BWD))) continue;
+    plan_splits(dir, kind, pairs_dir[dir], dir == 0 ? &pl->split_f : &pl->split_b);
+    pairs_alt[dir].push_back(pairs_dir[dir]);
+    for (int q4 = 0; q4 < 2; ++q4)
+      for (int pairs : pairs_alt[dir]) plan_splits(dir, std::vector<char>(n, (char)q4), pairs, nullptr);
   }
   size_t off = kWsHeader;
   pl->zero_bytes = off;
@@ -1534,7 +1565,7 @@ void layer_copy(const lora_proj* L, int n_per, uint8_t* su_scratch, std::vector<
 // ------------------------------------------------------------------ reduced-vocabulary cross entropy
 
 // Split partials of one contraction: splits happen only below kPlanPairs output
-// tiles (M x N < kPlanPairs 256 x 512 padded), at most 8 of them.
+// tiles of 256 x 512 (fp32 output: 2 kPlanPairs of 256 x 256), at most 8 of them.
 constexpr size_t kCeSplitFloats = (size_t)8 * kPlanPairs * 256 * 512 + 64 * 1024;
 
 struct CePlan {

@@ -38,14 +38,17 @@
 // Every wait is bounded.
 //
 // 4-bit weights (Algorithm 1's on-the-fly dequantization, W = s * W_q + b with
-// one (s, b) per output row and 64-wide group along d_in): three decoupled
-// rings per CTA.  Warp 0 streams the activation boxes (3 deep); warp 10
+// one (s, b) per output row and 64-wide group along d_in): tiles of 512 x 256,
+// their two segments being row halves that share one dequantized weight tile,
+// so a weight element is dequantized once per 512 rows of the output and a
+// contraction block moves 122 KB through a CTA's shared memory (132 KB with
+// 256 x 512 tiles, which dequantize twice as much per FLOP).  Three decoupled
+// rings per CTA.  Warp 0 streams the activation boxes (3 deep); the last warp
 // streams this CTA's codes and (s, b) pairs by TMA (a quarter of the bf16
-// weight bytes, 2 deep); warps 6..9 dequantize a block with packed bf16
+// weight bytes); warps 6..13 dequantize a block with packed bf16
 // FMAs straight into the 128-byte-swizzled operand layout the tensor core
-// reads, in a ring of 4 bf16 weight tiles, releasing the code slot at once;
-// warp 11 relays "tile dequantized" to the MMA issuer (one cluster-scope
-// arrive per block and CTA, kept off the dequantizing warps' path); the MMA
+// reads, in a ring of 4 bf16 weight tiles, releasing the code slot at once and
+// arriving on the MMA issuer's barrier; the MMA
 // waits for an activation stage and a weight tile.  Each ring has a
 // block of slack over its refill latency; the bf16 weight never exists in HBM.
 #include "common.cuh"
@@ -66,38 +69,53 @@ constexpr uint32_t kBox = 64 * kBK * 2;           // one 64 x 64 box of the weig
 constexpr int kEpiWarps = 8;                      // bf16 weights: two per TMEM lane quadrant
 constexpr uint32_t kEpiStage = 32 * 128;          // per-warp output block: 32 rows x 64 bf16, 4 KB
 constexpr uint32_t kTmemCols = 512;
-constexpr int kConvWarps = 4;                     // 4-bit weights: dequantizing warps per CTA
+constexpr int kConvWarps = 8;                     // 4-bit weights: dequantizing warps per CTA, in
+constexpr int kConvGroups = 2;                    // groups that take alternate contraction blocks
+constexpr int kGroupWarps = kConvWarps / kConvGroups;
 
 constexpr int kMaxStages = 6;
 constexpr uint32_t kStageBytes = kAHalf + 2 * kBSeg;  // bf16 weights: activation + weight boxes
-constexpr uint32_t kQCodes = 8192;                    // 4-bit block: 256 weight rows x 64 codes
-constexpr uint32_t kQSlot = kQCodes + 4096;           // + (s, b) boxes
-constexpr int kQStages = 2;                           // 4-bit: code slots
 constexpr int kWStages = 4;                           // 4-bit: dequantized bf16 weight tiles
-constexpr uint32_t kWTile = 2 * kBSeg;
+constexpr uint32_t kWTile = kBSeg;                    // this CTA's 128 weight rows of the tile
+constexpr int kQMaxStages = 6;
+constexpr uint32_t kQRing = 36864;                    // 4-bit: code slots
+
+// 4-bit code slots.  Forward: a slot holds 4 contraction blocks, the span of
+// the 16-byte (s, b) rows the TMA can address, so codes come in whole 128-byte
+// rows (128-byte swizzle) and each (s, b) row is loaded once.  Backward: one
+// block, 64 contraction rows x this CTA's 128 columns, and the (s, b) of the
+// 256 columns around them.
+template <bool kBMn>
+struct QSlot {
+  static constexpr int kBlocks = kBMn ? 1 : 4;              // contraction blocks per slot
+  static constexpr uint32_t kCodes = kBMn ? 4096 : 16384;   // code bytes
+  static constexpr uint32_t kParams = kBMn ? 1024 : 2048;   // (s, b) bytes
+  static constexpr uint32_t kBytes = kBMn ? 6144 : kCodes + kParams;
+  static constexpr int kStages = kBMn ? 6 : 2;
+  static_assert(kStages <= kQMaxStages && kStages * kBytes <= kQRing && kBytes % 1024 == 0, "code slots");
+};
 
 // Shared-memory layout and warps of the bf16-weight (kQ false) and
 // 4-bit-weight (kQ true) kernels.  bf16: 4 stages of [activation | weight],
-// 8 epilogue warps; 4-bit: 3 activation boxes, 4 bf16 weight tiles, 2 code
-// slots, 4 epilogue warps (its tiles take longer, so one warp per TMEM lane
-// quadrant drains in time) and 4 dequantizing warps.  (4-bit, Llama-shaped
-// layer: 4 weight tiles against 3 took T = 256 from 154 to 149 us and T = 2048
-// from 731 to 720 us; 2 weight tiles cost 15-30 %; the code ring's depth, 2 to
-// 8, changed nothing.)
+// 8 epilogue warps; 4-bit: 3 stages of two activation boxes, 4 bf16 weight
+// tiles, 36 KB of code slots, 4 epilogue warps and 8 dequantizing warps.
+// Measured on the 4-bit Llama-shaped layer, T = 2048 (forward / backward
+// contraction): 256 x 512 tiles with the weight tiles relayed by a cluster-scope
+// release 334 / 325 us; 512 x 256 tiles 295 / 321 us (the release, 800 to 1400
+// cycles a block, was then the limit); without it 239 / 232 us, the rate of the
+// bf16 form (231 / 225 us).
 template <bool kQ>
 struct Cfg {
   static constexpr int kStages = kQ ? 3 : 4;  // activation ring
   static constexpr int kEpi = kQ ? 4 : kEpiWarps;
   static constexpr int kParts = kEpi / 4;          // epilogue warps per TMEM lane quadrant
   static constexpr int kPartCols = kSeg / kParts;  // columns of a segment per epilogue warp
-  static constexpr uint32_t kRing = kQ ? kStages * kAHalf + kWStages * kWTile + kQStages * kQSlot
-                                       : kStages * kStageBytes;
-  static constexpr int kThreads = (2 + kEpi + (kQ ? kConvWarps + 2 : 0)) * 32;
-  __device__ static uint32_t a_addr(uint32_t base, int s) { return base + (uint32_t)s * (kQ ? kAHalf : kStageBytes); }
-  __device__ static uint32_t w_tile(uint32_t base, int w) { return base + kStages * kAHalf + (uint32_t)w * kWTile; }
-  __device__ static uint32_t q_slot(uint32_t base, int s) {
-    return base + kStages * kAHalf + kWStages * kWTile + (uint32_t)s * kQSlot;
-  }
+  static constexpr uint32_t kAStage = kQ ? 2 * kAHalf : kStageBytes;
+  static constexpr uint32_t kRing = kStages * kAStage + (kQ ? kWStages * kWTile + kQRing : 0);
+  static constexpr int kThreads = (2 + kEpi + (kQ ? kConvWarps + 1 : 0)) * 32;
+  __device__ static uint32_t a_addr(uint32_t base, int s) { return base + (uint32_t)s * kAStage; }
+  __device__ static uint32_t w_tile(uint32_t base, int w) { return base + kStages * kAStage + (uint32_t)w * kWTile; }
+  __device__ static uint32_t q_ring(uint32_t base) { return base + kStages * kAStage + kWStages * kWTile; }
 };
 constexpr int kTileRing = 4;  // tile ids handed from the scheduler to the other roles
 constexpr int kDefer = 2;     // wide tiles: blocks whose segment-0 MMAs precede the first segment-1 MMA
@@ -108,10 +126,9 @@ constexpr long long kAbortDrainNs = 10000000ll;  // 10 ms per armed stage on the
 struct __align__(8) Ctl {
   uint64_t full[kMaxStages];       // even CTA: both CTAs' parts of a stage landed
   uint64_t empty[kMaxStages];      // both CTAs: the pair's MMAs finished reading a stage
-  uint64_t qfull[kQStages];        // both CTAs, 4-bit: this CTA's codes and (s, b) of a block landed
-  uint64_t qempty[kQStages];       // both CTAs, 4-bit: this CTA's dequantizers read a code slot
+  uint64_t qfull[kQMaxStages];     // both CTAs, 4-bit: this CTA's codes and (s, b) of a slot landed
+  uint64_t qempty[kQMaxStages];    // both CTAs, 4-bit: this CTA's dequantizers read a code slot
   uint64_t wfull[kWStages];        // even CTA, 4-bit: both CTAs' weight tile dequantized (or loaded)
-  uint64_t convd[kWStages];        // both CTAs, 4-bit: this CTA's dequantizing warps finished a weight tile
   uint64_t wempty[kWStages];       // both CTAs, 4-bit: the pair's MMAs finished reading a weight tile
   uint64_t tfull[2];               // both CTAs: accumulator (buffer) complete
   uint64_t tempty[2];              // even CTA: both CTAs' epilogues drained a segment (buffer)
@@ -135,7 +152,7 @@ constexpr size_t smem_bytes() {
 // that split's contraction blocks [kb0, kb1).  cs_half >= 0 (cluster split):
 // the tile is unsplit in the list and the pair takes half cs_half of its
 // contraction blocks (the first half rounded up).
-template <int kTileN = kBN>
+template <int kTileN = kBN, int kTileM = kBM>
 __device__ __forceinline__ void decode_tile(const GemmBatch& b, int t, int& p, int& m0, int& n0, int& ks, int& kb0,
                                             int& kb1, int cs_half = -1) {
   p = 0;
@@ -153,10 +170,10 @@ __device__ __forceinline__ void decode_tile(const GemmBatch& b, int t, int& p, i
     kb1 = min(Q.kb_total, kb0 + L);
   }
   if (Q.m_fast) {
-    m0 = (local % Q.num_m_tiles) * kBM;
+    m0 = (local % Q.num_m_tiles) * kTileM;
     n0 = (local / Q.num_m_tiles) * kTileN;
   } else {
-    m0 = (local / Q.num_n_tiles) * kBM;
+    m0 = (local / Q.num_n_tiles) * kTileM;
     n0 = (local % Q.num_n_tiles) * kTileN;
   }
 }
@@ -174,47 +191,49 @@ __device__ __forceinline__ uint32_t dq_pair(uint32_t w, uint32_t s2, uint32_t b2
 
 // Dequantizes this CTA's weight operand of one contraction block from the
 // staged codes and (s, b) pairs into the 128-byte-swizzled bf16 boxes the MMA
-// reads.  Row rho of box (h, j) is weight column / row col0 = n0 + 256 h +
-// 128 c + 64 j of the tile: the forward's rows are W rows col0 + rho at
-// k-group kb; the backward's are W rows 64 kb + rho at k-group col0 / 64.
-// Staged boxes: forward, codes (h, j) 64 rows x 32 B at 2 KB (2 h + j), (s, b)
-// h 128 rows x 4 groups at 2 KB h; backward, codes h 64 rows x 64 B at 4 KB h,
-// (s, b) h 64 rows x 4 groups at 1 KB h.  A thread takes half rows (32 codes,
-// 16 bytes) ordered so that a warp reads 512 contiguous bytes of codes.
+// reads: 128 output columns from n0 + 128 c on, as two boxes of 64.  Forward:
+// row rho (0..127) is W row n0 + 128 c + rho at k-group kb; its codes are 32
+// bytes of the slot's 128-byte row (chunk u at u ^ (rho mod 8)).  Backward: row
+// rho (0..63) of box j is W row 64 kb + rho at columns n0 + 128 c + 64 j ..; its
+// codes are 32 bytes of the slot's 64-byte row.  A thread takes half rows (32
+// codes, 16 bytes).  Lanes are ordered so that the 16-byte stores of a quarter
+// warp fall on the eight chunk positions once (forward: eight rows of one
+// half, backward: four rows of both halves), as do the forward's loads.
 template <bool kBMn>
 __device__ __forceinline__ void dequant_stage(uint32_t slot, uint32_t wdst, int ct, int c, int n0, int kb,
                                               int ncols) {
-  constexpr int kThr = kConvWarps * 32;
+  constexpr int kThr = kGroupWarps * 32;
   const uint32_t codes = slot;
-  const uint32_t params = slot + kQCodes;
+  const uint32_t params = slot + QSlot<kBMn>::kCodes;
+  const int colh = n0 + c * kHalf;
 #pragma unroll
-  for (int rep = 0; rep < 512 / kThr; ++rep) {
+  for (int rep = 0; rep < 256 / kThr; ++rep) {
     const int hu = ct + rep * kThr;  // half row
-    const int half = hu & 1, h = hu >> 8;
-    const int j = kBMn ? (hu >> 1) & 1 : (hu >> 7) & 1;
-    const int rho = kBMn ? (hu >> 2) & 63 : (hu >> 1) & 63;
-    const int colh = n0 + h * kSeg + c * kHalf;
-    if (colh + j * 64 >= ncols) continue;  // box not loaded: its MMA columns are never stored
+    const int half = kBMn ? hu & 1 : (hu >> 3) & 1;
+    const int row = kBMn ? hu >> 1 : (hu >> 4) * 8 + (hu & 7);  // 0..127
+    const int j = row >> 6, rho = row & 63;
+    if (colh + j * 64 >= ncols) continue;  // its MMA columns are never stored
     uint32_t csrc, psrc;
     if (kBMn) {
-      const int g = (colh >> 6) + j, gb = (colh >> 6) & ~3;
-      csrc = codes + (uint32_t)(h * 4096 + rho * 64 + j * 32 + half * 16);
-      psrc = params + (uint32_t)(h * 1024 + rho * 16 + (g - gb) * 4);
+      const int g = (colh >> 6) + j;
+      csrc = codes + (uint32_t)(rho * 64 + j * 32 + half * 16);
+      psrc = params + (uint32_t)(rho * 16 + (g & 3) * 4);
     } else {
-      csrc = codes + (uint32_t)((h * 2 + j) * 2048 + rho * 32 + half * 16);
-      psrc = params + (uint32_t)(h * 2048 + (j * 64 + rho) * 16 + (kb & 3) * 4);
+      const int u = (kb & 3) * 2 + half;
+      csrc = codes + (uint32_t)(row * 128 + ((u ^ (row & 7)) << 4));
+      psrc = params + (uint32_t)(row * 16 + (kb & 3) * 4);
     }
     uint32_t w[4], sb;
     asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
                  : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(csrc) : "memory");
     asm volatile("ld.shared.b32 %0, [%1];" : "=r"(sb) : "r"(psrc) : "memory");
     const uint32_t s2 = (sb & 0xFFFFu) * 0x10001u, b2 = (sb >> 16) * 0x10001u;
-    const uint32_t row = wdst + (uint32_t)(h * kBSeg + j * kBox + rho * 128);
+    const uint32_t dst_row = wdst + (uint32_t)(j * kBox + rho * 128);
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
       const uint32_t o0 = dq_pair(w[m], s2, b2), o1 = dq_pair(w[m] >> 4, s2, b2);
       const uint32_t o2 = dq_pair(w[m] >> 8, s2, b2), o3 = dq_pair(w[m] >> 12, s2, b2);
-      const uint32_t dst = row + (uint32_t)((((half * 4 + m) ^ (rho & 7)) & 7) << 4);
+      const uint32_t dst = dst_row + (uint32_t)((((half * 4 + m) ^ (rho & 7)) & 7) << 4);
       asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(o0), "r"(o1), "r"(o2), "r"(o3)
                    : "memory");
     }
@@ -234,8 +253,12 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
   constexpr bool kNarrow = kF32 || kCS;
   static_assert(!kNarrow || !kQ, "256 x 256 tiles: bf16 weights only");
   static_assert(!kF32 || (!kBMn && !kCS), "fp32 output is the plain forward form");
-  constexpr int kSegs = kNarrow ? 1 : 2;  // 256-column segments per tile
-  constexpr int kTileN = kSegs * kSeg;
+  // segments per tile, one 256 x 256 accumulator each: column halves of a 256 x 512 tile, or with 4-bit
+  // weights row halves of a 512 x 256 tile
+  constexpr int kSegs = kNarrow ? 1 : 2;
+  constexpr int kTileN = kQ ? kSeg : kSegs * kSeg;
+  constexpr int kTileM = kQ ? kSegs * kBM : kBM;
+  using QS = QSlot<kBMn>;
   constexpr int kStages = kNarrow ? 6 : Cfg<kQ>::kStages;
   constexpr uint32_t kStageB = kNarrow ? kAHalf + kBSeg : kStageBytes;
   static_assert(kStages <= kMaxStages && (!kNarrow || kStages * kStageB <= Cfg<kQ>::kRing), "ring");
@@ -265,13 +288,12 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
       mbar_init(smem_u32(&ctl->full[s]), 1);
       mbar_init(smem_u32(&ctl->empty[s]), 1);
     }
-    for (int q = 0; q < kQStages; ++q) {
+    for (int q = 0; q < QS::kStages; ++q) {
       mbar_init(smem_u32(&ctl->qfull[q]), 1);
       mbar_init(smem_u32(&ctl->qempty[q]), kConvWarps);
     }
     for (int w = 0; w < kWStages; ++w) {
-      mbar_init(smem_u32(&ctl->wfull[w]), 2);  // the relay of each CTA
-      mbar_init(smem_u32(&ctl->convd[w]), kConvWarps);
+      mbar_init(smem_u32(&ctl->wfull[w]), 2 * kGroupWarps);  // one group's dequantizing warps of both CTAs
       mbar_init(smem_u32(&ctl->wempty[w]), 1);
     }
     mbar_init(smem_u32(&ctl->tfull[0]), 1);
@@ -279,8 +301,8 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
     for (int h = 0; h < 2; ++h) mbar_init(smem_u32(&ctl->tempty[h]), 2 * kEpi);
     for (int k = 0; k < kTileRing; ++k) {
       mbar_init(smem_u32(&ctl->tile_full[k]), 1);
-      // MMA thread, epilogue (and dequantizing, code producer, relay) warps of both CTAs, producer of the odd CTA
-      mbar_init(smem_u32(&ctl->tile_empty[k]), 2 + 2 * kEpi + (kQ ? 2 * kConvWarps + 4 : 0));
+      // MMA thread, epilogue (and dequantizing, code producer) warps of both CTAs, producer of the odd CTA
+      mbar_init(smem_u32(&ctl->tile_empty[k]), 2 + 2 * kEpi + (kQ ? 2 * kConvWarps + 2 : 0));
     }
     mbar_init(smem_u32(&ctl->drain), 1);
     mbar_init(smem_u32(&ctl->xchg), 1);
@@ -332,7 +354,7 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
         if (kCS) {
           t = it == 0 ? cs_tile : -1;  // one tile, no scheduler
         } else if (c == 0) {
-          if (!mbar_wait_cluster(smem_u32(&ctl->tile_empty[slot]), par ^ 1u, wc, abort_flag)) break;
+          if (!mbar_wait(smem_u32(&ctl->tile_empty[slot]), par ^ 1u, wc, abort_flag)) break;
           t = atomicAdd(b.tile_counter, 1);
           if (t >= b.total_tiles) t = -1;
           ctl->tile_id[slot] = t;
@@ -342,29 +364,31 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
         } else {
           if (!mbar_wait_cluster(smem_u32(&ctl->tile_full[slot]), par, wc, abort_flag)) break;
           t = *reinterpret_cast<volatile int*>(&ctl->tile_id[slot]);
-          mbar_arrive_cluster(tile_empty_root + (uint32_t)slot * 8u);
+          mbar_arrive_remote(tile_empty_root + (uint32_t)slot * 8u);
         }
         if (t < 0) {
           griddep_launch_dependents();  // no tile left for this pair
           break;
         }
         int p, m0, n0, ks, kb0, kb1;
-        decode_tile<kTileN>(b, t, p, m0, n0, ks, kb0, kb1, cs_half);
+        decode_tile<kTileN, kTileM>(b, t, p, m0, n0, ks, kb0, kb1, cs_half);
         const GemmProblem& Q = b.prob[p];
         const int my_m = m0 + c * kHalf;
         const bool a_mine = my_m < Q.M;
+        const bool a_mine2 = kQ && my_m + kBM < Q.M;  // the second row segment
         // weight box (segment h, pair position cc, j): columns n0 + 256 h + 128 cc + 64 j
         auto box_ok = [&](int h, int cc, int j) { return n0 + h * kSeg + cc * kHalf + j * 64 < Q.N; };
         uint32_t boxes = 0;
-        for (int h = 0; h < kSegs; ++h)
+        for (int h = 0; !kQ && h < kSegs; ++h)
           for (int cc = 0; cc < 2; ++cc)
             for (int j = 0; j < 2; ++j) boxes += box_ok(h, cc, j) ? 1u : 0u;
         // bytes landing in this pair per stage (signalled on the even CTA)
-        const uint32_t tx_a = (m0 < Q.M ? kAHalf : 0u) + (m0 + kHalf < Q.M ? kAHalf : 0u);
+        uint32_t tx_a = (m0 < Q.M ? kAHalf : 0u) + (m0 + kHalf < Q.M ? kAHalf : 0u);
+        if (kQ) tx_a += (m0 + kBM < Q.M ? kAHalf : 0u) + (m0 + kBM + kHalf < Q.M ? kAHalf : 0u);
         const uint32_t tx_pair = tx_a + kBox * boxes;
         bool ok = true;
         for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait_cluster(smem_u32(&ctl->empty[stage]), phase ^ 1u, wc, abort_flag)) {
+          if (!mbar_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, wc, abort_flag)) {
             ok = false;
             break;
           }
@@ -384,6 +408,7 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
           const CUtensorMap* ta = main ? &b.tmA[p] : &b.tmA2[p];
           const CUtensorMap* tb = main ? &b.tmB[p] : &b.tmB2[p];
           if (a_mine) tma_load_2d_pair(a_dst, ta, bar, kc, my_m);
+          if (a_mine2) tma_load_2d_pair(a_dst + kAHalf, ta, bar, kc, my_m + kBM);
           if (w_tma) {
 #pragma unroll
             for (int h = 0; h < kSegs; ++h) {
@@ -406,7 +431,14 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (even CTA)
-    if (c == 0 && lane == 0) {
+    // The whole warp runs the loop, so that its state (stages, descriptors, tile shapes) stays uniform and
+    // in uniform registers, where the MMA and commit instructions take their operands; one elected lane
+    // issues.  Waits are made uniform by a vote.  (Against one thread running the loop: Llama q projection at
+    // T = 512 46.7 -> 45.5 us, the 4-bit layer at T = 64 129.5 -> 124.3 us, layers at T = 2048 -0.5 %.)
+    if (c == 0) {
+      auto wait_all = [&](uint32_t bar, uint32_t ph) {
+        return __all_sync(0xffffffffu, mbar_wait(bar, ph, wc, abort_flag)) != 0;
+      };
       constexpr uint32_t idesc = idesc_bf16_f32(kBM, kSeg, 0, kBMn ? 1 : 0);
       const uint16_t pair_mask = (uint16_t)(0x3u << pb);
       int stage = 0;
@@ -419,123 +451,129 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
         if (kCS) {
           t = it == 0 ? cs_tile : -1;
         } else {
-          if (!mbar_wait_cluster(smem_u32(&ctl->tile_full[slot]), (uint32_t)((it / kTileRing) & 1), wc, abort_flag))
-            break;
+          bool got = mbar_wait_cluster(smem_u32(&ctl->tile_full[slot]), (uint32_t)((it / kTileRing) & 1), wc, abort_flag);
+          got = __all_sync(0xffffffffu, got);
+          if (!got) break;
           t = *reinterpret_cast<volatile int*>(&ctl->tile_id[slot]);
-          mbar_arrive_cluster(tile_empty_root + (uint32_t)slot * 8u);
+          t = __shfl_sync(0xffffffffu, t, 0);
+          if (lane == 0) mbar_arrive_remote(tile_empty_root + (uint32_t)slot * 8u);
         }
         if (t < 0) {
           griddep_launch_dependents();  // no tile left for this pair
           break;
         }
         int p, m0, n0, ks, kb0, kb1;
-        decode_tile<kTileN>(b, t, p, m0, n0, ks, kb0, kb1, cs_half);
+        decode_tile<kTileN, kTileM>(b, t, p, m0, n0, ks, kb0, kb1, cs_half);
         const GemmProblem& Q = b.prob[p];
-        const int nseg = kNarrow ? 1 : (Q.N - n0 > kSeg ? 2 : 1);  // segments holding any column < N
+        // segments holding any column < N (4-bit weights: any row < M)
+        const int nseg = kNarrow ? 1 : kQ ? (Q.M - m0 > kBM ? 2 : 1) : (Q.N - n0 > kSeg ? 2 : 1);
         // accumulator buffer of this tile; a segment (buffer) is free once both epilogues drained
         // it for its previous tile (the previous tile, or with two buffers the one before)
         const int buf = kNarrow ? (it & 1) : 0;
         const uint32_t drained_par = kNarrow ? (uint32_t)(((it >> 1) & 1) ^ 1) : (uint32_t)((it & 1) ^ 1);
         int kb = kb0;
-        if (!kQ && kSegs == 2) {
-          // Start of a wide tile: segment 0's MMAs of the first kDefer blocks go first, and only then
-          // does the issuer need segment 1's accumulator (the epilogue drains segment 0 first).  Each
-          // segment still accumulates its blocks in order, so the sums are unchanged.
+        // one contraction block's operands: waits until they are in shared memory
+        auto wait_block = [&](int st, uint32_t ph, uint32_t ws) {
+          bool got = mbar_wait(smem_u32(&ctl->full[st]), ph, wc, abort_flag);
+          if (kQ && got) got = mbar_wait(smem_u32(&ctl->wfull[ws % kWStages]), (ws / kWStages) & 1u, wc, abort_flag);
+          got = __all_sync(0xffffffffu, got);
+          tc_fence_after();
+          return got;
+        };
+        // segment h's operands of the block in ring stage st (4-bit: weight tile wt)
+        auto a_desc = [&](int st, int h) {
+          return sw128_desc(a_addr_of(base, st) + (kQ ? (uint32_t)h * kAHalf : 0u), 16, 1024);
+        };
+        auto b_desc = [&](int st, int wt, int h) {
+          const uint32_t addr = kQ ? Cfg<kQ>::w_tile(base, wt) : a_addr_of(base, st) + kAHalf + (uint32_t)h * kBSeg;
+          return kBMn ? sw128_desc(addr, kBox, 1024) : sw128_desc(addr, 16, 1024);
+        };
+        auto depth = [&](int k) { return k < Q.kb_main ? kBK / 16 : min(kBK / 16, (Q.r - (k - Q.kb_main) * kBK + 15) / 16); };
+        // the MMAs of segment h on that block, `first` starting the accumulator
+        auto issue = [&](int st, int wt, int h, int nk, bool first) {
+          const uint64_t ad = a_desc(st, h), bd = b_desc(st, wt, h);
+          if (!elect_one()) return;
+          for (int k = 0; k < nk; ++k)
+            umma_bf16_pair(tmem_base + (uint32_t)((buf + h) * kSeg), ad + (uint64_t)(2 * k),
+                           bd + (uint64_t)((kBMn ? 128 : 2) * k), idesc, (!first || k != 0) ? 1u : 0u);
+        };
+        auto release = [&](int st, int wt) {
+          if (!elect_one()) return;
+          umma_commit_pair_mc(smem_u32(&ctl->empty[st]), pair_mask);
+          if (kQ) umma_commit_pair_mc(smem_u32(&ctl->wempty[wt]), pair_mask);
+        };
+        if (kSegs == 2) {
+          // Start of a two-segment tile: segment 0's MMAs of the first kDefer blocks go first, and only
+          // then does the issuer need segment 1's accumulator (the epilogue drains segment 0 first).
+          // Each segment still accumulates its blocks in order, so the sums are unchanged.
           const int nd = min(kDefer, kb1 - kb0);
-          int dst[kDefer];
+          int dst[kDefer], dwt[kDefer];
           for (int i = 0; i < nd && ok; ++i, ++kb) {
-            if (!mbar_wait(smem_u32(&ctl->full[stage]), phase, wc, abort_flag) ||
-                (i == 0 && !mbar_wait_cluster(smem_u32(&ctl->tempty[buf]), drained_par, wc, abort_flag))) {
+            if (!wait_block(stage, phase, wseq) ||
+                (i == 0 && !wait_all(smem_u32(&ctl->tempty[buf]), drained_par))) {
               ok = false;
               break;
             }
             tc_fence_after();
             dst[i] = stage;
-            const uint32_t a_addr = a_addr_of(base, stage);
-            const int nk = kb < Q.kb_main ? kBK / 16 : min(kBK / 16, (Q.r - (kb - Q.kb_main) * kBK + 15) / 16);
-            const uint64_t ad = sw128_desc(a_addr, 16, 1024);
-            const uint64_t bd = kBMn ? sw128_desc(a_addr + kAHalf, kBox, 1024) : sw128_desc(a_addr + kAHalf, 16, 1024);
-            for (int k = 0; k < nk; ++k)
-              umma_bf16_pair(tmem_base + (uint32_t)(buf * kSeg), ad + (uint64_t)(2 * k),
-                             bd + (uint64_t)((kBMn ? 128 : 2) * k), idesc, (kb != kb0 || k != 0) ? 1u : 0u);
+            dwt[i] = (int)(wseq % kWStages);
+            ++wseq;
+            issue(stage, dwt[i], 0, depth(kb), kb == kb0);
             if (++stage == kStages) {
               stage = 0;
               phase ^= 1u;
             }
           }
-          if (ok && !mbar_wait_cluster(smem_u32(&ctl->tempty[buf + 1]), drained_par, wc, abort_flag)) ok = false;
+          if (ok && !wait_all(smem_u32(&ctl->tempty[buf + 1]), drained_par)) ok = false;
           if (!ok) break;
           tc_fence_after();
           for (int i = 0; i < nd; ++i) {
-            const int kbi = kb0 + i;
-            const uint32_t a_addr = a_addr_of(base, dst[i]);
-            const int nk = kbi < Q.kb_main ? kBK / 16 : min(kBK / 16, (Q.r - (kbi - Q.kb_main) * kBK + 15) / 16);
-            if (nseg > 1) {
-              const uint64_t ad = sw128_desc(a_addr, 16, 1024);
-              const uint64_t bd = kBMn ? sw128_desc(a_addr + kAHalf + kBSeg, kBox, 1024)
-                                       : sw128_desc(a_addr + kAHalf + kBSeg, 16, 1024);
-              for (int k = 0; k < nk; ++k)
-                umma_bf16_pair(tmem_base + (uint32_t)((buf + 1) * kSeg), ad + (uint64_t)(2 * k),
-                               bd + (uint64_t)((kBMn ? 128 : 2) * k), idesc, (kbi != kb0 || k != 0) ? 1u : 0u);
-            }
-            umma_commit_pair_mc(smem_u32(&ctl->empty[dst[i]]), pair_mask);
+            if (nseg > 1) issue(dst[i], dwt[i], 1, depth(kb0 + i), i == 0);
+            release(dst[i], dwt[i]);
           }
         }
-        // wide bf16 tiles with both segments: the last kEndDefer blocks are issued below
-        const int kb_end = (!kQ && kSegs == 2 && nseg == 2 && kb1 - kb >= kEndDefer) ? kb1 - kEndDefer : kb1;
+        // tiles with both segments: the last kEndDefer blocks are issued below
+        const int kb_end = (kSegs == 2 && nseg == 2 && kb1 - kb >= kEndDefer) ? kb1 - kEndDefer : kb1;
         for (; kb < kb_end; ++kb) {
-          if (!mbar_wait(smem_u32(&ctl->full[stage]), phase, wc, abort_flag)) {
+          if (!wait_block(stage, phase, wseq)) {
             ok = false;
             break;
           }
           const int wt = (int)(wseq % kWStages);
-          if (kQ && !mbar_wait_cluster(smem_u32(&ctl->wfull[wt]), (wseq / kWStages) & 1u, wc, abort_flag)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t a_addr = a_addr_of(base, stage);
-          const uint32_t b_addr = kQ ? Cfg<kQ>::w_tile(base, wt) : a_addr + kAHalf;
-          const int nk = kb < Q.kb_main ? kBK / 16 : min(kBK / 16, (Q.r - (kb - Q.kb_main) * kBK + 15) / 16);
-          if (kb != kb0 && nk == kBK / 16 && nseg == kSegs) {
-            // Steady state (every segment, full depth, accumulating).  The one issuing thread paces
+          const int nk = depth(kb);
+          if (kb != kb0 && nk == kBK / 16) {
+            // Steady state (full depth, accumulating).  The one issuing thread paces
             // the main loop, so its instructions per MMA are kept to a minimum: each operand's
             // descriptor is built once per block and advanced by the 16-deep step in its start-address
             // field (address >> 4; 32 bytes of a K-major row, 2048 bytes = 16 rows of an MN-major
             // operand; shared addresses stay below the field's 2^18-byte range).  The same MMAs as the
             // general form below; this form took the Llama-shaped layer's two contractions from 271 /
             // 251 us to 242 / 232 us per step.
-            const uint64_t ad = sw128_desc(a_addr, 16, 1024);
+            if (elect_one()) {
 #pragma unroll
-            for (int h = 0; h < kSegs; ++h) {
-              const uint64_t bd = kBMn ? sw128_desc(b_addr + (uint32_t)h * kBSeg, kBox, 1024)
-                                       : sw128_desc(b_addr + (uint32_t)h * kBSeg, 16, 1024);
+              for (int h = 0; h < kSegs; ++h) {
+                if (h >= nseg) break;
+                const uint64_t ad = a_desc(stage, h), bd = b_desc(stage, wt, h);
 #pragma unroll
-              for (int k = 0; k < kBK / 16; ++k)
-                umma_bf16_pair(tmem_base + (uint32_t)((buf + h) * kSeg), ad + (uint64_t)(2 * k),
-                               bd + (uint64_t)((kBMn ? 128 : 2) * k), idesc, 1u);
-            }
-          } else
-          for (int h = 0; h < kSegs; ++h) {
-            if (kb == kb0) {
-              if (!mbar_wait_cluster(smem_u32(&ctl->tempty[buf + h]), drained_par, wc, abort_flag)) {
-                ok = false;
-                break;
+                for (int k = 0; k < kBK / 16; ++k)
+                  umma_bf16_pair(tmem_base + (uint32_t)((buf + h) * kSeg), ad + (uint64_t)(2 * k),
+                                 bd + (uint64_t)((kBMn ? 128 : 2) * k), idesc, 1u);
               }
-              tc_fence_after();
             }
-            if (h >= nseg) continue;
-            const uint32_t d_tmem = tmem_base + (uint32_t)((buf + h) * kSeg);
-            const uint32_t bseg = b_addr + (uint32_t)h * kBSeg;
-            for (int k = 0; k < nk; ++k) {
-              const uint64_t adesc = sw128_desc(a_addr + k * 32, 16, 1024);
-              const uint64_t bdesc = kBMn ? sw128_desc(bseg + k * 2048, kBox, 1024) : sw128_desc(bseg + k * 32, 16, 1024);
-              umma_bf16_pair(d_tmem, adesc, bdesc, idesc, (kb != kb0 || k != 0) ? 1u : 0u);
+          } else {
+            for (int h = 0; h < nseg; ++h) {
+              if (kb == kb0) {  // two-segment tiles start above
+                if (!wait_all(smem_u32(&ctl->tempty[buf + h]), drained_par)) {
+                  ok = false;
+                  break;
+                }
+                tc_fence_after();
+              }
+              issue(stage, wt, h, nk, kb == kb0);
             }
           }
           if (!ok) break;
-          umma_commit_pair_mc(smem_u32(&ctl->empty[stage]), pair_mask);
-          if (kQ) umma_commit_pair_mc(smem_u32(&ctl->wempty[wt]), pair_mask);
+          release(stage, wt);
           ++wseq;
           if (++stage == kStages) {
             stage = 0;
@@ -544,55 +582,43 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
         }
         if (!ok) break;
         if (kSegs == 2) {
-          // End of a wide tile: segment 0's MMAs of the last blocks go first and segment 0 is signalled
-          // complete before segment 1, so its drain overlaps segment 1's last MMAs.  Each segment still
-          // accumulates its blocks in order.
-          int dst2[kEndDefer];
-          const int ne = kQ ? 0 : kb1 - kb;
+          // End of a two-segment tile: segment 0's MMAs of the last blocks go first and segment 0 is
+          // signalled complete before segment 1, so its drain overlaps segment 1's last MMAs.  Each
+          // segment still accumulates its blocks in order.
+          int dst2[kEndDefer], dwt2[kEndDefer];
+          const int ne = kb1 - kb;
           for (int i = 0; i < ne && ok; ++i, ++kb) {
-            if (!mbar_wait(smem_u32(&ctl->full[stage]), phase, wc, abort_flag)) {
+            if (!wait_block(stage, phase, wseq)) {
               ok = false;
               break;
             }
-            tc_fence_after();
             dst2[i] = stage;
-            const uint32_t a_addr = a_addr_of(base, stage);
-            const int nk = kb < Q.kb_main ? kBK / 16 : min(kBK / 16, (Q.r - (kb - Q.kb_main) * kBK + 15) / 16);
-            const uint64_t ad = sw128_desc(a_addr, 16, 1024);
-            const uint64_t bd = kBMn ? sw128_desc(a_addr + kAHalf, kBox, 1024) : sw128_desc(a_addr + kAHalf, 16, 1024);
-            for (int k = 0; k < nk; ++k)
-              umma_bf16_pair(tmem_base, ad + (uint64_t)(2 * k), bd + (uint64_t)((kBMn ? 128 : 2) * k), idesc, 1u);
+            dwt2[i] = (int)(wseq % kWStages);
+            ++wseq;
+            issue(stage, dwt2[i], 0, depth(kb), false);
             if (++stage == kStages) {
               stage = 0;
               phase ^= 1u;
             }
           }
           if (!ok) break;
-          umma_commit_pair_mc(smem_u32(&ctl->tfull[0]), pair_mask);
+          if (elect_one()) umma_commit_pair_mc(smem_u32(&ctl->tfull[0]), pair_mask);
           for (int i = 0; i < ne; ++i) {
-            const int kbi = kb1 - ne + i;
-            const uint32_t a_addr = a_addr_of(base, dst2[i]);
-            const int nk = kbi < Q.kb_main ? kBK / 16 : min(kBK / 16, (Q.r - (kbi - Q.kb_main) * kBK + 15) / 16);
-            const uint64_t ad = sw128_desc(a_addr, 16, 1024);
-            const uint64_t bd = kBMn ? sw128_desc(a_addr + kAHalf + kBSeg, kBox, 1024)
-                                     : sw128_desc(a_addr + kAHalf + kBSeg, 16, 1024);
-            for (int k = 0; k < nk; ++k)
-              umma_bf16_pair(tmem_base + (uint32_t)kSeg, ad + (uint64_t)(2 * k), bd + (uint64_t)((kBMn ? 128 : 2) * k),
-                             idesc, 1u);
-            umma_commit_pair_mc(smem_u32(&ctl->empty[dst2[i]]), pair_mask);
+            issue(dst2[i], dwt2[i], 1, depth(kb1 - ne + i), false);
+            release(dst2[i], dwt2[i]);
           }
-          umma_commit_pair_mc(smem_u32(&ctl->tfull[1]), pair_mask);
+          if (elect_one()) umma_commit_pair_mc(smem_u32(&ctl->tfull[1]), pair_mask);
         } else {
-          umma_commit_pair_mc(smem_u32(&ctl->tfull[buf]), pair_mask);
+          if (elect_one()) umma_commit_pair_mc(smem_u32(&ctl->tfull[buf]), pair_mask);
         }
       }
       // completes in both CTAs of the pair once every MMA issued above has finished
-      umma_commit_pair_mc(smem_u32(&ctl->drain), pair_mask);
+      if (elect_one()) umma_commit_pair_mc(smem_u32(&ctl->drain), pair_mask);
     }
   } else if (kCS && warp < 2 + kEpi) {
     // ------------------------------------------------------------ epilogue, cluster split: wait for the
     // pair's accumulator; the exchange of the halves follows below, after every role
-    bool ok = mbar_wait_cluster(smem_u32(&ctl->tfull[0]), 0u, wc, abort_flag);
+    bool ok = mbar_wait(smem_u32(&ctl->tfull[0]), 0u, wc, abort_flag);
     ok = __all_sync(0xffffffffu, ok);
     tc_fence_after();
   } else if (warp < 2 + kEpi) {
@@ -607,23 +633,24 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
       if (!got) break;
       const int t = *reinterpret_cast<volatile int*>(&ctl->tile_id[slot]);
       __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(tile_empty_root + (uint32_t)slot * 8u);
+      if (lane == 0) mbar_arrive_remote(tile_empty_root + (uint32_t)slot * 8u);
       if (t < 0) break;
       int p, m0, n0, ks, kb0, kb1;
-      decode_tile<kTileN>(b, t, p, m0, n0, ks, kb0, kb1);
+      decode_tile<kTileN, kTileM>(b, t, p, m0, n0, ks, kb0, kb1);
       const GemmProblem& Q = b.prob[p];
       const int buf = kNarrow ? (it & 1) : 0;  // accumulator buffer of this tile
       const uint32_t tpar = kNarrow ? (uint32_t)((it >> 1) & 1) : (uint32_t)(it & 1);
-      // wide tiles signal each segment's accumulator complete on its own (tfull[h])
-      bool ok = kSegs == 2 || mbar_wait_cluster(smem_u32(&ctl->tfull[buf]), tpar, wc, abort_flag);
+      // two-segment tiles signal each segment's accumulator complete on its own (tfull[h])
+      bool ok = kSegs == 2 || mbar_wait(smem_u32(&ctl->tfull[buf]), tpar, wc, abort_flag);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
-      const int row0 = m0 + c * kHalf + q * 32;  // first of this warp's 32 rows
       const uint32_t stg = epi_base + (uint32_t)(warp - 2) * kEpiStage;
       for (int h = 0; h < kSegs; ++h) {
+        const int row0 = m0 + (kQ ? h * kBM : 0) + c * kHalf + q * 32;  // first of this warp's 32 rows
+        const int seg_col = kQ ? 0 : h * kSeg;                          // the segment's first tile column
         if (kSegs == 2) {
-          bool okh = mbar_wait_cluster(smem_u32(&ctl->tfull[h]), tpar, wc, abort_flag);
+          bool okh = mbar_wait(smem_u32(&ctl->tfull[h]), tpar, wc, abort_flag);
           okh = __all_sync(0xffffffffu, okh);
           if (!okh) {
             ok = false;
@@ -761,7 +788,7 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
           }
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive_cluster(tempty_pl + (uint32_t)(buf + h) * 8u);
+          if (lane == 0) mbar_arrive_remote(tempty_pl + (uint32_t)(buf + h) * 8u);
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
             const int col0 = c00 + 64 * u;
@@ -786,9 +813,10 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
           continue;
         }
         for (int cc = 0; !app && cc < Cfg<kQ>::kPartCols; cc += block_cols) {
-          const int col0 = h * kSeg + part * Cfg<kQ>::kPartCols + cc;  // tile column of this block
+          const int col0 = seg_col + part * Cfg<kQ>::kPartCols + cc;  // tile column of this block
           if (n0 + col0 >= Q.N || row0 >= Q.M) break;     // uniform across the warp
-          const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * kSeg + col0);
+          const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) +
+                                 (uint32_t)((buf + (kQ ? h : 0)) * kSeg + col0);
           uint32_t v[32], w[32];
           tmem_ld_32x32b_x32(taddr, v);
           if (!f32) tmem_ld_32x32b_x32(taddr + 32u, w);
@@ -845,7 +873,7 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
         }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(tempty_pl + (uint32_t)(buf + h) * 8u);
+        if (lane == 0) mbar_arrive_remote(tempty_pl + (uint32_t)(buf + h) * 8u);
       }
       if (!ok) break;
     }
@@ -853,9 +881,12 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
     if (lane == 0) bulk_wait0();
   } else if (kQ && warp < 2 + kEpi + kConvWarps) {
     // ------------------------------------------------------------ weight dequantizers (both CTAs)
-    const int cw = warp - 2 - kEpi;
+    // Two groups of four warps take alternate blocks: a warp's waits, proxy fence and shared-memory
+    // latency per block (about 250 of its 650 cycles when all eight share each block) then overlap the
+    // other group's conversion.
+    const int cw = (warp - 2 - kEpi) % kGroupWarps, grp = (warp - 2 - kEpi) / kGroupWarps;
     const int ct = cw * 32 + lane;
-    const uint32_t wfull_pl = mapa_shared(smem_u32(&ctl->wfull[0]), 0);  // adapter-block TMA completions
+    const uint32_t wfull_pl = mapa_shared(smem_u32(&ctl->wfull[0]), 0);  // the MMA issuer's barriers
     int qs = 0;          // code slot of the next main block
     uint32_t qpar = 0;   // its qfull parity
     uint32_t wseq = 0;   // contraction blocks so far: weight tile wseq % kWStages
@@ -866,88 +897,65 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
       if (!got) break;
       const int t = *reinterpret_cast<volatile int*>(&ctl->tile_id[slot]);
       __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(tile_empty_root + (uint32_t)slot * 8u);
+      if (lane == 0) mbar_arrive_remote(tile_empty_root + (uint32_t)slot * 8u);
       if (t < 0) break;
       int p, m0, n0, ks, kb0, kb1;
-      decode_tile(b, t, p, m0, n0, ks, kb0, kb1);
+      decode_tile<kTileN, kTileM>(b, t, p, m0, n0, ks, kb0, kb1);
       const GemmProblem& Q = b.prob[p];
-      auto box_ok = [&](int h, int cc, int j) { return n0 + h * kSeg + cc * kHalf + j * 64 < Q.N; };
+      auto box_ok = [&](int cc, int j) { return n0 + cc * kHalf + j * 64 < Q.N; };
+      const int kq1 = min(kb1, Q.kb_main);  // end of the blocks taken from codes
       bool ok = true;
-      for (int kb = kb0; kb < kb1; ++kb) {
+      for (int kb = kb0; kb < kb1; ++kb, ++wseq) {
         const bool main = kb < Q.kb_main;
         const int wt = (int)(wseq % kWStages);
-        // the weight tile's previous contents are consumed by the MMAs
-        ok = mbar_wait_cluster(smem_u32(&ctl->wempty[wt]), ((wseq / kWStages) & 1u) ^ 1u, wc, abort_flag);
-        if (ok && main) ok = mbar_wait(smem_u32(&ctl->qfull[qs]), qpar, wc, abort_flag);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
+        const bool mine = (int)(wseq % kConvGroups) == grp;
         const uint32_t wdst = Cfg<kQ>::w_tile(base, wt);
+        if (mine) {
+          // the weight tile's previous contents are consumed by the MMAs
+          ok = mbar_wait(smem_u32(&ctl->wempty[wt]), ((wseq / kWStages) & 1u) ^ 1u, wc, abort_flag);
+          // (waiting again for a slot already seen full returns at once)
+          if (ok && main) ok = mbar_wait(smem_u32(&ctl->qfull[qs]), qpar, wc, abort_flag);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+        }
         if (main) {
-          dequant_stage<kBMn>(Cfg<kQ>::q_slot(base, qs), wdst, ct, c, n0, kb, Q.N);
-          fence_proxy_async_smem();  // the tensor core reads what these threads wrote
-          __syncwarp();
-          if (lane == 0) {
-            mbar_arrive(smem_u32(&ctl->qempty[qs]));  // the code slot may be refilled
-            mbar_arrive(smem_u32(&ctl->convd[wt]));
+          if (mine) {
+            dequant_stage<kBMn>(Cfg<kQ>::q_ring(base) + (uint32_t)qs * QS::kBytes, wdst, ct, c, n0, kb, Q.N);
+            fence_proxy_async_smem();  // the tensor core reads what these threads wrote
+            __syncwarp();
           }
-          if (++qs == kQStages) {
-            qs = 0;
-            qpar ^= 1u;
+          // past the slot's last block of this tile: every warp of both groups lets it be refilled (a
+          // group cannot be a whole ring ahead: its next weight tile waits for the other group's blocks)
+          if ((kb + 1) % QS::kBlocks == 0 || kb + 1 == kq1) {
+            if (lane == 0) mbar_arrive(smem_u32(&ctl->qempty[qs]));
+            if (++qs == QS::kStages) {
+              qs = 0;
+              qpar ^= 1u;
+            }
           }
-        } else {
+        } else if (mine) {
           // adapter block: the bf16 rank-side boxes go straight into the weight tile by TMA
           if (cw == 0 && lane == 0) {
             const int kc = (kb - Q.kb_main) * kBK;
             const uint32_t bar = wfull_pl + (uint32_t)wt * 8u;
             if (c == 0) {
-              // before this CTA's relay can arrive: the phase cannot complete without these bytes
+              // before this warp arrives: the phase cannot complete without these bytes
               uint32_t boxes = 0;
-              for (int h = 0; h < 2; ++h)
-                for (int cc = 0; cc < 2; ++cc)
-                  for (int j = 0; j < 2; ++j) boxes += box_ok(h, cc, j) ? 1u : 0u;
+              for (int cc = 0; cc < 2; ++cc)
+                for (int j = 0; j < 2; ++j) boxes += box_ok(cc, j) ? 1u : 0u;
               mbar_expect_tx(smem_u32(&ctl->wfull[wt]), kBox * boxes);
             }
-            for (int h = 0; h < 2; ++h) {
-              for (int j = 0; j < 2; ++j) {
-                if (!box_ok(h, c, j)) continue;
-                const int col = n0 + h * kSeg + c * kHalf + j * 64;
-                tma_load_2d_pair(wdst + h * kBSeg + j * kBox, &b.tmB2[p], bar, kBMn ? col : kc, kBMn ? kc : col);
-              }
+            for (int j = 0; j < 2; ++j) {
+              if (!box_ok(c, j)) continue;
+              const int col = n0 + c * kHalf + j * 64;
+              tma_load_2d_pair(wdst + j * kBox, &b.tmB2[p], bar, kBMn ? col : kc, kBMn ? kc : col);
             }
           }
           __syncwarp();
-          if (lane == 0) mbar_arrive(smem_u32(&ctl->convd[wt]));
         }
-        ++wseq;
+        if (mine && lane == 0) mbar_arrive_remote(wfull_pl + (uint32_t)wt * 8u);
       }
       if (!ok) break;
-    }
-  } else if (kQ && warp == 2 + kEpi + kConvWarps + 1) {
-    // ------------------------------------------------------------ relay (both CTAs)
-    if (lane == 0) {
-      const uint32_t wfull_pl = mapa_shared(smem_u32(&ctl->wfull[0]), 0);
-      uint32_t wseq = 0;
-      for (int it = 0;; ++it) {
-        const int slot = it % kTileRing;
-        if (!mbar_wait_cluster(smem_u32(&ctl->tile_full[slot]), (uint32_t)((it / kTileRing) & 1), wc, abort_flag))
-          break;
-        const int t = *reinterpret_cast<volatile int*>(&ctl->tile_id[slot]);
-        mbar_arrive_cluster(tile_empty_root + (uint32_t)slot * 8u);
-        if (t < 0) break;
-        int p, m0, n0, ks, kb0, kb1;
-        decode_tile(b, t, p, m0, n0, ks, kb0, kb1);
-        bool ok = true;
-        for (int kb = kb0; kb < kb1; ++kb, ++wseq) {
-          const int wt = (int)(wseq % kWStages);
-          if (!mbar_wait(smem_u32(&ctl->convd[wt]), (wseq / kWStages) & 1u, wc, abort_flag)) {
-            ok = false;
-            break;
-          }
-          // cumulative release: covers the dequantizing warps' writes this thread acquired
-          mbar_arrive_cluster(wfull_pl + (uint32_t)wt * 8u);
-        }
-        if (!ok) break;
-      }
     }
   } else if (kQ) {
     // ------------------------------------------------------------ code producer (both CTAs)
@@ -960,47 +968,37 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
         if (!mbar_wait_cluster(smem_u32(&ctl->tile_full[slot]), (uint32_t)((it / kTileRing) & 1), wc, abort_flag))
           break;
         const int t = *reinterpret_cast<volatile int*>(&ctl->tile_id[slot]);
-        mbar_arrive_cluster(tile_empty_root + (uint32_t)slot * 8u);
+        mbar_arrive_remote(tile_empty_root + (uint32_t)slot * 8u);
         if (t < 0) break;
         int p, m0, n0, ks, kb0, kb1;
-        decode_tile(b, t, p, m0, n0, ks, kb0, kb1);
+        decode_tile<kTileN, kTileM>(b, t, p, m0, n0, ks, kb0, kb1);
         const GemmProblem& Q = b.prob[p];
-        auto box_ok = [&](int h, int j) { return n0 + h * kSeg + c * kHalf + j * 64 < Q.N; };
-        // bytes of this CTA's code and (s, b) boxes per block
-        uint32_t tx_q = 0;
-        for (int h = 0; h < 2; ++h) {
-          if (kBMn) {
-            tx_q += box_ok(h, 0) ? 4096u + 1024u : 0u;
-          } else {
-            tx_q += box_ok(h, 0) ? 2048u : 0u;
-            for (int j = 0; j < 2; ++j) tx_q += box_ok(h, j) ? 2048u : 0u;
-          }
-        }
+        const int colh = n0 + c * kHalf;  // this CTA's first output column
+        // a slot of columns past N loads nothing, but still passes through the ring
+        const bool any = colh < Q.N;
         bool ok = true;
-        for (int kb = kb0; kb < min(kb1, Q.kb_main); ++kb) {
+        for (int kb = kb0; kb < min(kb1, Q.kb_main); kb = (kb / QS::kBlocks + 1) * QS::kBlocks) {
           if (!mbar_wait(smem_u32(&ctl->qempty[qs]), qpar ^ 1u, wc, abort_flag)) {
             ok = false;
             break;
           }
           const uint32_t qbar = smem_u32(&ctl->qfull[qs]);
-          const uint32_t codes = Cfg<kQ>::q_slot(base, qs);
-          const uint32_t params = codes + kQCodes;
-          mbar_arrive_expect_tx(qbar, tx_q);
+          const uint32_t codes = Cfg<kQ>::q_ring(base) + (uint32_t)qs * QS::kBytes;
+          const uint32_t params = codes + QS::kCodes;
+          mbar_arrive_expect_tx(qbar, any ? QS::kCodes + QS::kParams : 0u);
           ++qfills;
-          for (int h = 0; h < 2; ++h) {
-            const int colh = n0 + h * kSeg + c * kHalf;
-            if (!box_ok(h, 0)) continue;
+          if (any) {
             if (kBMn) {
-              // W rows 64 kb ..; this CTA's 128 output columns = 64 code bytes, 2 groups
-              tma_load_2d(codes + h * 4096, &b.tmQ[p], qbar, colh / 2, kb * kBK);
-              tma_load_2d(params + h * 1024, &b.tmP[p], qbar, ((colh >> 6) & ~3) * 2, kb * kBK);
+              // W rows 64 kb ..; this CTA's 128 output columns = 64 code bytes; (s, b) of 4 groups
+              tma_load_2d(codes, &b.tmQ[p], qbar, colh / 2, kb * kBK);
+              tma_load_2d(params, &b.tmP[p], qbar, ((colh >> 6) & ~3) * 2, kb * kBK);
             } else {
-              for (int j = 0; j < 2; ++j)
-                if (box_ok(h, j)) tma_load_2d(codes + (h * 2 + j) * 2048, &b.tmQ[p], qbar, kb * 32, colh + j * 64);
-              tma_load_2d(params + h * 2048, &b.tmP[p], qbar, (kb & ~3) * 2, colh);
+              // the 4 blocks around kb: 128 code bytes and 4 (s, b) groups of this CTA's 128 W rows
+              tma_load_2d(codes, &b.tmQ[p], qbar, (kb & ~3) * 32, colh);
+              tma_load_2d(params, &b.tmP[p], qbar, (kb & ~3) * 2, colh);
             }
           }
-          if (++qs == kQStages) {
+          if (++qs == QS::kStages) {
             qs = 0;
             qpar ^= 1u;
           }
@@ -1119,8 +1117,8 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
           if (!mbar_wait_drain(smem_u32(&ctl->full[i % kStages]), (uint32_t)((i / kStages) & 1), kAbortDrainNs))
             atomicCAS(b.status, 0, kStatusTimeout);
       if (kQ)
-        for (int i = nq - 1; i >= 0 && i >= nq - kQStages; --i)
-          if (!mbar_wait_drain(smem_u32(&ctl->qfull[i % kQStages]), (uint32_t)((i / kQStages) & 1), kAbortDrainNs))
+        for (int i = nq - 1; i >= 0 && i >= nq - QS::kStages; --i)
+          if (!mbar_wait_drain(smem_u32(&ctl->qfull[i % QS::kStages]), (uint32_t)((i / QS::kStages) & 1), kAbortDrainNs))
             atomicCAS(b.status, 0, kStatusTimeout);
       const uint64_t t0 = global_timer_ns();
       while (global_timer_ns() - t0 < 50000ull) {
@@ -1305,6 +1303,8 @@ cudaError_t launch_fused_gemm(const GemmBatch& batch, bool b_mn_major, bool q4, 
 }
 
 int gemm_tile_m() { return kBM; }
+int gemm_tile_m_q4() { return 2 * kBM; }
+int gemm_tile_n_q4() { return kSeg; }
 int gemm_lse_group() { return kLseGroup; }
 int gemm_tile_n() { return kBN; }
 int gemm_tile_n_f32() { return kSeg; }

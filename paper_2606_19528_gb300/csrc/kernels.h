@@ -154,6 +154,8 @@ int gemm_cs_max_clusters(bool b_mn_major);
 // of the batch with splits > 1 (bf16 or fp32 per out_f32).
 cudaError_t launch_split_reduce(const GemmBatch& batch, cudaStream_t stream);
 int gemm_tile_m();
+int gemm_tile_m_q4();   // tile rows and columns with 4-bit weights
+int gemm_tile_n_q4();
 int gemm_tile_n_f32();  // tile columns of the fp32-output form (two accumulator buffers)
 int gemm_lse_group();  // columns of one log-sum-exp partial
 int gemm_tile_n();

@@ -511,3 +511,17 @@ def test_few_tile_contractions(T, K, N, r):
     for n in ("y", "su", "dx"):
         assert torch.equal(getattr(p, n).view(torch.int16), getattr(q, n).view(torch.int16)), n
     assert torch.equal(p.dA, q.dA) and torch.equal(p.dB, q.dB)
+
+
+def test_unequal_depths_are_cut():
+    """A batch of 76 to 151 output tiles of unequal depth, whose deep problem is cut into partials (80 tiles of
+    5 blocks, 2 of 129): every output against the oracle."""
+    ps = [G.DevProj(*gen_proj(34, 1, 0, 512, 256, 20480, 8, 2.0), 2.0),
+          G.DevProj(*gen_proj(34, 2, 0, 512, 8192, 512, 8, 2.0), 2.0)]
+    before = lora.lora_launch_count()
+    G.run_stack(ps, lora.LORA_FWD)
+    # su, its partial sum, the contractions and the sum of the cut one's partials
+    assert lora.lora_launch_count() - before == 4
+    G.run_stack(ps)
+    for p in ps:
+        check_full(p)

@@ -68,6 +68,19 @@ def check_q4_full(p: DevQ4Proj):
     return errs
 
 
+# around the 512 x 256 tiles (one row segment, both, a second row tile; a column tile of a few columns), and
+# few tiles over a long contraction, whose split ranges start inside a 4-block code slot of the forward
+Q4_EDGES = [(8, 256, 8, 1), (264, 512, 264, 8), (512, 256, 136, 16), (520, 768, 520, 16), (776, 1024, 248, 64),
+            (64, 4352, 512, 16), (64, 1024, 4360, 16)]
+
+
+@pytest.mark.parametrize("T,K,N,r", Q4_EDGES, ids=[f"T{T}_K{K}_N{N}_r{r}" for T, K, N, r in Q4_EDGES])
+def test_q4_tile_edges(T, K, N, r):
+    p = gen_q4_proj(23, 1, 0, T, K, N, r, 2.0)
+    run_q4_single(p)
+    check_q4_full(p)
+
+
 def test_q4_handworked_exact():
     """The hand-worked dequantization (2 rows x 128 columns) embedded in a
     T = 8, d_in = 256, d_out = 8, r = 1 problem with A = B = 0 (zero codes and
