@@ -594,7 +594,8 @@ int choose_unit_chunks(const std::vector<Spec>& specs, size_t i0, size_t i1, int
 }
 
 // Row products of one phase on `ctas` persistent CTAs (one per SM).
-int launch_rows(const std::vector<RowSpec>& specs, const Arena& ar, const DeviceInfo* d, int ctas, cudaStream_t st) {
+int launch_rows(const std::vector<RowSpec>& specs, const Arena& ar, const DeviceInfo* d, int ctas, cudaStream_t st,
+                bool early_next = false) {
   const int tile = rank_mma_tile();
   size_t pf = 0;
   int rc;
@@ -603,6 +604,7 @@ int launch_rows(const std::vector<RowSpec>& specs, const Arena& ar, const Device
     RowBatch b;
     memset(&b, 0, sizeof(b));
     b.tile_rows = tile;
+    b.early_next = early_next ? 1 : 0;
     // one persistent CTA per SM; (tiles, reduction length) of a row problem
     b.unit_chunks = choose_unit_chunks(specs, i0, i1, ctas, [&](const RowSpec& q) {
       return std::make_pair(cdiv(q.T, tile), q.C);
@@ -1323,7 +1325,11 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
     }
     {
       ProfScope ps(LORA_KERNEL_ROWPROJ, st);
-      if ((rc = launch_rows(rows, arena(ws, pl, kPhFwdRows), d, d->num_sms, st)) != LORA_OK) return rc;
+      // Without a side stream the contraction may start beside these products (Llama-shaped layer forward,
+      // T = 32: 56.7 -> 53.5 us).  With one it must not: its CTA pairs would take the free SMs first and its
+      // last pairs then wait for SM pairs that the side stream's CTAs have split up (Llama layer T = 256:
+      // 124 -> 130 us; q projection T = 512: 45.6 -> 47.9 us).
+      if ((rc = launch_rows(rows, arena(ws, pl, kPhFwdRows), d, d->num_sms, st, !ov.on)) != LORA_OK) return rc;
     }
     if (!rows.empty()) prior_main = true;
     // the backward's rank-r work needs su only: it may start now, beside the forward contractions
@@ -1368,6 +1374,9 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
         return rc;
       if (any_adapter(projs, n)) prior_main = true;  // the pass over dy or the row products ran here
     }
+    // with no adapter the dx contraction follows the forward's directly: it must not start on its tiles
+    // before that one's partials, whose buffers it may reuse, are summed
+    if (mode == LORA_FWD_BWD && !any_adapter(projs, n)) prior_main = false;
     // the dx contraction reads sv: when the side stream computed it, wait for it
     if (mode == LORA_FWD_BWD && ov.on && (rc = ov.wait_sv()) != LORA_OK) return rc;
     std::vector<Operands>& ops = bops;

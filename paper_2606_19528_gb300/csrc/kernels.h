@@ -199,6 +199,12 @@ struct RowBatch {
   int tile_rows;    // tokens per tile
   int unit_chunks;  // 64-wide reduction chunks per unit
   int red_total;    // elements of the partial-sum pass (0: none)
+  // 1: the next grid may start as soon as this one has (the kernel signals right after its wait for the
+  // previous grid, its partial-sum pass even before that wait): the contraction that follows a few-CTA row
+  // product then loads and contracts its base operands on the SMs left free.  Every grid waits for its
+  // predecessor before it reads anything but the call's inputs and before it ends, and the row product
+  // itself has waited for everything before the call.
+  int early_next;
   float* partials;  // [tile][unit][tile_rows][rpad] per problem
   int* status;
   long long limit_ns;
@@ -228,6 +234,7 @@ struct ColBatch {
   int tile_rows;    // columns per tile
   int unit_chunks;
   int red_total;
+  int early_next;   // as in RowBatch
   float* partials;
   int* status;
   long long limit_ns;

@@ -16,8 +16,9 @@ namespace {
 // row); the loads of all units are independent and issued together.
 template <typename Batch, bool kRow>
 __global__ void __launch_bounds__(256) reduce_partials_kernel(const __grid_constant__ Batch b, int total4) {
+  if (b.early_next) griddep_launch_dependents();
   griddep_wait();
-  griddep_launch_dependents();
+  if (!b.early_next) griddep_launch_dependents();
   const int i4 = blockIdx.x * blockDim.x + threadIdx.x;
   if (i4 >= total4) return;
   const int i = i4 * 4;

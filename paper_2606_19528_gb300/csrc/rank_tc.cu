@@ -126,6 +126,7 @@ __global__ void __launch_bounds__(kThreads, 1) rank_mma_kernel(const __grid_cons
   __syncthreads();
   tc_fence_after();
   griddep_wait();  // X and the rank sides may come from the previous grid
+  if (b.early_next && threadIdx.x == 0) griddep_launch_dependents();
   const uint32_t tmem_base = ctl->tmem_base;
   long long issued = 0;     // producer: stages issued
   bool issued_any = false;  // MMA issuer: any MMA issued
@@ -174,7 +175,7 @@ __global__ void __launch_bounds__(kThreads, 1) rank_mma_kernel(const __grid_cons
           }
         }
       }
-      griddep_launch_dependents();  // every load of this CTA is issued
+      if (!b.early_next) griddep_launch_dependents();  // every load of this CTA is issued
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
