@@ -13,6 +13,7 @@
 #include <cstdlib>
 #include <functional>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <vector>
 
@@ -215,6 +216,10 @@ Ws plan_ws(const lora_shape& s, int mode) {
 // most the sum of its members').
 enum { kPhFwdRows = 0, kPhBwdRows = 1, kPhBwdCols = 2, kPhases = 3 };
 
+struct SideWidths {
+  int w1 = 0, w2 = 0;  // beside the forward contraction, beside the dx contraction
+};
+
 struct Plan {
   std::vector<Ws> ws;
   std::vector<size_t> offs;
@@ -223,12 +228,10 @@ struct Plan {
   // backward contraction and its fp32 partial buffer (planned from the shapes)
   std::vector<int> split_f, split_b;
   std::vector<size_t> split_off;
-  size_t zero_bytes = 0;  // [0, zero_bytes) is cleared at the start of a call
+  size_t zero_bytes = 0;  // [0, zero_bytes) is cleared at the start of a call that uses tile counters
+  bool counters = false;  // a contraction has more tiles than CTA pairs (on kPlanSms SMs): it takes them from a counter
+  SideWidths side;        // the side stream's SMs on kPlanSms SMs (mode with a backward)
   size_t total = 0;
-  // the fused passes over dy cut for the whole device, as a backward call cuts them, even where a
-  // side stream runs them on a few SMs (the checkpointed stack, whose re-forward-and-backward calls
-  // must sum sv and dB exactly as the saved schedule's backward calls)
-  bool dy_cut_device = false;
 };
 
 template <typename T>
@@ -1056,10 +1059,6 @@ constexpr double kSideAdapter1 = 12.0;  // bytes per r N
 constexpr double kSideAdapter2 = 8.0;   // bytes per r K
 constexpr double kSideSecondPass = 0.6;  // the unfused dB pass over dy: its kernel streams faster per byte
 
-struct SideWidths {
-  int w1 = 0, w2 = 0;
-};
-
 int env_int(const char* name) {
   const char* e = getenv(name);
   return e ? atoi(e) : 0;
@@ -1153,7 +1152,7 @@ struct Overlap {
   int side_ctas2 = 0;  // beside the dx contraction
   cudaStream_t main = nullptr, side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_sv = nullptr, ev_done = nullptr;
-  int init(const DeviceInfo* d, cudaStream_t st, const lora_proj* projs, int n) {
+  int init(const DeviceInfo* d, cudaStream_t st, const lora_proj* projs, int n, const SideWidths& planned) {
     if (!overlap_enabled() || !any_adapter(projs, n)) return LORA_OK;
     SideCtx& c = t_side.dev[d - g_dev];
     if (!c.side && cudaStreamCreateWithFlags(&c.side, cudaStreamNonBlocking) != cudaSuccess) return LORA_ECUDA;
@@ -1164,7 +1163,7 @@ struct Overlap {
     ev_fork = c.ev[0];
     ev_sv = c.ev[1];
     ev_done = c.ev[2];
-    const SideWidths w = side_widths(d->num_sms, projs, n);
+    const SideWidths w = d->num_sms == kPlanSms ? planned : side_widths(d->num_sms, projs, n);
     side_ctas = w.w1;
     side_ctas2 = w.w2;
     on = true;
@@ -1190,14 +1189,19 @@ struct Overlap {
 };
 
 // Runs the given projections in `mode`; every argument already validated.
-int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, DeviceInfo* d, cudaStream_t st) {
+// dy_cut_device: the fused passes over dy are cut for the whole device, as a backward call cuts them, even
+// where a side stream runs them on a few SMs (the checkpointed stack, whose re-forward-and-backward calls
+// must sum sv and dB exactly as the saved schedule's backward calls).
+int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, DeviceInfo* d, cudaStream_t st,
+             bool dy_cut_device = false) {
   int rc;
   const std::vector<Ws>& plans = pl.ws;
   auto W_ = [&](int i) { return at<uint8_t>(ws, pl.offs[i]); };
   // tile counters of the fused-GEMM launches
   int* counters = at<int>(ws, 0);
   int next_counter = 0;
-  if (cudaMemsetAsync(ws, 0, pl.zero_bytes, st) != cudaSuccess) return LORA_ECUDA;
+  if ((pl.counters || d->num_sms != kPlanSms) && cudaMemsetAsync(ws, 0, pl.zero_bytes, st) != cudaSuccess)
+    return LORA_ECUDA;
   // whether a kernel of this call already ran on the main stream: a contraction launched after one may
   // load its base operands (inputs of the call) before the previous grid ends
   bool prior_main = false;
@@ -1207,7 +1211,7 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
   // dB where the pass over dy is not fused) on the side stream beside the dx
   // contraction
   Overlap ov;
-  if ((mode & LORA_BWD) && (rc = ov.init(d, st, projs, n)) != LORA_OK) return rc;
+  if ((mode & LORA_BWD) && (rc = ov.init(d, st, projs, n, pl.side)) != LORA_OK) return rc;
   const int gemm_sms = ov.on ? d->num_sms - ov.side_ctas : d->num_sms;      // forward contraction
   const int gemm_sms_b = ov.on ? d->num_sms - ov.side_ctas2 : d->num_sms;  // dx contraction
   // backward rank-r work: B^T, su^T, sv (and sv^T), then dB and dA; on `rs`
@@ -1269,7 +1273,7 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
     {
       // sv (and dB where fused) before the event the dx contraction waits for
       ProfScope ps(LORA_KERNEL_ROWPROJ, rs);
-      if ((rc = launch_dy_pass(dys, arena(ws, pl, kPhBwdRows), d, ctas, pl.dy_cut_device ? d->num_sms : ctas, rs)) !=
+      if ((rc = launch_dy_pass(dys, arena(ws, pl, kPhBwdRows), d, ctas, dy_cut_device ? d->num_sms : ctas, rs)) !=
           LORA_OK)
         return rc;
       if ((rc = launch_rows(rows, arena(ws, pl, kPhBwdRows), d, ctas, rs)) != LORA_OK) return rc;
@@ -1453,7 +1457,7 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
   // covers a call of either weight kind in any mode
   std::vector<int> pairs_alt[2] = {{kPlanPairs}, {kPlanPairs}};
   if ((mode & LORA_BWD) && overlap_enabled() && any_adapter(projs, n)) {
-    const SideWidths w = side_widths(kPlanSms, projs, n);
+    const SideWidths w = pl->side = side_widths(kPlanSms, projs, n);
     if (mode == LORA_FWD_BWD) pairs_dir[0] = (kPlanSms - w.w1) / 2;
     pairs_dir[1] = (kPlanSms - w.w2) / 2;
     static const uint8_t kAnyCodes = 0;  // a non-null code pointer marks a projection 4-bit for the widths
@@ -1491,11 +1495,15 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
         choose_splits(b, sp, pairs);
         if (!allow_split)
           for (int q = 0; q < b.num_problems; ++q) sp[q] = 1;
+        long long units = 0;
         for (int q = 0; q < b.num_problems; ++q) {
           const int pi = order[i0 + q];
+          units += (long long)b.prob[q].num_m_tiles * b.prob[q].num_n_tiles * sp[q];
           if (keep) (*keep)[pi] = sp[q];
           split_need[pi] = std::max(split_need[pi], split_floats(b.prob[q], sp[q]));
         }
+        // (the backward's launches may leave out projections without dx: never more tiles)
+        if (keep && units > pairs) pl->counters = true;
       }
     }
   };
@@ -1535,6 +1543,53 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
 }
 
 
+// The plan of a call, made once per set of shapes: it depends on the mode, and per projection on its shape,
+// the kind of its weight and which projections share an activation (not on any address).  Planning took 8 to
+// 12 us of the host per call (the tile walks simulated for the splits and the side widths are cached, but a
+// call looked a dozen of them up), as long as a small projection's forward takes on the GPU.  Plans are
+// never changed once made; at most kMaxPlans are kept.
+constexpr size_t kMaxPlans = 512;
+
+int cached_plan(const lora_proj* projs, int n, int mode, std::shared_ptr<const Plan>* out, bool allow_split = true) {
+  std::vector<int64_t> key;
+  key.reserve(2 + 6 * (size_t)n);  // (the length tells n)
+  int dev = -1;  // the side widths ask the device how many clusters fit
+  if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
+  key.push_back(mode + (allow_split ? 4 : 0));
+  key.push_back(dev);
+  for (int i = 0; i < n; ++i) {
+    const lora_shape& sh = projs[i].shape;
+    int first = i;  // the first projection reading this x (its own index without a pointer)
+    if (projs[i].x != nullptr)
+      for (int k = 0; k < i; ++k)
+        if (projs[k].x == projs[i].x) {
+          first = k;
+          break;
+        }
+    key.insert(key.end(), {sh.T, sh.d_in, sh.d_out, sh.rank, is_q4(projs[i]) ? 1 : 0, first});
+  }
+  static std::mutex mu;
+  static std::map<std::vector<int64_t>, std::shared_ptr<const Plan>> cache;
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = cache.find(key);
+    if (it != cache.end()) {
+      for (int i = 0; i < n; ++i)
+        if (!isfinite(projs[i].shape.scale)) return LORA_EINVAL;  // the only part of a shape the key leaves out
+      *out = it->second;
+      return LORA_OK;
+    }
+  }
+  auto pl = std::make_shared<Plan>();
+  const int rc = plan_all(projs, n, mode, pl.get(), allow_split);
+  if (rc != LORA_OK) return rc;
+  *out = pl;
+  std::lock_guard<std::mutex> lk(mu);
+  if (cache.size() >= kMaxPlans) cache.clear();
+  cache.emplace(std::move(key), std::move(pl));
+  return LORA_OK;
+}
+
 // Checkpointed stack (Algorithm 2): scratch for one layer's saved su (the
 // largest layer) and for one stack step.
 int ckpt_layout(const lora_proj* projs, int n_layers, int n_per, size_t* su_bytes, size_t* step_bytes) {
@@ -1549,11 +1604,11 @@ int ckpt_layout(const lora_proj* projs, int n_layers, int n_per, size_t* su_byte
       if (rc != LORA_OK) return rc;
       su += up256((size_t)L[i].shape.T * (size_t)L[i].shape.rank * 2);
     }
-    Plan pl;
-    int rc = plan_all(L, n_per, LORA_FWD_BWD, &pl);  // bounds the su-less forward's needs too
+    std::shared_ptr<const Plan> pl;
+    int rc = cached_plan(L, n_per, LORA_FWD_BWD, &pl);  // bounds the su-less forward's needs too
     if (rc != LORA_OK) return rc;
     sb = std::max(sb, su);
-    wb = std::max(wb, pl.total);
+    wb = std::max(wb, pl->total);
   }
   *su_bytes = up256(sb);
   *step_bytes = wb;
@@ -1823,10 +1878,10 @@ int lora_workspace_size(const lora_shape* shape, int mode, size_t* bytes) {
 int lora_stack_workspace_size(const lora_proj* projs, int n_proj, int mode, size_t* bytes) {
   if (!projs || !bytes) return rec(LORA_ENULL);
   if (n_proj < 1 || n_proj > 64 || mode < LORA_FWD || mode > LORA_FWD_BWD) return rec(LORA_EINVAL);
-  Plan pl;
-  int rc = plan_all(projs, n_proj, mode, &pl);
+  std::shared_ptr<const Plan> pl;
+  int rc = cached_plan(projs, n_proj, mode, &pl);
   if (rc != LORA_OK) return rec(rc);
-  *bytes = pl.total;
+  *bytes = pl->total;
   return rec(LORA_OK);
 }
 
@@ -1848,9 +1903,9 @@ int stack_step(const lora_proj* projs, int n_proj, int mode, void* workspace, si
   DeviceInfo* d = nullptr;
   int rc = device_info(&d);
   if (rc != LORA_OK) return rec(rc);
-  Plan pl;
-  if ((rc = plan_all(projs, n_proj, mode, &pl)) != LORA_OK) return rec(rc);
-  const size_t need = pl.total;
+  std::shared_ptr<const Plan> pl;
+  if ((rc = cached_plan(projs, n_proj, mode, &pl)) != LORA_OK) return rec(rc);
+  const size_t need = pl->total;
   for (int i = 0; i < n_proj; ++i) {
     if ((mode & LORA_FWD) && (rc = check_fwd_ptrs(projs[i])) != LORA_OK) return rec(rc);
     if ((mode & LORA_BWD) && (rc = check_bwd_ptrs(projs[i])) != LORA_OK) return rec(rc);
@@ -1858,8 +1913,7 @@ int stack_step(const lora_proj* projs, int n_proj, int mode, void* workspace, si
       return rec(LORA_ENULL);  // the backward needs the saved su
   }
   if ((rc = check_ws(workspace, workspace_bytes, need)) != LORA_OK) return rec(rc);
-  pl.dy_cut_device = dy_cut_device;
-  return rec(run_step(projs, n_proj, mode, workspace, pl, d, static_cast<cudaStream_t>(stream)));
+  return rec(run_step(projs, n_proj, mode, workspace, *pl, d, static_cast<cudaStream_t>(stream), dy_cut_device));
 }
 }  // namespace
 
@@ -2260,10 +2314,10 @@ extern "C" int lora_linear_fwd_noalloc(const lora_shape* shape, const lora_bf16*
   p.B = B;
   p.y = y;
   p.su = su;
-  Plan pl;
-  if ((rc = plan_all(&p, 1, LORA_FWD, &pl, false)) != LORA_OK) return rec(rc);
+  std::shared_ptr<const Plan> pl;
+  if ((rc = cached_plan(&p, 1, LORA_FWD, &pl, false)) != LORA_OK) return rec(rc);
   if ((rc = check_fwd_ptrs(p)) != LORA_OK) return rec(rc);  // argument errors first, as lora_stack_step
-  if (pl.total > kNoAllocScratchBytes) return rec(LORA_ESCRATCH);
+  if (pl->total > kNoAllocScratchBytes) return rec(LORA_ESCRATCH);
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return rec(LORA_ECUDA);
   void* scratch = nullptr;
@@ -2278,5 +2332,5 @@ extern "C" int lora_linear_fwd_noalloc(const lora_shape* shape, const lora_bf16*
     scratch = g_noalloc_addr[dev];
   }
   // run_step clears the part of the scratch that must start at zero
-  return rec(run_step(&p, 1, LORA_FWD, scratch, pl, d, static_cast<cudaStream_t>(stream)));
+  return rec(run_step(&p, 1, LORA_FWD, scratch, *pl, d, static_cast<cudaStream_t>(stream)));
 }

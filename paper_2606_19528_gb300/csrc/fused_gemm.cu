@@ -355,7 +355,11 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
           t = it == 0 ? cs_tile : -1;  // one tile, no scheduler
         } else if (c == 0) {
           if (!mbar_wait(smem_u32(&ctl->tile_empty[slot]), par ^ 1u, wc, abort_flag)) break;
-          t = atomicAdd(b.tile_counter, 1);
+          // at most one tile per pair: no counter (and no counter to clear before the launch)
+          if (b.total_tiles <= (int)(gridDim.x >> 1))
+            t = it == 0 ? (int)(blockIdx.x >> 1) : b.total_tiles;
+          else
+            t = atomicAdd(b.tile_counter, 1);
           if (t >= b.total_tiles) t = -1;
           ctl->tile_id[slot] = t;
           st_cluster_u32(mapa_shared(smem_u32(&ctl->tile_id[slot]), pb + 1), (uint32_t)t);

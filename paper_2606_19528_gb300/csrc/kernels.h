@@ -126,7 +126,7 @@ struct GemmBatch {
   GemmProblem prob[kMaxProblems];
   int num_problems;
   int total_tiles;
-  int* tile_counter;   // zero at launch; hands out tiles in list order
+  int* tile_counter;   // zero at launch; hands out tiles in list order (unused with at most one tile per CTA pair)
   int* status;
   long long limit_ns;
   // 1: an earlier kernel of the same call precedes this launch on its stream, so the call's inputs
