@@ -152,16 +152,16 @@ int make_map(CUtensorMap* m, const void* ptr, uint64_t inner, uint64_t outer, ui
 }
 
 // 2-D tensor map of `dtype` elements over a row-major [outer, inner] matrix
-// with row stride `ld` elements, no swizzle or the 128-byte swizzle (staging boxes read by threads).
+// with row stride `ld` elements, no swizzle or the given one (staging boxes read by threads).
 int make_map_plain(CUtensorMap* m, CUtensorMapDataType dtype, int esize, const void* ptr, uint64_t inner,
-                   uint64_t outer, uint64_t ld, uint32_t box_inner, uint32_t box_outer, bool swizzle = false) {
+                   uint64_t outer, uint64_t ld, uint32_t box_inner, uint32_t box_outer,
+                   CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_NONE) {
   cuuint64_t dims[2] = {inner, outer};
   cuuint64_t strides[1] = {ld * (uint64_t)esize};
   cuuint32_t box[2] = {box_inner, box_outer};
   cuuint32_t estr[2] = {1, 1};
   CUresult r = g_encode(m, dtype, 2, const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
-                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? LORA_OK : LORA_ECUDA;
 }
@@ -227,6 +227,7 @@ struct Plan {
   // split contractions: per projection, the split counts of its forward and
   // backward contraction and its fp32 partial buffer (planned from the shapes)
   std::vector<int> split_f, split_b;
+  std::vector<char> small_f, small_b;  // whether they run on the few-rows kernel
   std::vector<size_t> split_off;
   size_t zero_bytes = 0;  // [0, zero_bytes) is cleared at the start of a call that uses tile counters
   bool counters = false;  // a contraction has more tiles than CTA pairs (on kPlanSms SMs): it takes them from a counter
@@ -278,9 +279,12 @@ void gemm_shape(GemmProblem& g, int64_t M, int64_t N, int64_t Kc, int64_t r, int
   g.row_off = g.col_off = g.sym = 0;
 }
 
-// The same for the contraction of one projection, whose tile depends on its weight type.
-void proj_gemm_shape(GemmProblem& g, int64_t M, int64_t N, int64_t Kc, int64_t r, bool q4) {
-  if (q4)
+// The same for the contraction of one projection, whose tile depends on its weight type and on whether it
+// runs on the few-rows kernel.
+void proj_gemm_shape(GemmProblem& g, int64_t M, int64_t N, int64_t Kc, int64_t r, bool q4, bool small) {
+  if (small)
+    gemm_shape(g, M, N, Kc, r, gemm_tile_n_small(), gemm_small_rows());
+  else if (q4)
     gemm_shape(g, M, N, Kc, r, gemm_tile_n_q4(), gemm_tile_m_q4());
   else
     gemm_shape(g, M, N, Kc, r);
@@ -312,8 +316,10 @@ constexpr double kBytesPerBlock = 5.0e6;  // HBM bytes moved in one block time
 
 // A problem's block in those units: a 4-bit problem's 512 x 256 tile holds as many MMAs, half as many when
 // the problem has one 256-row segment only; so does the 256 x 256 tile of fp32 output.
+constexpr double kSmallBlockCost = 1.0;  // 128 x 256 tiles of the few-rows kernel, one CTA: the weight stream
 double block_cost(const GemmProblem& g) {
   const bool q4 = g.m_pad == g.num_m_tiles * gemm_tile_m_q4();
+  if (g.m_pad == g.num_m_tiles * gemm_small_rows()) return kSmallBlockCost;
   return g.out_f32 ? 0.6 : q4 && g.M <= gemm_tile_m() ? 0.8 : 1.0;
 }
 
@@ -917,52 +923,59 @@ Arena arena(void* ws, const Plan& pl, int phase) {
 }
 
 // ------------------------------------------------------------------ forward
-int add_fwd_problem(GemmBatch& b, const lora_proj& p, const Operands& o) {
+int add_fwd_problem(GemmBatch& b, const lora_proj& p, const Operands& o, bool small) {
   const lora_shape& s = p.shape;
   const int i = b.num_problems;
   const int64_t T = s.T, K = s.d_in, N = s.d_out, r = s.rank;
   int rc;
-  // activation boxes: one CTA's 128 rows x 64 contraction elements; weight
-  // boxes: 64 rows x 64 (two per CTA)
-  if ((rc = make_map(&b.tmA[i], p.x, K, T, K, 64, 128)) != LORA_OK) return rc;
+  // activation boxes: one CTA's 128 rows x 64 contraction elements (few rows: the rows there are); weight
+  // boxes: 64 rows x 64 (two per CTA; few rows: the tile's 256 rows)
+  const uint32_t rows = small ? (uint32_t)rup(T, 8) : 128u, wrows = small ? 256u : 64u;
+  if ((rc = make_map(&b.tmA[i], p.x, K, T, K, 64, rows)) != LORA_OK) return rc;
   // rank 0: no adapter slab (kb_total = kb_main), so the slab maps are never read
-  if ((rc = r > 0 ? make_map(&b.tmA2[i], o.s_in, r, T, o.ld_s, 64, 128) : (b.tmA2[i] = b.tmA[i], LORA_OK)) != LORA_OK)
+  if ((rc = r > 0 ? make_map(&b.tmA2[i], o.s_in, r, T, o.ld_s, 64, rows) : (b.tmA2[i] = b.tmA[i], LORA_OK)) != LORA_OK)
     return rc;
   if (is_q4(p)) {
-    // 4-bit W: a box is 128 rows x 256 codes (128 bytes, swizzled); (s, b) boxes are 128 rows x 4 groups
-    if ((rc = make_map_plain(&b.tmQ[i], CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, p.Wq.codes, K / 2, N, K / 2, 128, 128,
-                             true)) != LORA_OK)
+    // 4-bit W: a box is 128 rows x 256 codes (128 bytes, swizzled), with few rows 256 x 128; (s, b) boxes
+    // are as many rows x 4 groups
+    const uint32_t qrows = small ? 256u : 128u;
+    if ((rc = make_map_plain(&b.tmQ[i], CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, p.Wq.codes, K / 2, N, K / 2,
+                             small ? 64 : 128, qrows,
+                             small ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B)) != LORA_OK)
       return rc;
     if ((rc = make_map_plain(&b.tmP[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, p.Wq.params, K / 32, N, K / 32, 8,
-                             128)) != LORA_OK)
+                             qrows)) != LORA_OK)
       return rc;
-  } else if ((rc = make_map(&b.tmB[i], p.W, K, N, K, 64, 64)) != LORA_OK) {
+  } else if ((rc = make_map(&b.tmB[i], p.W, K, N, K, 64, wrows)) != LORA_OK) {
     return rc;
   }
-  if ((rc = r > 0 ? make_map(&b.tmB2[i], o.B, r, N, o.ld_b, 64, 64) : (b.tmB2[i] = b.tmA[i], LORA_OK)) != LORA_OK)
+  if ((rc = r > 0 ? make_map(&b.tmB2[i], o.B, r, N, o.ld_b, 64, wrows) : (b.tmB2[i] = b.tmA[i], LORA_OK)) != LORA_OK)
     return rc;
   if ((rc = make_map(&b.tmOut[i], p.y, N, T, N, 64, 32)) != LORA_OK) return rc;
   GemmProblem& g = b.prob[i];
-  proj_gemm_shape(g, T, N, K, r, is_q4(p));
+  proj_gemm_shape(g, T, N, K, r, is_q4(p), small);
   g.out = mb(p.y);
   add_problem(b);
   return LORA_OK;
 }
 
 // ------------------------------------------------------------------ backward
-int add_bwd_problem(GemmBatch& b, const lora_proj& p, const Operands& o) {
+int add_bwd_problem(GemmBatch& b, const lora_proj& p, const Operands& o, bool small) {
   const lora_shape& s = p.shape;
   const int i = b.num_problems;
   const int64_t T = s.T, K = s.d_in, N = s.d_out, r = s.rank;
   int rc;
-  if ((rc = make_map(&b.tmA[i], p.dy, N, T, N, 64, 128)) != LORA_OK) return rc;
-  if ((rc = r > 0 ? make_map(&b.tmA2[i], o.s_in, r, T, o.ld_s, 64, 128) : (b.tmA2[i] = b.tmA[i], LORA_OK)) != LORA_OK)
+  const uint32_t rows = small ? (uint32_t)rup(T, 8) : 128u;
+  if ((rc = make_map(&b.tmA[i], p.dy, N, T, N, 64, rows)) != LORA_OK) return rc;
+  if ((rc = r > 0 ? make_map(&b.tmA2[i], o.s_in, r, T, o.ld_s, 64, rows) : (b.tmA2[i] = b.tmA[i], LORA_OK)) != LORA_OK)
     return rc;
   // W [N, K] read MN-major: inner dimension K (the GEMM's output columns), rows = contraction
   if (is_q4(p)) {
-    // 4-bit W: a box is 64 rows x 128 codes (64 bytes); (s, b) boxes are 64 rows x 4 groups
-    if ((rc = make_map_plain(&b.tmQ[i], CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, p.Wq.codes, K / 2, N, K / 2, 64, 64)) !=
-        LORA_OK)
+    // 4-bit W: a box is 64 rows x 128 codes (64 bytes), with few rows x 256 (128 bytes, swizzled); (s, b)
+    // boxes are 64 rows x 4 groups
+    if ((rc = make_map_plain(&b.tmQ[i], CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, p.Wq.codes, K / 2, N, K / 2,
+                             small ? 128 : 64, 64,
+                             small ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE)) != LORA_OK)
       return rc;
     if ((rc = make_map_plain(&b.tmP[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, p.Wq.params, K / 32, N, K / 32, 8,
                              64)) != LORA_OK)
@@ -974,7 +987,7 @@ int add_bwd_problem(GemmBatch& b, const lora_proj& p, const Operands& o) {
     return rc;
   if ((rc = make_map(&b.tmOut[i], p.dx, K, T, K, 64, 32)) != LORA_OK) return rc;
   GemmProblem& g = b.prob[i];
-  proj_gemm_shape(g, T, K, N, r, is_q4(p));
+  proj_gemm_shape(g, T, K, N, r, is_q4(p), small);
   g.out = mb(p.dx);
   add_problem(b);
   return LORA_OK;
@@ -1034,6 +1047,25 @@ bool overlap_enabled() {
     return !(e && e[0] == '0' && e[1] == 0);
   }();
   return on;
+}
+
+// Tiles of 256 x 256 when the whole call's contraction in one direction runs as a cluster split on `pairs`
+// CTA pairs (use_cluster_split), 0 when it does not.  4-bit weights keep their own tiles.
+template <typename Q4>
+int call_cluster_tiles(int n, Q4 q4, const lora_proj* projs, bool bwd, int pairs) {
+  if (n > kMaxProblems) return 0;
+  long long wide = 0, narrow = 0;
+  for (int i = 0; i < n; ++i) {
+    if (q4(i)) return 0;
+    const lora_shape& sh = projs[i].shape;
+    const int64_t out = bwd ? sh.d_in : sh.d_out, depth = bwd ? sh.d_out : sh.d_in;
+    const int kb = cdiv(depth, 64) + (sh.rank > 0 ? cdiv(sh.rank, 64) : 0);
+    if (kb < kCsMinBlocks || kb > kCsMaxBlocks) return 0;
+    wide += (long long)cdiv(sh.T, 256) * cdiv(out, gemm_tile_n());
+    narrow += (long long)cdiv(sh.T, 256) * cdiv(out, gemm_tile_n_f32());
+  }
+  if (wide == 0 || wide >= pairs || 2 * narrow > pairs || narrow > gemm_cs_max_clusters(bwd)) return 0;
+  return (int)narrow;
 }
 
 // Widths of the side stream in its two phases.  Beside the forward
@@ -1096,19 +1128,7 @@ SideWidths side_widths(int num_sms, const lora_proj* projs, int n) {
   // A contraction with few output tiles runs as a cluster split, four CTAs per 256 x 256 tile, and leaves
   // the other SMs idle: the side stream takes them (the split still fits beside it).
   auto cs_sms = [&](bool bwd, int side) {
-    long long wide = 0, narrow = 0;
-    for (int i = 0; i < n; ++i) {
-      if (is_q4(projs[i])) return 0;  // 4-bit weights keep the wide tiles
-      const lora_shape& sh = projs[i].shape;
-      const int out = bwd ? sh.d_in : sh.d_out, depth = bwd ? sh.d_out : sh.d_in;
-      const int kb = cdiv(depth, 64) + (sh.rank > 0 ? cdiv(sh.rank, 64) : 0);
-      if (kb < kCsMinBlocks || kb > kCsMaxBlocks) return 0;
-      wide += (long long)cdiv(sh.T, 256) * cdiv(out, gemm_tile_n());
-      narrow += (long long)cdiv(sh.T, 256) * cdiv(out, gemm_tile_n_f32());
-    }
-    const int pairs = (num_sms - side) / 2;
-    if (wide == 0 || wide >= pairs || 2 * narrow > pairs || narrow > gemm_cs_max_clusters(bwd)) return 0;
-    return (int)(4 * narrow);
+    return 4 * call_cluster_tiles(n, [&](int i) { return is_q4(projs[i]); }, projs, bwd, (num_sms - side) / 2);
   };
   if (v1 <= 0) {
     const int used = cs_sms(false, w.w1);
@@ -1339,12 +1359,13 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
     // the backward's rank-r work needs su only: it may start now, beside the forward contractions
     if (ov.on && (rc = ov.fork()) != LORA_OK) return rc;
     if (ov.on && (rc = bwd_rank(ov.side, ov.side_ctas, ov.side, ov.side_ctas2)) != LORA_OK) return rc;
-    // one launch per batch of bf16-weight, then of 4-bit-weight problems;
+    // one launch per batch of bf16-weight, then of 4-bit-weight problems, of many rows, then of few;
     // heavier problems first so that the tile walk ends balanced
-    for (int q4 = 0; q4 < 2; ++q4) {
+    for (int cls = 0; cls < 4; ++cls) {
+      const bool q4 = (cls & 1) != 0, small = cls >= 2;
       std::vector<int> order;
       for (int i = 0; i < n; ++i)
-        if (is_q4(projs[i]) == (q4 != 0)) order.push_back(i);
+        if (is_q4(projs[i]) == q4 && (pl.small_f[i] != 0) == small) order.push_back(i);
       std::stable_sort(order.begin(), order.end(),
                        [&](int a, int b) { return projs[a].shape.d_in > projs[b].shape.d_in; });
       for (size_t i0 = 0; i0 < order.size(); i0 += kMaxProblems) {
@@ -1356,17 +1377,19 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
         int sp[kMaxProblems];
         float* parts[kMaxProblems];
         for (size_t i = i0; i < order.size() && i < i0 + kMaxProblems; ++i) {
-          if ((rc = add_fwd_problem(b, projs[order[i]], ops[order[i]])) != LORA_OK) return rc;
+          if ((rc = add_fwd_problem(b, projs[order[i]], ops[order[i]], small)) != LORA_OK) return rc;
           sp[i - i0] = pl.split_f[order[i]];
           parts[i - i0] = at<float>(ws, pl.split_off[order[i]]);
         }
         ProfScope ps(LORA_KERNEL_GEMM_FWD, st);
-        if (q4 == 0 && use_cluster_split(b, false, gemm_sms / 2)) {
+        if (!q4 && !small && use_cluster_split(b, false, gemm_sms / 2)) {
           if (launch_fused_gemm_cs(b, false, st) != cudaSuccess) return LORA_ECUDA;
           continue;
         }
         if ((rc = apply_splits(b, sp, parts)) != LORA_OK) return rc;
-        if (launch_fused_gemm(b, false, q4 != 0, gemm_sms, st) != cudaSuccess) return LORA_ECUDA;
+        if ((small ? launch_small_gemm(b, false, q4, gemm_sms, st) : launch_fused_gemm(b, false, q4, gemm_sms, st)) !=
+            cudaSuccess)
+          return LORA_ECUDA;
         if (launch_split_reduce(b, st) != cudaSuccess) return LORA_ECUDA;
       }
     }
@@ -1384,10 +1407,11 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
     // the dx contraction reads sv: when the side stream computed it, wait for it
     if (mode == LORA_FWD_BWD && ov.on && (rc = ov.wait_sv()) != LORA_OK) return rc;
     std::vector<Operands>& ops = bops;
-    for (int q4 = 0; q4 < 2; ++q4) {
+    for (int cls = 0; cls < 4; ++cls) {
+      const bool q4 = (cls & 1) != 0, small = cls >= 2;
       std::vector<int> order;
       for (int i = 0; i < n; ++i)
-        if (projs[i].dx && is_q4(projs[i]) == (q4 != 0)) order.push_back(i);
+        if (projs[i].dx && is_q4(projs[i]) == q4 && (pl.small_b[i] != 0) == small) order.push_back(i);
       std::stable_sort(order.begin(), order.end(),
                        [&](int a, int b) { return projs[a].shape.d_out > projs[b].shape.d_out; });
       for (size_t i0 = 0; i0 < order.size(); i0 += kMaxProblems) {
@@ -1399,17 +1423,19 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
         int sp[kMaxProblems];
         float* parts[kMaxProblems];
         for (size_t i = i0; i < order.size() && i < i0 + kMaxProblems; ++i) {
-          if ((rc = add_bwd_problem(b, projs[order[i]], ops[order[i]])) != LORA_OK) return rc;
+          if ((rc = add_bwd_problem(b, projs[order[i]], ops[order[i]], small)) != LORA_OK) return rc;
           sp[i - i0] = pl.split_b[order[i]];
           parts[i - i0] = at<float>(ws, pl.split_off[order[i]]);
         }
         ProfScope ps(LORA_KERNEL_GEMM_BWD, st);
-        if (q4 == 0 && use_cluster_split(b, true, gemm_sms_b / 2)) {
+        if (!q4 && !small && use_cluster_split(b, true, gemm_sms_b / 2)) {
           if (launch_fused_gemm_cs(b, true, st) != cudaSuccess) return LORA_ECUDA;
           continue;
         }
         if ((rc = apply_splits(b, sp, parts)) != LORA_OK) return rc;
-        if (launch_fused_gemm(b, true, q4 != 0, gemm_sms_b, st) != cudaSuccess) return LORA_ECUDA;
+        if ((small ? launch_small_gemm(b, true, q4, gemm_sms_b, st) : launch_fused_gemm(b, true, q4, gemm_sms_b, st)) !=
+            cudaSuccess)
+          return LORA_ECUDA;
         if (launch_split_reduce(b, st) != cudaSuccess) return LORA_ECUDA;
       }
     }
@@ -1449,6 +1475,8 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
   // split contractions: batches as run_step forms them (every projection counted for the backward)
   pl->split_f.assign(n, 1);
   pl->split_b.assign(n, 1);
+  pl->small_f.assign(n, 0);
+  pl->small_b.assign(n, 0);
   // the side stream's SMs are left out of the contractions they run beside: the
   // forward's in a forward-and-backward call, the dx contraction's in any call with a backward
   int pairs_dir[2] = {kPlanPairs, kPlanPairs};
@@ -1473,10 +1501,18 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
   // The splits of direction `dir` on `pairs` pairs with the projections' weights as `kind` says (0 bf16,
   // 1 4-bit, which has tiles of its own): raises split_need, and keeps the counts when `keep` is given.
   auto plan_splits = [&](int dir, const std::vector<char>& kind, int pairs, std::vector<int>* keep) {
-    for (int q4 = 0; q4 < 2; ++q4) {
+    // at most gemm_small_rows() tokens go to the few-rows kernel, but for a call that is cut within clusters
+    // (few bf16 tiles), whose sums the forward without a workspace reproduces
+    const bool cs = call_cluster_tiles(n, [&](int i) { return kind[i] != 0; }, projs, dir == 1, pairs) > 0;
+    auto is_small = [&](int i) { return projs[i].shape.T <= gemm_small_rows() && !cs; };
+    if (keep)
+      for (int i = 0; i < n; ++i) (dir == 0 ? pl->small_f : pl->small_b)[i] = is_small(i) ? 1 : 0;
+    for (int cls = 0; cls < 4; ++cls) {
+      const bool q4 = (cls & 1) != 0, small = cls >= 2;
+      const int workers = small ? 2 * pairs : pairs;
       std::vector<int> order;
       for (int i = 0; i < n; ++i)
-        if (kind[i] == q4) order.push_back(i);
+        if ((kind[i] != 0) == q4 && is_small(i) == small) order.push_back(i);
       std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
         return dir == 0 ? projs[a].shape.d_in > projs[b].shape.d_in : projs[a].shape.d_out > projs[b].shape.d_out;
       });
@@ -1486,13 +1522,13 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
         for (size_t i = i0; i < order.size() && i < i0 + kMaxProblems; ++i) {
           const lora_shape& sh = projs[order[i]].shape;
           if (dir == 0)
-            proj_gemm_shape(b.prob[b.num_problems], sh.T, sh.d_out, sh.d_in, sh.rank, q4 != 0);
+            proj_gemm_shape(b.prob[b.num_problems], sh.T, sh.d_out, sh.d_in, sh.rank, q4, small);
           else
-            proj_gemm_shape(b.prob[b.num_problems], sh.T, sh.d_in, sh.d_out, sh.rank, q4 != 0);
+            proj_gemm_shape(b.prob[b.num_problems], sh.T, sh.d_in, sh.d_out, sh.rank, q4, small);
           add_problem(b);
         }
         int sp[kMaxProblems];
-        choose_splits(b, sp, pairs);
+        choose_splits(b, sp, workers);
         if (!allow_split)
           for (int q = 0; q < b.num_problems; ++q) sp[q] = 1;
         long long units = 0;
@@ -1503,7 +1539,7 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
           split_need[pi] = std::max(split_need[pi], split_floats(b.prob[q], sp[q]));
         }
         // (the backward's launches may leave out projections without dx: never more tiles)
-        if (keep && units > pairs) pl->counters = true;
+        if (keep && units > workers) pl->counters = true;
       }
     }
   };

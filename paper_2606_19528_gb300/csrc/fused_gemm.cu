@@ -178,17 +178,6 @@ __device__ __forceinline__ void decode_tile(const GemmBatch& b, int t, int& p, i
   }
 }
 
-// Two 4-bit codes -> bf16x2 (s * q + b): the codes sit at bits 0..3 and
-// 16..19 of `w`; OR-ing in the exponent of 128 gives exactly 128 + q per half,
-// the first FMA takes 128 off (exact), the second rounds s * q + b once.
-__device__ __forceinline__ uint32_t dq_pair(uint32_t w, uint32_t s2, uint32_t b2) {
-  const uint32_t v = (w & 0x000F000Fu) | 0x43004300u;
-  uint32_t q, r;
-  asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(q) : "r"(v), "r"(0x3F803F80u), "r"(0xC300C300u));
-  asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(q), "r"(s2), "r"(b2));
-  return r;
-}
-
 // Dequantizes this CTA's weight operand of one contraction block from the
 // staged codes and (s, b) pairs into the 128-byte-swizzled bf16 boxes the MMA
 // reads: 128 output columns from n0 + 128 c on, as two boxes of 64.  Forward:

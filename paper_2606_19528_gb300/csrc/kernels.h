@@ -153,6 +153,12 @@ int gemm_cs_max_clusters(bool b_mn_major);
 // out = sum over s of the split partials, in split order, for every problem
 // of the batch with splits > 1 (bf16 or fp32 per out_f32).
 cudaError_t launch_split_reduce(const GemmBatch& batch, cudaStream_t stream);
+// Contractions of at most gemm_small_rows() rows (small_gemm.cu): the batch's tiles are 256 columns wide
+// with one row tile per problem, the activation maps' boxes hold the rows rounded up to 8, and the forward's
+// weight maps' boxes 256 rows (codes: 64 swizzled bytes of 256 rows, backward 128 swizzled bytes of 64 rows).
+cudaError_t launch_small_gemm(const GemmBatch& batch, bool b_mn_major, bool q4, int num_sms, cudaStream_t stream);
+int gemm_small_rows();
+int gemm_tile_n_small();
 int gemm_tile_m();
 int gemm_tile_m_q4();   // tile rows and columns with 4-bit weights
 int gemm_tile_n_q4();

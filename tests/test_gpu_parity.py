@@ -525,3 +525,26 @@ def test_unequal_depths_are_cut():
     G.run_stack(ps)
     for p in ps:
         check_full(p)
+
+
+# at most 128 tokens: one row tile of 128 x 256 tiles, each CTA by itself (8, 128 and in between; columns and
+# depth off the tile, a padded rank, ranks over one and two 64-deep adapter blocks), alone and with a deep
+# problem that is cut into partials
+FEW_ROWS = [(8, 64, 16, 1), (40, 3080, 9992, 12), (120, 200, 264, 128), (128, 11008, 2056, 64)]
+
+
+@pytest.mark.parametrize("T,K,N,r", FEW_ROWS, ids=[f"T{t}_K{k}_N{n}_r{r}" for t, k, n, r in FEW_ROWS])
+def test_few_rows(T, K, N, r):
+    p = G.DevProj(*gen_proj(35, r, T, T, K, N, r, 2.0), 2.0)
+    G.run_single(p)
+    check_full(p)
+
+
+def test_few_rows_layer():
+    """A layer at T = 72 with frozen projections among the adapted ones, forward and backward in one call."""
+    ps = [G.DevProj(*gen_proj(36, i, 0, 72, K, N, 16, 2.0), 2.0)
+          for i, (K, N) in enumerate([(1024, 1024), (1024, 264), (8200, 520), (520, 16392)])]
+    G.run_stack(ps)
+    for p in ps:
+        check_full(p)
+

@@ -70,8 +70,10 @@ def check_q4_full(p: DevQ4Proj):
 
 # around the 512 x 256 tiles (one row segment, both, a second row tile; a column tile of a few columns), and
 # few tiles over a long contraction, whose split ranges start inside a 4-block code slot of the forward
+# (at most 128 tokens: 128 x 256 tiles, one row tile)
 Q4_EDGES = [(8, 256, 8, 1), (264, 512, 264, 8), (512, 256, 136, 16), (520, 768, 520, 16), (776, 1024, 248, 64),
-            (64, 4352, 512, 16), (64, 1024, 4360, 16)]
+            (136, 4352, 512, 16), (64, 4352, 512, 16), (64, 1024, 4360, 16), (128, 768, 8200, 128),
+            (40, 11008, 248, 12)]
 
 
 @pytest.mark.parametrize("T,K,N,r", Q4_EDGES, ids=[f"T{T}_K{K}_N{N}_r{r}" for T, K, N, r in Q4_EDGES])
