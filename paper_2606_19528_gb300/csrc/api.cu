@@ -865,7 +865,7 @@ size_t dy_plan_floats(const std::vector<DySpec>& specs) {
 // The fused passes over dy on `ctas` persistent CTAs (one per SM), then their reduce; the cuts are
 // the cheapest ones for `plan_ctas` CTAs (the cut decides how sv and dB are summed).
 int launch_dy_pass(const std::vector<DySpec>& specs, const Arena& ar, const DeviceInfo* d, int ctas, int plan_ctas,
-                   cudaStream_t st) {
+                   cudaStream_t st, bool early_next) {
   size_t pf = 0;
   int rc;
   for (size_t i0 = 0; i0 < specs.size(); i0 += kMaxRankProblems) {
@@ -873,6 +873,7 @@ int launch_dy_pass(const std::vector<DySpec>& specs, const Arena& ar, const Devi
     const std::vector<DyCut> cuts = dy_choose(specs, i0, i1, plan_ctas);
     DyBatch b;
     memset(&b, 0, sizeof(b));
+    b.early_next = early_next ? 1 : 0;
     for (size_t i = i0; i < i1; ++i) {
       const DySpec& s = specs[i];
       const DyCut& c = cuts[i - i0];
@@ -1217,6 +1218,12 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
   int rc;
   const std::vector<Ws>& plans = pl.ws;
   auto W_ = [&](int i) { return at<uint8_t>(ws, pl.offs[i]); };
+  // every contraction on the few-rows kernel, whose CTAs need no SM pairs
+  bool small_fwd = true, small_bwd = true;
+  for (int i = 0; i < n; ++i) {
+    small_fwd = small_fwd && pl.small_f[i] != 0;
+    small_bwd = small_bwd && pl.small_b[i] != 0;
+  }
   // tile counters of the fused-GEMM launches
   int* counters = at<int>(ws, 0);
   int next_counter = 0;
@@ -1231,21 +1238,22 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
   // dB where the pass over dy is not fused) on the side stream beside the dx
   // contraction
   Overlap ov;
-  if ((mode & LORA_BWD) && (rc = ov.init(d, st, projs, n, pl.side)) != LORA_OK) return rc;
+  // (a backward alone of few rows stays on the caller's stream: its dA takes a few microseconds after the dx
+  // contraction, less than the events of a second stream cost the host)
+  if ((mode & LORA_BWD) && !(mode == LORA_BWD && small_bwd) && (rc = ov.init(d, st, projs, n, pl.side)) != LORA_OK) return rc;
   const int gemm_sms = ov.on ? d->num_sms - ov.side_ctas : d->num_sms;      // forward contraction
   const int gemm_sms_b = ov.on ? d->num_sms - ov.side_ctas2 : d->num_sms;  // dx contraction
   // backward rank-r work: B^T, su^T, sv (and sv^T), then dB and dA; on `rs`
   // with `ctas` persistent CTAs; the operands of the dx contraction go to bops
   std::vector<Operands> bops(n);
-  // ctas: CTAs of the transposes and the passes over dy, on rs; ctas2: of dA (and
-  // the second pass over dy where it is not fused), on rs2 (after rs's first phase)
-  auto bwd_rank = [&](cudaStream_t rs, int ctas, cudaStream_t rs2, int ctas2) -> int {
+  // ctas: CTAs of the transposes and the passes over dy, on rs; rs2: the stream bwd_cols runs on
+  std::vector<bf*> sut(n), svt(n);
+  std::vector<char> fused(n);
+  // early_next: the dx contraction follows on the same stream and may start beside these
+  auto bwd_rank = [&](cudaStream_t rs, int ctas, cudaStream_t rs2, bool early_next) -> int {
     int rc;
     std::vector<RowSpec> rows;
-    std::vector<ColSpec> cols;
     std::vector<DySpec> dys;
-    std::vector<bf*> sut(n), svt(n);
-    std::vector<char> fused(n);
     for (int i = 0; i < n; ++i)
       fused[i] = projs[i].shape.rank > 0 &&
                  dy_fusable((int)projs[i].shape.T, (int)projs[i].shape.d_out, (int)projs[i].shape.rank);
@@ -1293,14 +1301,20 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
     {
       // sv (and dB where fused) before the event the dx contraction waits for
       ProfScope ps(LORA_KERNEL_ROWPROJ, rs);
-      if ((rc = launch_dy_pass(dys, arena(ws, pl, kPhBwdRows), d, ctas, dy_cut_device ? d->num_sms : ctas, rs)) !=
-          LORA_OK)
+      if ((rc = launch_dy_pass(dys, arena(ws, pl, kPhBwdRows), d, ctas, dy_cut_device ? d->num_sms : ctas, rs,
+                               early_next)) != LORA_OK)
         return rc;
-      if ((rc = launch_rows(rows, arena(ws, pl, kPhBwdRows), d, ctas, rs)) != LORA_OK) return rc;
+      if ((rc = launch_rows(rows, arena(ws, pl, kPhBwdRows), d, ctas, rs, early_next)) != LORA_OK) return rc;
     }
     // sv is complete: the dx contraction may start (on the main stream: at once, or after this event)
     if (ov.on && rs != ov.main && cudaEventRecord(ov.ev_sv, rs) != cudaSuccess) return LORA_ECUDA;
     if (ov.on && rs == ov.main && rs2 != rs && (rc = ov.fork()) != LORA_OK) return rc;
+    return LORA_OK;
+  };
+  // dA (and the second pass over dy where it is not fused) on rs2 with ctas2 persistent CTAs, after the above
+  auto bwd_cols = [&](cudaStream_t rs2, int ctas2) -> int {
+    int rc;
+    std::vector<ColSpec> cols;
     for (int i = 0; i < n; ++i) {
       if (fused[i] || projs[i].shape.rank == 0) continue;
       const lora_proj& p = projs[i];
@@ -1353,12 +1367,14 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
       // T = 32: 56.7 -> 53.5 us).  With one it must not: its CTA pairs would take the free SMs first and its
       // last pairs then wait for SM pairs that the side stream's CTAs have split up (Llama layer T = 256:
       // 124 -> 130 us; q projection T = 512: 45.6 -> 47.9 us).
-      if ((rc = launch_rows(rows, arena(ws, pl, kPhFwdRows), d, d->num_sms, st, !ov.on)) != LORA_OK) return rc;
+      if ((rc = launch_rows(rows, arena(ws, pl, kPhFwdRows), d, d->num_sms, st, !ov.on || small_fwd)) != LORA_OK) return rc;
     }
     if (!rows.empty()) prior_main = true;
     // the backward's rank-r work needs su only: it may start now, beside the forward contractions
     if (ov.on && (rc = ov.fork()) != LORA_OK) return rc;
-    if (ov.on && (rc = bwd_rank(ov.side, ov.side_ctas, ov.side, ov.side_ctas2)) != LORA_OK) return rc;
+    if (ov.on && ((rc = bwd_rank(ov.side, ov.side_ctas, ov.side, false)) != LORA_OK ||
+                  (rc = bwd_cols(ov.side, ov.side_ctas2)) != LORA_OK))
+      return rc;
     // one launch per batch of bf16-weight, then of 4-bit-weight problems, of many rows, then of few;
     // heavier problems first so that the tile walk ends balanced
     for (int cls = 0; cls < 4; ++cls) {
@@ -1397,8 +1413,8 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
   if (mode & LORA_BWD) {
     // (a forward-and-backward call without the side stream runs it here too, on every SM)
     if (!(mode == LORA_FWD_BWD && ov.on)) {
-      if ((rc = bwd_rank(st, d->num_sms, ov.on ? ov.side : st, ov.on ? ov.side_ctas2 : d->num_sms)) != LORA_OK)
-        return rc;
+      if ((rc = bwd_rank(st, d->num_sms, ov.on ? ov.side : st, !ov.on && small_bwd)) != LORA_OK) return rc;
+      if (ov.on && (rc = bwd_cols(ov.side, ov.side_ctas2)) != LORA_OK) return rc;
       if (any_adapter(projs, n)) prior_main = true;  // the pass over dy or the row products ran here
     }
     // with no adapter the dx contraction follows the forward's directly: it must not start on its tiles
@@ -1440,6 +1456,7 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
       }
     }
   }
+  if ((mode & LORA_BWD) && !ov.on && (rc = bwd_cols(st, d->num_sms)) != LORA_OK) return rc;
   // the call ends when the side stream's dA and dB are done
   if (ov.on && (rc = ov.join()) != LORA_OK) return rc;
   return LORA_OK;

@@ -276,6 +276,7 @@ struct DyBatch {
   DyProb p[kMaxRankProblems];
   int n, units;
   float* partials;
+  int early_next;      // as in RowBatch
   int red_sv, red_db;  // items of the reduce pass: T x pad8(r) / 8 (pieces > 1), N x ceil(r / 4) (groups > 1)
   int* status;
   long long limit_ns;

@@ -158,6 +158,7 @@ __global__ void __launch_bounds__(kThreads, 1) rank_dy_kernel(const __grid_const
   __syncthreads();
   tc_fence_after();
   griddep_wait();  // dy, B^T and su^T may come from the previous grid
+  if (b.early_next && threadIdx.x == 0) griddep_launch_dependents();
   const uint32_t tmem_base = ctl->tmem_base;
   long long issued = 0;     // producer: stages issued
   bool issued_any = false;  // MMA issuer: any MMA issued
@@ -199,7 +200,7 @@ __global__ void __launch_bounds__(kThreads, 1) rank_dy_kernel(const __grid_const
           }
         }
       }
-      griddep_launch_dependents();  // every load of this CTA is issued
+      if (!b.early_next) griddep_launch_dependents();  // every load of this CTA is issued
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
@@ -376,6 +377,7 @@ __global__ void __launch_bounds__(kThreads, 1) rank_dy_kernel(const __grid_const
 // turn take consecutive tokens, so the sv^T stores coalesce) or 4 of one dB
 // row, and issues the loads of every piece before it sums them.
 __global__ void __launch_bounds__(256) dy_reduce_kernel(const __grid_constant__ DyBatch b) {
+  if (b.early_next) griddep_launch_dependents();
   griddep_wait();
   const long long total = (long long)b.red_sv + b.red_db;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
@@ -440,7 +442,7 @@ __global__ void __launch_bounds__(256) dy_reduce_kernel(const __grid_constant__ 
         if (j + k < P.r) d[k] = o[k];
     }
   }
-  griddep_launch_dependents();
+  if (!b.early_next) griddep_launch_dependents();
 }
 
 template <int R>
