@@ -227,7 +227,8 @@ struct Plan {
   // split contractions: per projection, the split counts of its forward and
   // backward contraction and its fp32 partial buffer (planned from the shapes)
   std::vector<int> split_f, split_b;
-  std::vector<char> small_f, small_b;  // whether they run on the few-rows kernel
+  std::vector<char> small_f, small_b;  // whether they run on the few-rows kernel, and there the CTAs of a
+  std::vector<char> cl_f, cl_b;        // cluster that share a tile (1: none)
   std::vector<size_t> split_off;
   size_t zero_bytes = 0;  // [0, zero_bytes) is cleared at the start of a call that uses tile counters
   bool counters = false;  // a contraction has more tiles than CTA pairs (on kPlanSms SMs): it takes them from a counter
@@ -438,6 +439,29 @@ bool use_cluster_split(GemmBatch& b, bool b_mn, int pairs) {
     b.total_tiles += g.num_m_tiles * g.num_n_tiles;
   }
   return true;
+}
+
+// CTAs of a cluster that share each tile of a few-rows batch (1: none): the most of 8, 4 and 2 whose clusters
+// all run at once on the launch's `workers` CTAs, that leave every CTA two blocks, and whose exchange fits
+// shared memory.  (3080 x 9992 projection, T = 64, forward and backward as two calls: 75.8 us with the pairs'
+// cluster split, four CTAs per 256 x 256 tile, and partials in memory; 49.9 us this way.)
+int small_cluster(const GemmBatch& b, bool b_mn, bool q4, int workers) {
+  long long tiles = 0;
+  int rows = 0, depth = 1 << 30;
+  for (int p = 0; p < b.num_problems; ++p) {
+    const GemmProblem& g = b.prob[p];
+    tiles += g.num_n_tiles;
+    rows = std::max(rows, g.M);
+    depth = std::min(depth, g.kb_total);
+  }
+  for (int s : {8, 4, 2}) {
+    bool full = true;  // every CTA has blocks of every problem
+    for (int p = 0; p < b.num_problems; ++p) full = full && (s - 1) * cdiv(b.prob[p].kb_total, s) < b.prob[p].kb_total;
+    if (full && depth >= std::max(kCsMinBlocks, 2 * s) && rows <= gemm_small_cluster_rows(s) && tiles * s <= workers &&
+        tiles <= gemm_small_max_clusters(b_mn, q4, s))
+      return s;
+  }
+  return 1;
 }
 
 // fp32 partial elements of a problem cut into `sp` splits.
@@ -1051,7 +1075,8 @@ bool overlap_enabled() {
 }
 
 // Tiles of 256 x 256 when the whole call's contraction in one direction runs as a cluster split on `pairs`
-// CTA pairs (use_cluster_split), 0 when it does not.  4-bit weights keep their own tiles.
+// CTA pairs (use_cluster_split), 0 when it does not.  4-bit weights keep their own tiles.  (Calls of more
+// rows than the few-rows kernel takes.)
 template <typename Q4>
 int call_cluster_tiles(int n, Q4 q4, const lora_proj* projs, bool bwd, int pairs) {
   if (n > kMaxProblems) return 0;
@@ -1126,10 +1151,27 @@ SideWidths side_widths(int num_sms, const lora_proj* projs, int n) {
   SideWidths w;
   w.w1 = std::max(2, std::min(num_sms / 4, v1 > 0 ? v1 : width(kSideKappa1, b1)));
   w.w2 = std::max(2, std::min(num_sms / 4, v2 > 0 ? v2 : width(kSideKappa2, b2)));
-  // A contraction with few output tiles runs as a cluster split, four CTAs per 256 x 256 tile, and leaves
-  // the other SMs idle: the side stream takes them (the split still fits beside it).
+  // A contraction with few output tiles runs as a cluster split, four CTAs per 256 x 256 tile (few rows: 2
+  // to 8 per 128 x 256 tile), and leaves the other SMs idle: the side stream takes them (the split still fits
+  // beside it).
   auto cs_sms = [&](bool bwd, int side) {
-    return 4 * call_cluster_tiles(n, [&](int i) { return is_q4(projs[i]); }, projs, bwd, (num_sms - side) / 2);
+    int few = 0, q4 = 0;
+    for (int i = 0; i < n; ++i) {
+      few += projs[i].shape.T <= gemm_small_rows() ? 1 : 0;
+      q4 += is_q4(projs[i]) ? 1 : 0;
+    }
+    if (few == 0) return 4 * call_cluster_tiles(n, [&](int i) { return is_q4(projs[i]); }, projs, bwd, (num_sms - side) / 2);
+    if (few < n || (q4 != 0 && q4 < n) || n > kMaxProblems) return 0;
+    GemmBatch b;
+    memset(&b, 0, sizeof(b));
+    for (int i = 0; i < n; ++i) {
+      const lora_shape& sh = projs[i].shape;
+      proj_gemm_shape(b.prob[b.num_problems], sh.T, bwd ? sh.d_in : sh.d_out, bwd ? sh.d_out : sh.d_in, sh.rank, q4 != 0,
+                      true);
+      add_problem(b);
+    }
+    const int s = small_cluster(b, bwd, q4 != 0, num_sms - side);
+    return s > 1 ? s * b.total_tiles : 0;
   };
   if (v1 <= 0) {
     const int used = cs_sms(false, w.w1);
@@ -1227,7 +1269,8 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
   // tile counters of the fused-GEMM launches
   int* counters = at<int>(ws, 0);
   int next_counter = 0;
-  if ((pl.counters || d->num_sms != kPlanSms) && cudaMemsetAsync(ws, 0, pl.zero_bytes, st) != cudaSuccess)
+  // (more projections than a launch holds: without some dx the backward's launches group them differently)
+  if ((pl.counters || n > kMaxProblems || d->num_sms != kPlanSms) && cudaMemsetAsync(ws, 0, pl.zero_bytes, st) != cudaSuccess)
     return LORA_ECUDA;
   // whether a kernel of this call already ran on the main stream: a contraction launched after one may
   // load its base operands (inputs of the call) before the previous grid ends
@@ -1390,9 +1433,11 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
         b.tile_counter = counters + next_counter++;
         b.early_inputs = prior_main ? 1 : 0;
         prior_main = true;
+        b.cluster = 8;
         int sp[kMaxProblems];
         float* parts[kMaxProblems];
         for (size_t i = i0; i < order.size() && i < i0 + kMaxProblems; ++i) {
+          b.cluster = std::min(b.cluster, (int)pl.cl_f[order[i]]);
           if ((rc = add_fwd_problem(b, projs[order[i]], ops[order[i]], small)) != LORA_OK) return rc;
           sp[i - i0] = pl.split_f[order[i]];
           parts[i - i0] = at<float>(ws, pl.split_off[order[i]]);
@@ -1436,9 +1481,11 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
         b.tile_counter = counters + next_counter++;
         b.early_inputs = prior_main ? 1 : 0;
         prior_main = true;
+        b.cluster = 8;
         int sp[kMaxProblems];
         float* parts[kMaxProblems];
         for (size_t i = i0; i < order.size() && i < i0 + kMaxProblems; ++i) {
+          b.cluster = std::min(b.cluster, (int)pl.cl_b[order[i]]);
           if ((rc = add_bwd_problem(b, projs[order[i]], ops[order[i]], small)) != LORA_OK) return rc;
           sp[i - i0] = pl.split_b[order[i]];
           parts[i - i0] = at<float>(ws, pl.split_off[order[i]]);
@@ -1494,6 +1541,8 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
   pl->split_b.assign(n, 1);
   pl->small_f.assign(n, 0);
   pl->small_b.assign(n, 0);
+  pl->cl_f.assign(n, 1);
+  pl->cl_b.assign(n, 1);
   // the side stream's SMs are left out of the contractions they run beside: the
   // forward's in a forward-and-backward call, the dx contraction's in any call with a backward
   int pairs_dir[2] = {kPlanPairs, kPlanPairs};
@@ -1518,10 +1567,7 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
   // The splits of direction `dir` on `pairs` pairs with the projections' weights as `kind` says (0 bf16,
   // 1 4-bit, which has tiles of its own): raises split_need, and keeps the counts when `keep` is given.
   auto plan_splits = [&](int dir, const std::vector<char>& kind, int pairs, std::vector<int>* keep) {
-    // at most gemm_small_rows() tokens go to the few-rows kernel, but for a call that is cut within clusters
-    // (few bf16 tiles), whose sums the forward without a workspace reproduces
-    const bool cs = call_cluster_tiles(n, [&](int i) { return kind[i] != 0; }, projs, dir == 1, pairs) > 0;
-    auto is_small = [&](int i) { return projs[i].shape.T <= gemm_small_rows() && !cs; };
+    auto is_small = [&](int i) { return projs[i].shape.T <= gemm_small_rows(); };
     if (keep)
       for (int i = 0; i < n; ++i) (dir == 0 ? pl->small_f : pl->small_b)[i] = is_small(i) ? 1 : 0;
     for (int cls = 0; cls < 4; ++cls) {
@@ -1545,14 +1591,20 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
           add_problem(b);
         }
         int sp[kMaxProblems];
+        const int cl = small ? small_cluster(b, dir == 1, q4, workers) : 1;
         choose_splits(b, sp, workers);
+        if (cl > 1)
+          for (int q = 0; q < b.num_problems; ++q) sp[q] = 1;
         if (!allow_split)
           for (int q = 0; q < b.num_problems; ++q) sp[q] = 1;
         long long units = 0;
         for (int q = 0; q < b.num_problems; ++q) {
           const int pi = order[i0 + q];
           units += (long long)b.prob[q].num_m_tiles * b.prob[q].num_n_tiles * sp[q];
-          if (keep) (*keep)[pi] = sp[q];
+          if (keep) {
+            (*keep)[pi] = sp[q];
+            (dir == 0 ? pl->cl_f : pl->cl_b)[pi] = (char)cl;
+          }
           split_need[pi] = std::max(split_need[pi], split_floats(b.prob[q], sp[q]));
         }
         // (the backward's launches may leave out projections without dx: never more tiles)

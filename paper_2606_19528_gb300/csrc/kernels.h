@@ -133,6 +133,7 @@ struct GemmBatch {
   // (the base contraction's operands) were complete before this grid started and its main blocks may
   // be loaded before the previous grid ends; only the adapter slab's activations (su or sv) wait
   int early_inputs;
+  int cluster;  // few-rows kernel: > 1, clusters of that many CTAs share a tile (one tile per cluster, unsplit)
 };
 
 // b_mn_major: the weight operand is contracted over its rows (backward);
@@ -158,6 +159,10 @@ cudaError_t launch_split_reduce(const GemmBatch& batch, cudaStream_t stream);
 // weight maps' boxes 256 rows (codes: 64 swizzled bytes of 256 rows, backward 128 swizzled bytes of 64 rows).
 cudaError_t launch_small_gemm(const GemmBatch& batch, bool b_mn_major, bool q4, int num_sms, cudaStream_t stream);
 int gemm_small_rows();
+// Clusters of `size` (2, 4, 8) CTAs of it that run at once on this device (0 if the query fails), and the
+// rows up to which that size may be used.
+int gemm_small_max_clusters(bool b_mn_major, bool q4, int size);
+int gemm_small_cluster_rows(int size);
 int gemm_tile_n_small();
 int gemm_tile_m();
 int gemm_tile_m_q4();   // tile rows and columns with 4-bit weights

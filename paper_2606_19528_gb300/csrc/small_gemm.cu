@@ -25,6 +25,14 @@
 //   4-bit:      warps 6..13 dequantize, two groups of four taking alternate
 //               blocks; warp 14 streams codes and (s, b) pairs by TMA
 // Every wait is bounded.
+//
+// Cluster form (kCl), for launches whose tiles leave most CTAs idle (one
+// projection): a cluster of S = 2, 4 or 8 CTAs shares a tile, CTA j contracting
+// the j-th part of its blocks.  Then every CTA's ring is idle and the parts are
+// summed through distributed shared memory: CTA j owns 256 / S of the tile's
+// columns, gets the other CTAs' fp32 values for them by bulk copies, adds them
+// in CTA order, rounds once and stores.  No partials in memory, no reduce
+// launch, and a forward without a workspace gives the same bits.
 #include "common.cuh"
 #include "kernels.h"
 
@@ -83,6 +91,7 @@ struct __align__(8) Ctl {
   uint64_t tfull[2], tempty[2];    // accumulator complete / drained
   uint64_t tile_full[kTileRing], tile_empty[kTileRing];
   uint64_t drain;
+  uint64_t xchg;                   // kCl: the other CTAs' values of this CTA's columns arrived
   int tile_id[kTileRing];
   uint32_t tmem_base;
   int abort;
@@ -162,7 +171,7 @@ __device__ __forceinline__ void dequant_block(uint32_t slot, uint32_t wdst, int 
   }
 }
 
-template <bool kBMn, bool kQ>
+template <bool kBMn, bool kQ, bool kCl>
 __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) small_lora_gemm(const __grid_constant__ GemmBatch b) {
   using C = Cfg<kQ>;
   using QS = QSlot<kBMn>;
@@ -198,6 +207,7 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) small_lora_gemm(const __
       mbar_init(smem_u32(&ctl->tile_empty[k]), 1 + kEpi + (kQ ? kConvWarps + 1 : 0));
     }
     mbar_init(smem_u32(&ctl->drain), 1);
+    mbar_init(smem_u32(&ctl->xchg), 1);
     ctl->abort = 0;
     ctl->fills = 0;
     ctl->qfills = 0;
@@ -219,6 +229,18 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) small_lora_gemm(const __
   // with early inputs only the producers of the adapter slab wait for the previous grid, and every CTA before it ends
   if (!b.early_inputs) griddep_wait();
   const uint32_t tmem_base = ctl->tmem_base;
+  // kCl: cluster size, this CTA's part of the tile's blocks
+  const int S = kCl ? b.cluster : 1;
+  const int crank = kCl ? (int)cluster_ctarank() : 0;
+  auto tile_of = [&](int t) {
+    Tile w = decode(b, t);
+    if (kCl) {
+      const int kt = b.prob[w.p].kb_total, L = (kt + S - 1) / S;
+      w.kb0 = crank * L;
+      w.kb1 = min(kt, w.kb0 + L);
+    }
+    return w;
+  };
 
   // tile of the consumers' iteration `it`, or -1 (all tiles done, or a wait gave up); whole warps call it
   auto next_tile = [&](int it) {
@@ -254,7 +276,9 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) small_lora_gemm(const __
         const int slot = it % kTileRing;
         if (!mbar_wait(smem_u32(&ctl->tile_empty[slot]), (uint32_t)(((it / kTileRing) & 1) ^ 1), wc, abort_flag)) break;
         int t;
-        if (b.total_tiles <= (int)gridDim.x)  // at most one tile per CTA: no counter
+        if (kCl)
+          t = it == 0 ? (int)blockIdx.x / S : b.total_tiles;
+        else if (b.total_tiles <= (int)gridDim.x)  // at most one tile per CTA: no counter
           t = it == 0 ? (int)blockIdx.x : b.total_tiles;
         else
           t = atomicAdd(b.tile_counter, 1);
@@ -265,7 +289,7 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) small_lora_gemm(const __
           griddep_launch_dependents();
           break;
         }
-        const Tile w = decode(b, t);
+        const Tile w = tile_of(t);
         const GemmProblem& Q = b.prob[w.p];
         const uint32_t a_bytes = (uint32_t)((Q.M + 7) & ~7) * 128u;  // the map's box rows
         const uint32_t tx = a_bytes + (kQ ? 0u : w_bytes(w.n0, Q.N));
@@ -304,7 +328,7 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) small_lora_gemm(const __
     for (int it = 0; ok; ++it) {
       const int t = next_tile(it);
       if (t < 0) break;
-      const Tile w = decode(b, t);
+      const Tile w = tile_of(t);
       const GemmProblem& Q = b.prob[w.p];
       const int buf = it & 1;
       ok = mbar_wait(smem_u32(&ctl->tempty[buf]), (uint32_t)(((it >> 1) & 1) ^ 1), wc, abort_flag);
@@ -355,13 +379,14 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) small_lora_gemm(const __
     for (int it = 0;; ++it) {
       const int t = next_tile(it);
       if (t < 0) break;
-      const Tile w = decode(b, t);
+      const Tile w = tile_of(t);
       const GemmProblem& Q = b.prob[w.p];
       const int buf = it & 1;
       bool ok = mbar_wait(smem_u32(&ctl->tfull[buf]), (uint32_t)((it >> 1) & 1), wc, abort_flag);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
+      if (kCl) continue;                 // the exchange follows below, after every role
       const bool f32 = Q.splits > 1;  // the fp32 partial of one split: 32-column blocks
       const int block_cols = f32 ? 32 : 64;
       const int row_st = (f32 ? w.ks * Q.m_pad : 0) + row0;
@@ -415,7 +440,7 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) small_lora_gemm(const __
     for (int it = 0; ok; ++it) {
       const int t = next_tile(it);
       if (t < 0) break;
-      const Tile w = decode(b, t);
+      const Tile w = tile_of(t);
       const GemmProblem& Q = b.prob[w.p];
       const int kq1 = min(w.kb1, Q.kb_main);  // end of the blocks taken from codes
       for (int kb = w.kb0; kb < w.kb1; ++kb, ++wseq) {
@@ -469,7 +494,7 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) small_lora_gemm(const __
     for (int it = 0; ok; ++it) {
       const int t = next_tile(it);
       if (t < 0) break;
-      const Tile w = decode(b, t);
+      const Tile w = tile_of(t);
       const GemmProblem& Q = b.prob[w.p];
       for (int kb = w.kb0; kb < min(w.kb1, Q.kb_main); kb = (kb / QS::kBlocks + 1) * QS::kBlocks) {
         ok = mbar_wait(smem_u32(&ctl->qempty[qs]), qpar ^ 1u, wc, abort_flag);
@@ -495,6 +520,95 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) small_lora_gemm(const __
       }
     }
     if (lane == 0) ctl->qfills = qfills;
+  }
+
+  if constexpr (kCl) {
+    // ------------------------------------------------------------ sum of the parts
+    // Send and receive areas lie in the idle ring, each (S - 1) / S of rows x 1 KB (the host keeps both
+    // within it): one region per peer of `rows` rows x 1024 / S bytes, 16-byte chunk u of row r at
+    // u ^ (r mod 8).
+    tc_fence_before();
+    cluster_sync_all();
+    tc_fence_after();
+    if (warp >= 2 && warp < 2 + kEpi && !*abort_flag) {
+      const Tile w = tile_of((int)blockIdx.x / S);
+      const GemmProblem& Q = b.prob[w.p];
+      const int q = warp & 3, part = (warp - 2) >> 2;
+      const int row0 = q * 32, row = row0 + lane;
+      const int groups = (Q.M + 31) / 32;                // 32-row groups holding rows
+      const uint32_t cols = (uint32_t)(kN / S), row_b = cols * 4u, region = (uint32_t)groups * 32u * row_b;
+      const uint32_t recv = base, send = base + (uint32_t)(S - 1) * region;
+      auto slot = [&](int owner, int from) { return (uint32_t)(from < owner ? from : from - 1) * region; };
+      auto chunk = [&](uint32_t u) { return (uint32_t)row * row_b + (((u ^ (uint32_t)row) & 7u) | (u & ~7u)) * 16u; };
+      const uint32_t tl = tmem_base + ((uint32_t)row0 << 16);
+      if (row0 < Q.M) {  // uniform across the warp
+        // the slices of this warp's columns that other CTAs own
+        for (int k = 0; k < S; ++k) {
+          const int c0 = k * (int)cols;
+          if (k == crank || c0 >= (part + 1) * C::kPartCols || c0 + (int)cols <= part * C::kPartCols) continue;
+          const uint32_t dst = send + slot(crank, k);
+          for (uint32_t cc = 0; cc < cols; cc += 32) {
+            uint32_t v[32];
+            tmem_ld_32x32b_x32(tl + (uint32_t)c0 + cc, v);
+            tmem_ld_wait();
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + chunk(cc / 4 + (uint32_t)u)),
+                           "r"(v[4 * u]), "r"(v[4 * u + 1]), "r"(v[4 * u + 2]), "r"(v[4 * u + 3])
+                           : "memory");
+          }
+          fence_proxy_async_smem();  // the bulk copy reads what these threads wrote
+          __syncwarp();
+          if (lane == 0) {
+            const uint32_t off = (uint32_t)row0 * row_b;
+            bulk_copy_to_peer(mapa_shared(recv + slot(k, crank) + off, (uint32_t)k), dst + off, 32u * row_b,
+                              mapa_shared(smem_u32(&ctl->xchg), (uint32_t)k));
+          }
+        }
+        // this CTA's own columns
+        const int c0 = crank * (int)cols;
+        if (c0 < (part + 1) * C::kPartCols && c0 + (int)cols > part * C::kPartCols) {
+          if (q == 0 && lane == 0) mbar_arrive_expect_tx(smem_u32(&ctl->xchg), (uint32_t)(S - 1) * region);
+          bool got = mbar_wait(smem_u32(&ctl->xchg), 0u, wc, abort_flag);
+          got = __all_sync(0xffffffffu, got);
+          __nv_bfloat16* out = static_cast<__nv_bfloat16*>(Q.out) + (size_t)row * Q.ldo + w.n0 + c0;
+          for (uint32_t cc = 0; got && cc < cols; cc += 32) {
+            uint32_t v[32];
+            tmem_ld_32x32b_x32(tl + (uint32_t)c0 + cc, v);
+            tmem_ld_wait();
+            float a[32];
+#pragma unroll
+            for (int e = 0; e < 32; ++e) a[e] = 0.f;
+            for (int s = 0; s < S; ++s) {  // in CTA order
+              if (s == crank) {
+#pragma unroll
+                for (int e = 0; e < 32; ++e) a[e] += __uint_as_float(v[e]);
+              } else {
+                const uint32_t src = recv + slot(crank, s);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                  float o[4];
+                  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                               : "=f"(o[0]), "=f"(o[1]), "=f"(o[2]), "=f"(o[3])
+                               : "r"(src + chunk(cc / 4 + (uint32_t)u))
+                               : "memory");
+#pragma unroll
+                  for (int e = 0; e < 4; ++e) a[4 * u + e] += o[e];
+                }
+              }
+            }
+            if (row < Q.M) {
+#pragma unroll
+              for (int u = 0; u < 4; ++u)  // N is a multiple of 8: whole 16-byte pieces
+                if (w.n0 + c0 + (int)cc + 8 * u < Q.N)
+                  *reinterpret_cast<uint4*>(out + cc + 8 * u) =
+                      make_uint4(pack_bf16x2(a[8 * u], a[8 * u + 1]), pack_bf16x2(a[8 * u + 2], a[8 * u + 3]),
+                                 pack_bf16x2(a[8 * u + 4], a[8 * u + 5]), pack_bf16x2(a[8 * u + 6], a[8 * u + 7]));
+            }
+          }
+        }
+      }
+    }
   }
 
   // ------------------------------------------------------------ teardown
@@ -523,6 +637,7 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) small_lora_gemm(const __
     if (b.early_inputs) griddep_wait();
   }
   __syncthreads();
+  if (kCl) cluster_sync_all();  // no copy into or out of a peer is pending
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, kTmemCols);
@@ -532,13 +647,67 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) small_lora_gemm(const __
 template <bool kBMn, bool kQ>
 cudaError_t launch_variant(const GemmBatch& batch, int ctas, cudaStream_t stream) {
   constexpr size_t smem = smem_bytes<kQ>();
+  if (batch.cluster > 1) {
+    static std::atomic<unsigned long long> cl_done{0};
+    const cudaError_t e = set_smem_once(small_lora_gemm<kBMn, kQ, true>, (int)smem, cl_done);
+    if (e != cudaSuccess) return e;
+    return launch_kernel(small_lora_gemm<kBMn, kQ, true>, dim3((unsigned)(batch.total_tiles * batch.cluster)),
+                         dim3(Cfg<kQ>::kThreads), smem, stream, batch.cluster, batch);
+  }
   static std::atomic<unsigned long long> attr_done{0};
-  const cudaError_t e = set_smem_once(small_lora_gemm<kBMn, kQ>, (int)smem, attr_done);
+  const cudaError_t e = set_smem_once(small_lora_gemm<kBMn, kQ, false>, (int)smem, attr_done);
   if (e != cudaSuccess) return e;
-  return launch_kernel(small_lora_gemm<kBMn, kQ>, dim3((unsigned)ctas), dim3(Cfg<kQ>::kThreads), smem, stream, 1, batch);
+  return launch_kernel(small_lora_gemm<kBMn, kQ, false>, dim3((unsigned)ctas), dim3(Cfg<kQ>::kThreads), smem, stream, 1,
+                       batch);
+}
+
+template <bool kBMn, bool kQ>
+int query_clusters(int size) {
+  constexpr size_t smem = smem_bytes<kQ>();
+  static std::atomic<unsigned long long> attr_done{0};
+  if (set_smem_once(small_lora_gemm<kBMn, kQ, true>, (int)smem, attr_done) != cudaSuccess) return 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(size * 128));
+  cfg.blockDim = dim3(Cfg<kQ>::kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)size;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int k = 0;
+  if (cudaOccupancyMaxActiveClusters(&k, small_lora_gemm<kBMn, kQ, true>, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return k;
 }
 
 }  // namespace
+
+int gemm_small_max_clusters(bool b_mn_major, bool q4, int size) {
+  // per device, form and cluster size 2, 4, 8; 0: not asked yet, -1: none
+  static std::atomic<int> cache[64][4][3];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  std::atomic<int>& c = cache[dev][(b_mn_major ? 2 : 0) + (q4 ? 1 : 0)][size == 8 ? 2 : size == 4 ? 1 : 0];
+  int v = c.load(std::memory_order_acquire);
+  if (v == 0) {
+    v = b_mn_major ? (q4 ? query_clusters<true, true>(size) : query_clusters<true, false>(size))
+                   : (q4 ? query_clusters<false, true>(size) : query_clusters<false, false>(size));
+    if (v <= 0) v = -1;
+    c.store(v, std::memory_order_release);
+  }
+  return v > 0 ? v : 0;
+}
+
+// Rows whose send and receive areas, (size - 1) / size of 2 KB each, fit the ring.
+int gemm_small_cluster_rows(int size) {
+  const int rows = (int)(Cfg<false>::kRing / (2u * 1024u * (unsigned)(size - 1) / (unsigned)size));
+  return rows / 32 * 32 < kM ? rows / 32 * 32 : kM;
+}
 
 cudaError_t launch_small_gemm(const GemmBatch& batch, bool b_mn_major, bool q4, int num_sms, cudaStream_t stream) {
   if (batch.total_tiles <= 0) return cudaSuccess;

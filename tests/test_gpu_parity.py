@@ -530,14 +530,22 @@ def test_unequal_depths_are_cut():
 # at most 128 tokens: one row tile of 128 x 256 tiles, each CTA by itself (8, 128 and in between; columns and
 # depth off the tile, a padded rank, ranks over one and two 64-deep adapter blocks), alone and with a deep
 # problem that is cut into partials
-FEW_ROWS = [(8, 64, 16, 1), (40, 3080, 9992, 12), (120, 200, 264, 128), (128, 11008, 2056, 64)]
+# (few tiles: clusters of 8, 4 and 2 CTAs share a tile; 96 and 104 rows are the last with 8 and the first with 4)
+FEW_ROWS = [(8, 64, 16, 1), (40, 3080, 9992, 12), (120, 200, 264, 128), (128, 11008, 2056, 64), (96, 4104, 520, 8),
+            (104, 4104, 520, 8), (32, 3072, 3072, 16), (72, 1032, 16392, 0)]
 
 
 @pytest.mark.parametrize("T,K,N,r", FEW_ROWS, ids=[f"T{t}_K{k}_N{n}_r{r}" for t, k, n, r in FEW_ROWS])
 def test_few_rows(T, K, N, r):
+    if r == 0:
+        test_few_tile_contractions(T, K, N, r)
+        return
     p = G.DevProj(*gen_proj(35, r, T, T, K, N, r, 2.0), 2.0)
     G.run_single(p)
     check_full(p)
+    y, dx = p.y.clone(), p.dx.clone()
+    G.run_single(p)  # the parts are added in CTA order: the same bits again
+    assert torch.equal(p.y, y) and torch.equal(p.dx, dx)
 
 
 def test_few_rows_layer():
