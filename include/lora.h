@@ -265,7 +265,7 @@ int lora_ce_fwd_bwd(const lora_ce_args* args, void* workspace, size_t workspace_
  * matrix is never formed.  Below V = 32768 similarities are computed 512 rows
  * at a time in fp32 on the tensor cores and each row's top k is selected from
  * them.  From V = 32768 on, each row first gets a threshold from its
- * similarities to 8192 evenly spread tokens, the similarity contraction keeps
+ * similarities to up to 8192 evenly spread tokens, the similarity contraction keeps
  * only the values at or above it (at most 4096 per row, in workspace), and
  * those are sorted; rows left with fewer than k or more than 4096 such values
  * are redone exactly on the 512-row path, which needs one synchronization of

@@ -354,8 +354,9 @@ cudaError_t launch_scatter_rows(const __nv_bfloat16* src, const int32_t* tpos, i
                                 cudaStream_t stream);
 
 // ---------------------------------------------------------------- top-k similarity table
-// En[i] = bf16(E[i] / ||E[i]||), the norm's sum of squares in fp32 in index order.
-cudaError_t launch_normalize_rows(const __nv_bfloat16* E, int V, int d, __nv_bfloat16* En, cudaStream_t stream);
+// En[i] = bf16(E[i] / norm[i]), norm[i] = ||E[i]|| with the sum of squares in fp32 in index order.
+cudaError_t launch_normalize_rows(const __nv_bfloat16* E, int V, int d, float* norm, __nv_bfloat16* En,
+                                  cudaStream_t stream);
 // Rows row0 .. row0 + nrows - 1 of the table from their similarities S [nrows, lds] fp32:
 // the k largest per row, descending, lower index first on ties; *status =
 // kStatusTopkTies when a row has too many candidates tied at its k-th value.
@@ -363,17 +364,18 @@ cudaError_t launch_normalize_rows(const __nv_bfloat16* E, int V, int d, __nv_bfl
 // row rows[r], or row0 + r when rows is null).
 cudaError_t launch_topk_select(const float* S, long long lds, int V, int k, int row0, const int32_t* rows, int nrows,
                                int32_t* table, int* status, cudaStream_t stream);
-// Thresholds of nrows rows from their sample similarities Z [nrows, topk_sample()].
-cudaError_t launch_topk_tau(const float* Z, int V, int k, int nrows, float* tau, cudaStream_t stream);
+// Thresholds of nrows rows from their sample similarities Z [nrows, ns].
+cudaError_t launch_topk_tau(const float* Z, int V, int k, int ns, int nrows, float* tau, cudaStream_t stream);
 // Sorts each row's appended candidates into the table (a warp per row, a block for
 // lists over 1024: big_rows / big_count, a zeroed count), or lists the row for the fallback.
 cudaError_t launch_topk_sort(const uint2* cand, int* cnt, int cap, int k, int row0, int nrows, int32_t* table,
                              int32_t* big_rows, int* big_count, int32_t* fail_rows, int* fail_count, int num_sms,
                              cudaStream_t stream);
-// Es [topk_sample(), d] = the evenly spread sample rows of En [V, d].
-cudaError_t launch_topk_gather_sample(const __nv_bfloat16* En, int V, int d, __nv_bfloat16* Es, int num_sms,
+// Es [ns, d] = the evenly spread sample rows of En [V, d].
+cudaError_t launch_topk_gather_sample(const __nv_bfloat16* En, int V, int d, int ns, __nv_bfloat16* Es, int num_sms,
                                       cudaStream_t stream);
-int topk_sample();        // sample tokens per row
+int topk_sample();        // most sample tokens per row (sizes the workspace)
+int topk_sample_for(int V, int k);  // sample tokens per row of a table, a multiple of 512
 int topk_sample_min_v();  // shortest rows that take the sampled selection
 int topk_cap();           // candidate slots per row
 int topk_max_k();

@@ -3,7 +3,7 @@
 // normalised, C = E~ E~^T holds the cosine similarities, and row i of the
 // table lists the k most similar tokens in descending order (lower index
 // first on ties).  The V x V matrix is never formed.
-//   normalize_rows      E~_i = bf16(E_i / ||E_i||), the sum of squares
+//   row_norms,          E~_i = bf16(E_i / ||E_i||), the sum of squares
 //                       accumulated in fp32 in index order (squares of bf16
 //                       are exact), correctly rounded sqrt and division
 // Rows shorter than 32768 tokens (the host runs 512-row chunks):
@@ -15,7 +15,7 @@
 //                       sort on (similarity descending, index ascending); it
 //                       also serves the longer rows' fallback
 // Rows of at least 32768 tokens:
-//   topk_gather_sample  8192 evenly spread tokens
+//   topk_gather_sample  up to 8192 evenly spread tokens
 //   topk_tau            each row's threshold from its similarities to them
 //   (fused_gemm.cu)     the upper triangle of C, each value appended to the
 //                       candidate lists of both its rows when it reaches
@@ -34,41 +34,115 @@ namespace {
 constexpr int kSelThreads = 1024;
 constexpr int kCap = 4096;  // candidates held in shared memory
 
-__global__ void normalize_rows_kernel(const __nv_bfloat16* __restrict__ E, int V, int d,
-                                      __nv_bfloat16* __restrict__ En) {
-  griddep_wait();
-  griddep_launch_dependents();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= V) return;
-  const uint4* row = reinterpret_cast<const uint4*>(E + (long long)i * d);
-  const int nv = d / 8;
-  float s = 0.f;
-  for (int v = 0; v < nv; ++v) {
-    const uint4 q = __ldg(row + v);
-    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float lo = __uint_as_float(w[e] << 16), hi = __uint_as_float(w[e] & 0xFFFF0000u);
-      s = __fadd_rn(s, __fmul_rn(lo, lo));  // each square is exact; index order
-      s = __fadd_rn(s, __fmul_rn(hi, hi));
-    }
-  }
-  const float n = __fsqrt_rn(s);
-  uint4* out = reinterpret_cast<uint4*>(En + (long long)i * d);
-  for (int v = 0; v < nv; ++v) {
-    const uint4 q = __ldg(row + v);
-    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-    uint32_t o[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float lo = __uint_as_float(w[e] << 16), hi = __uint_as_float(w[e] & 0xFFFF0000u);
-      const float a = n > 0.f ? __fdiv_rn(lo, n) : 0.f, b = n > 0.f ? __fdiv_rn(hi, n) : 0.f;
-      o[e] = pack_bf16x2(a, b);
-    }
-    out[v] = make_uint4(o[0], o[1], o[2], o[3]);
-  }
+// Row norms, one warp per 32 rows.  The sum of squares is a chain in index
+// order, so a row belongs to one lane; the warp stages 64 columns of its 32 rows
+// at a time through shared memory with coalesced 16-byte copies (cp.async,
+// kNormStages chunks in flight) and each lane adds its own row's.  Then one
+// element-wise pass divides (scale_rows).  HBM-bound: E twice in, E~ once out (735
+// MB at V = 40000, d = 3072).  Measured there: one thread per row, reading its row
+// straight from memory and dividing it, 355 us; these two 46 + 99 us.
+
+// bf16(x / n) with the division correctly rounded to fp32 first, as
+// __float2bfloat16_rn(__fdiv_rn(x, n)).  x * (1 / n), both rounded, is within 2
+// units in the last place of x / n and the rounded quotient within half of
+// one, so both round to the same bf16 unless the product's low 16 bits are within
+// 3 of the midpoint 0x8000: those elements (1 in 9000) are divided.  `fast` is false
+// for a divisor whose reciprocal or quotients could leave the normal range;
+// quotients below 2^-100 are divided as well.
+__device__ __forceinline__ float divide_bf16(float x, float n, float rn, bool fast) {
+  const float q = x * rn;
+  const uint32_t u = __float_as_uint(q), lo = (u & 0xFFFFu) - (0x8000u - 4u);
+  if (fast && lo > 8u && (fabsf(q) >= 0x1p-100f || x == 0.f)) return q;
+  return __fdiv_rn(x, n);
 }
 
+constexpr int kNormWarps = 2, kNormStages = 4;
+constexpr int kNormPitch = 144;  // bytes of a staged row: 128 + 16, so that lanes reading 16 bytes of 32 rows spread
+
+__global__ void __launch_bounds__(kNormWarps * 32) row_norms_kernel(const __nv_bfloat16* __restrict__ E, int V, int d,
+                                                                   float* __restrict__ norm) {
+  griddep_wait();
+  griddep_launch_dependents();
+  __shared__ __align__(16) uint8_t stage[kNormWarps][kNormStages][32 * kNormPitch];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int i0 = (blockIdx.x * kNormWarps + warp) * 32;
+  if (i0 >= V) return;  // whole warps
+  const int rows = min(32, V - i0);
+  const int nv = d / 8, chunks = (nv + 7) / 8;  // 16-byte vectors of a row, 8 per chunk
+  const uint4* src = reinterpret_cast<const uint4*>(E) + (long long)i0 * nv;
+  const int cr = lane >> 3, cv = lane & 7;  // this lane's row (of four) and vector in a copy step
+  auto fetch = [&](int c) {
+    if (c < chunks && c * 8 + cv < nv) {
+      const uint32_t dst = smem_u32(stage[warp][c % kNormStages]) + (uint32_t)cv * 16u;
+#pragma unroll
+      for (int r = 0; r < 32; r += 4)
+        if (r + cr < rows)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (uint32_t)((r + cr) * kNormPitch)),
+                       "l"(src + (long long)(r + cr) * nv + c * 8 + cv)
+                       : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll
+  for (int c = 0; c < kNormStages - 1; ++c) fetch(c);
+  float s = 0.f;
+  for (int c = 0; c < chunks; ++c) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kNormStages - 2) : "memory");
+    __syncwarp();  // every lane's copies of chunk c have landed, and chunk c - 1 is read
+    fetch(c + kNormStages - 1);
+    const uint4* row = reinterpret_cast<const uint4*>(stage[warp][c % kNormStages] + lane * kNormPitch);
+    const int n = min(8, nv - c * 8);
+    if (lane < rows)
+      for (int v = 0; v < n; ++v) {
+        const uint4 q = row[v];
+        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float lo = __uint_as_float(w[e] << 16), hi = __uint_as_float(w[e] & 0xFFFF0000u);
+          s = __fadd_rn(s, __fmul_rn(lo, lo));  // each square is exact; index order
+          s = __fadd_rn(s, __fmul_rn(hi, hi));
+        }
+      }
+  }
+  if (lane < rows) norm[i0 + lane] = __fsqrt_rn(s);
+}
+
+// En[i] = bf16(E[i] / norm[i]) (zero rows stay zero): eight 16-byte vectors per thread, all loads first.
+__global__ void __launch_bounds__(256) scale_rows_kernel(const __nv_bfloat16* __restrict__ E, int V, int d,
+                                                         const float* __restrict__ norm,
+                                                         __nv_bfloat16* __restrict__ En) {
+  griddep_wait();
+  griddep_launch_dependents();
+  constexpr int kU = 8;
+  const int nv = d / 8;
+  const long long total = (long long)V * nv, e0 = (long long)blockIdx.x * (256 * kU) + threadIdx.x;
+  const uint4* src = reinterpret_cast<const uint4*>(E);
+  uint4* dst = reinterpret_cast<uint4*>(En);
+  uint4 q[kU];
+  float nr[kU];
+#pragma unroll
+  for (int u = 0; u < kU; ++u) {
+    const long long e = e0 + 256 * u;
+    q[u] = e < total ? __ldg(src + e) : make_uint4(0u, 0u, 0u, 0u);
+    nr[u] = e < total ? __ldg(norm + e / nv) : 1.f;
+  }
+#pragma unroll
+  for (int u = 0; u < kU; ++u) {
+    const long long e = e0 + 256 * u;
+    const float n = nr[u];
+    const bool fast = n > 0x1p-60f && n < 0x1p60f;
+    const float rn = __frcp_rn(n);
+    const uint32_t w[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
+    uint32_t o[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const float lo = __uint_as_float(w[h] << 16), hi = __uint_as_float(w[h] & 0xFFFF0000u);
+      const float x = n > 0.f ? divide_bf16(lo, n, rn, fast) : 0.f, y = n > 0.f ? divide_bf16(hi, n, rn, fast) : 0.f;
+      o[h] = pack_bf16x2(x, y);
+    }
+    if (e < total) dst[e] = make_uint4(o[0], o[1], o[2], o[3]);
+  }
+}
 
 // Exclusive scan of one value per thread over the block; returns the total.
 __device__ __forceinline__ int scan_block(int v, int* excl, int* warp_tot) {
@@ -145,7 +219,7 @@ __device__ __forceinline__ int cand_index(uint64_t v) { return (int)(0xffffffffu
 template <int kT, int E>
 __device__ void bitonic_sort(uint64_t (&v)[E], uint64_t* x) {
   constexpr int p2 = kT * E;
-  const int tid = kT == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;  // kT = 32: one warp, no barrier
+  const int tid = (int)threadIdx.x;
   // fully unrolled: every stage's exchange form and masks are compile-time constants
 #pragma unroll
   for (int size = 2; size <= p2; size <<= 1) {
@@ -191,11 +265,75 @@ __device__ void bitonic_sort(uint64_t (&v)[E], uint64_t* x) {
   }
 }
 
+// One warp sorts 32 * E packed candidates, descending: slot e of lane l is
+// position l * E + e, so every exchange at a stride below E stays within a lane
+// and only the log2(32) + ... + 1 = 15 steps at strides E .. 16 E are warp
+// shuffles (with position e * 32 + l, 40 of the 55 steps of 1024 candidates
+// shuffled two words of every slot, and the shuffle unit set the pace: 1092 us
+// for 40000 rows of about 800 candidates).
+template <int E>
+__device__ __forceinline__ void warp_sort(uint64_t (&v)[E]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int size = 2; size <= 32 * E; size <<= 1) {
+#pragma unroll
+    for (int stride = size >> 1; stride > 0; stride >>= 1) {
+      if (stride >= E) {
+        const bool up = size > 16 * E || (lane & (size / E)) == 0, lo = (lane & (stride / E)) == 0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const uint64_t q = __shfl_xor_sync(0xffffffffu, v[e], stride / E);
+          // the lower position of the pair keeps the larger in a descending run
+          if ((q > v[e]) == (lo == up)) v[e] = q;
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const int f = e | stride;
+          if ((e & stride) == 0 && f < E) {
+            const bool up = size < E ? (e & size) == 0 : size > 16 * E || (lane & (size / E)) == 0;
+            if ((v[f] > v[e]) == up) {
+              const uint64_t t = v[e];
+              v[e] = v[f];
+              v[f] = t;
+            }
+          }
+        }
+      }
+    }
+  }
+}
+
+// A warp loads n <= 32 * E candidates, sorts them and writes the first k
+// indices to out through its 32 * E words of shared memory (whole lines).
+template <int E>
+__device__ void warp_sort_write(const uint2* __restrict__ c, int n, int k, int32_t* __restrict__ buf,
+                                int32_t* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  uint64_t v[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) {  // any order will do: the loads coalesce
+    const int p = lane + e * 32;
+    v[e] = 0ull;
+    if (p < n) {
+      const uint2 q = c[p];
+      v[e] = pack_cand(q.x, (int)q.y);
+    }
+  }
+  warp_sort<E>(v);
+  // position l * E + e at word (l * E + e) ^ l: lanes write to different banks
+#pragma unroll
+  for (int e = 0; e < E; ++e) buf[(lane * E + e) ^ lane] = cand_index(v[e]);
+  __syncwarp();
+  for (int p = lane; p < k; p += 32) out[p] = buf[p ^ (p / E)];
+  __syncwarp();
+}
+
 // Loads n <= kT * E candidates (get(p) -> (key, index)), sorts them and writes
 // the first k indices to out; padding sorts below every real candidate.
 template <int kT, int E, typename Get>
 __device__ void sort_write_e(Get get, int n, int k, uint64_t* x, int32_t* __restrict__ out) {
-  const int tid = kT == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
+  const int tid = (int)threadIdx.x;
   uint64_t v[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) {
@@ -207,7 +345,7 @@ __device__ void sort_write_e(Get get, int n, int k, uint64_t* x, int32_t* __rest
       v[e] = 0ull;
     }
   }
-  if (kT > 32) __syncthreads();  // the candidates may live in the exchange buffer
+  __syncthreads();  // the candidates may live in the exchange buffer
   bitonic_sort<kT, E>(v, x);
 #pragma unroll
   for (int e = 0; e < E; ++e) {
@@ -243,9 +381,9 @@ constexpr int kSampleMinV = 4 * kSample;
 constexpr float kOver = 1.6f;
 
 // Rank of the sample value that sets the threshold: about kOver * k of a
-// row's V values are expected at or above the rs-th largest of kSample.
-__device__ __forceinline__ int sample_rank(int V, int k) {
-  return min(kSample, max(1, (int)ceilf(kOver * (float)k * (float)kSample / (float)V)));
+// row's V values are expected at or above the rs-th largest of ns sampled ones.
+__device__ __forceinline__ int sample_rank(int V, int k, int ns) {
+  return min(ns, max(1, (int)ceilf(kOver * (float)k * (float)ns / (float)V)));
 }
 
 // The smallest value whose order key shares the top 22 bits of the rs-th
@@ -287,7 +425,7 @@ __device__ bool sampled_select(SelShared& sh, const float* __restrict__ s, int V
     sk[4 * u + 2] = ord_key(q.z);
     sk[4 * u + 3] = ord_key(q.w);
   }
-  const float tf = sample_threshold(sh, sk, sample_rank(V, k));
+  const float tf = sample_threshold(sh, sk, sample_rank(V, k, kSample));
   if (threadIdx.x == 0) sh.ncand = 0;
   __syncthreads();
   // appends this lane's hits among its first nv values of q (positions j0 + e); whole warps call it
@@ -449,15 +587,25 @@ __global__ void __launch_bounds__(kSelThreads, 2) topk_select_kernel(const float
   sort_and_write(sh, sh.ncand, k, table + trow * k);
 }
 
-// Rows of the sample similarities Z [rows, kSample]: each row's threshold,
+// Sample tokens of the rows' thresholds (topk_sample_for): about kSampleRank of
+// them lie at or above the threshold, so the candidates above it number kOver k
+// give or take 1 / sqrt(kSampleRank) (13 %): one row in 700 falls short of k and
+// is redone on the fallback path, about a batch of rows for tables of 30000 to
+// 130000 tokens, a few tens of microseconds there.  At V = 40000, k = 500 that
+// is 3072 tokens: against 8192 (a fifth of V) the sample contractions take 512 us
+// instead of 1253 and the thresholds 245 us instead of 368; 3 rows fell short and
+// took 85 us.
+constexpr int kSampleRank = 56;
+
+// Rows of the sample similarities Z [rows, ns]: each row's threshold,
 // the smallest sample value in the bin of a 2048-bin linear histogram over
 // [min, max] of the row's sample that holds its rs-th largest value, so that
 // between rs and rs + (that bin's count) sample values are at or above it.
-// 256 threads, 32 values each.
+// 256 threads, up to 32 values each (ns a multiple of 512).
 constexpr int kTauThreads = 256;
-constexpr int kTauPer = kSample / kTauThreads;
 
-__global__ void __launch_bounds__(kTauThreads, 4) topk_tau_kernel(const float* __restrict__ Z, int V, int k,
+template <int kTauPer>  // values per thread: ns <= kTauPer * kTauThreads
+__global__ void __launch_bounds__(kTauThreads, kTauPer > 16 ? 4 : 6) topk_tau_kernel(const float* __restrict__ Z, int V, int k, int ns,
                                                                 float* __restrict__ tau) {
   griddep_wait();
   griddep_launch_dependents();
@@ -465,11 +613,13 @@ __global__ void __launch_bounds__(kTauThreads, 4) topk_tau_kernel(const float* _
   __shared__ float red[2][kTauThreads / 32];
   __shared__ int s_bin;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const float4* z4 = reinterpret_cast<const float4*>(Z + (long long)blockIdx.x * kSample);
+  const float4* z4 = reinterpret_cast<const float4*>(Z + (long long)blockIdx.x * ns);
+  // values u of this thread beyond the sample repeat its first one, and are not counted (mine: how many count)
+  const int mine = tid * 4 < ns ? ((ns / 4 - tid + kTauThreads - 1) / kTauThreads) * 4 : 0;
   float v[kTauPer];
 #pragma unroll
   for (int u = 0; u < kTauPer / 4; ++u) {
-    const float4 q = __ldcs(z4 + tid + u * kTauThreads);
+    const float4 q = __ldcs(z4 + (u * 4 < mine ? tid + u * kTauThreads : tid * 4 < ns ? tid : 0));
     v[4 * u] = q.x;
     v[4 * u + 1] = q.y;
     v[4 * u + 2] = q.z;
@@ -502,10 +652,11 @@ __global__ void __launch_bounds__(kTauThreads, 4) topk_tau_kernel(const float* _
   const float scale = hi > lo ? 2048.f / (hi - lo) : 0.f;
   auto bin_of = [&](float x) { return min(2047, max(0, (int)((x - lo) * scale))); };
 #pragma unroll
-  for (int e = 0; e < kTauPer; ++e) atomicAdd(&hist[bin_of(v[e])], 1);
+  for (int e = 0; e < kTauPer; ++e)
+    if (e < mine) atomicAdd(&hist[bin_of(v[e])], 1);
   __syncthreads();
   // bins by descending index: thread t holds bins 2047 - 8t .. 2040 - 8t
-  const int rs = sample_rank(V, k);
+  const int rs = sample_rank(V, k, ns);
   int local = 0;
 #pragma unroll
   for (int q = 0; q < 8; ++q) local += hist[2047 - 8 * tid - q];
@@ -553,8 +704,7 @@ __global__ void __launch_bounds__(kTauThreads, 4) topk_tau_kernel(const float* _
 
 // Each row's cnt[r] candidates (order key, token) appended by the similarity
 // contraction; with k <= n <= cap they hold the exact top k.  One warp per row
-// sorts lists of up to 1024 in registers (32 lanes x up to 32 slots: shuffles
-// below stride 32, in-thread swaps above, no barrier); longer lists go to a
+// sorts lists of up to 1024 in registers (32 lanes x up to 32 slots); longer lists go to a
 // list for the block sort below; rows outside [k, cap] join the fallback list.
 constexpr int kWarpSortMax = 1024;
 constexpr int kSortThreads = 256;
@@ -565,6 +715,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) topk_sort_warp_kernel(
     int32_t* __restrict__ fail_rows, int* __restrict__ fail_count) {
   griddep_wait();
   griddep_launch_dependents();
+  __shared__ int32_t buf[kSortThreads / 32][kWarpSortMax];
   const int r = blockIdx.x * (kSortThreads / 32) + (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (r >= nrows) return;  // whole warps
   const int n = cnt[r];
@@ -577,16 +728,16 @@ __global__ void __launch_bounds__(kSortThreads, 2) topk_sort_warp_kernel(
     return;
   }
   const uint2* c = cand + (long long)r * cap;
-  auto get = [&](int p) { return c[p]; };
   int32_t* out = table + (long long)(row0 + r) * k;
+  int32_t* x = buf[threadIdx.x >> 5];
   if (n <= 128)
-    sort_write_e<32, 4>(get, n, k, nullptr, out);
+    warp_sort_write<4>(c, n, k, x, out);
   else if (n <= 256)
-    sort_write_e<32, 8>(get, n, k, nullptr, out);
+    warp_sort_write<8>(c, n, k, x, out);
   else if (n <= 512)
-    sort_write_e<32, 16>(get, n, k, nullptr, out);
+    warp_sort_write<16>(c, n, k, x, out);
   else
-    sort_write_e<32, 32>(get, n, k, nullptr, out);
+    warp_sort_write<32>(c, n, k, x, out);
 }
 
 // The rows the warp sort listed (more than 1024 candidates): one block of 256
@@ -614,25 +765,31 @@ __global__ void __launch_bounds__(kSortThreads, 4) topk_sort_kernel(const uint2*
   }
 }
 
-// Es[i, :] = En[floor(i * V / kSample), :]: the sample tokens, evenly spread.
-__global__ void topk_gather_sample_kernel(const __nv_bfloat16* __restrict__ En, int V, int d,
+// Es[i, :] = En[floor(i * V / ns), :] for i < ns: the sample tokens, evenly spread.
+__global__ void topk_gather_sample_kernel(const __nv_bfloat16* __restrict__ En, int V, int d, int ns,
                                           __nv_bfloat16* __restrict__ Es) {
   griddep_wait();
   griddep_launch_dependents();
   const int vpr = d / 8;
-  const long long total = (long long)kSample * vpr;
+  const long long total = (long long)ns * vpr;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
        e += (long long)gridDim.x * blockDim.x) {
     const int i = (int)(e / vpr), v = (int)(e % vpr);
-    const long long src = (long long)i * V / kSample;
+    const long long src = (long long)i * V / ns;
     reinterpret_cast<uint4*>(Es + (long long)i * d)[v] = reinterpret_cast<const uint4*>(En + src * d)[v];
   }
 }
 
 }  // namespace
 
-cudaError_t launch_normalize_rows(const __nv_bfloat16* E, int V, int d, __nv_bfloat16* En, cudaStream_t st) {
-  return launch_kernel(normalize_rows_kernel, dim3((V + 127) / 128), dim3(128), 0, st, 1, E, V, d, En);
+cudaError_t launch_normalize_rows(const __nv_bfloat16* E, int V, int d, float* norm, __nv_bfloat16* En,
+                                  cudaStream_t st) {
+  const int per = 32 * kNormWarps;
+  const cudaError_t e = launch_kernel(row_norms_kernel, dim3((V + per - 1) / per), dim3(kNormWarps * 32), 0, st, 1, E, V, d,
+                                      norm);
+  if (e != cudaSuccess) return e;
+  const long long blocks = ((long long)V * (d / 8) + 256 * 8 - 1) / (256 * 8);
+  return launch_kernel(scale_rows_kernel, dim3((unsigned)blocks), dim3(256), 0, st, 1, E, V, d, (const float*)norm, En);
 }
 
 // Sets the dynamic shared-memory size of the selection kernel (once per device).
@@ -649,8 +806,9 @@ cudaError_t launch_topk_select(const float* S, long long lds, int V, int k, int 
                        k, row0, rows, table, status);
 }
 
-cudaError_t launch_topk_tau(const float* Z, int V, int k, int nrows, float* tau, cudaStream_t st) {
-  return launch_kernel(topk_tau_kernel, dim3(nrows), dim3(kTauThreads), 0, st, 1, Z, V, k, tau);
+cudaError_t launch_topk_tau(const float* Z, int V, int k, int ns, int nrows, float* tau, cudaStream_t st) {
+  auto kernel = ns <= 16 * kTauThreads ? topk_tau_kernel<16> : topk_tau_kernel<kSample / kTauThreads>;
+  return launch_kernel(kernel, dim3(nrows), dim3(kTauThreads), 0, st, 1, Z, V, k, ns, tau);
 }
 
 cudaError_t launch_topk_sort(const uint2* cand, int* cnt, int cap, int k, int row0, int nrows, int32_t* table,
@@ -665,12 +823,16 @@ cudaError_t launch_topk_sort(const uint2* cand, int* cnt, int cap, int k, int ro
                        (const int*)cnt, cap, k, row0, (const int32_t*)big_rows, (const int*)big_count, table);
 }
 
-cudaError_t launch_topk_gather_sample(const __nv_bfloat16* En, int V, int d, __nv_bfloat16* Es, int num_sms,
+cudaError_t launch_topk_gather_sample(const __nv_bfloat16* En, int V, int d, int ns, __nv_bfloat16* Es, int num_sms,
                                       cudaStream_t st) {
-  return launch_kernel(topk_gather_sample_kernel, dim3(num_sms * 4), dim3(256), 0, st, 1, En, V, d, Es);
+  return launch_kernel(topk_gather_sample_kernel, dim3(num_sms * 4), dim3(256), 0, st, 1, En, V, d, ns, Es);
 }
 
 int topk_sample() { return kSample; }
+int topk_sample_for(int V, int k) {
+  const long long n = (long long)((double)kSampleRank * V / (kOver * (double)k)) + 1;
+  return (int)std::min<long long>(kSample, std::max<long long>(1024, (n + 511) / 512 * 512));
+}
 int topk_sample_min_v() { return kSampleMinV; }
 int topk_cap() { return kCap; }
 

@@ -78,6 +78,21 @@ def test_topk_table_parity(V, d, k):
     check_rows(bits, table, k, rows)
 
 
+# partial row groups and column chunks of the norms, several chunks of short rows, large k (a short sample)
+@pytest.mark.parametrize("V,d,k", [(2001, 72, 16), (9003, 200, 130), (33001, 72, 1024)],
+                         ids=["V2001_d72_k16", "V9003_d200_k130", "V33001_d72_k1024"])
+def test_topk_table_edges(V, d, k):
+    """The oracle's checks, and the same table when rows are scaled by powers of two (2^62 and 2^-50 take the two
+    division paths of the normalisation; a scaled row normalises to the same bits)."""
+    bits = synth.gen_E(0, 52, V, d)
+    table = run_table(bits, k)
+    rng = np.random.default_rng(V)
+    check_rows(bits, table, k, np.unique(np.concatenate([[0, V - 1, 511, 512], rng.integers(0, V, 20)])))
+    scale = np.array([1.0, 2.0 ** 62, 2.0 ** -50])[rng.integers(0, 3, V)]
+    scaled = synth.to_bf16_bits(synth.bf16_bits_to_f64(bits) * scale[:, None])
+    assert np.array_equal(run_table(scaled, k), table)
+
+
 def test_topk_argument_errors():
     with pytest.raises(lora.LoraError) as e:
         lora.lora_topk_workspace_size(100, 12, 5)  # d not a multiple of 8

@@ -60,3 +60,22 @@ def test_topk_pins_catch_planted_mistake(name):
         except AssertionError:
             failed = True
     assert failed, f"no pin caught the planted mistake {name}"
+
+
+def test_division_shortcut_rounds_alike():
+    """The normalisation's shortcut in fp32 arithmetic: x * (1 / n) rounds to the same bf16 as x / n wherever its low
+    16 bits are more than 4 from the midpoint, for every bf16 mantissa x against random divisors."""
+    rng = np.random.default_rng(5)
+    x = (np.arange(128, 256, dtype=np.float32) / np.float32(128))[:, None]
+    n = np.concatenate([rng.uniform(1, 2, 40000), 1 + 2.0 ** -rng.integers(1, 24, 2000)]).astype(np.float32)[None, :]
+    q, p = (x / n).astype(np.float32), (x * (np.float32(1) / n)).astype(np.float32)
+    qb, pb = q.view(np.uint32), p.view(np.uint32)
+    assert np.abs(qb.astype(np.int64) - pb.astype(np.int64)).max() <= 3
+    low = (pb & 0xFFFF).astype(np.int64)
+    safe = np.abs(low - 0x8000) > 4
+
+    def bf16(b):
+        return (b + 0x7FFF + ((b >> 16) & 1)) >> 16
+
+    assert safe.mean() > 0.999 and np.array_equal(bf16(qb)[safe], bf16(pb)[safe])
+
