@@ -228,7 +228,7 @@ int lora_stack_ckpt(const lora_proj* projs, int n_layers, int n_per_layer, void*
  *     dh_t = sum_{j in J} (softmax_J(z_t)[j] - [j == y_t]) E_j for t in T_set, 0 elsewhere.
  * Row i of the top-k table lists tokens by descending similarity to token i
  * and starts with i (so every trainable target is in J); it is the table
- * lora_topk_table builds.  The call synchronizes `stream` once, after the
+ * lora_topk_table builds.  The call waits once on the host for the
  * index pass, to size the two contractions by |T_set| and |J| (so it cannot
  * be captured into a CUDA graph).  Logits are accumulated in fp32 and kept in
  * fp32; softmax - onehot enters the dh contraction in bf16; dh is bf16.

@@ -1209,6 +1209,16 @@ struct ThreadSide {
 
 thread_local ThreadSide t_side;
 
+// The calling thread's side stream and events on device d, created on its first use.
+int side_ctx(const DeviceInfo* d, SideCtx** out) {
+  SideCtx& c = t_side.dev[d - g_dev];
+  if (!c.side && cudaStreamCreateWithFlags(&c.side, cudaStreamNonBlocking) != cudaSuccess) return LORA_ECUDA;
+  for (cudaEvent_t& e : c.ev)
+    if (!e && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return LORA_ECUDA;
+  *out = &c;
+  return LORA_OK;
+}
+
 struct Overlap {
   bool on = false, forked = false, joined = false;
   int side_ctas = 0;   // beside the forward contraction
@@ -1217,10 +1227,10 @@ struct Overlap {
   cudaEvent_t ev_fork = nullptr, ev_sv = nullptr, ev_done = nullptr;
   int init(const DeviceInfo* d, cudaStream_t st, const lora_proj* projs, int n, const SideWidths& planned) {
     if (!overlap_enabled() || !any_adapter(projs, n)) return LORA_OK;
-    SideCtx& c = t_side.dev[d - g_dev];
-    if (!c.side && cudaStreamCreateWithFlags(&c.side, cudaStreamNonBlocking) != cudaSuccess) return LORA_ECUDA;
-    for (cudaEvent_t& e : c.ev)
-      if (!e && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return LORA_ECUDA;
+    SideCtx* ctx = nullptr;
+    const int rc = side_ctx(d, &ctx);
+    if (rc != LORA_OK) return rc;
+    SideCtx& c = *ctx;
     main = st;
     side = c.side;
     ev_fork = c.ev[0];
@@ -1738,7 +1748,7 @@ void layer_copy(const lora_proj* L, int n_per, uint8_t* su_scratch, std::vector<
 constexpr size_t kCeSplitFloats = (size_t)8 * kPlanPairs * 256 * 512 + 64 * 1024;
 
 struct CePlan {
-  size_t flags, counts, segs, J, pos, tl, tpos, ycol, rowloss, lse, ht, ej, z, lse_part, g, dht, part, tiles, total;
+  size_t flags, counts, segs, J, tl, tpos, ycol, rowloss, ht, ej, z, lse_part, g, dht, part, tiles, total;
   int ld_lse;
 };
 
@@ -1764,12 +1774,10 @@ int ce_check(const lora_ce_args* a, CePlan* pl) {
   pl->segs = take(128 * 4);
   pl->flags = take((size_t)V);
   pl->J = take((size_t)V * 4);
-  pl->pos = take((size_t)V * 4);
   pl->tl = take((size_t)T * 4);
   pl->tpos = take((size_t)T * 4);
   pl->ycol = take((size_t)T * 4);
   pl->rowloss = take((size_t)T * 4);
-  pl->lse = take((size_t)T * 4);
   pl->ht = take((size_t)T * d * 2);
   // J is the whole vocabulary without a top-k table: E is read in place
   pl->ej = take(a->topk ? (size_t)V * d * 2 : 0);
@@ -2209,18 +2217,28 @@ int lora_ce_fwd_bwd(const lora_ce_args* a, void* workspace, size_t workspace_byt
   ix.k = (int)a->k;
   ix.flags = ws + pl.flags;
   ix.J = at<int32_t>(ws, pl.J);
-  ix.pos = at<int32_t>(ws, pl.pos);
   ix.tl = at<int32_t>(ws, pl.tl);
   ix.tpos = at<int32_t>(ws, pl.tpos);
   ix.ycol = at<int32_t>(ws, pl.ycol);
   ix.counts = at<int32_t>(ws, pl.counts);
   ix.seg_counts = at<int32_t>(ws, pl.segs);
   if (launch_ce_index(ix, st) != cudaSuccess) return rec(LORA_ECUDA);
-  // |T_set| and |J| size the contractions
+  // |T_set| and |J| size the contractions: the host reads them on the thread's side stream while the
+  // dense rows, whose kernel takes them from device memory, are made on the caller's
   int32_t counts[3] = {0, 0, 0};
-  if (cudaMemcpyAsync(counts, ix.counts, sizeof(counts), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-      cudaStreamSynchronize(st) != cudaSuccess)
-    return rec(LORA_ECUDA);
+  {
+    SideCtx* side = nullptr;
+    if ((rc = side_ctx(d, &side)) != LORA_OK) return rec(rc);
+    if (cudaEventRecord(side->ev[0], st) != cudaSuccess || cudaStreamWaitEvent(side->side, side->ev[0], 0) != cudaSuccess)
+      return rec(LORA_ECUDA);
+    if (launch_ce_prepare(ix, cb(a->h), cb(a->E), D, at<bf>(ws, pl.ht), at<bf>(ws, pl.ej), mb(a->dh), a->token_loss,
+                          d->num_sms, st) !=
+        cudaSuccess)
+      return rec(LORA_ECUDA);
+    if (cudaMemcpyAsync(counts, ix.counts, sizeof(counts), cudaMemcpyDeviceToHost, side->side) != cudaSuccess ||
+        cudaStreamSynchronize(side->side) != cudaSuccess)
+      return rec(LORA_ECUDA);
+  }
   if (counts[2]) return rec(LORA_EINVAL);
   const int nT = counts[0], nJ = counts[1];
   if (a->counts) {
@@ -2236,20 +2254,15 @@ int lora_ce_fwd_bwd(const lora_ce_args* a, void* workspace, size_t workspace_byt
     const int ldz = (int)rup(nJ, 4), ldg = (int)rup(nJ, 8);
     int* tiles = at<int>(ws, pl.tiles);
     // J sorted ascending with |J| = V is every token in order: E serves as E_J
-    const bf* ej = cb(a->E);
-    bf* ejw = at<bf>(ws, pl.ej);
-    if (launch_gather_rows2(cb(a->h), D, ix.tl, nT, ht, cb(a->E), D, ix.J, nJ < V ? nJ : 0, ejw, D, st) !=
-        cudaSuccess)
-      return rec(LORA_ECUDA);
-    if (nJ < V) ej = ejw;
+    const bf* ej = nJ < V ? at<bf>(ws, pl.ej) : cb(a->E);
     {
       ProfScope ps(LORA_KERNEL_GEMM_FWD, st);
       if ((rc = ce_gemm(d, tiles, ht, D, ej, D, z, ldz, nT, nJ, D, false, true, at<float>(ws, pl.part), st, lse_part,
                         pl.ld_lse)) != LORA_OK)
         return rec(rc);
     }
-    if (launch_ce_rows(lse_part, pl.ld_lse, z, ldz, nJ, ix.ycol, nT, at<float>(ws, pl.lse), rowloss, ix.tpos, T,
-                       a->token_loss, a->loss, ix.counts + 5, g, ldg, d->num_sms, st) != cudaSuccess)
+    if (launch_ce_rows(lse_part, pl.ld_lse, z, ldz, nJ, ix.ycol, nT, rowloss, ix.tl, a->token_loss, a->loss,
+                       ix.counts + 5, g, ldg, d->num_sms, st) != cudaSuccess)
       return rec(LORA_ECUDA);
     if (a->dh) {
       bf* dht = at<bf>(ws, pl.dht);
@@ -2259,10 +2272,9 @@ int lora_ce_fwd_bwd(const lora_ce_args* a, void* workspace, size_t workspace_byt
         return rec(rc);
     }
   }
-  // with trainable positions the log-sum-exp launch's last block has written the losses
-  if (nT == 0 && launch_ce_finish(rowloss, nT, ix.tpos, T, a->token_loss, a->loss, st) != cudaSuccess)
-    return rec(LORA_ECUDA);
-  if (a->dh && launch_scatter_rows(at<bf>(ws, pl.dht), ix.tpos, T, D, mb(a->dh), st) != cudaSuccess)
+  // with trainable positions the launch over the logits' rows has written the loss
+  if (nT == 0 && cudaMemsetAsync(a->loss, 0, sizeof(float), st) != cudaSuccess) return rec(LORA_ECUDA);
+  if (a->dh && launch_scatter_rows(at<bf>(ws, pl.dht), ix.tl, nT, D, mb(a->dh), st) != cudaSuccess)
     return rec(LORA_ECUDA);
   if (a->vocab && nJ > 0 &&
       cudaMemcpyAsync(a->vocab, ix.J, (size_t)nJ * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess)

@@ -313,10 +313,11 @@ cudaError_t launch_transposes(const TransposeJobs& jobs, cudaStream_t stream);
 
 // ---------------------------------------------------------------- reduced-vocabulary cross entropy
 // Index pass: J (ascending) = union of the trainable targets' first k top-k
-// entries (every token when topk is null), pos[v] = column of v in J or -1,
-// tl = trainable positions (ascending), tpos[t] = row of t in tl or -1,
-// ycol[i] = column in J of the target of tl[i]; counts = {|tl|, |J|, bad
-// input flag}.  flags (V bytes) and counts must be zero at launch.
+// entries (every token when topk is null), tl = trainable positions (ascending),
+// tpos[t] = row of t in tl or -1; counts = {|tl|, |J|, bad input flag (a table
+// entry out of range, a trainable target out of range or outside J)}.  flags (V
+// bytes) and counts must be zero at launch.  ycol[i] = column in J of the target
+// of tl[i] (launch_ce_prepare).
 struct CeIndex {
   const int32_t* targets;
   const uint8_t* mask;  // null: every position trainable
@@ -325,32 +326,30 @@ struct CeIndex {
   long long ld_topk;
   int k;
   uint8_t* flags;
-  int32_t *J, *pos, *tl, *tpos, *ycol;
-  int32_t* counts;      // [8]: |T_set|, |J|, error flag, -, two last-block counters
+  int32_t *J, *tl, *tpos, *ycol;
+  int32_t* counts;      // [8]: |T_set|, |J|, error flag, -, -, a last-block counter
   int32_t* seg_counts;  // 128 per-segment counts of the vocabulary compaction
 };
 cudaError_t launch_ce_index(const CeIndex& a, cudaStream_t stream);
+// After it, with the counts still on the device: ht = rows tl of h, ej = rows J of E (unless |J| = V), ycol, and
+// zeros in the rows of dh and token_loss (both optional) outside tl; nothing when the bad input flag is set.
+cudaError_t launch_ce_prepare(const CeIndex& a, const __nv_bfloat16* h, const __nv_bfloat16* E, int d,
+                              __nv_bfloat16* ht, __nv_bfloat16* ej, __nv_bfloat16* dh, float* token_loss, int num_sms,
+                              cudaStream_t stream);
 // dst[i, :] = src[idx[i], :] for i < n (rows of d bf16, d a multiple of 8).
 cudaError_t launch_gather_rows(const __nv_bfloat16* src, long long ld, const int32_t* idx, int n, int d,
                                __nv_bfloat16* dst, cudaStream_t stream);
-// Two such gathers in one launch.
-cudaError_t launch_gather_rows2(const __nv_bfloat16* src_a, long long ld_a, const int32_t* idx_a, int n_a,
-                                __nv_bfloat16* dst_a, const __nv_bfloat16* src_b, long long ld_b,
-                                const int32_t* idx_b, int n_b, __nv_bfloat16* dst_b, int d, cudaStream_t stream);
 // Per row i < nT of the fp32 logits Z [nT, ldz] with their log-sum-exp
 // partials lse_part [nT, ld_part] (one per gemm_lse_group() columns), nT >= 1:
-// lse[i], rowloss[i] = lse - z[ycol[i]] and G[i, :] = bf16(softmax - onehot),
+// rowloss[i] = lse_i - z[ycol[i]] and G[i, :] = bf16(softmax - onehot),
 // zero in columns [nJ, ldg).
-// The last block also writes token_loss (optional) and *loss (as launch_ce_finish);
+// token_loss[tl[i]] (optional) = rowloss[i], *loss = their sum in a fixed order;
 // done: a zeroed counter.
 cudaError_t launch_ce_rows(const float2* lse_part, int ld_part, const float* Z, int ldz, int nJ, const int32_t* ycol,
-                           int nT, float* lse, float* rowloss, const int32_t* tpos, int T, float* token_loss,
-                           float* loss, int* done, __nv_bfloat16* G, int ldg, int num_sms, cudaStream_t stream);
-// token_loss[t] (optional) and *loss = sum of rowloss in a fixed order.
-cudaError_t launch_ce_finish(const float* rowloss, int nT, const int32_t* tpos, int T, float* token_loss,
-                             float* loss, cudaStream_t stream);
-// dst[t, :] = src[tpos[t], :] or zeros when tpos[t] < 0.
-cudaError_t launch_scatter_rows(const __nv_bfloat16* src, const int32_t* tpos, int T, int d, __nv_bfloat16* dst,
+                           int nT, float* rowloss, const int32_t* tl, float* token_loss, float* loss, int* done,
+                           __nv_bfloat16* G, int ldg, int num_sms, cudaStream_t stream);
+// dst[idx[i], :] = src[i, :] for i < n.
+cudaError_t launch_scatter_rows(const __nv_bfloat16* src, const int32_t* idx, int n, int d, __nv_bfloat16* dst,
                                 cudaStream_t stream);
 
 // ---------------------------------------------------------------- top-k similarity table

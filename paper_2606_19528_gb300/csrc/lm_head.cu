@@ -4,19 +4,22 @@
 // compute the logits of the trainable positions over the reduced vocabulary
 // J and the hidden-state gradient.
 //   vocab_mark      J = union of the trainable targets' first k top-k entries
-//   vocab_count,    J and the trainable positions as ascending lists and
-//   compact         their inverse maps (128 vocabulary segments counted, then
-//                   compacted in parallel); the last block places each
-//                   trainable target in J
-//   gather_rows(2)  rows of h (trainable positions) and of E (J) made dense
-//   ce_lse          per trainable position: log-sum-exp over J merged from the
-//                   logits contraction's per-group partials, and its loss; the
-//                   last block writes the per-position losses and their sum
-//                   in a fixed order
-//   ce_grad         G = softmax_J - onehot(target) in bf16 for the dh
-//                   contraction, one streaming pass over the logits
-//   ce_finish       the losses when no position is trainable
-//   scatter_rows    dh rows of trainable positions, zeros elsewhere
+//   compact         J and the trainable positions as ascending lists and the
+//                   latter's inverse map: 128 blocks take a vocabulary segment
+//                   each, counting the flags before it themselves (tables past
+//                   2^20 tokens: vocab_count first), one block the positions,
+//                   with the check of their targets
+//   prepare_rows    rows of h (trainable positions) and of E (J) made dense, each
+//                   trainable target's column in J, zeros in the other rows of dh
+//                   and the other positions' losses;
+//                   it reads the counts on the device, so it runs while the host
+//                   waits for them
+//   ce_rows         per trainable position: log-sum-exp over J merged from the
+//                   logits contraction's per-group partials, its loss, and G =
+//                   softmax_J - onehot(target) in bf16 for the dh contraction in
+//                   one streaming pass over the logits; the last block writes the
+//                   losses' sum in a fixed order
+//   scatter_rows    dh rows of trainable positions
 #include <math.h>
 
 #include <algorithm>
@@ -99,10 +102,10 @@ __device__ __forceinline__ int block_scan(int v, int* excl) {
   return total;
 }
 
-// Ascending compaction of the set entries of [0, n) (flag(i) != 0) into
-// list, with inv[i] = position in list or -1.  One block.
+// Ascending compaction of the set entries of [0, n) (flag(i) != 0): list[k] =
+// first + the k-th set i, and inv[i] = its position or -1.  One block.
 template <typename Flag>
-__device__ int compact(int n, Flag flag, int32_t* list, int32_t* inv) {
+__device__ int compact(int n, Flag flag, int first, int32_t* list, int32_t* inv) {
   const int per = (n + kScanThreads - 1) / kScanThreads;
   const int b0 = min(n, (int)threadIdx.x * per), b1 = min(n, b0 + per);
   int cnt = 0;
@@ -111,7 +114,7 @@ __device__ int compact(int n, Flag flag, int32_t* list, int32_t* inv) {
   const int total = block_scan(cnt, &off);
   for (int i = b0; i < b1; ++i) {
     if (flag(i)) {
-      list[off] = i;
+      list[off] = first + i;
       if (inv) inv[i] = off;
       ++off;
     } else if (inv) {
@@ -144,74 +147,56 @@ __global__ void __launch_bounds__(256) vocab_count_kernel(const uint8_t* __restr
   }
 }
 
-// Blocks 0 .. kSegs-1: their segment of J (ascending) and pos; block kSegs:
-// the trainable positions, their inverse map and the counts.
-// The last block to finish also places each trainable target in J (ycol).
-__device__ void ycol_rows(const int32_t* __restrict__ targets, const int32_t* tl, const int32_t* pos, int V,
-                          int32_t* ycol, int32_t* counts) {
-  const int nT = counts[0];
-  for (int i = threadIdx.x; i < nT; i += blockDim.x) {
-    const int y = targets[tl[i]];
-    const int c = (y >= 0 && y < V) ? pos[y] : -1;
-    if (c < 0) counts[2] = 1;  // a trainable target outside J (or out of range)
-    ycol[i] = c < 0 ? 0 : c;
+// Set flags (bytes 0 or 1) in [0, n), by the whole block; every thread gets the sum.
+__device__ int count_flags(const uint8_t* __restrict__ flags, int n) {
+  const int n16 = n / 16;
+  const uint4* f4 = reinterpret_cast<const uint4*>(flags);
+  int c = 0;
+  for (int i = threadIdx.x; i < n16; i += kScanThreads) {
+    const uint4 q = f4[i];
+    c += __popc(q.x) + __popc(q.y) + __popc(q.z) + __popc(q.w);
   }
+  const int t = 16 * n16 + (int)threadIdx.x;
+  if (threadIdx.x < 16 && t < n) c += flags[t];
+  int excl;
+  return block_scan(c, &excl);
 }
 
-__device__ void compact_part(const uint8_t* __restrict__ flags, int V, int full, const int32_t* __restrict__ seg_counts,
-                             const uint8_t* __restrict__ mask, int T, int32_t* J, int32_t* pos, int32_t* tl,
-                             int32_t* tpos, int32_t* counts, int* s_base_p) {
-  int& s_base = *s_base_p;
-  if (blockIdx.x < kSegs) {
-    const int seg = (V + kSegs - 1) / kSegs;
-    const int b0 = min(V, (int)blockIdx.x * seg), b1 = min(V, b0 + seg);
-    if (threadIdx.x == 0) {
-      int base = 0;
-      for (int b = 0; b < (int)blockIdx.x; ++b) base += seg_counts[b];
-      s_base = base;
-    }
-    __syncthreads();
-    const int base = s_base;
-    compact(b1 - b0, [&](int i) { return full || flags[b0 + i] != 0; }, J + base, nullptr);
-    __syncthreads();
-    // pos over the segment: J[base .. base + cnt) are ascending tokens of [b0, b1)
-    for (int i = b0 + threadIdx.x; i < b1; i += kScanThreads) pos[i] = -1;
-    __syncthreads();
-    const int cnt = seg_counts[blockIdx.x];
-    for (int q = threadIdx.x; q < cnt; q += kScanThreads) {
-      J[base + q] += b0;  // compact wrote segment-relative indices
-      pos[J[base + q]] = base + q;
-    }
-    return;
-  }
-  const int nT = compact(T, [&](int t) { return !mask || mask[t] != 0; }, tl, tpos);
-  if (threadIdx.x == 0) {
-    int nJ = 0;
-    for (int b = 0; b < kSegs; ++b) nJ += seg_counts[b];
-    counts[0] = nT;
-    counts[1] = nJ;
-  }
-}
-
+// Blocks 0 .. kSegs - 1: their segment of J (ascending); block kSegs: the
+// trainable positions, their inverse map, the counts, and the check that every
+// trainable target lies in J.  seg_counts null: each block counts the flags
+// before its segment (at most 2^20 bytes, from L2) instead of a launch of its own
+// counting the segments first.
 __global__ void __launch_bounds__(kScanThreads) compact_kernel(const uint8_t* __restrict__ flags, int V, int full,
                                                                const int32_t* __restrict__ seg_counts,
                                                                const uint8_t* __restrict__ mask, int T,
-                                                               int32_t* J, int32_t* pos, int32_t* tl, int32_t* tpos,
-                                                               int32_t* counts, const int32_t* __restrict__ targets,
-                                                               int32_t* ycol, int32_t* done) {
+                                                               const int32_t* __restrict__ targets, int32_t* J,
+                                                               int32_t* tl, int32_t* tpos, int32_t* counts) {
   griddep_wait();
   griddep_launch_dependents();
-  __shared__ int s_base, s_last;
-  compact_part(flags, V, full, seg_counts, mask, T, J, pos, tl, tpos, counts, &s_base);
-  // the last block to finish (every J, pos, tl written and visible) places the targets
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(done, 1) == (int)gridDim.x - 1;
-  __syncthreads();
-  if (s_last) {
-    __threadfence();
-    ycol_rows(targets, tl, pos, V, ycol, counts);
+  if (blockIdx.x < kSegs) {
+    const int seg = (V + kSegs - 1) / kSegs;
+    const int b0 = min(V, (int)blockIdx.x * seg), b1 = min(V, b0 + seg);
+    int base = b0;
+    if (!full) {
+      base = 0;
+      if (seg_counts)
+        for (int b = 0; b < (int)blockIdx.x; ++b) base += seg_counts[b];
+      else
+        base = count_flags(flags, b0);
+    }
+    const int n = compact(b1 - b0, [&](int i) { return full || flags[b0 + i] != 0; }, b0, J + base, nullptr);
+    if (blockIdx.x == kSegs - 1 && threadIdx.x == 0) counts[1] = base + n;
+    return;
   }
+  auto trainable = [&](int t) { return !mask || mask[t] != 0; };
+  const int nT = compact(T, trainable, 0, tl, tpos);
+  for (int t = threadIdx.x; t < T; t += kScanThreads) {
+    if (!trainable(t)) continue;
+    const int y = targets[t];
+    if (y < 0 || y >= V || (!full && flags[y] == 0)) counts[2] = 1;  // out of range or outside J
+  }
+  if (threadIdx.x == 0) counts[0] = nT;
 }
 
 __global__ void gather_rows_kernel(const __nv_bfloat16* __restrict__ src, long long ld,
@@ -228,26 +213,44 @@ __global__ void gather_rows_kernel(const __nv_bfloat16* __restrict__ src, long l
   }
 }
 
-// Two gathers in one launch (blockIdx.y selects the row set): one warp per
-// row, four 16-byte loads in flight per lane.
-__global__ void gather_rows2_kernel(const __nv_bfloat16* __restrict__ src_a, long long ld_a,
-                                    const int32_t* __restrict__ idx_a, int n_a, __nv_bfloat16* __restrict__ dst_a,
-                                    const __nv_bfloat16* __restrict__ src_b, long long ld_b,
-                                    const int32_t* __restrict__ idx_b, int n_b, __nv_bfloat16* __restrict__ dst_b,
-                                    int d) {
+// One warp per row, four 16-byte loads in flight per lane: the trainable rows of
+// h (and their targets' columns in the ascending J, by a 32-way search), the rows
+// of E in J (not when J is the whole vocabulary: E is read in place), and zeros in
+// the rows of dh and the losses outside the trainable set (not after a failed check: the call's
+// outputs stay untouched).
+__global__ void __launch_bounds__(256) prepare_rows_kernel(const __nv_bfloat16* __restrict__ h,
+                                                           const __nv_bfloat16* __restrict__ E, int d, int T, int V,
+                                                           const int32_t* __restrict__ tl,
+                                                           const int32_t* __restrict__ tpos,
+                                                           const int32_t* __restrict__ J,
+                                                           const int32_t* __restrict__ targets,
+                                                           const int32_t* __restrict__ counts,
+                                                           __nv_bfloat16* __restrict__ ht, __nv_bfloat16* __restrict__ ej,
+                                                           int32_t* __restrict__ ycol, __nv_bfloat16* __restrict__ dh,
+                                                           float* __restrict__ token_loss) {
   griddep_wait();
   griddep_launch_dependents();
-  const bool b = blockIdx.y == 1;
-  const __nv_bfloat16* src = b ? src_b : src_a;
-  const long long ld = b ? ld_b : ld_a;
-  const int32_t* idx = b ? idx_b : idx_a;
-  const int n = b ? n_b : n_a;
-  __nv_bfloat16* dst = b ? dst_b : dst_a;
+  const int nT = counts[0], nJ = counts[1];
+  if (counts[2] != 0) return;
+  const int nE = nJ < V ? nJ : 0;
   const int vpr = d / 8, lane = threadIdx.x & 31;
-  const int warps = gridDim.x * (blockDim.x >> 5);
-  for (int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
-    const uint4* s = reinterpret_cast<const uint4*>(src + (long long)idx[i] * ld);
-    uint4* o = reinterpret_cast<uint4*>(dst + (long long)i * d);
+  const long long warps = (long long)gridDim.x * 8, total = (long long)nT + nE + (dh || token_loss ? T : 0);
+  for (long long w = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); w < total; w += warps) {
+    if (w >= (long long)nT + nE) {
+      const int t = (int)(w - nT - nE);
+      if (tpos[t] < 0) {
+        if (dh)
+          for (int v = lane; v < vpr; v += 32)
+            reinterpret_cast<uint4*>(dh + (long long)t * d)[v] = make_uint4(0u, 0u, 0u, 0u);
+        if (token_loss && lane == 0) token_loss[t] = 0.f;
+      }
+      continue;
+    }
+    const bool isT = w < nT;
+    const int i = (int)(isT ? w : w - nT);
+    const int src = isT ? tl[i] : J[i];
+    const uint4* s = reinterpret_cast<const uint4*>((isT ? h : E) + (long long)src * d);
+    uint4* o = reinterpret_cast<uint4*>((isT ? ht : ej) + (long long)i * d);
     for (int v0 = lane; v0 < vpr; v0 += 4 * 32) {
       uint4 q[4];
 #pragma unroll
@@ -256,6 +259,20 @@ __global__ void gather_rows2_kernel(const __nv_bfloat16* __restrict__ src_a, lon
 #pragma unroll
       for (int u = 0; u < 4; ++u)
         if (v0 + u * 32 < vpr) o[v0 + u * 32] = q[u];
+    }
+    if (isT) {
+      // J[lo] <= y < J[hi] (J[nJ] beyond every token); y is in J
+      const int y = targets[src];
+      int lo = 0, hi = nJ;
+      while (hi - lo > 1) {  // uniform across the warp
+        const int step = (hi - lo + 31) / 32, p = lo + lane * step;
+        const unsigned le = __ballot_sync(0xffffffffu, p < hi && J[min(p, nJ - 1)] <= y);
+        const int k = 31 - __clz((int)le);  // lane 0's probe, J[lo], always counts
+        const int l2 = lo + k * step;
+        hi = min(hi, l2 + step);
+        lo = l2;
+      }
+      if (lane == 0) ycol[i] = lo;
     }
   }
 }
@@ -270,13 +287,9 @@ __device__ __forceinline__ void lse_merge(float& m, float& s, float m2, float s2
   }
 }
 
-// Per-position losses (zeros off the trainable set) and their sum in a fixed
-// order (fp64), by one block of 256 threads.
-__device__ void finish_body(const float* rowloss, int nT, const int32_t* tpos, int T, float* token_loss,
-                            float* loss) {
+// The losses' sum in a fixed order (fp64), by one block of 256 threads.
+__device__ void finish_body(const float* rowloss, int nT, float* loss) {
   __shared__ double part[256];
-  if (token_loss)
-    for (int t = threadIdx.x; t < T; t += blockDim.x) token_loss[t] = tpos[t] >= 0 ? rowloss[tpos[t]] : 0.f;
   double acc = 0.0;
   for (int i = threadIdx.x; i < nT; i += blockDim.x) acc += (double)rowloss[i];
   part[threadIdx.x] = acc;
@@ -288,108 +301,106 @@ __device__ void finish_body(const float* rowloss, int nT, const int32_t* tpos, i
   if (threadIdx.x == 0) *loss = (float)part[0];
 }
 
-// One block per trainable position i: its log-sum-exp over J from the logits
-// contraction's per-group (max, sum of exp) partials, and its loss
-// lse - z[i, ycol[i]].
-__global__ void __launch_bounds__(256) ce_lse_kernel(const float2* __restrict__ part, int ld_part, int ngroups,
-                                                     const float* __restrict__ Z, int ldz,
-                                                     const int32_t* __restrict__ ycol, float* __restrict__ lse_out,
-                                                     float* rowloss, const int32_t* __restrict__ tpos, int T,
-                                                     float* __restrict__ token_loss, float* __restrict__ loss,
-                                                     int* __restrict__ done) {
+// One block per (trainable position i, chunk of its logits).  It merges the
+// row's log-sum-exp from the logits contraction's per-group (max, sum of exp)
+// partials (every block of a row the same way, so the same bits; its first logits
+// are on their way meanwhile) and writes G[i, :] = bf16(exp(z - lse_i) - [j ==
+// ycol_i]) of its chunk, zeros in [nJ, ldg): one read of the fp32 logits, 16-byte
+// loads and 8-byte stores.  The block of a row's first chunk also writes its loss
+// lse - z[i, ycol[i]]; the last of those to finish sums them.  Rows are cut so that
+// about eight blocks per SM run, in multiples of kGradStep columns: more blocks
+// would repeat the merge.  (As two launches, one for the rows and one for G: 12.2
+// + 9.8 us for 614 positions and 8648 tokens; this 17.5 us.)
+constexpr int kGradStep = 4096;  // four 16-byte loads per thread
+
+__global__ void __launch_bounds__(256) ce_rows_kernel(const float2* __restrict__ part, int ld_part, int ngroups,
+                                                      const float* __restrict__ Z, int ldz, int nJ,
+                                                      const int32_t* __restrict__ ycol, int nT, int chunk,
+                                                      __nv_bfloat16* __restrict__ G, int ldg, float* rowloss,
+                                                      const int32_t* __restrict__ tl, float* __restrict__ token_loss,
+                                                      float* __restrict__ loss, int* __restrict__ done) {
   griddep_wait();
   griddep_launch_dependents();
   __shared__ float sm[8], ss[8];
-  const int i = blockIdx.x;
+  __shared__ int s_last;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int chunks = (ldg + chunk - 1) / chunk;
+  const int i = (int)blockIdx.x / chunks, c = (int)blockIdx.x % chunks;
+  const float* z = Z + (long long)i * ldz;
+  __nv_bfloat16* g = G + (long long)i * ldg;
+  const int j_end = min(ldg, (c + 1) * chunk);
+  float4 q[4];
+  auto fetch = [&](int j0) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int j = j0 + 1024 * u;
+      // ldz >= j + 4: inside the row
+      q[u] = j < nJ && j < j_end ? __ldcs(reinterpret_cast<const float4*>(z + j)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  int j0 = c * chunk + 4 * (int)threadIdx.x;
+  fetch(j0);
   const float2* pr = part + (long long)i * ld_part;
   float m = -INFINITY, s = 0.f;
-  for (int g = threadIdx.x; g < ngroups; g += blockDim.x) {
-    const float2 q = pr[g];
-    lse_merge(m, s, q.x, q.y);
+  for (int p = threadIdx.x; p < ngroups; p += blockDim.x) {
+    const float2 w = pr[p];
+    lse_merge(m, s, w.x, w.y);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const float m2 = __shfl_xor_sync(0xffffffffu, m, o), s2 = __shfl_xor_sync(0xffffffffu, s, o);
     lse_merge(m, s, m2, s2);
   }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (lane == 0) {
     sm[warp] = m;
     ss[warp] = s;
   }
+  const int yc = ycol[i];
   __syncthreads();
-  if (threadIdx.x == 0) {
-    float M = sm[0], S = ss[0];
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) lse_merge(M, S, sm[w], ss[w]);
-    const float lse = M + logf(S);
-    lse_out[i] = lse;
-    rowloss[i] = lse - Z[(long long)i * ldz + ycol[i]];
-  }
-  // the last block to finish (every rowloss written and visible) sums the losses
-  __shared__ int s_last;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(done, 1) == (int)gridDim.x - 1;
-  __syncthreads();
-  if (s_last) {
-    __threadfence();
-    finish_body(rowloss, (int)gridDim.x, tpos, T, token_loss, loss);
-  }
-}
-
-// G[i, :] = bf16(exp(z - lse_i) - [j == ycol_i]) with zeros in [nJ, ldg): one
-// read of the fp32 logits, 16-byte loads and 8-byte stores; work items are
-// (row, 4096-column chunk) pairs over a grid-stride loop.
-constexpr int kGradChunk = 4096;
-
-__global__ void __launch_bounds__(256) ce_grad_kernel(const float* __restrict__ Z, int ldz, int nJ,
-                                                      const int32_t* __restrict__ ycol,
-                                                      const float* __restrict__ lse_in, int nT,
-                                                      __nv_bfloat16* __restrict__ G, int ldg) {
-  griddep_wait();
-  griddep_launch_dependents();
-  const int chunks = (ldg + kGradChunk - 1) / kGradChunk;
-  const long long items = (long long)nT * chunks;
-  for (long long e = blockIdx.x; e < items; e += gridDim.x) {
-    const int i = (int)(e / chunks), c = (int)(e % chunks);
-    const float lse = lse_in[i];
-    const int yc = ycol[i];
-    const float* z = Z + (long long)i * ldz;
-    __nv_bfloat16* g = G + (long long)i * ldg;
-    const int j_end = min(ldg, (c + 1) * kGradChunk);
-#pragma unroll 4
-    for (int j = c * kGradChunk + 4 * (int)threadIdx.x; j < j_end; j += 4 * (int)blockDim.x) {
-      float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (j < nJ) q = __ldcs(reinterpret_cast<const float4*>(z + j));  // ldz >= j + 4: inside the row
-      const float zv[4] = {q.x, q.y, q.z, q.w};
-      float o[4];
+  float M = sm[0], Sm = ss[0];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) o[u] = j + u < nJ ? expf(zv[u] - lse) - (j + u == yc ? 1.f : 0.f) : 0.f;
-      *reinterpret_cast<uint2*>(g + j) = make_uint2(pack_bf16x2(o[0], o[1]), pack_bf16x2(o[2], o[3]));
+  for (int w = 1; w < 8; ++w) lse_merge(M, Sm, sm[w], ss[w]);
+  const float lse = M + logf(Sm);
+  for (; j0 < j_end; j0 += kGradStep) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int j = j0 + 1024 * u;
+      if (j < j_end) {
+        const float zv[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
+        float o[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[e] = j + e < nJ ? expf(zv[e] - lse) - (j + e == yc ? 1.f : 0.f) : 0.f;
+        *reinterpret_cast<uint2*>(g + j) = make_uint2(pack_bf16x2(o[0], o[1]), pack_bf16x2(o[2], o[3]));
+      }
     }
+    if (j0 + kGradStep < j_end) fetch(j0 + kGradStep);
+  }
+  if (c != 0) return;  // uniform across the block
+  if (threadIdx.x == 0) {
+    const float l = lse - z[yc];
+    rowloss[i] = l;
+    if (token_loss) token_loss[tl[i]] = l;
+    __threadfence();
+    s_last = atomicAdd(done, 1) == nT - 1;
+  }
+  __syncthreads();
+  if (s_last) {  // every rowloss is written and visible
+    __threadfence();
+    finish_body(rowloss, nT, loss);
   }
 }
 
-__global__ void __launch_bounds__(256) ce_finish_kernel(const float* __restrict__ rowloss, int nT,
-                                                        const int32_t* __restrict__ tpos, int T,
-                                                        float* __restrict__ token_loss, float* __restrict__ loss) {
-  griddep_wait();
-  griddep_launch_dependents();
-  finish_body(rowloss, nT, tpos, T, token_loss, loss);
-}
-
-__global__ void scatter_rows_kernel(const __nv_bfloat16* __restrict__ src, const int32_t* __restrict__ tpos, int T,
-                                    int d, __nv_bfloat16* __restrict__ dst) {
+// dst[idx[i], :] = src[i, :] for i < n.
+__global__ void scatter_rows_kernel(const __nv_bfloat16* __restrict__ src, const int32_t* __restrict__ idx, int n, int d,
+                                    __nv_bfloat16* __restrict__ dst) {
   griddep_wait();
   griddep_launch_dependents();
   const int vpr = d / 8;
-  const long long total = (long long)T * vpr;
+  const long long total = (long long)n * vpr;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
        e += (long long)gridDim.x * blockDim.x) {
-    const int t = (int)(e / vpr), v = (int)(e % vpr);
-    const int i = tpos[t];
-    const uint4 x = i >= 0 ? reinterpret_cast<const uint4*>(src + (long long)i * d)[v] : make_uint4(0u, 0u, 0u, 0u);
-    reinterpret_cast<uint4*>(dst + (long long)t * d)[v] = x;
+    const int i = (int)(e / vpr), v = (int)(e % vpr);
+    reinterpret_cast<uint4*>(dst + (long long)idx[i] * d)[v] = reinterpret_cast<const uint4*>(src + (long long)i * d)[v];
   }
 }
 
@@ -410,21 +421,23 @@ cudaError_t launch_ce_index(const CeIndex& a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
   }
   const int full = a.topk ? 0 : 1;
-  e = launch_kernel(vocab_count_kernel, dim3(kSegs), dim3(256), 0, st, 1, (const uint8_t*)a.flags, a.V, full,
-                    a.seg_counts);
-  if (e != cudaSuccess) return e;
+  const bool counted = !full && a.V > (1 << 20);
+  if (counted) {
+    e = launch_kernel(vocab_count_kernel, dim3(kSegs), dim3(256), 0, st, 1, (const uint8_t*)a.flags, a.V, full,
+                      a.seg_counts);
+    if (e != cudaSuccess) return e;
+  }
   return launch_kernel(compact_kernel, dim3(kSegs + 1), dim3(kScanThreads), 0, st, 1, (const uint8_t*)a.flags, a.V,
-                       full, (const int32_t*)a.seg_counts, a.mask, a.T, a.J, a.pos, a.tl, a.tpos, a.counts, a.targets,
-                       a.ycol, a.counts + 4);
+                       full, (const int32_t*)(counted ? a.seg_counts : nullptr), a.mask, a.T, a.targets, a.J, a.tl,
+                       a.tpos, a.counts);
 }
 
-cudaError_t launch_gather_rows2(const __nv_bfloat16* src_a, long long ld_a, const int32_t* idx_a, int n_a,
-                                __nv_bfloat16* dst_a, const __nv_bfloat16* src_b, long long ld_b,
-                                const int32_t* idx_b, int n_b, __nv_bfloat16* dst_b, int d, cudaStream_t st) {
-  if (n_b <= 0) return launch_gather_rows(src_a, ld_a, idx_a, n_a, d, dst_a, st);
-  if (n_a <= 0) return launch_gather_rows(src_b, ld_b, idx_b, n_b, d, dst_b, st);
-  return launch_kernel(gather_rows2_kernel, dim3(grid_for(std::max(n_a, n_b), 8, 4096), 2), dim3(256), 0, st, 1,
-                       src_a, ld_a, idx_a, n_a, dst_a, src_b, ld_b, idx_b, n_b, dst_b, d);
+cudaError_t launch_ce_prepare(const CeIndex& a, const __nv_bfloat16* h, const __nv_bfloat16* E, int d,
+                              __nv_bfloat16* ht, __nv_bfloat16* ej, __nv_bfloat16* dh, float* token_loss, int num_sms,
+                              cudaStream_t st) {
+  return launch_kernel(prepare_rows_kernel, dim3(num_sms * 8), dim3(256), 0, st, 1, h, E, d, a.T, a.V,
+                       (const int32_t*)a.tl, (const int32_t*)a.tpos, (const int32_t*)a.J, a.targets,
+                       (const int32_t*)a.counts, ht, ej, a.ycol, dh, token_loss);
 }
 
 cudaError_t launch_gather_rows(const __nv_bfloat16* src, long long ld, const int32_t* idx, int n, int d,
@@ -435,27 +448,23 @@ cudaError_t launch_gather_rows(const __nv_bfloat16* src, long long ld, const int
 }
 
 cudaError_t launch_ce_rows(const float2* lse_part, int ld_part, const float* Z, int ldz, int nJ, const int32_t* ycol,
-                           int nT, float* lse, float* rowloss, const int32_t* tpos, int T, float* token_loss,
-                           float* loss, int* done, __nv_bfloat16* G, int ldg, int num_sms, cudaStream_t st) {
+                           int nT, float* rowloss, const int32_t* tl, float* token_loss, float* loss, int* done,
+                           __nv_bfloat16* G, int ldg, int num_sms, cudaStream_t st) {
   if (nT <= 0) return cudaSuccess;
   const int ngroups = (nJ + gemm_lse_group() - 1) / gemm_lse_group();
-  cudaError_t e = launch_kernel(ce_lse_kernel, dim3(nT), dim3(256), 0, st, 1, lse_part, ld_part, ngroups, Z, ldz,
-                                ycol, lse, rowloss, tpos, T, token_loss, loss, done);
-  if (e != cudaSuccess) return e;
-  const long long items = (long long)nT * ((ldg + kGradChunk - 1) / kGradChunk);
-  const int grid = (int)std::min<long long>(items, (long long)num_sms * 8);
-  return launch_kernel(ce_grad_kernel, dim3(grid), dim3(256), 0, st, 1, Z, ldz, nJ, ycol, lse, nT, G, ldg);
+  // columns per block: rows cut into as many parts as give eight blocks per SM
+  const int steps = (ldg + kGradStep - 1) / kGradStep, parts = std::min(steps, std::max(1, (8 * num_sms + nT - 1) / nT));
+  const int chunk = (steps + parts - 1) / parts * kGradStep;
+  const long long blocks = (long long)nT * ((ldg + chunk - 1) / chunk);
+  return launch_kernel(ce_rows_kernel, dim3((unsigned)blocks), dim3(256), 0, st, 1, lse_part, ld_part, ngroups, Z, ldz,
+                       nJ, ycol, nT, chunk, G, ldg, rowloss, tl, token_loss, loss, done);
 }
 
-cudaError_t launch_ce_finish(const float* rowloss, int nT, const int32_t* tpos, int T, float* token_loss,
-                             float* loss, cudaStream_t st) {
-  return launch_kernel(ce_finish_kernel, dim3(1), dim3(256), 0, st, 1, rowloss, nT, tpos, T, token_loss, loss);
-}
-
-cudaError_t launch_scatter_rows(const __nv_bfloat16* src, const int32_t* tpos, int T, int d, __nv_bfloat16* dst,
+cudaError_t launch_scatter_rows(const __nv_bfloat16* src, const int32_t* idx, int n, int d, __nv_bfloat16* dst,
                                 cudaStream_t st) {
-  return launch_kernel(scatter_rows_kernel, dim3(grid_for((long long)T * (d / 8), 256, 8192)), dim3(256), 0, st, 1,
-                       src, tpos, T, d, dst);
+  if (n <= 0) return cudaSuccess;
+  return launch_kernel(scatter_rows_kernel, dim3(grid_for((long long)n * (d / 8), 256, 8192)), dim3(256), 0, st, 1,
+                       src, idx, n, d, dst);
 }
 
 }  // namespace lora
