@@ -229,6 +229,7 @@ struct Plan {
   std::vector<int> split_f, split_b;
   std::vector<char> small_f, small_b;  // whether they run on the few-rows kernel, and there the CTAs of a
   std::vector<char> cl_f, cl_b;        // cluster that share a tile (1: none)
+  std::vector<char> nar_f, nar_b;      // whether their batch runs on 256 x 256 tiles
   std::vector<size_t> split_off;
   size_t zero_bytes = 0;  // [0, zero_bytes) is cleared at the start of a call that uses tile counters
   bool counters = false;  // a contraction has more tiles than CTA pairs (on kPlanSms SMs): it takes them from a counter
@@ -282,8 +283,10 @@ void gemm_shape(GemmProblem& g, int64_t M, int64_t N, int64_t Kc, int64_t r, int
 
 // The same for the contraction of one projection, whose tile depends on its weight type and on whether it
 // runs on the few-rows kernel.
-void proj_gemm_shape(GemmProblem& g, int64_t M, int64_t N, int64_t Kc, int64_t r, bool q4, bool small) {
-  if (small)
+void proj_gemm_shape(GemmProblem& g, int64_t M, int64_t N, int64_t Kc, int64_t r, bool q4, bool small, bool narrow) {
+  if (narrow)
+    gemm_shape(g, M, N, Kc, r, gemm_tile_n_f32());
+  else if (small)
     gemm_shape(g, M, N, Kc, r, gemm_tile_n_small(), gemm_small_rows());
   else if (q4)
     gemm_shape(g, M, N, Kc, r, gemm_tile_n_q4(), gemm_tile_m_q4());
@@ -311,16 +314,18 @@ constexpr int kPlanPairs = kPlanSms / 2;  // CTA pairs of a launch on all of the
 // partial epilogue, and the reduce launch plus its traffic; the cheapest
 // candidate wins (fewer splits on ties).  Choices are cached per shape set.
 constexpr double kUnitFixBlocks = 3.0;    // per unit: pipeline fill and epilogue
-constexpr double kPartEpiBlocks = 1.0;    // per split unit: fp32 partial tile instead of bf16
+constexpr double kPartEpiBlocks = 6.0;    // per split unit: fp32 partial tile instead of bf16
 constexpr double kReduceFixBlocks = 6.0;  // the reduce launch
 constexpr double kBytesPerBlock = 5.0e6;  // HBM bytes moved in one block time
 
 // A problem's block in those units: a 4-bit problem's 512 x 256 tile holds as many MMAs, half as many when
 // the problem has one 256-row segment only; so does the 256 x 256 tile of fp32 output.
+constexpr double kNarrowBlockCost = 0.75;  // 256 x 256 tiles, bf16: ~820 cycles a block against ~1090 for 256 x 512
 constexpr double kSmallBlockCost = 1.0;  // 128 x 256 tiles of the few-rows kernel, one CTA: the weight stream
 double block_cost(const GemmProblem& g) {
   const bool q4 = g.m_pad == g.num_m_tiles * gemm_tile_m_q4();
   if (g.m_pad == g.num_m_tiles * gemm_small_rows()) return kSmallBlockCost;
+  if (!g.out_f32 && !q4 && g.num_n_tiles > cdiv(g.N, gemm_tile_n())) return kNarrowBlockCost;
   return g.out_f32 ? 0.6 : q4 && g.M <= gemm_tile_m() ? 0.8 : 1.0;
 }
 
@@ -948,7 +953,7 @@ Arena arena(void* ws, const Plan& pl, int phase) {
 }
 
 // ------------------------------------------------------------------ forward
-int add_fwd_problem(GemmBatch& b, const lora_proj& p, const Operands& o, bool small) {
+int add_fwd_problem(GemmBatch& b, const lora_proj& p, const Operands& o, bool small, bool narrow) {
   const lora_shape& s = p.shape;
   const int i = b.num_problems;
   const int64_t T = s.T, K = s.d_in, N = s.d_out, r = s.rank;
@@ -978,14 +983,14 @@ int add_fwd_problem(GemmBatch& b, const lora_proj& p, const Operands& o, bool sm
     return rc;
   if ((rc = make_map(&b.tmOut[i], p.y, N, T, N, 64, 32)) != LORA_OK) return rc;
   GemmProblem& g = b.prob[i];
-  proj_gemm_shape(g, T, N, K, r, is_q4(p), small);
+  proj_gemm_shape(g, T, N, K, r, is_q4(p), small, narrow);
   g.out = mb(p.y);
   add_problem(b);
   return LORA_OK;
 }
 
 // ------------------------------------------------------------------ backward
-int add_bwd_problem(GemmBatch& b, const lora_proj& p, const Operands& o, bool small) {
+int add_bwd_problem(GemmBatch& b, const lora_proj& p, const Operands& o, bool small, bool narrow) {
   const lora_shape& s = p.shape;
   const int i = b.num_problems;
   const int64_t T = s.T, K = s.d_in, N = s.d_out, r = s.rank;
@@ -1012,7 +1017,7 @@ int add_bwd_problem(GemmBatch& b, const lora_proj& p, const Operands& o, bool sm
     return rc;
   if ((rc = make_map(&b.tmOut[i], p.dx, K, T, K, 64, 32)) != LORA_OK) return rc;
   GemmProblem& g = b.prob[i];
-  proj_gemm_shape(g, T, K, N, r, is_q4(p), small);
+  proj_gemm_shape(g, T, K, N, r, is_q4(p), small, narrow);
   g.out = mb(p.dx);
   add_problem(b);
   return LORA_OK;
@@ -1167,7 +1172,7 @@ SideWidths side_widths(int num_sms, const lora_proj* projs, int n) {
     for (int i = 0; i < n; ++i) {
       const lora_shape& sh = projs[i].shape;
       proj_gemm_shape(b.prob[b.num_problems], sh.T, bwd ? sh.d_in : sh.d_out, bwd ? sh.d_out : sh.d_in, sh.rank, q4 != 0,
-                      true);
+                      true, false);
       add_problem(b);
     }
     const int s = small_cluster(b, bwd, q4 != 0, num_sms - side);
@@ -1444,11 +1449,15 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
         b.early_inputs = prior_main ? 1 : 0;
         prior_main = true;
         b.cluster = 8;
+        b.narrow = 1;  // (planned together, unless projections without dx moved others into this launch)
+        for (size_t i = i0; i < order.size() && i < i0 + kMaxProblems; ++i) {
+          b.cluster = std::min(b.cluster, (int)pl.cl_f[order[i]]);
+          b.narrow = std::min(b.narrow, (int)pl.nar_f[order[i]]);
+        }
         int sp[kMaxProblems];
         float* parts[kMaxProblems];
         for (size_t i = i0; i < order.size() && i < i0 + kMaxProblems; ++i) {
-          b.cluster = std::min(b.cluster, (int)pl.cl_f[order[i]]);
-          if ((rc = add_fwd_problem(b, projs[order[i]], ops[order[i]], small)) != LORA_OK) return rc;
+          if ((rc = add_fwd_problem(b, projs[order[i]], ops[order[i]], small, b.narrow != 0)) != LORA_OK) return rc;
           sp[i - i0] = pl.split_f[order[i]];
           parts[i - i0] = at<float>(ws, pl.split_off[order[i]]);
         }
@@ -1492,11 +1501,15 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
         b.early_inputs = prior_main ? 1 : 0;
         prior_main = true;
         b.cluster = 8;
+        b.narrow = 1;  // (planned together, unless projections without dx moved others into this launch)
+        for (size_t i = i0; i < order.size() && i < i0 + kMaxProblems; ++i) {
+          b.cluster = std::min(b.cluster, (int)pl.cl_b[order[i]]);
+          b.narrow = std::min(b.narrow, (int)pl.nar_b[order[i]]);
+        }
         int sp[kMaxProblems];
         float* parts[kMaxProblems];
         for (size_t i = i0; i < order.size() && i < i0 + kMaxProblems; ++i) {
-          b.cluster = std::min(b.cluster, (int)pl.cl_b[order[i]]);
-          if ((rc = add_bwd_problem(b, projs[order[i]], ops[order[i]], small)) != LORA_OK) return rc;
+          if ((rc = add_bwd_problem(b, projs[order[i]], ops[order[i]], small, b.narrow != 0)) != LORA_OK) return rc;
           sp[i - i0] = pl.split_b[order[i]];
           parts[i - i0] = at<float>(ws, pl.split_off[order[i]]);
         }
@@ -1551,6 +1564,8 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
   pl->split_b.assign(n, 1);
   pl->small_f.assign(n, 0);
   pl->small_b.assign(n, 0);
+  pl->nar_f.assign(n, 0);
+  pl->nar_b.assign(n, 0);
   pl->cl_f.assign(n, 1);
   pl->cl_b.assign(n, 1);
   // the side stream's SMs are left out of the contractions they run beside: the
@@ -1590,22 +1605,41 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
         return dir == 0 ? projs[a].shape.d_in > projs[b].shape.d_in : projs[a].shape.d_out > projs[b].shape.d_out;
       });
       for (size_t i0 = 0; i0 < order.size(); i0 += kMaxProblems) {
-        GemmBatch b;
-        memset(&b, 0, sizeof(b));
-        for (size_t i = i0; i < order.size() && i < i0 + kMaxProblems; ++i) {
-          const lora_shape& sh = projs[order[i]].shape;
-          if (dir == 0)
-            proj_gemm_shape(b.prob[b.num_problems], sh.T, sh.d_out, sh.d_in, sh.rank, q4, small);
-          else
-            proj_gemm_shape(b.prob[b.num_problems], sh.T, sh.d_in, sh.d_out, sh.rank, q4, small);
-          add_problem(b);
-        }
+        auto batch = [&](bool narrow) {
+          GemmBatch b;
+          memset(&b, 0, sizeof(b));
+          for (size_t i = i0; i < order.size() && i < i0 + kMaxProblems; ++i) {
+            const lora_shape& sh = projs[order[i]].shape;
+            if (dir == 0)
+              proj_gemm_shape(b.prob[b.num_problems], sh.T, sh.d_out, sh.d_in, sh.rank, q4, small, narrow);
+            else
+              proj_gemm_shape(b.prob[b.num_problems], sh.T, sh.d_in, sh.d_out, sh.rank, q4, small, narrow);
+            add_problem(b);
+          }
+          return b;
+        };
+        GemmBatch b = batch(false);
         int sp[kMaxProblems];
         const int cl = small ? small_cluster(b, dir == 1, q4, workers) : 1;
         choose_splits(b, sp, workers);
-        if (cl > 1)
-          for (int q = 0; q < b.num_problems; ++q) sp[q] = 1;
         if (!allow_split)
+          for (int q = 0; q < b.num_problems; ++q) sp[q] = 1;
+        // 256 x 256 tiles where they finish sooner, below one 256 x 512 tile per pair (3080 x 4104 projection, T =
+        // 1000: 36 wide tiles cut in two, 29.5 us and a 12 us reduce, or 68 narrow ones, 28.5 us)
+        bool narrow = false;
+        if (!q4 && !small && b.total_tiles < pairs) {
+          GemmBatch nb = batch(true);
+          int nsp[kMaxProblems];
+          choose_splits(nb, nsp, workers);
+          if (!allow_split)
+            for (int q = 0; q < nb.num_problems; ++q) nsp[q] = 1;
+          if (simulate_splits(nb, nsp, workers) < simulate_splits(b, sp, workers)) {
+            narrow = true;
+            b = nb;
+            std::copy(nsp, nsp + nb.num_problems, sp);
+          }
+        }
+        if (cl > 1)
           for (int q = 0; q < b.num_problems; ++q) sp[q] = 1;
         long long units = 0;
         for (int q = 0; q < b.num_problems; ++q) {
@@ -1614,6 +1648,7 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
           if (keep) {
             (*keep)[pi] = sp[q];
             (dir == 0 ? pl->cl_f : pl->cl_b)[pi] = (char)cl;
+            (dir == 0 ? pl->nar_f : pl->nar_b)[pi] = narrow ? 1 : 0;
           }
           split_need[pi] = std::max(split_need[pi], split_floats(b.prob[q], sp[q]));
         }

@@ -229,7 +229,7 @@ __device__ __forceinline__ void dequant_stage(uint32_t slot, uint32_t wdst, int 
   }
 }
 
-template <bool kBMn, bool kQ, bool kF32 = false, bool kCS = false>
+template <bool kBMn, bool kQ, bool kF32 = false, bool kCS = false, bool kN256 = false>
 __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __grid_constant__ GemmBatch b) {
   // fp32 output: 256 x 256 tiles whose accumulator alternates between two TMEM
   // buffers, so one tile's epilogue overlaps the next tile's contraction (the
@@ -239,7 +239,9 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
   // halves are summed through distributed shared memory (each pair finishes
   // and stores its own 128 columns): no fp32 partials in global memory, no
   // reduce launch.  For launches with too few tiles to fill the GPU.
-  constexpr bool kNarrow = kF32 || kCS;
+  // kN256 (bf16 output): 256 x 256 tiles with two accumulators as for fp32 output, for launches whose 256 x
+  // 512 tiles would leave pairs idle or have to be cut into partials.
+  constexpr bool kNarrow = kF32 || kCS || kN256;
   static_assert(!kNarrow || !kQ, "256 x 256 tiles: bf16 weights only");
   static_assert(!kF32 || (!kBMn && !kCS), "fp32 output is the plain forward form");
   // segments per tile, one 256 x 256 accumulator each: column halves of a 256 x 512 tile, or with 4-bit
@@ -1224,15 +1226,15 @@ cudaError_t launch_split_reduce(const GemmBatch& batch, cudaStream_t stream) {
 
 size_t fused_gemm_smem_bytes() { return smem_bytes<false>(); }
 
-template <bool kBMn, bool kQ, bool kF32, bool kCS = false>
+template <bool kBMn, bool kQ, bool kF32, bool kCS = false, bool kN256 = false>
 cudaError_t launch_variant(const GemmBatch& batch, int pairs, cudaStream_t stream) {
   constexpr size_t smem = smem_bytes<kQ>();
   static std::atomic<unsigned long long> attr_done{0};
-  const cudaError_t e = set_smem_once(fused_lora_gemm<kBMn, kQ, kF32, kCS>, (int)smem, attr_done);
+  const cudaError_t e = set_smem_once(fused_lora_gemm<kBMn, kQ, kF32, kCS, kN256>, (int)smem, attr_done);
   if (e != cudaSuccess) return e;
   // kCS: one tile per cluster of two pairs; otherwise persistent pairs
   const unsigned grid = kCS ? (unsigned)(4 * batch.total_tiles) : (unsigned)(2 * pairs);
-  return launch_kernel(fused_lora_gemm<kBMn, kQ, kF32, kCS>, dim3(grid), dim3(Cfg<kQ>::kThreads), smem, stream,
+  return launch_kernel(fused_lora_gemm<kBMn, kQ, kF32, kCS, kN256>, dim3(grid), dim3(Cfg<kQ>::kThreads), smem, stream,
                        kCS ? 4 : 2, batch);
 }
 
@@ -1291,6 +1293,9 @@ cudaError_t launch_fused_gemm(const GemmBatch& batch, bool b_mn_major, bool q4, 
   if (q4)
     return b_mn_major ? launch_variant<true, true, false>(batch, pairs, stream)
                       : launch_variant<false, true, false>(batch, pairs, stream);
+  if (batch.narrow)
+    return b_mn_major ? launch_variant<true, false, false, false, true>(batch, pairs, stream)
+                      : launch_variant<false, false, false, false, true>(batch, pairs, stream);
   return b_mn_major ? launch_variant<true, false, false>(batch, pairs, stream)
                     : launch_variant<false, false, false>(batch, pairs, stream);
 }

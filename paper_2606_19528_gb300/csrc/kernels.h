@@ -133,6 +133,7 @@ struct GemmBatch {
   // (the base contraction's operands) were complete before this grid started and its main blocks may
   // be loaded before the previous grid ends; only the adapter slab's activations (su or sv) wait
   int early_inputs;
+  int narrow;   // bf16 weights and output: the tiles are listed with gemm_tile_n_f32() columns
   int cluster;  // few-rows kernel: > 1, clusters of that many CTAs share a tile (one tile per cluster, unsplit)
 };
 

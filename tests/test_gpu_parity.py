@@ -484,7 +484,9 @@ def test_token_shards_sum_to_the_unsharded_gradients():
 # shared by the two CTA pairs of a cluster (halves of the contraction summed in distributed shared
 # memory): ragged tokens and columns, the smallest depth the library cuts this way (8 blocks: the
 # backward of the first shape, 392 + 24 deep), a rank that pads, and a frozen projection.
-CS_SHAPES = [(264, 520, 392, 24), (136, 1032, 520, 3), (512, 3072, 3072, 16), (392, 2056, 1544, 0)]
+# (the last two: 256 x 256 tiles that each pair contracts whole, and a ragged last column tile of 8 columns)
+CS_SHAPES = [(264, 520, 392, 24), (136, 1032, 520, 3), (512, 3072, 3072, 16), (392, 2056, 1544, 0),
+             (1000, 2056, 4104, 12), (264, 3080, 10248, 16)]
 
 
 @pytest.mark.parametrize("T,K,N,r", CS_SHAPES, ids=[f"T{t}_K{k}_N{n}_r{r}" for t, k, n, r in CS_SHAPES])
