@@ -601,29 +601,40 @@ struct Arena {
   size_t n_partials;
 };
 
+struct UnitLen {
+  long long tiles;  // 128-row output tiles of a problem
+  int red, rpad;    // its reduction length and padded rank
+};
+
 constexpr int kMinUnitChunks = 8;  // smallest work unit (64-wide chunks); sizes the partial arenas
 
 // Chunks per unit for a launch.  The persistent grid (max_ctas CTAs) takes
 // units round-robin, so the launch lasts about ceil(units / CTAs) units; the
-// cost of a size is that makespan in chunks, plus a fixed charge for the
-// partial-sum pass when any tile needs several units.  Ties go to the larger
-// unit (fewer partials).
+// cost of a size is that makespan in chunks, plus, when any tile needs several
+// units, the partial sums: 128 rows x the padded rank per unit, written and read
+// again at the CTAs' streaming rate (16 KB per chunk time), and a launch.  Ties
+// go to the larger unit (fewer partials).  (With a flat charge of 4 chunks a
+// width of 18 instead of 22 side SMs cut the column products of the Qwen-shaped
+// layer at T = 4096, r = 64 into partials: 954 against 884 us per step.)
+constexpr double kUnitReduceChunks = 12.0;
+
 template <typename Spec, typename LenFn>
 int choose_unit_chunks(const std::vector<Spec>& specs, size_t i0, size_t i1, int max_ctas, LenFn len) {
   int best = kMinUnitChunks;
-  long long best_cost = -1;
+  double best_cost = -1.0;
   for (int u : {64, 32, 16, 8}) {
     long long units = 0;
-    bool partials = false;
+    double partials = 0.0;
     for (size_t i = i0; i < i1; ++i) {
-      const auto tl = len(specs[i]);  // (tiles, reduction length)
-      const long long upt = cdiv(cdiv(tl.second, 64), u);
-      units += (long long)tl.first * upt;
-      partials = partials || upt > 1;
+      const UnitLen tl = len(specs[i]);
+      const long long upt = cdiv(cdiv(tl.red, 64), u);
+      units += tl.tiles * upt;
+      if (upt > 1) partials += (double)tl.tiles * upt * rank_mma_tile() * tl.rpad * 4.0;
     }
     const long long ctas = std::min<long long>(units, (long long)max_ctas);
-    const long long cost = (units + ctas - 1) / ctas * u + (partials ? 4 : 0);
-    if (best_cost < 0 || cost < best_cost) {
+    const double cost = (double)((units + ctas - 1) / ctas * u) +
+                        (partials > 0.0 ? kUnitReduceChunks + 2.0 * partials / 16384.0 / max_ctas : 0.0);
+    if (best_cost < 0.0 || cost < best_cost) {
       best_cost = cost;
       best = u;
     }
@@ -643,9 +654,9 @@ int launch_rows(const std::vector<RowSpec>& specs, const Arena& ar, const Device
     memset(&b, 0, sizeof(b));
     b.tile_rows = tile;
     b.early_next = early_next ? 1 : 0;
-    // one persistent CTA per SM; (tiles, reduction length) of a row problem
+    // one persistent CTA per SM
     b.unit_chunks = choose_unit_chunks(specs, i0, i1, ctas, [&](const RowSpec& q) {
-      return std::make_pair(cdiv(q.T, tile), q.C);
+      return UnitLen{cdiv(q.T, tile), q.C, rank_pad16(used_rank(q.rw, q.nblk))};
     });
     int rmax = 16;
     for (size_t i = i0; i < i1; ++i) {
@@ -702,9 +713,8 @@ int launch_cols(const std::vector<ColSpec>& specs, const Arena& ar, const Device
     ColBatch b;
     memset(&b, 0, sizeof(b));
     b.tile_rows = tile;
-    // (tiles, reduction length) of a column problem
     b.unit_chunks = choose_unit_chunks(specs, i0, i1, ctas, [&](const ColSpec& q) {
-      return std::make_pair(cdiv(q.C, tile), q.T);
+      return UnitLen{cdiv(q.C, tile), q.T, rank_pad16(used_rank(q.rs, q.nblk))};
     });
     int rmax = 16;
     for (size_t i = i0; i < i1; ++i) {
@@ -714,8 +724,8 @@ int launch_cols(const std::vector<ColSpec>& specs, const Arena& ar, const Device
       p.C = sp.C;
       p.nblk = sp.nblk;
       p.out_cr = sp.out_cr;
-      // X^T tiles: two boxes of 64 columns x 64 tokens
-      if ((rc = make_map(&p.tmX, sp.X, sp.C, sp.T, sp.ldx, 64, 64)) != LORA_OK) return rc;
+      // X^T tiles: boxes of 64 columns x 128 tokens (two chunks)
+      if ((rc = make_map(&p.tmX, sp.X, sp.C, sp.T, sp.ldx, 64, 128)) != LORA_OK) return rc;
       int bytes = tile * 64 * 2;
       for (int k = 0; k < sp.nblk; ++k) {
         p.rs[k] = sp.rs[k];
@@ -1104,7 +1114,7 @@ int call_cluster_tiles(int n, Q4 q4, const lora_proj* projs, bool bwd, int pairs
 // slower per FLOP) it transposes B and su and reads dy once: the fused pass
 // (sv and dB, r <= 16) or the sv pass; the dx contraction waits for sv.
 // Beside the dx contraction it runs dA = sv^T x (2TK bytes per distinct x) and,
-// where the pass over dy was not fused, dB (dy read again, 0.6 x as costly
+// where the pass over dy was not fused, dB (dy read again, 0.3 x as costly
 // per byte).  The rank-r kernels are issue-bound, costlier per byte as r
 // grows.  Each phase gets the share of SMs that ends it with the contraction
 // beside it:
@@ -1113,14 +1123,14 @@ int call_cluster_tiles(int n, Q4 q4, const lora_proj* projs, bool bwd, int pairs
 // partial sums, fp32 gradients).  kappa1 gives the Llama-3.2-3B layer at
 // r = 16 12 SMs, kappa2 8 SMs, the measured best pair at T = 2048; the same
 // constants give 16 / 8 for the Qwen-2.5-3B layer at r = 16 (best measured
-// 16-18 / 8) and 22 / 20 at r = 64 (best 16-20 / 20-24).  Rounded to even
+// 16-18 / 8) and 22 / 16 at r = 64 (18-22 / 16: 851 us, 22 / 22: 862 us).  Rounded to even
 // counts so the contractions keep whole CTA pairs; LORA_SIDE_SMS and
 // LORA_SIDE_SMS2 override.
 constexpr double kSideKappa1 = 290.0;
 constexpr double kSideKappa2 = 245.0;
 constexpr double kSideAdapter1 = 12.0;  // bytes per r N
 constexpr double kSideAdapter2 = 8.0;   // bytes per r K
-constexpr double kSideSecondPass = 0.6;  // the unfused dB pass over dy: its kernel streams faster per byte
+constexpr double kSideSecondPass = 0.3;  // the unfused dB pass over dy: its kernel streams faster per byte
 
 int env_int(const char* name) {
   const char* e = getenv(name);
@@ -1334,7 +1344,7 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
         tj.r[k] = r;
         tj.ld[k] = r;
         tj.r8[k] = rank_pad8(r);
-        tj.max_elems = std::max(tj.max_elems, (long long)rows_ * tj.r8[k]);
+        tj.max_n = std::max(tj.max_n, rows_);
         return LORA_OK;
       };
       for (int i = 0; i < n; ++i) {

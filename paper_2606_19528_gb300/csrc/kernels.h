@@ -199,7 +199,7 @@ struct RowProb {
   __nv_bfloat16* outT[kMaxRankBlocks];
   float scale;
   int rpad;            // concatenated rank, rounded up to 16
-  int tx_bytes;        // bytes one chunk stage receives (X box + rank-side boxes)
+  int tx_bytes;        // bytes of a chunk: one 16 KB X box + rank-side boxes
   int upt;             // work units per 128-token tile (each unit_chunks x 64 columns)
   int unit_begin;      // first unit of this problem in the launch
   int red_begin;       // first element of this problem in the partial-sum pass (upt > 1)
@@ -226,7 +226,7 @@ struct RowBatch {
 // block b sharing X [T, C]; S_b is given transposed, S_b^T [rs_b, T]
 // row-major.  out_cr: out_b[c * rs_b + j] (dB), else out_b[j * C + c] (dA).
 struct ColProb {
-  CUtensorMap tmX;                   // X [T, C]: box 64 columns x 64 tokens, 128-byte swizzle
+  CUtensorMap tmX;                   // X [T, C]: box 64 columns x 128 tokens, 128-byte swizzle
   CUtensorMap tmS[kMaxRankBlocks];   // S_b^T [rs_b, T]: box 64 tokens x pad8(rs_b) rows, 128-byte swizzle
   int T, C;
   int nblk;
@@ -234,7 +234,7 @@ struct ColProb {
   float* out[kMaxRankBlocks];
   int out_cr;
   int rpad;
-  int tx_bytes;        // bytes of a full chunk stage (both X boxes + rank-side boxes)
+  int tx_bytes;        // bytes of a chunk: 16 KB of X + rank-side boxes
   int upt;             // work units per 128-column tile (each unit_chunks x 64 tokens)
   int unit_begin;
   int red_begin;
@@ -301,14 +301,14 @@ cudaError_t launch_colmma(const ColBatch& b, int rmax, int ctas, cudaStream_t st
 cudaError_t launch_reduce_rows(const RowBatch& b, cudaStream_t stream);
 cudaError_t launch_reduce_cols(const ColBatch& b, cudaStream_t stream);
 // Batched transposes: dst_i[j, n] = src_i[n, j] for j < r_i, 0 for r_i <= j < r8_i
-// (src_i [n_i, r_i] with row stride ld_i), every job in one launch.
+// (src_i [n_i, r_i] with row stride ld_i, 16-byte aligned; n_i a multiple of 8), every job in one launch.
 constexpr int kMaxTransposes = 128;
 struct TransposeJobs {
   const __nv_bfloat16* src[kMaxTransposes];
   __nv_bfloat16* dst[kMaxTransposes];
   int n[kMaxTransposes], r[kMaxTransposes], ld[kMaxTransposes], r8[kMaxTransposes];
   int count;
-  long long max_elems;  // largest n_i * r8_i
+  int max_n;  // largest n_i
 };
 cudaError_t launch_transposes(const TransposeJobs& jobs, cudaStream_t stream);
 

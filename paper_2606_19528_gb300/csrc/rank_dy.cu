@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kThreads, 1) rank_dy_kernel(const __grid_const
 
   if (warp == 0) {
     // ---------------------------------------------------------------- producer
-    if (lane == 0) {
+    {
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(kThreads, 1) rank_dy_kernel(const __grid_const
         for (int blk = w.blk0; blk < w.blk1 && ok; ++blk) {
           const int c0 = blk * kCols;
           for (int j = 0; j < w.nt; ++j) {
-            if (!mbar_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, wc, abort_flag)) {
+            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, wc, abort_flag))) {
               ok = false;
               break;
             }
@@ -185,13 +185,16 @@ __global__ void __launch_bounds__(kThreads, 1) rank_dy_kernel(const __grid_const
             const uint32_t xs = base + (uint32_t)stage * G::kStageBytes;
             const uint32_t rs = xs + kDyBytes;
             const int tk = (w.t0 + j) * kTok;
-            mbar_arrive_expect_tx(full, tx);
-            tma_load_2d(xs, &P.tmDy, full, c0, tk);
-            tma_load_2d(xs + kBox, &P.tmDy, full, c0 + 64, tk);
-            tma_load_2d(rs, &P.tmBt, full, c0, 0);
-            tma_load_2d(rs + G::kSideBox, &P.tmBt, full, c0 + 64, 0);
-            tma_load_2d(rs + 2 * G::kSideBox, &P.tmSuT, full, tk, 0);
-            tma_load_2d(rs + 3 * G::kSideBox, &P.tmSuT, full, tk + 64, 0);
+            if (elect_one()) {
+              mbar_arrive_expect_tx(full, tx);
+              tma_load_2d(xs, &P.tmDy, full, c0, tk);
+              tma_load_2d(xs + kBox, &P.tmDy, full, c0 + 64, tk);
+              tma_load_2d(rs, &P.tmBt, full, c0, 0);
+              tma_load_2d(rs + G::kSideBox, &P.tmBt, full, c0 + 64, 0);
+              tma_load_2d(rs + 2 * G::kSideBox, &P.tmSuT, full, tk, 0);
+              tma_load_2d(rs + 3 * G::kSideBox, &P.tmSuT, full, tk + 64, 0);
+            }
+            __syncwarp();
             ++issued;
             if (++stage == G::kStages) {
               stage = 0;
@@ -204,7 +207,11 @@ __global__ void __launch_bounds__(kThreads, 1) rank_dy_kernel(const __grid_const
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
+    // (the whole warp, converged, one elected lane issuing: the operands then come from uniform registers)
+    {
+      auto wait_all = [&](uint32_t bar, uint32_t ph) {
+        return __all_sync(0xffffffffu, mbar_wait(bar, ph, wc, abort_flag)) != 0;
+      };
       int stage = 0;
       uint32_t phase = 0;
       int di = 0;  // dB accumulators used so far
@@ -221,18 +228,18 @@ __global__ void __launch_bounds__(kThreads, 1) rank_dy_kernel(const __grid_const
         const uint32_t idesc_sv = idesc_bf16_f32(kTok, P.rpad, 0, 0);
         const uint32_t idesc_db = idesc_bf16_f32(kCols, P.rpad, 1, 0);
         // the previous unit's sv accumulators must be read out first
-        if (!mbar_wait(smem_u32(&ctl->sempty), (uint32_t)((ui & 1) ^ 1), wc, abort_flag)) break;
+        if (!wait_all(smem_u32(&ctl->sempty), (uint32_t)((ui & 1) ^ 1))) break;
         tc_fence_after();
         for (int blk = w.blk0; blk < w.blk1 && ok; ++blk, ++di) {
           const int buf = di & 1;
-          if (!mbar_wait(smem_u32(&ctl->dempty[buf]), (uint32_t)(((di >> 1) & 1) ^ 1), wc, abort_flag)) {
+          if (!wait_all(smem_u32(&ctl->dempty[buf]), (uint32_t)(((di >> 1) & 1) ^ 1))) {
             ok = false;
             break;
           }
           tc_fence_after();
           const uint32_t d_db = tmem_base + (uint32_t)((G::kTilesMax + buf) * R);
           for (int j = 0; j < w.nt; ++j) {
-            if (!mbar_wait(smem_u32(&ctl->full[stage]), phase, wc, abort_flag)) {
+            if (!wait_all(smem_u32(&ctl->full[stage]), phase)) {
               ok = false;
               break;
             }
@@ -245,33 +252,38 @@ __global__ void __launch_bounds__(kThreads, 1) rank_dy_kernel(const __grid_const
             const uint64_t a_db = desc_db_a + soff, b_db = desc_db_b + soff;
             const uint32_t d_sv = tmem_base + (uint32_t)(j * R);
             const uint32_t acc_sv = blk != w.blk0 ? 1u : 0u, acc_db = j != 0 ? 1u : 0u;
+            if (elect_one()) {
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-              // sv: 16 columns of dy per step (K-major, box k / 4) against the same columns of B^T
-              const uint32_t bx = (uint32_t)(k >> 2), kk = (uint32_t)(k & 3) * 32u;
-              umma_bf16(d_sv, a_sv + ((bx * kBox + kk) >> 4), b_sv + ((bx * G::kSideBox + kk) >> 4), idesc_sv,
-                        k != 0 ? 1u : acc_sv);
-            }
+              for (int k = 0; k < 8; ++k) {
+                // sv: 16 columns of dy per step (K-major, box k / 4) against the same columns of B^T
+                const uint32_t bx = (uint32_t)(k >> 2), kk = (uint32_t)(k & 3) * 32u;
+                umma_bf16(d_sv, a_sv + ((bx * kBox + kk) >> 4), b_sv + ((bx * G::kSideBox + kk) >> 4), idesc_sv,
+                          k != 0 ? 1u : acc_sv);
+              }
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-              // dB: 16 tokens of dy per step (MN-major: the two 64-column boxes kBox apart)
-              // against the same tokens of su^T
-              const uint32_t bx = (uint32_t)(k >> 2), kk = (uint32_t)(k & 3) * 32u;
-              umma_bf16(d_db, a_db + (((uint32_t)k * 2048u) >> 4), b_db + ((bx * G::kSideBox + kk) >> 4), idesc_db,
-                        k != 0 ? 1u : acc_db);
+              for (int k = 0; k < 8; ++k) {
+                // dB: 16 tokens of dy per step (MN-major: the two 64-column boxes kBox apart)
+                // against the same tokens of su^T
+                const uint32_t bx = (uint32_t)(k >> 2), kk = (uint32_t)(k & 3) * 32u;
+                umma_bf16(d_db, a_db + (((uint32_t)k * 2048u) >> 4), b_db + ((bx * G::kSideBox + kk) >> 4), idesc_db,
+                          k != 0 ? 1u : acc_db);
+              }
+              umma_commit(smem_u32(&ctl->empty[stage]));
             }
+            __syncwarp();
             issued_any = true;
-            umma_commit(smem_u32(&ctl->empty[stage]));
             if (++stage == G::kStages) {
               stage = 0;
               phase ^= 1u;
             }
           }
           if (!ok) break;
-          umma_commit(smem_u32(&ctl->dfull[buf]));
+          if (elect_one()) umma_commit(smem_u32(&ctl->dfull[buf]));
+          __syncwarp();
         }
         if (!ok) break;
-        umma_commit(smem_u32(&ctl->sfull));
+        if (elect_one()) umma_commit(smem_u32(&ctl->sfull));
+        __syncwarp();
       }
     }
   } else {

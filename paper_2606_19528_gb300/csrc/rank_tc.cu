@@ -14,18 +14,23 @@
 // M = 128 x N = rank x K = 16 with A = the X tile (K-major for row products;
 // MN-major, straight from X's row-major layout, for column products) and B =
 // the rank-side tile (always K-major).
-// Per CTA (persistent, one per SM): warp 0 streams X tiles (16 KB) and the
-// matching rank-side tiles by TMA into a deep ring of shared-memory stages;
+// Per CTA (persistent, one per SM): warp 0 streams X tiles (two 16 KB boxes a
+// stage) and the matching rank-side tiles by TMA into a ring of 3 to 6 stages;
 // one thread of warp 1 issues tcgen05.mma into a TMEM accumulator; warps 2..5
 // read the accumulator back (one output row per thread) and write the
 // outputs, or fp32 partials when a tile's reduction spans several work units
 // (summed in unit order by a second pass, so results never depend on
 // scheduling).  Two accumulators let the read-back of one unit overlap the
 // next unit's loads and MMAs.  The MMAs are tiny (N = rank), and a stream of
-// them from one thread takes ~47 cycles per MMA whatever N up to 64; one CTA
-// streams X at ~45-60 GB/s, bounded by the X bytes its ring keeps in flight
-// (16 KB boxes, 8 stages) against the load latency, so these kernels fill the
-// HBM bandwidth only on many SMs.  Every wait is bounded.
+// them from one thread takes ~47 cycles per MMA whatever N up to 64.  One CTA
+// streams X at 55-90 GB/s, so these kernels fill the HBM bandwidth only on many
+// SMs.  What bounds it is work per stage, in the producer and in the MMA thread:
+// dA of the Llama-shaped layer at T = 2048 (71 MB) took 157 us on 8 SMs with one
+// chunk per stage and one thread issuing its two to four copies, 136 us with the
+// copies issued by an elected lane of a converged warp, 100 us with two chunks
+// per stage (column products: 16 KB boxes of 128 tokens instead of 8 KB ones).
+// (Electing the MMA issuer in the same way gained nothing here, with 8 MMAs per
+// stage; the pass over dy, with 16, gained 15 %.)  Every wait is bounded.
 #include "rank_store.cuh"
 
 namespace lora {
@@ -33,22 +38,25 @@ namespace lora {
 namespace {
 
 constexpr int kRows = 128;                        // output rows per tile = TMEM lanes
-constexpr int kChunk = 64;                        // reduction length per stage
-constexpr uint32_t kXBytes = kRows * kChunk * 2;  // 16 KB
-constexpr uint32_t kXHalf = kXBytes / 2;          // one 64 x 64 box of a column product
+constexpr int kChunk = 64;                        // reduction length of a chunk; a stage holds two
+constexpr uint32_t kXBytes = kRows * kChunk * 2;  // one box: 128 rows x 64 (column products: 64 columns x 128 tokens)
 constexpr int kThreads = 192;
 constexpr long long kDrainNs = 1000000000ll;
 
 template <int R>
 struct TcRing {
-  static constexpr uint32_t kStageBytes = (kXBytes + 128u * R + 1023u) & ~1023u;
-  static constexpr int kStages = (int)(196608u / kStageBytes) < 12 ? (int)(196608u / kStageBytes) : 12;
+  static constexpr uint32_t kSide = 128u * R;  // rank side of a chunk
+  static constexpr uint32_t kStageBytes = (2u * (kXBytes + kSide) + 1023u) & ~1023u;
+  static constexpr int kStages = (int)(225u * 1024u / kStageBytes);
+  static_assert(kStages >= 3 && kStages <= 6, "ring");
   static constexpr uint32_t kTmemCols = 2 * R <= 32 ? 32 : 2 * R;  // two accumulators, power of two
 };
 
+constexpr int kMaxStages = 6;
+
 struct __align__(8) TcCtl {
-  uint64_t full[12];
-  uint64_t empty[12];
+  uint64_t full[kMaxStages];
+  uint64_t empty[kMaxStages];
   uint64_t tfull[2];
   uint64_t tempty[2];
   uint64_t drain;
@@ -133,7 +141,9 @@ __global__ void __launch_bounds__(kThreads, 1) rank_mma_kernel(const __grid_cons
 
   if (warp == 0) {
     // ---------------------------------------------------------------- producer
-    if (lane == 0) {
+    // (the whole warp, converged, one elected lane issuing: the copies then take their operands from uniform
+    // registers; one thread spent 320 to 420 cycles on the two or three copies of a stage)
+    {
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
@@ -146,28 +156,37 @@ __global__ void __launch_bounds__(kThreads, 1) rank_mma_kernel(const __grid_cons
         const int nch = (min(S::red(P), k_begin + b.unit_chunks * kChunk) - k_begin + kChunk - 1) / kChunk;
         // a column tile whose second half lies past C loads only the first box
         const bool hi = !kCol || r0 + kChunk < S::rows(P);
-        const uint32_t tx = (uint32_t)P.tx_bytes - (hi ? 0u : kXHalf);
-        for (int ch = 0; ch < nch; ++ch) {
-          if (!mbar_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, wc, abort_flag)) {
+        for (int ch = 0; ch < nch; ch += 2) {
+          const int nsub = min(2, nch - ch);
+          // column products: boxes of 128 tokens whatever is left of them (zeros past T)
+          const uint32_t tx = (kCol ? (hi ? 2u : 1u) : (uint32_t)nsub) * kXBytes +
+                              (uint32_t)nsub * ((uint32_t)P.tx_bytes - kXBytes);
+          if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, wc, abort_flag))) {
             ok = false;
             break;
           }
           const uint32_t full = smem_u32(&ctl->full[stage]);
           const uint32_t xs = base + (uint32_t)stage * G::kStageBytes;
           const int k0 = k_begin + ch * kChunk;
-          mbar_arrive_expect_tx(full, tx);
-          if constexpr (kCol) {
-            // X^T as an MN-major operand: two 64-column x 64-token boxes
-            tma_load_2d(xs, &P.tmX, full, r0, k0);
-            if (hi) tma_load_2d(xs + kXHalf, &P.tmX, full, r0 + kChunk, k0);
-          } else {
-            tma_load_2d(xs, &P.tmX, full, k0, r0);
+          if (elect_one()) {
+            mbar_arrive_expect_tx(full, tx);
+            if constexpr (kCol) {
+              // X^T as an MN-major operand: two 64-column x 128-token boxes
+              tma_load_2d(xs, &P.tmX, full, r0, k0);
+              if (hi) tma_load_2d(xs + kXBytes, &P.tmX, full, r0 + kChunk, k0);
+            } else {
+              tma_load_2d(xs, &P.tmX, full, k0, r0);
+              if (nsub > 1) tma_load_2d(xs + kXBytes, &P.tmX, full, k0 + kChunk, r0);
+            }
+            int off = 0;
+            for (int k = 0; k < P.nblk; ++k) {
+              const uint32_t rs = xs + 2u * kXBytes + (uint32_t)off * 128u;
+              tma_load_2d(rs, S::rmap(P, k), full, k0, 0);
+              if (nsub > 1) tma_load_2d(rs + G::kSide, S::rmap(P, k), full, k0 + kChunk, 0);
+              off += pad8(S::rank(P, k));
+            }
           }
-          int off = 0;
-          for (int k = 0; k < P.nblk; ++k) {
-            tma_load_2d(xs + kXBytes + (uint32_t)off * 128u, S::rmap(P, k), full, k0, 0);
-            off += pad8(S::rank(P, k));
-          }
+          __syncwarp();
           ++issued;
           if (++stage == G::kStages) {
             stage = 0;
@@ -184,10 +203,10 @@ __global__ void __launch_bounds__(kThreads, 1) rank_mma_kernel(const __grid_cons
       uint32_t phase = 0;
       int it = 0;
       bool ok = true;
-      // stage 0's operand descriptors: X (K-major rows, or MN-major with the boxes kXHalf apart)
-      // and the rank side after it
-      const uint64_t desc_a = kCol ? sw128_desc(base, kXHalf, 1024) : sw128_desc(base, 16, 1024);
-      const uint64_t desc_b = sw128_desc(base + kXBytes, 16, 1024);
+      // stage 0's operand descriptors: X (K-major rows, or MN-major with the boxes kXBytes
+      // apart) and the rank side after it
+      const uint64_t desc_a = kCol ? sw128_desc(base, kXBytes, 1024) : sw128_desc(base, 16, 1024);
+      const uint64_t desc_b = sw128_desc(base + 2u * kXBytes, 16, 1024);
       for (int u = blockIdx.x; u < b.units && ok; u += gridDim.x, ++it) {
         int pi, tile, piece;
         decode_unit(b, u, pi, tile, piece);
@@ -199,7 +218,7 @@ __global__ void __launch_bounds__(kThreads, 1) rank_mma_kernel(const __grid_cons
         if (!mbar_wait(smem_u32(&ctl->tempty[acc]), (uint32_t)(((it >> 1) & 1) ^ 1), wc, abort_flag)) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * R);
-        for (int ch = 0; ch < nch; ++ch) {
+        for (int ch = 0; ch < nch; ch += 2) {
           if (!mbar_wait(smem_u32(&ctl->full[stage]), phase, wc, abort_flag)) {
             ok = false;
             break;
@@ -209,11 +228,15 @@ __global__ void __launch_bounds__(kThreads, 1) rank_mma_kernel(const __grid_cons
           // low 14 bits of the descriptor; shared-memory offsets never carry out of them)
           const uint32_t soff = (uint32_t)stage * (G::kStageBytes >> 4);
           const uint64_t ad = desc_a + soff, bd = desc_b + soff;
+          const bool two = ch + 1 < nch;
 #pragma unroll
-          for (int k = 0; k < kChunk / 16; ++k) {
-            // MN-major A: 16 reduction rows of 128 B per step, the two 64-wide boxes 8 KB apart
-            umma_bf16(d_tmem, ad + (uint32_t)(kCol ? k * 128 : k * 2), bd + (uint32_t)(k * 2), idesc,
-                      (ch | k) != 0 ? 1u : 0u);
+          for (int k = 0; k < 2 * kChunk / 16; ++k) {
+            if (k >= kChunk / 16 && !two) break;
+            // second chunk: the next box of X rows (column products: the same boxes' tokens 64 on), the next
+            // rank side; MN-major A: 16 reduction rows of 128 B per step
+            const uint32_t sub = (uint32_t)k / (kChunk / 16), kk = (uint32_t)k % (kChunk / 16);
+            umma_bf16(d_tmem, ad + (kCol ? (uint32_t)k * 128u : sub * (kXBytes >> 4) + kk * 2u),
+                      bd + sub * (G::kSide >> 4) + kk * 2u, idesc, (ch | k) != 0 ? 1u : 0u);
           }
           issued_any = true;
           umma_commit(smem_u32(&ctl->empty[stage]));
