@@ -1487,7 +1487,7 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
   if (mode & LORA_BWD) {
     // (a forward-and-backward call without the side stream runs it here too, on every SM)
     if (!(mode == LORA_FWD_BWD && ov.on)) {
-      if ((rc = bwd_rank(st, d->num_sms, ov.on ? ov.side : st, !ov.on && small_bwd)) != LORA_OK) return rc;
+      if ((rc = bwd_rank(st, d->num_sms, ov.on ? ov.side : st, mode == LORA_BWD)) != LORA_OK) return rc;
       if (ov.on && (rc = bwd_cols(ov.side, ov.side_ctas2)) != LORA_OK) return rc;
       if (any_adapter(projs, n)) prior_main = true;  // the pass over dy or the row products ran here
     }
