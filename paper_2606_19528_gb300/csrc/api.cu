@@ -1266,6 +1266,7 @@ struct Overlap {
   }
   // what follows on the side stream comes after the main stream's work so far
   int side_after_main() {
+    forked = true;
     return cudaEventRecord(ev_fwd, main) == cudaSuccess && cudaStreamWaitEvent(side, ev_fwd, 0) == cudaSuccess
                ? LORA_OK
                : LORA_ECUDA;
@@ -1325,6 +1326,37 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
   std::vector<bf*> sut(n), svt(n);
   std::vector<char> fused(n);
   // early_next: the dx contraction follows on the same stream and may start beside these
+  // rank sides as K-major tensor-core operands: B^T for sv = s dy B (bit 0 of `which`) and su^T for dB =
+  // dy^T su (bit 1), zero rows past r
+  auto transposes = [&](cudaStream_t rs, int which) -> int {
+    ProfScope ps(LORA_KERNEL_PAD, rs);
+    TransposeJobs tj;
+    memset(&tj, 0, sizeof(tj));
+    for (int i = 0; i < n; ++i) {
+      const lora_proj& p = projs[i];
+      const int T = (int)p.shape.T, N = (int)p.shape.d_out, r = (int)p.shape.rank;
+      if (r == 0) continue;  // frozen: dx = dy W only
+      for (int w = 0; w < 2; ++w) {
+        if (!((which >> w) & 1)) continue;
+        if (tj.count == kMaxTransposes) {
+          if (launch_transposes(tj, rs) != cudaSuccess) return LORA_ECUDA;
+          memset(&tj, 0, sizeof(tj));
+        }
+        const int k = tj.count++, rows = w == 0 ? N : T;
+        tj.src[k] = w == 0 ? cb(p.B) : cb(p.su);
+        tj.dst[k] = at<bf>(W_(i), w == 0 ? plans[i].bt : plans[i].sut);
+        tj.n[k] = rows;
+        tj.r[k] = r;
+        tj.ld[k] = r;
+        tj.r8[k] = rank_pad8(r);
+        tj.max_n = std::max(tj.max_n, rows);
+      }
+    }
+    return launch_transposes(tj, rs) == cudaSuccess ? LORA_OK : LORA_ECUDA;
+  };
+  long long bt_elems = 0;
+  for (int i = 0; i < n; ++i) bt_elems += projs[i].shape.d_out * rank_pad8((int)projs[i].shape.rank);
+  const bool bt_early = bt_elems >= (1 << 17);
   auto bwd_rank = [&](cudaStream_t rs, int ctas, cudaStream_t rs2, bool early_next) -> int {
     int rc;
     std::vector<RowSpec> rows;
@@ -1333,27 +1365,11 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
       fused[i] = projs[i].shape.rank > 0 &&
                  dy_fusable((int)projs[i].shape.T, (int)projs[i].shape.d_out, (int)projs[i].shape.rank);
     std::vector<Operands>& ops = bops;
-    TransposeJobs tj;
-    memset(&tj, 0, sizeof(tj));
+    // (with the side stream the forward made su^T already, and a large B^T)
+    if (rs == st || !bt_early) {
+      if ((rc = transposes(rs, rs == st ? 3 : 1)) != LORA_OK) return rc;
+    }
     {
-      ProfScope ps(LORA_KERNEL_PAD, rs);
-      // rank sides as K-major tensor-core operands: B^T for sv = s dy B and
-      // su^T for dB = dy^T su, zero rows past r
-      auto transpose = [&](const bf* src, int rows_, int r, bf* dst) -> int {
-        if (tj.count == kMaxTransposes) {
-          if (launch_transposes(tj, rs) != cudaSuccess) return LORA_ECUDA;
-          memset(&tj, 0, sizeof(tj));
-        }
-        const int k = tj.count++;
-        tj.src[k] = src;
-        tj.dst[k] = dst;
-        tj.n[k] = rows_;
-        tj.r[k] = r;
-        tj.ld[k] = r;
-        tj.r8[k] = rank_pad8(r);
-        tj.max_n = std::max(tj.max_n, rows_);
-        return LORA_OK;
-      };
       for (int i = 0; i < n; ++i) {
         const lora_proj& p = projs[i];
         const int T = (int)p.shape.T, N = (int)p.shape.d_out, r = (int)p.shape.rank, r8 = rank_pad8(r);
@@ -1361,8 +1377,6 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
         bf* bt = at<bf>(W_(i), plans[i].bt);
         sut[i] = at<bf>(W_(i), plans[i].sut);
         svt[i] = at<bf>(W_(i), plans[i].svt);
-        if ((rc = transpose(cb(p.B), N, r, bt)) != LORA_OK) return rc;
-        if ((rc = transpose(cb(p.su), T, r, sut[i])) != LORA_OK) return rc;
         bf* sv = at<bf>(W_(i), plans[i].sv);
         if (fused[i])
           dys.push_back(DySpec{cb(p.dy), T, N, r, p.shape.scale, bt, sut[i], sv, svt[i], p.dB});
@@ -1371,7 +1385,6 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
         ops[i].s_in = sv;
         ops[i].ld_s = r8;
       }
-      if (launch_transposes(tj, rs) != cudaSuccess) return LORA_ECUDA;
     }
     {
       // sv (and dB where fused) before the event the dx contraction waits for
@@ -1408,6 +1421,12 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
     return LORA_OK;
   };
   if (mode & LORA_FWD) {
+    // The pass over dy needs B^T and su^T.  The row products write su^T beside su; B^T is made on the side
+    // stream while they run, or after them where it is small: the events that start the side stream with the
+    // call cost the main stream about 2 us (Qwen layer T = 32, r = 4, 229k elements: 92.9 us after, 86.4 us
+    // beside; 4-bit Llama layer T = 64, q and v, 65k elements: 80.8 and 83.3 us).
+    if (ov.on && bt_early && ((rc = ov.side_after_main()) != LORA_OK || (rc = transposes(ov.side, 1)) != LORA_OK))
+      return rc;
     std::vector<Operands> ops(n);
     std::vector<RowSpec> rows;
     {
@@ -1421,8 +1440,8 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
         bf* su_gemm = (p.su && !pad) ? mb(p.su) : at<bf>(W_(i), plans[i].su_pad);
         const int ld_gemm = (p.su && !pad) ? r : r8;
         bf* su_user2 = (p.su && pad) ? mb(p.su) : nullptr;
-        add_row_block(rows, cb(p.x), K, T, K, p.shape.scale, cb(p.A), K, r, su_gemm, ld_gemm, su_user2, r, nullptr,
-                      true);
+        add_row_block(rows, cb(p.x), K, T, K, p.shape.scale, cb(p.A), K, r, su_gemm, ld_gemm, su_user2, r,
+                      ov.on ? at<bf>(W_(i), plans[i].sut) : nullptr, true);
         ops[i].s_in = su_gemm;
         ops[i].ld_s = ld_gemm;
         if (pad) {

@@ -10,45 +10,44 @@ namespace lora {
 
 namespace {
 
-// Second pass: out = sum of a tile's unit partials, in unit order.  One
-// thread per 4 consecutive elements of [tile][tile_rows][rpad] of every
-// problem with several units (rpad is a multiple of 16, so the 4 share a
-// row); the loads of all units are independent and issued together.
+// Second pass: out = sum of a tile's unit partials, in unit order.  One thread
+// per 8 consecutive rank columns (a sector of each partial) of one row of
+// [tile][tile_rows][rpad], lanes along the rows, so that the transposed outputs
+// (su^T, sv^T and dA) are stored in whole lines; the loads of all units are
+// independent and issued together.
 template <typename Batch, bool kRow>
-__global__ void __launch_bounds__(256) reduce_partials_kernel(const __grid_constant__ Batch b, int total4) {
+__global__ void __launch_bounds__(256) reduce_partials_kernel(const __grid_constant__ Batch b, int total8) {
   if (b.early_next) griddep_launch_dependents();
   griddep_wait();
   if (!b.early_next) griddep_launch_dependents();
-  const int i4 = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i4 >= total4) return;
-  const int i = i4 * 4;
+  const int i8 = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i8 >= total8) return;
   int pi = 0;
-  while (pi + 1 < b.n && i >= (int)b.p[pi + 1].red_begin) ++pi;
+  while (pi + 1 < b.n && i8 >= (int)b.p[pi + 1].red_begin / 8) ++pi;
   const auto& P = b.p[pi];
-  const int e = i - P.red_begin;
-  const int rpad = P.rpad, upt = P.upt;
-  const int blk = b.tile_rows * rpad;
-  const int tile = e / blk, k = e % blk;
-  const float4* src = reinterpret_cast<const float4*>(b.partials + P.part_off + (size_t)tile * upt * blk + k);
-  const size_t stride4 = (size_t)blk / 4;
-  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 8
+  const int e = i8 - P.red_begin / 8;
+  const int rpad = P.rpad, upt = P.upt, tr = b.tile_rows;
+  const int per = tr * (rpad / 8);  // threads of a tile
+  const int tile = e / per, k = e % per;
+  const int j = k / tr * 8, lr = k % tr;
+  const size_t blk = (size_t)tr * rpad;
+  const float* src = b.partials + P.part_off + (size_t)tile * upt * blk + (size_t)lr * rpad + j;
+  float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
   for (int u = 0; u < upt; ++u) {
-    const float4 w = __ldcg(src + (size_t)u * stride4);
-    v.x += w.x;
-    v.y += w.y;
-    v.z += w.z;
-    v.w += w.w;
+    const float4 lo = __ldcg(reinterpret_cast<const float4*>(src + (size_t)u * blk));
+    const float4 hi = __ldcg(reinterpret_cast<const float4*>(src + (size_t)u * blk) + 1);
+    v[0] += lo.x, v[1] += lo.y, v[2] += lo.z, v[3] += lo.w;
+    v[4] += hi.x, v[5] += hi.y, v[6] += hi.z, v[7] += hi.w;
   }
-  const int row = tile * b.tile_rows + k / rpad, j = k % rpad;
-  const float vv[4] = {v.x, v.y, v.z, v.w};
+  uint32_t w[8];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    if constexpr (kRow) {
-      if (row < P.T) row_store(P, row, j + q, vv[q]);
-    } else {
-      if (row < P.C) col_store(P, row, j + q, vv[q]);
-    }
+  for (int q = 0; q < 8; ++q) w[q] = __float_as_uint(v[q]);
+  const int row = tile * tr + lr;
+  if constexpr (kRow) {
+    if (row < P.T) row_store8(P, row, j, w);
+  } else {
+    if (row < P.C) col_store8(P, row, j, w);
   }
 }
 
@@ -141,9 +140,9 @@ cudaError_t launch_transposes(const TransposeJobs& jobs, cudaStream_t st) {
 
 cudaError_t launch_reduce_rows(const RowBatch& b, cudaStream_t st) {
   if (b.red_total <= 0) return cudaSuccess;
-  const int total4 = b.red_total / 4;
-  return launch_kernel(reduce_partials_kernel<RowBatch, true>, dim3((total4 + 255) / 256), dim3(256), 0, st, 1, b,
-                       total4);
+  const int total8 = b.red_total / 8;
+  return launch_kernel(reduce_partials_kernel<RowBatch, true>, dim3((total8 + 255) / 256), dim3(256), 0, st, 1, b,
+                       total8);
 }
 
 cudaError_t launch_wait_probe(int* status, long long limit_ns, cudaStream_t st) {
@@ -152,9 +151,9 @@ cudaError_t launch_wait_probe(int* status, long long limit_ns, cudaStream_t st) 
 
 cudaError_t launch_reduce_cols(const ColBatch& b, cudaStream_t st) {
   if (b.red_total <= 0) return cudaSuccess;
-  const int total4 = b.red_total / 4;
-  return launch_kernel(reduce_partials_kernel<ColBatch, false>, dim3((total4 + 255) / 256), dim3(256), 0, st, 1, b,
-                       total4);
+  const int total8 = b.red_total / 8;
+  return launch_kernel(reduce_partials_kernel<ColBatch, false>, dim3((total8 + 255) / 256), dim3(256), 0, st, 1, b,
+                       total8);
 }
 
 cudaError_t launch_pad_cols(const __nv_bfloat16* src, int rows, int r, __nv_bfloat16* dst, int ld_dst,

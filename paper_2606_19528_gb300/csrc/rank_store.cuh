@@ -27,35 +27,13 @@ __device__ __forceinline__ int find_block(const int* rw, int nblk, int j, int* j
   return -1;
 }
 
-// Row product element (t, j), unscaled: bf16 of scale * v into out [T, ld_out],
-// the optional copy out2 and the optional transposed copy outT [pad8(r), T];
-// the padding columns j in [r, pad8(r)) are written as zeros.
-__device__ __forceinline__ void row_store(const RowProb& P, int t, int j, float v) {
-  int jj;
-  const int b = find_block(P.rw, P.nblk, j, &jj);
-  if (b < 0) return;
-  const __nv_bfloat16 o = __float2bfloat16_rn(jj < P.rw[b] ? P.scale * v : 0.f);
-  if (jj < P.ld_out[b]) P.out[b][(size_t)t * P.ld_out[b] + jj] = o;
-  if (P.out2[b] != nullptr && jj < P.ld_out2[b]) P.out2[b][(size_t)t * P.ld_out2[b] + jj] = o;
-  if (P.outT[b] != nullptr) P.outT[b][(size_t)jj * P.T + t] = o;
-}
-
-// Column product element (c, j) in fp32: out [C, r] (out_cr) or [r, C].
-__device__ __forceinline__ void col_store(const ColProb& P, int c, int j, float v) {
-  int jj;
-  const int b = find_block(P.rs, P.nblk, j, &jj);
-  if (b < 0 || jj >= P.rs[b]) return;
-  if (P.out_cr)
-    P.out[b][(size_t)c * P.rs[b] + jj] = v;
-  else
-    P.out[b][(size_t)jj * P.C + c] = v;
-}
-
 __device__ __forceinline__ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-// Row product elements (t, j .. j + 7), j a multiple of 8 (so one rank block
-// holds all eight): as row_store, with one 16-byte store per output row where
-// its layout allows.
+// Row product elements (t, j .. j + 7), unscaled, j a multiple of 8 (so one rank
+// block holds all eight): bf16 of scale * v into out [T, ld_out], the optional
+// copy out2 and the optional transposed copy outT [pad8(r), T]; the padding
+// columns in [r, pad8(r)) are written as zeros.  One 16-byte store per output row
+// where its layout allows.
 __device__ __forceinline__ void row_store8(const RowProb& P, int t, int j, const uint32_t* v) {
   int jj;
   const int b = find_block(P.rw, P.nblk, j, &jj);
@@ -85,8 +63,8 @@ __device__ __forceinline__ void row_store8(const RowProb& P, int t, int j, const
     for (int e = 0; e < 8; ++e) P.outT[b][(size_t)(jj + e) * P.T + t] = o[e];
 }
 
-// Column product elements (c, j .. j + 7), j a multiple of 8: as col_store,
-// with 16-byte stores into the [C, r] layout where it allows.
+// Column product elements (c, j .. j + 7) in fp32, j a multiple of 8: out [C, r]
+// (out_cr), with 16-byte stores where it allows, or [r, C].
 __device__ __forceinline__ void col_store8(const ColProb& P, int c, int j, const uint32_t* v) {
   int jj;
   const int b = find_block(P.rs, P.nblk, j, &jj);
