@@ -1989,7 +1989,8 @@ int topk_check(const lora_bf16* E, int64_t V, int64_t d, int64_t k, TopkPlan* pl
     return o;
   };
   // zeroed at the start of a call: tile counters, status, fallback count, candidate counts
-  const int nctr = pl->sampled ? pl->sblocks + pl->achunks + pl->fmax : pl->chunks;
+  // (short rows: per chunk a tile counter and the counts of rows for the block sort and the radix select)
+  const int nctr = pl->sampled ? pl->sblocks + pl->achunks + pl->fmax : 3 * pl->chunks;
   pl->counters = take((size_t)nctr * 4);
   pl->status = take(4);
   pl->fail_count = take(4);
@@ -2000,6 +2001,12 @@ int topk_check(const lora_bf16* E, int64_t V, int64_t d, int64_t k, TopkPlan* pl
   pl->s = take((size_t)pl->chunk_rows * pl->lds * 4);
   pl->part = take(kCeSplitFloats * 4);  // short rows: few tiles per chunk
   pl->es = pl->zs = pl->tau = pl->cand = pl->fail_rows = pl->big_rows = 0;
+  if (V <= topk_short_max_v()) {
+    pl->cand = take((size_t)pl->chunk_rows * topk_short_cap() * 8);
+    pl->tau = take((size_t)pl->chunk_rows * 4);  // the lists' lengths
+    pl->fail_rows = take((size_t)pl->chunk_rows * 4);
+    pl->big_rows = take((size_t)pl->chunk_rows * 4);
+  }
   if (pl->sampled) {
     pl->es = take((size_t)topk_sample() * d * 2);  // later the gathered rows of a fallback batch
     pl->zs = take((size_t)std::min<int64_t>(V, kTopkSampleRows) * topk_sample() * 4);
@@ -2396,8 +2403,21 @@ int lora_topk_table(const lora_bf16* E, int64_t V, int64_t d, int64_t k, int32_t
             LORA_OK)
           return rec(rc);
       }
-      if (launch_topk_select(S, pl.lds, (int)V, (int)k, (int)r0, nullptr, (int)rows, table, dv->status, st) !=
-          cudaSuccess)
+      if (V > topk_short_max_v()) {
+        if (launch_topk_select(S, pl.lds, (int)V, (int)k, (int)r0, nullptr, (int)rows, nullptr, table, dv->status, st) !=
+            cudaSuccess)
+          return rec(LORA_ECUDA);
+        continue;
+      }
+      int* n_big = ctr + pl.chunks + c;
+      int* n_fail = ctr + 2 * pl.chunks + c;
+      int32_t* fail = at<int32_t>(ws, pl.fail_rows);
+      if (launch_topk_short(S, pl.lds, (int)V, (int)k, (int)rows, at<uint2>(ws, pl.cand), topk_short_cap(),
+                            at<int>(ws, pl.tau), st) != cudaSuccess ||
+          launch_topk_sort(at<uint2>(ws, pl.cand), at<int>(ws, pl.tau), topk_short_cap(), (int)k, (int)r0, (int)rows,
+                           table, at<int32_t>(ws, pl.big_rows), n_big, fail, n_fail, dv->num_sms, st) != cudaSuccess ||
+          launch_topk_select(S, pl.lds, (int)V, (int)k, (int)r0, fail, std::min((int)rows, dv->num_sms), n_fail, table,
+                             dv->status, st) != cudaSuccess)
         return rec(LORA_ECUDA);
     }
     return rec(LORA_OK);
@@ -2447,7 +2467,7 @@ int lora_topk_table(const lora_bf16* E, int64_t V, int64_t d, int64_t k, int32_t
       if ((rc = ce_gemm(dv, ctr + next++, es, d, en, d, S, pl.lds, n, V, d, false, true, part, st)) != LORA_OK)
         return rec(rc);
     }
-    if (launch_topk_select(S, pl.lds, (int)V, (int)k, 0, fail_rows + f0, n, table, dv->status, st) != cudaSuccess)
+    if (launch_topk_select(S, pl.lds, (int)V, (int)k, 0, fail_rows + f0, n, nullptr, table, dv->status, st) != cudaSuccess)
       return rec(LORA_ECUDA);
   }
   return rec(LORA_OK);

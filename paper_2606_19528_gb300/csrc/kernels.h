@@ -357,13 +357,16 @@ cudaError_t launch_scatter_rows(const __nv_bfloat16* src, const int32_t* idx, in
 // En[i] = bf16(E[i] / norm[i]), norm[i] = ||E[i]|| with the sum of squares in fp32 in index order.
 cudaError_t launch_normalize_rows(const __nv_bfloat16* E, int V, int d, float* norm, __nv_bfloat16* En,
                                   cudaStream_t stream);
-// Rows row0 .. row0 + nrows - 1 of the table from their similarities S [nrows, lds] fp32:
-// the k largest per row, descending, lower index first on ties; *status =
-// kStatusTopkTies when a row has too many candidates tied at its k-th value.
-// Top-k selection per row of similarities S [nrows, lds] (row r goes to table
-// row rows[r], or row0 + r when rows is null).
+// Radix selection per row of similarities S [.., lds] into table rows rows[r] (row0 + r when rows is null) of S's row
+// r < nrows; with n_list
+// (device) of the first *n_list rows of the list instead, whose similarities are S's rows rows[i] - row0, on nrows
+// blocks.  The k largest per row, descending, lower index first on ties; *status = kStatusTopkTies when a row has
+// too many candidates tied at its k-th value.
 cudaError_t launch_topk_select(const float* S, long long lds, int V, int k, int row0, const int32_t* rows, int nrows,
-                               int32_t* table, int* status, cudaStream_t stream);
+                               const int* n_list, int32_t* table, int* status, cudaStream_t stream);
+// Candidate lists (order key, token) [nrows, cap] and their lengths cnt of nrows short rows of similarities.
+cudaError_t launch_topk_short(const float* S, long long lds, int V, int k, int nrows, uint2* cand, int cap, int* cnt,
+                              cudaStream_t stream);
 // Thresholds of nrows rows from their sample similarities Z [nrows, ns].
 cudaError_t launch_topk_tau(const float* Z, int V, int k, int ns, int nrows, float* tau, cudaStream_t stream);
 // Sorts each row's appended candidates into the table (a warp per row, a block for
@@ -378,6 +381,8 @@ int topk_sample();        // most sample tokens per row (sizes the workspace)
 int topk_sample_for(int V, int k);  // sample tokens per row of a table, a multiple of 512
 int topk_sample_min_v();  // shortest rows that take the sampled selection
 int topk_cap();           // candidate slots per row
+int topk_short_cap();     // of rows of at most topk_short_max_v() tokens
+int topk_short_max_v();
 int topk_max_k();
 
 // One bounded wait on a barrier nothing arrives on (failure-detection self-check).

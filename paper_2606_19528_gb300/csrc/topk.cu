@@ -6,14 +6,17 @@
 //   row_norms,          E~_i = bf16(E_i / ||E_i||), the sum of squares
 //                       accumulated in fp32 in index order (squares of bf16
 //                       are exact), correctly rounded sqrt and division
-// Rows shorter than 32768 tokens (the host runs 512-row chunks):
-//   topk_select         per row of a chunk's fp32 similarities (tcgen05
-//                       contraction in fused_gemm.cu): radix select on an
+// Rows shorter than 32768 tokens (the host runs chunks of rows):
+//   topk_short          (up to 8192 tokens) per row of a chunk's fp32 similarities
+//                       (tcgen05 contraction in fused_gemm.cu): the values from
+//                       the k-th largest one's histogram bin up, sorted as the
+//                       long rows' candidates are
+//   topk_select         (over 8192 tokens, and any row whose list came out short
+//                       or long) radix select on an
 //                       order-preserving uint32 image (11-bit histograms,
 //                       then 11, then 10 bits) until the candidates at or
 //                       above the chosen prefix fit in shared memory, then a
-//                       sort on (similarity descending, index ascending); it
-//                       also serves the longer rows' fallback
+//                       sort on (similarity descending, index ascending)
 // Rows of at least 32768 tokens:
 //   topk_gather_sample  up to 8192 evenly spread tokens
 //   topk_tau            each row's threshold from its similarities to them
@@ -478,17 +481,9 @@ __device__ bool sampled_select(SelShared& sh, const float* __restrict__ s, int V
   return true;
 }
 
-__global__ void __launch_bounds__(kSelThreads, 2) topk_select_kernel(const float* __restrict__ S, long long lds, int V,
-                                                                  int k, int row0, const int32_t* __restrict__ rows,
-                                                                  int32_t* __restrict__ table,
-                                                                  int* __restrict__ status) {
-  griddep_wait();
-  griddep_launch_dependents();
-  extern __shared__ uint8_t smem_raw[];
-  SelShared& sh = *reinterpret_cast<SelShared*>(smem_raw);
-  const int r = blockIdx.x;
-  const long long trow = rows ? rows[r] : row0 + r;  // table row of similarity row r
-  const float* s = S + (long long)r * lds;  // lds is a multiple of 4: 16-byte aligned rows
+// Similarity row s to table row trow.
+__device__ __forceinline__ void select_row(SelShared& sh, const float* __restrict__ s, int V, int k, long long trow,
+                           int32_t* __restrict__ table, int* __restrict__ status) {
   if (V >= kSampleMinV) {
     if (sampled_select(sh, s, V, k, table + trow * k)) return;
     __syncthreads();  // the fallback reuses the shared buffers
@@ -585,6 +580,152 @@ __global__ void __launch_bounds__(kSelThreads, 2) topk_select_kernel(const float
   for (int j = (V & ~3) + (int)threadIdx.x; j < V; j += kSelThreads) take(s[j], j);
   __syncthreads();
   sort_and_write(sh, sh.ncand, k, table + trow * k);
+}
+
+// One block per row r of S [.., lds], for table row rows[r] (row0 + r without
+// rows); kList: the first *n_list entries of rows are table rows whose similarities
+// are S's rows rows[i] - row0 (a short launch that usually finds none).
+template <bool kList>
+__global__ void __launch_bounds__(kSelThreads, 2) topk_select_kernel(const float* __restrict__ S, long long lds, int V,
+                                                                  int k, int row0, const int32_t* __restrict__ rows,
+                                                                  const int* __restrict__ n_list,
+                                                                  int32_t* __restrict__ table,
+                                                                  int* __restrict__ status) {
+  griddep_wait();
+  griddep_launch_dependents();
+  extern __shared__ uint8_t smem_raw[];
+  SelShared& sh = *reinterpret_cast<SelShared*>(smem_raw);
+  // lds is a multiple of 4: 16-byte aligned rows
+  if constexpr (!kList) {
+    select_row(sh, S + (long long)blockIdx.x * lds, V, k,
+               rows ? rows[blockIdx.x] : row0 + (int)blockIdx.x, table, status);
+  } else {
+    const int n = *n_list;
+    for (int i = blockIdx.x; i < n; i += gridDim.x) {
+      select_row(sh, S + (long long)(rows[i] - row0) * lds, V, k, rows[i], table, status);
+      __syncthreads();  // the shared buffers are free for the next row
+    }
+  }
+}
+
+// Candidates of rows of at most kShortMaxV values: one block per row of S, the row
+// in registers.  A linear histogram of 2048 bins over the row's [min, max] gives
+// the bin of its k-th largest value; every value from that bin up goes to the
+// row's list (a value left out is in a lower bin, so below every candidate: with
+// k to cap of them they hold the exact top k, and the warp sort finishes; any
+// other row, for instance thousands of ties, goes to the radix select).  The radix
+// select alone, a 1024-thread block with a three-level histogram and a block sort
+// per row, took 118 us for 2048 rows of 8000 (k = 200); this 39 us, the sort 8 us.
+// For longer rows (512 rows of 24000, k = 800) the radix select's 49 us a chunk were
+// less than this on 1024 threads (47 us) and a sort of few rows (31 us).
+constexpr int kShortThreads = 256;
+constexpr int kShortRegs = 8;  // float4 per thread
+constexpr int kShortMaxV = 4 * kShortRegs * kShortThreads;
+
+__global__ void __launch_bounds__(kShortThreads, 4) topk_short_kernel(const float* __restrict__ S, long long lds, int V,
+                                                                     int k, uint2* __restrict__ cand, int cap,
+                                                                     int* __restrict__ cnt) {
+  griddep_wait();
+  griddep_launch_dependents();
+  __shared__ int hist[2048];
+  __shared__ float red[2][kShortThreads / 32];
+  __shared__ int wsum[kShortThreads / 32];
+  __shared__ int s_bin, s_n;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const float* s = S + (long long)blockIdx.x * lds;
+  const float4* s4 = reinterpret_cast<const float4*>(s);
+  const int n4 = (V + 3) / 4;  // lds is a multiple of 4: the last group is readable, its tail not counted
+  float4 v[kShortRegs];
+#pragma unroll
+  for (int u = 0; u < kShortRegs; ++u) {
+    const int j4 = tid + u * kShortThreads;
+    v[u] = j4 < n4 ? __ldg(s4 + j4) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  // f(value, index) over this thread's values
+  auto each = [&](auto f) {
+#pragma unroll
+    for (int u = 0; u < kShortRegs; ++u) {
+      const float x[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+      const int j = 4 * (tid + u * kShortThreads);
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (j + e < V) f(x[e], j + e);
+    }
+  };
+  float lo = INFINITY, hi = -INFINITY;
+  bool nan = false;
+  each([&](float x, int) {
+    lo = fminf(lo, x);
+    hi = fmaxf(hi, x);
+    nan = nan || x != x;
+  });
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  if (__syncthreads_or(nan)) {  // the radix select orders NaNs by their keys
+    if (tid == 0) cnt[blockIdx.x] = cap + 1;
+    return;
+  }
+  for (int b = tid; b < 2048; b += kShortThreads) hist[b] = 0;
+  if (lane == 0) {
+    red[0][warp] = lo;
+    red[1][warp] = hi;
+  }
+  if (tid == 0) {
+    s_bin = 0;
+    s_n = 0;
+  }
+  __syncthreads();
+  lo = red[0][0];
+  hi = red[1][0];
+#pragma unroll
+  for (int w = 1; w < kShortThreads / 32; ++w) {
+    lo = fminf(lo, red[0][w]);
+    hi = fmaxf(hi, red[1][w]);
+  }
+  const float scale = hi > lo ? 2048.f / (hi - lo) : 0.f;
+  auto bin_of = [&](float x) { return min(2047, max(0, (int)((x - lo) * scale))); };
+  each([&](float x, int) { atomicAdd(&hist[bin_of(x)], 1); });
+  __syncthreads();
+  // bins by descending index: thread t holds bins 2047 - 8t .. 2040 - 8t
+  int local = 0;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) local += hist[2047 - 8 * tid - q];
+  int x = local;  // inclusive scan over the block
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) wsum[warp] = x;
+  __syncthreads();
+  int excl = x - local;
+  for (int w = 0; w < warp; ++w) excl += wsum[w];
+  if (excl < k && k <= excl + local) {
+    int acc = excl;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int h = hist[2047 - 8 * tid - q];
+      if (k <= acc + h) {
+        s_bin = 2047 - 8 * tid - q;
+        break;
+      }
+      acc += h;
+    }
+  }
+  __syncthreads();
+  const int bstar = s_bin;
+  uint2* dst = cand + (long long)blockIdx.x * cap;
+  each([&](float f, int j) {
+    if (bin_of(f) >= bstar) {
+      const int slot = atomicAdd(&s_n, 1);
+      if (slot < cap) dst[slot] = make_uint2(ord_key(f), (uint32_t)j);
+    }
+  });
+  __syncthreads();
+  if (tid == 0) cnt[blockIdx.x] = s_n;
 }
 
 // Sample tokens of the rows' thresholds (topk_sample_for): about kSampleRank of
@@ -793,17 +934,23 @@ cudaError_t launch_normalize_rows(const __nv_bfloat16* E, int V, int d, float* n
 }
 
 // Sets the dynamic shared-memory size of the selection kernel (once per device).
+template <bool kList>
 cudaError_t sel_attrs() {
   static std::atomic<unsigned long long> attr_done{0};
-  return set_smem_once(topk_select_kernel, (int)sizeof(SelShared), attr_done);
+  return set_smem_once(topk_select_kernel<kList>, (int)sizeof(SelShared), attr_done);
 }
 
 cudaError_t launch_topk_select(const float* S, long long lds, int V, int k, int row0, const int32_t* rows, int nrows,
-                               int32_t* table, int* status, cudaStream_t st) {
-  cudaError_t e = sel_attrs();
+                               const int* n_list, int32_t* table, int* status, cudaStream_t st) {
+  const cudaError_t e = n_list ? sel_attrs<true>() : sel_attrs<false>();
   if (e != cudaSuccess) return e;
-  return launch_kernel(topk_select_kernel, dim3(nrows), dim3(kSelThreads), (int)sizeof(SelShared), st, 1, S, lds, V,
-                       k, row0, rows, table, status);
+  return launch_kernel(n_list ? topk_select_kernel<true> : topk_select_kernel<false>, dim3(nrows), dim3(kSelThreads), (int)sizeof(SelShared), st, 1, S, lds, V,
+                       k, row0, rows, n_list, table, status);
+}
+
+cudaError_t launch_topk_short(const float* S, long long lds, int V, int k, int nrows, uint2* cand, int cap, int* cnt,
+                              cudaStream_t st) {
+  return launch_kernel(topk_short_kernel, dim3(nrows), dim3(kShortThreads), 0, st, 1, S, lds, V, k, cand, cap, cnt);
 }
 
 cudaError_t launch_topk_tau(const float* Z, int V, int k, int ns, int nrows, float* tau, cudaStream_t st) {
@@ -835,6 +982,8 @@ int topk_sample_for(int V, int k) {
 }
 int topk_sample_min_v() { return kSampleMinV; }
 int topk_cap() { return kCap; }
+int topk_short_cap() { return kCap / 2; }
+int topk_short_max_v() { return kShortMaxV; }
 
 int topk_max_k() { return kSelThreads; }
 

@@ -79,15 +79,17 @@ def test_topk_table_parity(V, d, k):
 
 
 # partial row groups and column chunks of the norms, several chunks of short rows, large k (a short sample)
-@pytest.mark.parametrize("V,d,k", [(2001, 72, 16), (9003, 200, 130), (33001, 72, 1024)],
-                         ids=["V2001_d72_k16", "V9003_d200_k130", "V33001_d72_k1024"])
+@pytest.mark.parametrize("V,d,k", [(2001, 72, 16), (9003, 200, 130), (33001, 72, 1024), (17001, 64, 1000),
+                                   (100, 8, 100)],
+                         ids=["V2001_d72_k16", "V9003_d200_k130", "V33001_d72_k1024", "V17001_d64_k1000", "V100_d8_k100"])
 def test_topk_table_edges(V, d, k):
     """The oracle's checks, and the same table when rows are scaled by powers of two (2^62 and 2^-50 take the two
     division paths of the normalisation; a scaled row normalises to the same bits)."""
     bits = synth.gen_E(0, 52, V, d)
     table = run_table(bits, k)
     rng = np.random.default_rng(V)
-    check_rows(bits, table, k, np.unique(np.concatenate([[0, V - 1, 511, 512], rng.integers(0, V, 20)])))
+    rows = [r for r in (0, V - 1, 511, 512) if r < V]
+    check_rows(bits, table, k, np.unique(np.concatenate([rows, rng.integers(0, V, 20)])))
     scale = np.array([1.0, 2.0 ** 62, 2.0 ** -50])[rng.integers(0, 3, V)]
     scaled = synth.to_bf16_bits(synth.bf16_bits_to_f64(bits) * scale[:, None])
     assert np.array_equal(run_table(scaled, k), table)
@@ -129,3 +131,23 @@ def test_topk_sampled_ties_and_fallback():
     for i in (2000, 4999):
         assert table[i].tolist() == list(range(2000, 3000)), i
     check_rows(bits, table, k, np.array([5000, 12345, V - 1]))
+
+
+def test_topk_short_rows_ties_and_nan():
+    """Short rows whose k-th similarity ties with thousands of others go to the radix select (lower index first), and
+    so do rows with a NaN similarity: rows 0..2999 are one vector, and with an infinite element in row 3500 (its
+    normalised row holds a NaN) every row of the table still lists k distinct tokens, each row's as without it but
+    for that token (its own row, 4000 tied NaNs, lists the first k)."""
+    V, d, k = 4000, 64, 100
+    bits = synth.gen_E(0, 53, V, d)
+    bits[:3000] = bits[7]
+    table = run_table(bits, k)
+    assert np.array_equal(table[[0, 1500, 2999]], np.tile(np.arange(k), (3, 1)))
+    check_rows(bits, table, k, np.array([3000, 3400, V - 1]))
+    bad = bits.copy()
+    bad[3500, 3] = 0x7F80
+    t2 = run_table(bad, k)
+    for i in (3000, 3400, V - 1):
+        rest = t2[i][t2[i] != 3500]
+        assert len(set(t2[i].tolist())) == k and len(rest) >= k - 1
+        assert np.array_equal(rest, table[i][table[i] != 3500][:len(rest)])
