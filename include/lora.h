@@ -262,8 +262,8 @@ int lora_ce_fwd_bwd(const lora_ce_args* args, void* workspace, size_t workspace_
  * row i of `table` [V, k] int32 lists the k tokens with the largest C[i, :],
  * in descending order, the lower index first on equal similarities (row i
  * starts with i unless another token has the same direction).  The V x V
- * matrix is never formed.  Below V = 32768 similarities are computed 512 rows
- * at a time in fp32 on the tensor cores and each row's top k is selected from
+ * matrix is never formed.  Below V = 32768 similarities are computed some
+ * hundreds of rows at a time in fp32 on the tensor cores and each row's top k is selected from
  * them.  From V = 32768 on, each row first gets a threshold from its
  * similarities to up to 8192 evenly spread tokens, the similarity contraction keeps
  * only the values at or above it (at most 4096 per row, in workspace), and

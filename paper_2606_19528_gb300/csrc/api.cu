@@ -1968,15 +1968,43 @@ struct TopkPlan {
   long long lds;
 };
 
+// Rows per chunk of a table of 8193 to 32767 tokens: multiples of 256 up to 96 MB
+// of similarities, the one whose chunks take least by this sum of whole waves: of
+// 256 x 256 tiles over the pairs (0.43 us per 64-deep block, 2 us epilogue) and of
+// rows over the selection's two blocks per SM (12 us at 30000 tokens), with 6 us
+// of ramps per chunk.  Against 64 MB rounded down to 512 rows: V = 29747, d = 1120:
+// 4986 -> 4443 us a table (512 rows are 234 tiles, 3.08 waves of 76 pairs; 768 rows
+// 4.6); V = 12000, d = 2048: 1200 -> 1100; V = 24000, d = 512: 4060 -> 3567.
+int topk_chunk_rows(int64_t V, int64_t d) {
+  const int64_t most = (int64_t)kTopkChunk * 3 / 2 * topk_sample_min_v() / rup(V, 4);
+  auto cost = [&](int64_t rows) {
+    return 6.0 + (double)cdiv(cdiv(rows, 256) * cdiv(V, 256), kPlanPairs) * (2.0 + 0.43 * (double)cdiv(d, 64)) +
+           (double)cdiv(rows, 4 * kPlanPairs) * 12.0 * (double)V / 30000.0;
+  };
+  int64_t best = 256;
+  double least = INFINITY;
+  for (int64_t rows = 256; rows <= std::min(most, rup(V, 256)); rows += 256) {
+    const int64_t last = V % rows;
+    const double c = (double)(V / rows) * cost(rows) + (last ? cost(last) : 0.0);
+    if (c < least) {
+      least = c;
+      best = rows;
+    }
+  }
+  return (int)std::min(best, V);
+}
+
 int topk_check(const lora_bf16* E, int64_t V, int64_t d, int64_t k, TopkPlan* pl) {
   if (V < 1 || d < 8 || (d % 8) || k < 1 || k > V || k > topk_max_k() || V > (1ll << 24) || d > (1ll << 20))
     return LORA_EINVAL;
   if (E && !aligned16(E)) return LORA_EALIGN;
   pl->sampled = V >= topk_sample_min_v();
-  // short rows: chunks of as many similarities as 512 rows of the longest of them have (64 MB), so that a
+  // up to 8192 tokens: chunks of as many similarities as 512 rows of 32768 have (64 MB), so that a
   // chunk's contraction fills the GPU (V = 8000, d = 1024, k = 200: 835 -> 618 us per table)
-  pl->chunk_rows = pl->sampled ? kTopkChunk
-                               : (int)std::min<int64_t>(V, (int64_t)kTopkChunk * topk_sample_min_v() / V / kTopkChunk * kTopkChunk);
+  pl->chunk_rows = pl->sampled                  ? kTopkChunk
+                   : V > topk_short_max_v() ? topk_chunk_rows(V, d)
+                                            : (int)std::min<int64_t>(V, (int64_t)kTopkChunk * topk_sample_min_v() / V /
+                                                                            kTopkChunk * kTopkChunk);
   pl->chunks = (int)cdiv(V, pl->chunk_rows);
   pl->sblocks = pl->sampled ? (int)cdiv(V, kTopkSampleRows) : 0;
   pl->achunks = pl->sampled ? (int)cdiv(V, kTopkAppendRows) : 0;

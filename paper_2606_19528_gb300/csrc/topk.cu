@@ -12,11 +12,14 @@
 //                       the k-th largest one's histogram bin up, sorted as the
 //                       long rows' candidates are
 //   topk_select         (over 8192 tokens, and any row whose list came out short
-//                       or long) radix select on an
+//                       or long) over 8192 tokens the values above a threshold
+//                       from a sample of the row, sorted on (similarity
+//                       descending, index ascending); otherwise, and where those
+//                       are too few or too many, radix select on an
 //                       order-preserving uint32 image (11-bit histograms,
 //                       then 11, then 10 bits) until the candidates at or
-//                       above the chosen prefix fit in shared memory, then a
-//                       sort on (similarity descending, index ascending)
+//                       above the chosen prefix fit in shared memory, then the
+//                       sort
 // Rows of at least 32768 tokens:
 //   topk_gather_sample  up to 8192 evenly spread tokens
 //   topk_tau            each row's threshold from its similarities to them
@@ -180,6 +183,7 @@ struct SelShared {
   int cidx[kCap];
   int warp_tot[32];
   int bin, above, ncand;
+  uint32_t smin, smax;
 };
 
 // Bin (of nbins, by descending bin index) where the k_rem-th largest falls,
@@ -370,15 +374,6 @@ __device__ void sort_and_write(SelShared& sh, int n, int k, int32_t* __restrict_
     sort_write_e<kSelThreads, 4>(get, n, k, x, out);
 }
 
-// Sampled threshold for long rows: the r-th largest of kSample evenly spread
-// row values (r sized so that about kOver * k of the row's values lie at or
-// above it), found to 22 key bits by two histogram levels over the sample
-// alone; then one streaming pass appends every value at or above that
-// threshold, one ballot per 16-byte load and, for a warp with hits, one
-// shared-memory atomic.  A value left out is strictly below every candidate,
-// so when the candidates number between k and kCap they contain the exact
-// top k.  Returns false (and the caller falls back to the full radix select)
-// otherwise.
 constexpr int kSample = 8 * kSelThreads;
 constexpr int kSampleMinV = 4 * kSample;
 constexpr float kOver = 1.6f;
@@ -389,51 +384,124 @@ __device__ __forceinline__ int sample_rank(int V, int k, int ns) {
   return min(ns, max(1, (int)ceilf(kOver * (float)k * (float)ns / (float)V)));
 }
 
-// The smallest value whose order key shares the top 22 bits of the rs-th
-// largest of the block's kSample sample keys (8 per thread): two histogram
-// levels of 11 bits over the sample.
-__device__ float sample_threshold(SelShared& sh, const uint32_t* sk, int rs) {
-  uint32_t prefix = 0;
-  int r_rem = rs;
-  for (int lvl = 0; lvl < 2; ++lvl) {
-    for (int b = threadIdx.x; b < 2048; b += kSelThreads) sh.hist[b] = 0;
-    __syncthreads();
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      if (lvl == 0)
-        atomicAdd(&sh.hist[sk[e] >> 21], 1);
-      else if ((sk[e] >> 21) == prefix)
-        atomicAdd(&sh.hist[(sk[e] >> 10) & 2047u], 1);
-    }
-    __syncthreads();
-    find_bin(sh, 2048, r_rem);
-    prefix = (lvl == 0 ? 0u : prefix << 11) | (uint32_t)sh.bin;
-    r_rem -= sh.above;
-    __syncthreads();
+// Sampled threshold for rows of more than kRowSampleMinV values: a linear
+// histogram of kRowSample evenly spread values over their [min, max] gives the
+// lower edge of the bin of their rs-th largest, rs four standard deviations
+// above the k * kRowSample / V of them expected among the row's top k (a row falls
+// short about once in 30000); then one streaming pass appends every value at or
+// above that edge, one ballot per 16-byte load and, for a warp with hits, one
+// shared-memory atomic.  A value left out is strictly below every candidate,
+// so when the candidates number between k and kCap they contain the exact
+// top k.  Returns false (and the caller falls back to the full radix select)
+// otherwise and for a row with a NaN, which the radix select orders by its key.
+// Bound by the row's reads from L2 (one and an eighth to one and a half times, the
+// radix select three times) and the block sort.  Whole tables, radix select before /
+// this: V = 29747, d = 1120, k = 150: 5570 / 4986 us; V = 12000, d = 2048, k = 64: 1269
+// / 1200; with more than 1024 candidates only once they are narrowed: V = 17003, d =
+// 512, k = 1000: 2939 / 2811 without, about 2410 with.
+constexpr int kRowSample = 4 * kSelThreads;
+constexpr int kRowSampleMinV = 2 * kRowSample;
+
+// The smallest and largest of the block's keys, each thread's own in kmin and
+// kmax, into sh.smin and sh.smax (read after the barrier it ends with).
+__device__ __forceinline__ void block_key_range(SelShared& sh, uint32_t kmin, uint32_t kmax) {
+  if (threadIdx.x == 0) {
+    sh.smin = 0xffffffffu;
+    sh.smax = 0u;
   }
-  const uint32_t key_lo = prefix << 10;
-  return __uint_as_float((key_lo & 0x80000000u) ? (key_lo & 0x7fffffffu) : ~key_lo);
+  kmin = __reduce_min_sync(0xffffffffu, kmin);
+  kmax = __reduce_max_sync(0xffffffffu, kmax);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) {
+    atomicMin(&sh.smin, kmin);
+    atomicMax(&sh.smax, kmax);
+  }
+  __syncthreads();
+}
+
+// Of the n candidates (k <= n <= kCap, all written before the caller's last
+// barrier) keeps those from the bin of the k-th largest up, in 2048 bins linear in
+// the keys; returns their number.  A sort of 2048 costs more than twice one of 1024.
+__device__ int narrow_candidates(SelShared& sh, int n, int k) {
+  const int t = threadIdx.x, lane = t & 31;
+  uint32_t key[4];
+  int idx[4];
+  uint32_t kmin = 0xffffffffu, kmax = 0u;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int p = t + e * kSelThreads;
+    key[e] = p < n ? sh.ckey[p] : 0u;
+    idx[e] = p < n ? sh.cidx[p] : 0;
+    if (p < n) {
+      kmin = min(kmin, key[e]);
+      kmax = max(kmax, key[e]);
+    }
+  }
+  sh.hist[t] = 0;
+  sh.hist[t + kSelThreads] = 0;
+  block_key_range(sh, kmin, kmax);
+  kmin = sh.smin;
+  const int shift = max(0, 21 - __clz((int)(sh.smax - kmin)));  // 11 bits of the range
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    if (t + e * kSelThreads < n) atomicAdd(&sh.hist[(key[e] - kmin) >> shift], 1);
+  if (t == 0) sh.ncand = 0;
+  __syncthreads();
+  find_bin(sh, 2048, k);
+  const uint32_t bin = (uint32_t)sh.bin;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const bool keep = t + e * kSelThreads < n && ((key[e] - kmin) >> shift) >= bin;
+    const uint32_t m = __ballot_sync(0xffffffffu, keep);
+    int base = 0;
+    if (lane == 0 && m) base = atomicAdd(&sh.ncand, __popc(m));
+    base = __shfl_sync(0xffffffffu, base, 0) + __popc(m & ((1u << lane) - 1u));
+    if (keep) {
+      sh.ckey[base] = key[e];
+      sh.cidx[base] = idx[e];
+    }
+  }
+  __syncthreads();
+  return sh.ncand;
+}
+
+// f: this thread's 4 sample values.
+__device__ float sample_threshold(SelShared& sh, const float (&f)[4], int rs) {
+  const int t = threadIdx.x;
+  sh.hist[t] = 0;
+  sh.hist[t + kSelThreads] = 0;
+  uint32_t kmin = 0xffffffffu, kmax = 0u;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    kmin = min(kmin, ord_key(f[e]));
+    kmax = max(kmax, ord_key(f[e]));
+  }
+  block_key_range(sh, kmin, kmax);
+  auto value = [](uint32_t key) { return __uint_as_float((key & 0x80000000u) ? (key & 0x7fffffffu) : ~key); };
+  const float lo = value(sh.smin), hi = value(sh.smax);
+  const float scale = hi > lo ? 2048.f / (hi - lo) : 0.f;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) atomicAdd(&sh.hist[min(2047, max(0, (int)((f[e] - lo) * scale)))], 1);
+  __syncthreads();
+  find_bin(sh, 2048, rs);
+  return lo + (float)sh.bin * ((hi - lo) / 2048.f);
 }
 
 __device__ bool sampled_select(SelShared& sh, const float* __restrict__ s, int V, int k, int32_t* __restrict__ out) {
   const float4* s4 = reinterpret_cast<const float4*>(s);
   const int n4 = V / 4;
   const int lane = threadIdx.x & 31;
-  uint32_t sk[8];  // this thread's sample keys, evenly spread over the row
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const float4 q = __ldg(s4 + (int)(((long long)(threadIdx.x + u * kSelThreads) * n4) / (2 * kSelThreads)));
-    sk[4 * u + 0] = ord_key(q.x);
-    sk[4 * u + 1] = ord_key(q.y);
-    sk[4 * u + 2] = ord_key(q.z);
-    sk[4 * u + 3] = ord_key(q.w);
-  }
-  const float tf = sample_threshold(sh, sk, sample_rank(V, k, kSample));
+  const float4 q0 = __ldg(s4 + (int)(((long long)threadIdx.x * n4) / kSelThreads));  // evenly spread over the row
+  const float sample[4] = {q0.x, q0.y, q0.z, q0.w};
+  const float rk = (float)k * (float)kRowSample / (float)V;
+  const float tf = sample_threshold(sh, sample, min(kRowSample, (int)ceilf(rk + 4.f * sqrtf(rk)) + 2));
+  bool nan = false;
   if (threadIdx.x == 0) sh.ncand = 0;
   __syncthreads();
   // appends this lane's hits among its first nv values of q (positions j0 + e); whole warps call it
   auto append4 = [&](const float4 q, int nv, int j0) {
     const float f[4] = {q.x, q.y, q.z, q.w};
+    nan = nan || !(q.x == q.x && q.y == q.y && q.z == q.z && q.w == q.w);
     const int c = (nv > 0 && f[0] >= tf) + (nv > 1 && f[1] >= tf) + (nv > 2 && f[2] >= tf) + (nv > 3 && f[3] >= tf);
     if (__ballot_sync(0xffffffffu, c > 0) == 0u) return;
     int x = c;  // inclusive scan of the hit counts over the warp
@@ -474,9 +542,10 @@ __device__ bool sampled_select(SelShared& sh, const float* __restrict__ s, int V
     const int j = 4 * n4 + lane;
     append4(make_float4(j < V ? s[j] : 0.f, 0.f, 0.f, 0.f), j < V ? 1 : 0, j);
   }
-  __syncthreads();
-  const int n = sh.ncand;
-  if (n < k || n > kCap) return false;  // uniform: read after the barrier
+  const bool any_nan = __syncthreads_or(nan);
+  int n = sh.ncand;
+  if (any_nan || n < k || n > kCap) return false;  // uniform: read after the barrier
+  if (n > kSelThreads) n = narrow_candidates(sh, n, k);
   sort_and_write(sh, n, k, out);
   return true;
 }
@@ -484,7 +553,7 @@ __device__ bool sampled_select(SelShared& sh, const float* __restrict__ s, int V
 // Similarity row s to table row trow.
 __device__ __forceinline__ void select_row(SelShared& sh, const float* __restrict__ s, int V, int k, long long trow,
                            int32_t* __restrict__ table, int* __restrict__ status) {
-  if (V >= kSampleMinV) {
+  if (V > kRowSampleMinV) {
     if (sampled_select(sh, s, V, k, table + trow * k)) return;
     __syncthreads();  // the fallback reuses the shared buffers
   }
@@ -616,8 +685,8 @@ __global__ void __launch_bounds__(kSelThreads, 2) topk_select_kernel(const float
 // other row, for instance thousands of ties, goes to the radix select).  The radix
 // select alone, a 1024-thread block with a three-level histogram and a block sort
 // per row, took 118 us for 2048 rows of 8000 (k = 200); this 39 us, the sort 8 us.
-// For longer rows (512 rows of 24000, k = 800) the radix select's 49 us a chunk were
-// less than this on 1024 threads (47 us) and a sort of few rows (31 us).
+// For longer rows (512 rows of 24000, k = 800) this form on 1024 threads (47 us) and a
+// sort of few rows (31 us) took longer than one block per row (topk_select).
 constexpr int kShortThreads = 256;
 constexpr int kShortRegs = 8;  // float4 per thread
 constexpr int kShortMaxV = 4 * kShortRegs * kShortThreads;

@@ -24,14 +24,14 @@ pytestmark = pytest.mark.gpu
 GOLDEN = os.path.join(os.path.dirname(os.path.abspath(__file__)), "golden")
 
 
-def run_table(bits, k):
+def run_table(bits, k, status=lora.LORA_OK):
     V, d = bits.shape
     E = G.dev_bf16(bits)
     table = torch.full((V, k), -1, dtype=torch.int32, device="cuda")
     ws = G.workspace(lora.lora_topk_workspace_size(V, d, k))
     lora.lora_topk_table(E, V, d, k, table, ws, ws.numel())
     torch.cuda.synchronize()
-    assert lora.lora_read_status() == lora.LORA_OK
+    assert lora.lora_read_status() == status
     return table.cpu().numpy()
 
 
@@ -151,3 +151,37 @@ def test_topk_short_rows_ties_and_nan():
         rest = t2[i][t2[i] != 3500]
         assert len(set(t2[i].tolist())) == k and len(rest) >= k - 1
         assert np.array_equal(rest, table[i][table[i] != 3500][:len(rest)])
+
+
+# just over the short rows, a length that is no multiple of 4, and the longest below the stored candidates
+@pytest.mark.parametrize("V,k", [(8193, 1000), (20481, 1000), (32766, 64)])
+def test_topk_row_sample_ties_and_nan(V, k):
+    """Rows whose threshold comes from a sample of the row itself: rows 0..nu-1 are one vector u, rows nu..3899 one
+    vector v with cos(u, v) about 0.9, so that u's k-th value is one of thousands of exact ties (the lower index
+    first). A random row whose k-th similarity is v's has at most k - 1 above it and 3900 - nu ties: 999 + 3000 at
+    k = 1000, 63 + 3880 at k = 64, so with a NaN at most 4000 of the 4096 candidates that the selection holds. With an
+    infinite element in the last row every other row holds a NaN, and goes to the radix select; that row itself (V
+    tied NaNs, more than the selection holds) is reported and left unwritten."""
+    d = 64
+    bits = synth.gen_E(0, 54, V, d)
+    x = synth.bf16_bits_to_f64(bits)
+    u = x[7] / np.linalg.norm(x[7])
+    w = x[11] - (x[11] @ u) * u
+    v = 0.9 * u + np.sqrt(1 - 0.81) * w / np.linalg.norm(w)
+    bits = bits.copy()
+    nu = max(k - 100, 20)
+    bits[:nu] = synth.to_bf16_bits(u[None, :])
+    bits[nu:3900] = synth.to_bf16_bits(v[None, :])
+    table = run_table(bits, k)
+    for i in (0, nu - 1):
+        assert np.array_equal(table[i], np.arange(k)), i
+    for i in (nu, 3899):
+        assert np.array_equal(table[i], np.arange(nu, nu + k)), i
+    check_rows(bits, table, k, np.array([4000, 7777, V - 1]))
+    bad = bits.copy()
+    bad[V - 1, 3] = 0x7F80
+    t2 = run_table(bad, k, lora.LORA_EINVAL)
+    for i in (0, nu, 4000, 7777):
+        rest = t2[i][t2[i] != V - 1]
+        assert len(set(t2[i].tolist())) == k and len(rest) >= k - 1, i
+        assert np.array_equal(rest, table[i][table[i] != V - 1][:len(rest)]), i
