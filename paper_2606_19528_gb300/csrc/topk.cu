@@ -221,15 +221,22 @@ __device__ __forceinline__ int cand_index(uint64_t v) { return (int)(0xffffffffu
 // Bitonic sort, descending, of p2 = kT * E packed candidates held in
 // registers: slot e of thread t is position t + e * kT.  Strides below 32 are
 // exchanged by warp shuffles, 32 .. kT / 2 through the shared buffer x (p2
-// entries), kT and up within the thread (fully unrolled, so the slots stay in
-// registers).  Every thread of the block takes part.
-template <int kT, int E>
-__device__ void bitonic_sort(uint64_t (&v)[E], uint64_t* x) {
+// entries; 2 p2 with kTwo, whose halves alternate so that a stage needs one barrier
+// instead of two), kT and up within the thread (fully unrolled, so the slots stay in
+// registers).  Only the first n positions hold candidates (the rest zeros, below
+// them all): the sort ends with the first runs of at least n.  Every thread of the
+// block takes part.  Bound by the barriers' latency: whole tables of V = 12000, d =
+// 2048, k = 64 with all sizes and two barriers a stage 1099 us, so 951; of V = 29747,
+// d = 1120, k = 150: 4414 / 4231; of V = 24000, d = 512, k = 800: 2976 / 2943.
+template <int kT, int E, bool kTwo>
+__device__ void bitonic_sort(uint64_t (&v)[E], uint64_t* x, int n) {
   constexpr int p2 = kT * E;
   const int tid = (int)threadIdx.x;
+  int half = 0;
   // fully unrolled: every stage's exchange form and masks are compile-time constants
 #pragma unroll
   for (int size = 2; size <= p2; size <<= 1) {
+    if (size >= 2 * n) break;
 #pragma unroll
     for (int stride = size >> 1; stride > 0; stride >>= 1) {
       if (stride >= kT) {
@@ -254,19 +261,20 @@ __device__ void bitonic_sort(uint64_t (&v)[E], uint64_t* x) {
         const bool via_smem = stride >= 32;
         if (via_smem) {
 #pragma unroll
-          for (int e = 0; e < E; ++e) x[tid + e * kT] = v[e];
+          for (int e = 0; e < E; ++e) x[half + tid + e * kT] = v[e];
           __syncthreads();
         }
 #pragma unroll
         for (int e = 0; e < E; ++e) {
           const int p = tid + e * kT;
-          const uint64_t q = via_smem ? x[p ^ stride] : __shfl_xor_sync(0xffffffffu, v[e], stride);
+          const uint64_t q = via_smem ? x[half + (p ^ stride)] : __shfl_xor_sync(0xffffffffu, v[e], stride);
           const bool up = (p & size) == 0, lo = (p & stride) == 0;
           const bool q_first = q > v[e];
           // an ascending run keeps the first of the pair at the lower position
           if (lo ? q_first == up : q_first != up) v[e] = q;
         }
-        if (via_smem) __syncthreads();
+        if (via_smem && !kTwo) __syncthreads();
+        if (via_smem && kTwo) half ^= p2;
       }
     }
   }
@@ -338,7 +346,7 @@ __device__ void warp_sort_write(const uint2* __restrict__ c, int n, int k, int32
 
 // Loads n <= kT * E candidates (get(p) -> (key, index)), sorts them and writes
 // the first k indices to out; padding sorts below every real candidate.
-template <int kT, int E, typename Get>
+template <int kT, int E, bool kTwo = false, typename Get>
 __device__ void sort_write_e(Get get, int n, int k, uint64_t* x, int32_t* __restrict__ out) {
   const int tid = (int)threadIdx.x;
   uint64_t v[E];
@@ -353,7 +361,7 @@ __device__ void sort_write_e(Get get, int n, int k, uint64_t* x, int32_t* __rest
     }
   }
   __syncthreads();  // the candidates may live in the exchange buffer
-  bitonic_sort<kT, E>(v, x);
+  bitonic_sort<kT, E, kTwo>(v, x, n);
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     const int p = tid + e * kT;
@@ -367,9 +375,9 @@ __device__ void sort_and_write(SelShared& sh, int n, int k, int32_t* __restrict_
   auto get = [&](int p) { return make_uint2(sh.ckey[p], (uint32_t)sh.cidx[p]); };
   uint64_t* x = reinterpret_cast<uint64_t*>(sh.ckey);  // ckey and cidx together: 4096 x 8 bytes
   if (n <= kSelThreads)
-    sort_write_e<kSelThreads, 1>(get, n, k, x, out);
+    sort_write_e<kSelThreads, 1, true>(get, n, k, x, out);
   else if (n <= 2 * kSelThreads)
-    sort_write_e<kSelThreads, 2>(get, n, k, x, out);
+    sort_write_e<kSelThreads, 2, true>(get, n, k, x, out);
   else
     sort_write_e<kSelThreads, 4>(get, n, k, x, out);
 }
@@ -397,7 +405,7 @@ __device__ __forceinline__ int sample_rank(int V, int k, int ns) {
 // Bound by the row's reads from L2 (one and an eighth to one and a half times, the
 // radix select three times) and the block sort.  Whole tables, radix select before /
 // this: V = 29747, d = 1120, k = 150: 5570 / 4986 us; V = 12000, d = 2048, k = 64: 1269
-// / 1200; with more than 1024 candidates only once they are narrowed: V = 17003, d =
+// / 1200 (with the sort's ten sizes); with more than 1024 candidates only once they are narrowed: V = 17003, d =
 // 512, k = 1000: 2939 / 2811 without, about 2410 with.
 constexpr int kRowSample = 4 * kSelThreads;
 constexpr int kRowSampleMinV = 2 * kRowSample;
