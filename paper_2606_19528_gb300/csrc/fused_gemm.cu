@@ -919,9 +919,18 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
             fence_proxy_async_smem();  // the tensor core reads what these threads wrote
             __syncwarp();
           }
-          // past the slot's last block of this tile: every warp of both groups lets it be refilled (a
-          // group cannot be a whole ring ahead: its next weight tile waits for the other group's blocks)
+          // Past the slot's last block of this tile: every warp of both groups lets it be refilled.  A warp
+          // arrives only once this fill of the slot has landed, also where its group owns no block of it: the
+          // fill before it is then released by all of them, so no warp's arrival counts for that one twice.
+          // (A split's range may start or end inside a slot's blocks, and slots of one block follow each other
+          // faster than the weight tiles hold a group back: [0, 33) and then [99, 132), slots of blocks 28..31,
+          // 32 and 99, the first and the third the same memory.)
           if ((kb + 1) % QS::kBlocks == 0 || kb + 1 == kq1) {
+            if (!mine) {
+              ok = mbar_wait(smem_u32(&ctl->qfull[qs]), qpar, wc, abort_flag);
+              ok = __all_sync(0xffffffffu, ok);
+              if (!ok) break;
+            }
             if (lane == 0) mbar_arrive(smem_u32(&ctl->qempty[qs]));
             if (++qs == QS::kStages) {
               qs = 0;

@@ -69,8 +69,8 @@ def check_q4_full(p: DevQ4Proj):
 
 
 # around the 512 x 256 tiles (one row segment, both, a second row tile; a column tile of a few columns), and
-# few tiles over a long contraction, whose split ranges start inside a 4-block code slot of the forward
-# (at most 128 tokens: 128 x 256 tiles, one row tile)
+# few tiles over a long contraction, whose split ranges start inside a 4-block code slot of the forward, one
+# range per pair (at most 128 tokens: 128 x 256 tiles, one row tile)
 Q4_EDGES = [(8, 256, 8, 1), (264, 512, 264, 8), (512, 256, 136, 16), (520, 768, 520, 16), (776, 1024, 248, 64),
             (136, 4352, 512, 16), (64, 4352, 512, 16), (64, 1024, 4360, 16), (128, 768, 8200, 128),
             (40, 11008, 248, 12)]
@@ -81,6 +81,29 @@ def test_q4_tile_edges(T, K, N, r):
     p = gen_q4_proj(23, 1, 0, T, K, N, r, 2.0)
     run_q4_single(p)
     check_q4_full(p)
+
+
+# Splits of 33 and of 35 blocks over more units than CTA pairs: a pair contracts several ranges in turn, which
+# start and end inside the forward's 4-block code slots, so slots of one block follow each other (33: blocks
+# 28..31, 32 and then 99 of the next unit).
+@pytest.mark.parametrize("T,K,N,r", [(560, 10240, 3096, 8), (776, 11008, 3096, 8)],
+                         ids=["T560_K10240_N3096_r8", "T776_K11008_N3096_r8"])
+def test_q4_units_off_the_code_slots(T, K, N, r):
+    p = gen_q4_proj(24, 1, 0, T, K, N, r, 2.0)
+    ws = G.workspace(lora.lora_workspace_size(p.shape, lora.LORA_FWD))
+
+    def forward():
+        p.y.fill_(float("nan"))
+        lora.lora_linear_fwd_q4(p.shape, p.x, p.Wq, p.A, p.B, p.y, p.su, ws, ws.numel())
+        torch.cuda.synchronize()
+        assert lora.lora_read_status() == lora.LORA_OK
+        return p.y.view(torch.int16).clone()
+
+    first = forward()
+    y, _ = oracle.lora_forward(p.f64("x"), p.W64, p.f64("A"), p.f64("B"), p.s)
+    assert G.rel_fro(G.host_f64(p.y), y) <= G.TOL_Y
+    for _ in range(20):
+        assert torch.equal(forward(), first)
 
 
 def test_q4_handworked_exact():
