@@ -919,14 +919,16 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
             fence_proxy_async_smem();  // the tensor core reads what these threads wrote
             __syncwarp();
           }
-          // Past the slot's last block of this tile: every warp of both groups lets it be refilled.  A warp
-          // arrives only once this fill of the slot has landed, also where its group owns no block of it: the
-          // fill before it is then released by all of them, so no warp's arrival counts for that one twice.
-          // (A split's range may start or end inside a slot's blocks, and slots of one block follow each other
-          // faster than the weight tiles hold a group back: [0, 33) and then [99, 132), slots of blocks 28..31,
-          // 32 and 99, the first and the third the same memory.)
+          // Past the slot's last block of this tile: every warp of both groups lets it be refilled.  A warp's
+          // arrival must count for this fill of the slot and no earlier one.  Forward: a warp arrives once the
+          // fill has landed, which the fill before it had to be released for; a slot of one block is waited for
+          // by the group that owns none of it as well.  (A split's range may start or end inside a slot, and
+          // slots of one block follow each other faster than the weight tiles hold a group back: [0, 33) and
+          // then [99, 132), slots of blocks 28..31, 32 and 99, the first and the third the same memory.)
+          // Backward, six slots of one block: when a warp passes block i, block i - 5 is consumed, so every
+          // warp is past block i - 6, the slot's last.
           if ((kb + 1) % QS::kBlocks == 0 || kb + 1 == kq1) {
-            if (!mine) {
+            if (!mine && !kBMn && kb == max(kb0, kb / QS::kBlocks * QS::kBlocks)) {
               ok = mbar_wait(smem_u32(&ctl->qfull[qs]), qpar, wc, abort_flag);
               ok = __all_sync(0xffffffffu, ok);
               if (!ok) break;

@@ -460,9 +460,18 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) small_lora_gemm(const __
             fence_proxy_async_smem();  // the tensor core reads what these threads wrote
             __syncwarp();
           }
-          // past the slot's last block of this tile (a group is never a whole ring ahead of the other: its
-          // next stage waits for the other group's blocks)
+          // Past the slot's last block of this tile.  A warp's arrival must count for this fill of the slot and no
+          // earlier one.  Forward: a warp arrives once the fill has landed, which the fill before it had to be
+          // released for; a slot of one block (a split's range that starts or ends inside a slot) is waited for
+          // by the group that owns none of it as well.  Backward: when a warp passes block i, block i - 4 is
+          // consumed, so every warp is past block i - 6, the slot's last (waiting there too took the 4-bit
+          // Llama-shaped layer at T = 64 from 81.7 to 87.0 us).
           if ((kb + 1) % QS::kBlocks == 0 || kb + 1 == kq1) {
+            if (!mine && !kBMn && kb == max(w.kb0, kb / QS::kBlocks * QS::kBlocks)) {
+              ok = mbar_wait(smem_u32(&ctl->qfull[qs]), qpar, wc, abort_flag);
+              ok = __all_sync(0xffffffffu, ok);
+              if (!ok) break;
+            }
             if (lane == 0) mbar_arrive(smem_u32(&ctl->qempty[qs]));
             if (++qs == QS::kStages) {
               qs = 0;

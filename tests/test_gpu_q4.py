@@ -85,9 +85,9 @@ def test_q4_tile_edges(T, K, N, r):
 
 # Splits of 33 and of 35 blocks over more units than CTA pairs: a pair contracts several ranges in turn, which
 # start and end inside the forward's 4-block code slots, so slots of one block follow each other (33: blocks
-# 28..31, 32 and then 99 of the next unit).
-@pytest.mark.parametrize("T,K,N,r", [(560, 10240, 3096, 8), (776, 11008, 3096, 8)],
-                         ids=["T560_K10240_N3096_r8", "T776_K11008_N3096_r8"])
+# 28..31, 32 and then 99 of the next unit).  At most 128 tokens: 43 blocks, off the 2-block slots.
+@pytest.mark.parametrize("T,K,N,r", [(560, 10240, 3096, 8), (776, 11008, 3096, 8), (64, 8192, 20488, 8)],
+                         ids=["T560_K10240_N3096_r8", "T776_K11008_N3096_r8", "T64_K8192_N20488_r8"])
 def test_q4_units_off_the_code_slots(T, K, N, r):
     p = gen_q4_proj(24, 1, 0, T, K, N, r, 2.0)
     ws = G.workspace(lora.lora_workspace_size(p.shape, lora.LORA_FWD))
