@@ -1209,6 +1209,10 @@ bool any_adapter(const lora_proj* projs, int n) {
 struct SideCtx {
   cudaStream_t side = nullptr;
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};  // fork, sv ready, side done, forward contracted
+  // copies that the host waits for: a stream without kernels, so that the wait is for the copy alone (the side
+  // stream may hold work that waits for another stream's calls of this thread)
+  cudaStream_t read = nullptr;
+  cudaEvent_t ev_read = nullptr;
 };
 
 struct ThreadSide {
@@ -1218,6 +1222,8 @@ struct ThreadSide {
       for (cudaEvent_t e : c.ev)
         if (e) cudaEventDestroy(e);
       if (c.side) cudaStreamDestroy(c.side);
+      if (c.ev_read) cudaEventDestroy(c.ev_read);
+      if (c.read) cudaStreamDestroy(c.read);
     }
   }
 };
@@ -1230,6 +1236,15 @@ int side_ctx(const DeviceInfo* d, SideCtx** out) {
   if (!c.side && cudaStreamCreateWithFlags(&c.side, cudaStreamNonBlocking) != cudaSuccess) return LORA_ECUDA;
   for (cudaEvent_t& e : c.ev)
     if (!e && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return LORA_ECUDA;
+  *out = &c;
+  return LORA_OK;
+}
+
+// Its read-back stream and event, created on their first use.
+int read_ctx(const DeviceInfo* d, SideCtx** out) {
+  SideCtx& c = t_side.dev[d - g_dev];
+  if (!c.read && cudaStreamCreateWithFlags(&c.read, cudaStreamNonBlocking) != cudaSuccess) return LORA_ECUDA;
+  if (!c.ev_read && cudaEventCreateWithFlags(&c.ev_read, cudaEventDisableTiming) != cudaSuccess) return LORA_ECUDA;
   *out = &c;
   return LORA_OK;
 }
@@ -2336,20 +2351,20 @@ int lora_ce_fwd_bwd(const lora_ce_args* a, void* workspace, size_t workspace_byt
   ix.counts = at<int32_t>(ws, pl.counts);
   ix.seg_counts = at<int32_t>(ws, pl.segs);
   if (launch_ce_index(ix, st) != cudaSuccess) return rec(LORA_ECUDA);
-  // |T_set| and |J| size the contractions: the host reads them on the thread's side stream while the
+  // |T_set| and |J| size the contractions: the host reads them on the thread's read-back stream while the
   // dense rows, whose kernel takes them from device memory, are made on the caller's
   int32_t counts[3] = {0, 0, 0};
   {
-    SideCtx* side = nullptr;
-    if ((rc = side_ctx(d, &side)) != LORA_OK) return rec(rc);
-    if (cudaEventRecord(side->ev[0], st) != cudaSuccess || cudaStreamWaitEvent(side->side, side->ev[0], 0) != cudaSuccess)
+    SideCtx* c = nullptr;
+    if ((rc = read_ctx(d, &c)) != LORA_OK) return rec(rc);
+    if (cudaEventRecord(c->ev_read, st) != cudaSuccess || cudaStreamWaitEvent(c->read, c->ev_read, 0) != cudaSuccess)
       return rec(LORA_ECUDA);
     if (launch_ce_prepare(ix, cb(a->h), cb(a->E), D, at<bf>(ws, pl.ht), at<bf>(ws, pl.ej), mb(a->dh), a->token_loss,
                           d->num_sms, st) !=
         cudaSuccess)
       return rec(LORA_ECUDA);
-    if (cudaMemcpyAsync(counts, ix.counts, sizeof(counts), cudaMemcpyDeviceToHost, side->side) != cudaSuccess ||
-        cudaStreamSynchronize(side->side) != cudaSuccess)
+    if (cudaMemcpyAsync(counts, ix.counts, sizeof(counts), cudaMemcpyDeviceToHost, c->read) != cudaSuccess ||
+        cudaStreamSynchronize(c->read) != cudaSuccess)
       return rec(LORA_ECUDA);
   }
   if (counts[2]) return rec(LORA_EINVAL);

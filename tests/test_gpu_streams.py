@@ -150,3 +150,37 @@ def test_forward_and_backward_call_without_the_side_stream():
                        timeout=600)
     assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
     assert "one-stream call ok" in r.stdout
+
+
+def test_cross_entropy_waits_for_its_own_stream_only():
+    """One thread, two streams: a layer call on stream a that cannot start (the device sleeps there first), then the
+    LM head's cross entropy on stream b, which reads its counts back on the host. It returns while a still sleeps:
+    the read-back stands behind b's work alone, not behind the layer call's side-stream work."""
+    from tests.test_gpu_ce import CeCase
+    wl = workloads.llama_sweep(256, 16)
+    ps = build_layer(wl, seed=11)
+    projs = [p.proj() for p in ps]
+    ws = G.workspace(lora.lora_stack_workspace_size(projs, lora.LORA_FWD_BWD))
+    case = CeCase(300, 256, 5000, k=37)
+    args = case.args()
+    cws = G.workspace(lora.lora_ce_workspace_size(args))
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    # once each: kernels loaded, the thread's streams and events made
+    lora.lora_stack_step(projs, lora.LORA_FWD_BWD, ws, ws.numel(), a)
+    lora.lora_ce_fwd_bwd(args, cws, cws.numel(), b)
+    torch.cuda.synchronize()
+    want, want_dh = snapshot(ps), case.dh.view(torch.int16).clone()
+    fill_nan(ps)
+    case.dh.fill_(float("nan"))
+    torch.cuda.synchronize()
+    awake = torch.cuda.Event()
+    with torch.cuda.stream(a):
+        torch.cuda._sleep(1_000_000_000)  # clock cycles: about half a second
+        awake.record()
+    lora.lora_stack_step(projs, lora.LORA_FWD_BWD, ws, ws.numel(), a)
+    lora.lora_ce_fwd_bwd(args, cws, cws.numel(), b)
+    assert not awake.query(), "the cross entropy waited for another stream"
+    torch.cuda.synchronize()
+    assert same(snapshot(ps), want) is None
+    assert torch.equal(case.dh.view(torch.int16), want_dh)
+    assert lora.lora_read_status() == lora.LORA_OK
