@@ -370,8 +370,10 @@ __global__ void __launch_bounds__(kThreads, 1) rank_dy_kernel(const __grid_const
       for (long long j = first; j < issued; ++j)
         mbar_wait_drain(smem_u32(&ctl->full[j % G::kStages]), (uint32_t)((j / G::kStages) & 1), kDrainNs);
     }
-    if (warp == 1 && lane == 0 && issued_any) {
-      umma_commit(smem_u32(&ctl->drain));
+    if (warp == 1 && issued_any) {  // uniform across the warp
+      // the lane that issued the MMAs: a commit follows its own thread's only
+      if (elect_one()) umma_commit(smem_u32(&ctl->drain));
+      __syncwarp();
       mbar_wait_drain(smem_u32(&ctl->drain), 0, kDrainNs);
     }
     tc_fence_before();
