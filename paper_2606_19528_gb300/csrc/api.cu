@@ -1713,17 +1713,21 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
     }
   };
   // The splits for the weights and the pairs of this call, and the partials sized for the largest of those
-  // splits and the ones of either weight kind on the other pair counts above: a forward-and-backward call's
-  // workspace, whose side stream may leave few pairs to a contraction, must also hold a forward or backward
-  // call of the same shapes.
+  // splits and the ones of either weight kind, and of the call's own, on the other pair counts above: a
+  // forward-and-backward call's workspace, whose side stream may leave few pairs to a contraction, must also
+  // hold a forward or backward call of the same shapes (the checkpointed stack makes such forwards).
   std::vector<char> kind(n);
   for (int i = 0; i < n; ++i) kind[i] = is_q4(projs[i]) ? 1 : 0;
   for (int dir = 0; dir < 2; ++dir) {
     if (!(mode & (dir == 0 ? LORA_FWD : LORA_BWD))) continue;
     plan_splits(dir, kind, pairs_dir[dir], dir == 0 ? &pl->split_f : &pl->split_b);
     pairs_alt[dir].push_back(pairs_dir[dir]);
-    for (int q4 = 0; q4 < 2; ++q4)
-      for (int pairs : pairs_alt[dir]) plan_splits(dir, std::vector<char>(n, (char)q4), pairs, nullptr);
+    const bool mixed = std::count(kind.begin(), kind.end(), 1) % n != 0;
+    for (int pairs : pairs_alt[dir]) {
+      for (int q4 = 0; q4 < 2; ++q4) plan_splits(dir, std::vector<char>(n, (char)q4), pairs, nullptr);
+      // weights of both kinds make two smaller batches, which may be cut into more partials than either's one
+      if (mixed) plan_splits(dir, kind, pairs, nullptr);
+    }
   }
   size_t off = kWsHeader;
   pl->zero_bytes = off;

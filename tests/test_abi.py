@@ -75,6 +75,25 @@ def test_stack_ckpt_workspace_covers_the_largest_layer(lib):
     assert lib.lora_stack_ckpt_workspace_size(arr, 1, 65, ctypes.byref(n_bad)) == lora.LORA_EINVAL
 
 
+@pytest.mark.parametrize("T,shapes", [
+    (272, [(9216, 9952, 0, 1), (10496, 1528, 16, 0), (5376, 984, 16, 0), (5120, 4232, 16, 1)]),
+    (1040, [(7680, 6816, 0, 0), (3328, 6176, 16, 1), (10240, 6112, 16, 1), (3840, 4904, 16, 1), (9984, 4064, 16, 0)]),
+    (264, [(6144, 9776, 16, 1), (512, 5200, 0, 0), (2816, 1248, 16, 0), (4864, 1816, 16, 0), (10752, 6560, 0, 1),
+           (4096, 2304, 16, 0)])])
+def test_forward_and_backward_workspace_covers_either_alone(lib, T, shapes):
+    """Layers of 4-bit (last field 1) and bf16 weights whose forward on every SM is cut into more partials than the
+    one beside a side stream, and than with weights of one kind: the forward-and-backward size, which is all that
+    the checkpointed stack has for its first stage's forwards, covers them."""
+    codes = ctypes.create_string_buffer(16)  # sizes only: nothing is read
+    layer = []
+    for K, N, r, q4 in shapes:
+        Wq = lora.lora_q4_weight(ctypes.addressof(codes), ctypes.addressof(codes)) if q4 else None
+        layer.append(lora.make_proj(lora.make_shape(T, K, N, r, 2.0), Wq=Wq))
+    both = lora.lora_stack_workspace_size(layer, lora.LORA_FWD_BWD)
+    assert lora.lora_stack_workspace_size(layer, lora.LORA_FWD) <= both
+    assert lora.lora_stack_workspace_size(layer, lora.LORA_BWD) <= both
+
+
 def test_q4_weights_validated_on_the_host(lib):
     st = lora.make_shape(128, 128, 256, 8, 2.0)  # d_in not a multiple of 256
     ws = ctypes.c_void_p(256)
