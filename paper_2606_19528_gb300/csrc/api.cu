@@ -1625,6 +1625,7 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
   pl->cl_b.assign(n, 1);
   // the side stream's SMs are left out of the contractions they run beside: the
   // forward's in a forward-and-backward call, the dx contraction's in any call with a backward
+  // but a backward alone of few rows, which has no side stream (run_step)
   int pairs_dir[2] = {kPlanPairs, kPlanPairs};
   // pair counts the partials are also sized for: every pair, and the side widths of the same shapes with
   // bf16 and with 4-bit weights, so that a size reported from the shapes alone (lora_workspace_size)
@@ -1633,7 +1634,8 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
   if ((mode & LORA_BWD) && overlap_enabled() && any_adapter(projs, n)) {
     const SideWidths w = pl->side = side_widths(kPlanSms, projs, n);
     if (mode == LORA_FWD_BWD) pairs_dir[0] = (kPlanSms - w.w1) / 2;
-    pairs_dir[1] = (kPlanSms - w.w2) / 2;
+    const bool few = std::all_of(projs, projs + n, [](const lora_proj& p) { return p.shape.T <= gemm_small_rows(); });
+    if (mode == LORA_FWD_BWD || !few) pairs_dir[1] = (kPlanSms - w.w2) / 2;
     static const uint8_t kAnyCodes = 0;  // a non-null code pointer marks a projection 4-bit for the widths
     for (int q4 = 0; q4 < 2; ++q4) {
       std::vector<lora_proj> as(projs, projs + n);

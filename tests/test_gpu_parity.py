@@ -558,3 +558,16 @@ def test_few_rows_layer():
     for p in ps:
         check_full(p)
 
+
+def test_few_rows_backward_alone_has_every_sm():
+    """A backward alone of few rows runs on the caller's stream, so its dx contraction is planned for all 152 SMs: 73
+    tiles in clusters of two CTAs, one launch (beside a side stream they do not fit, and are cut into partials)."""
+    p = G.DevProj(*gen_proj(37, 0, 0, 64, 18688, 8192, 16, 2.0), 2.0)
+    G.run_single(p, bwd=False)
+    lora.lora_profile_begin([lora.LORA_KERNEL_GEMM_BWD])
+    G.run_single(p, fwd=False)
+    _, launches = lora.lora_profile_end()
+    assert launches["gemm_bwd"] == 1
+    rows = G.sample_rows(64, 8, 5)
+    dx = oracle.lora_backward_dx_rows(rows, p.f64("dy"), p.f64("W"), p.f64("A"), p.f64("B"), p.s)
+    assert G.rel_fro(G.host_f64(p.dx)[rows], dx) <= G.TOL_DX
