@@ -958,6 +958,8 @@ def run_gpu(args, wl):
     flops = wl.flops()
     tflops = flops / (step_ms / 1e3) / 1e12
     f_fwd, f_bwd = gemm_flops(wl)
+    # (where the forward contraction is cut, T = 256 and 512, its partials are summed beside the dx contraction, and
+    # that span counts in both: the rate is then a lower bound)
     gemm_ms = kern_ms["gemm_fwd"] + kern_ms["gemm_bwd"]
     gemm_tflops = (f_fwd + f_bwd) / (gemm_ms / 1e3) / 1e12
     sustained = peaks.get("bf16_tflops_sustained", FALLBACK_PEAKS["bf16_tflops_sustained"])

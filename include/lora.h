@@ -318,6 +318,11 @@ int64_t lora_launch_count(void);
  * lora_profile_end waits for those events, writes the summed device time in
  * milliseconds and the kernel launches per kind into ms[LORA_KERNEL_KINDS]
  * and launches[LORA_KERNEL_KINDS] (either may be NULL), and stops recording.
+ * A group's time is the span between its events: groups on the side stream of
+ * a forward-and-backward call (the backward's rank-r work, and the sum of a
+ * cut forward contraction's partials, which is of kind GEMM_FWD) run beside a
+ * contraction and wait for free SMs in that span, so the kinds' times add up to
+ * more than the call's.
  * Returns LORA_OK, LORA_EINVAL (end without begin) or LORA_ECUDA. */
 int lora_profile_begin(void);
 /* As lora_profile_begin, but only the launch groups of the kinds whose bit

@@ -1514,21 +1514,27 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
         }
         bool split = false;
         for (int p = 0; p < b.num_problems; ++p) split = split || sp[p] > 1;
-        ProfScope ps(LORA_KERNEL_GEMM_FWD, st);
-        if (!q4 && !small && use_cluster_split(b, false, gemm_sms / 2)) {
-          if (launch_fused_gemm_cs(b, false, st) != cudaSuccess) return LORA_ECUDA;
-          continue;
-        }
-        if ((rc = apply_splits(b, sp, parts)) != LORA_OK) return rc;
-        if ((small ? launch_small_gemm(b, false, q4, gemm_sms, st) : launch_fused_gemm(b, false, q4, gemm_sms, st)) !=
-            cudaSuccess)
-          return LORA_ECUDA;
         // In a forward-and-backward call nothing before the call's end needs y: the partials are summed on the
         // side stream, beside the dx contraction (which has partials of its own), and the dx contraction starts
         // a launch earlier (Llama layer T = 256: 122.2 -> 118.2 us).
         const bool on_side = split && ov.on && mode == LORA_FWD_BWD;
-        if (on_side && (rc = ov.side_after_main()) != LORA_OK) return rc;
-        if (launch_split_reduce(b, on_side ? ov.side : st) != cudaSuccess) return LORA_ECUDA;
+        {
+          ProfScope ps(LORA_KERNEL_GEMM_FWD, st);
+          if (!q4 && !small && use_cluster_split(b, false, gemm_sms / 2)) {
+            if (launch_fused_gemm_cs(b, false, st) != cudaSuccess) return LORA_ECUDA;
+            continue;
+          }
+          if ((rc = apply_splits(b, sp, parts)) != LORA_OK) return rc;
+          if ((small ? launch_small_gemm(b, false, q4, gemm_sms, st) : launch_fused_gemm(b, false, q4, gemm_sms, st)) !=
+              cudaSuccess)
+            return LORA_ECUDA;
+          if (!on_side && launch_split_reduce(b, st) != cudaSuccess) return LORA_ECUDA;
+        }
+        if (on_side) {
+          if ((rc = ov.side_after_main()) != LORA_OK) return rc;
+          ProfScope ps(LORA_KERNEL_GEMM_FWD, ov.side);  // the events of the stream it runs on
+          if (launch_split_reduce(b, ov.side) != cudaSuccess) return LORA_ECUDA;
+        }
       }
     }
   }

@@ -106,6 +106,31 @@ def test_q4_units_off_the_code_slots(T, K, N, r):
         assert torch.equal(forward(), first)
 
 
+def test_q4_split_forward_is_profiled_with_its_partial_sum():
+    """The profiled time of a forward contraction cut into partials holds their sum in either mode: beside the dx
+    contraction (forward and backward in one call) the sum takes longer, so the kind's time is not below that of the
+    forward alone, where the sum follows on the same stream (a third of the time of these 8 cuts of 9 blocks)."""
+    p = gen_q4_proj(25, 1, 0, 136, 4352, 512, 16, 2.0)
+    projs = [p.proj()]
+    ws = G.workspace(lora.lora_stack_workspace_size(projs, lora.LORA_FWD_BWD))
+
+    def gemm_fwd(mode):
+        for _ in range(20):
+            lora.lora_stack_step(projs, mode, ws, ws.numel())
+        times = []
+        for _ in range(5):
+            torch.cuda.synchronize()
+            lora.lora_profile_begin([lora.LORA_KERNEL_GEMM_FWD])
+            for _ in range(20):
+                lora.lora_stack_step(projs, mode, ws, ws.numel())
+            ms, launches = lora.lora_profile_end()
+            assert launches["gemm_fwd"] == 40
+            times.append(ms["gemm_fwd"])
+        return sorted(times)[2]
+
+    assert gemm_fwd(lora.LORA_FWD_BWD) > gemm_fwd(lora.LORA_FWD)
+
+
 def test_q4_handworked_exact():
     """The hand-worked dequantization (2 rows x 128 columns) embedded in a
     T = 8, d_in = 256, d_out = 8, r = 1 problem with A = B = 0 (zero codes and
