@@ -98,6 +98,22 @@ def test_ce_full_vocab_parity():
     assert nJ == 4000
 
 
+def test_ce_vocabulary_past_2_20():
+    """A table of more than 2^20 tokens: the tokens before each of the 128 segments of J are counted in a launch of
+    its own. Targets at both ends and the segments' edges, table rows spread over the whole vocabulary."""
+    V, k = 2 ** 20 + 1003, 9
+    case = CeCase(64, 64, V, frac=0.7)
+    seg = -(-V // 128)
+    rng = np.random.default_rng(3)
+    case.targets = rng.integers(0, V, case.T).astype(np.int32)
+    case.targets[-6:] = [0, V - 1, seg - 1, seg, 127 * seg, 127 * seg - 1]
+    step = (np.arange(k, dtype=np.int64) * 116507)[None, :]
+    case.topk, case.k = ((np.arange(V, dtype=np.int64)[:, None] + step) % V).astype(np.int32), k
+    case.t_targets, case.t_topk = torch.from_numpy(case.targets).cuda(), torch.from_numpy(case.topk).cuda()
+    nT, nJ = check(case)
+    assert nT == 45 and 300 < nJ <= nT * k
+
+
 def test_ce_table_covering_the_whole_vocabulary():
     """A top-k table whose rows cover every token makes J the whole
     vocabulary: E is read in place although a table was given."""
