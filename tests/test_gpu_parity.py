@@ -551,12 +551,42 @@ def test_few_rows(T, K, N, r):
 
 
 def test_few_rows_layer():
-    """A layer at T = 72 with frozen projections among the adapted ones, forward and backward in one call."""
-    ps = [G.DevProj(*gen_proj(36, i, 0, 72, K, N, 16, 2.0), 2.0)
-          for i, (K, N) in enumerate([(1024, 1024), (1024, 264), (8200, 520), (520, 16392)])]
-    G.run_stack(ps)
-    for p in ps:
-        check_full(p)
+    """A layer at T = 72 with frozen projections among the adapted ones (CTAs with tiles of the frozen ones alone load
+    no adapter block): the forward alone, the backward alone (both start beside the kernels before them), then both
+    in one call, each against the oracle."""
+    sizes = [(1024, 1024, 16), (1024, 264, 0), (8200, 520, 16), (520, 16392, 0)]
+    ps = [G.DevProj(*gen_proj(36, i, 0, 72, K, N, max(r, 1), 2.0), 2.0) for i, (K, N, r) in enumerate(sizes)]
+
+    def proj(p, r):
+        if r:
+            return p.proj()
+        return lora.make_proj(lora.make_shape(p.T, p.K, p.N, 0, 1.0), x=p.x, W=p.W, dy=p.dy, y=p.y, dx=p.dx)
+
+    projs = [proj(p, r) for p, (_, _, r) in zip(ps, sizes)]
+    ws = G.workspace(lora.lora_stack_workspace_size(projs, lora.LORA_FWD_BWD))
+
+    def check(fwd, bwd):
+        torch.cuda.synchronize()
+        assert lora.lora_read_status() == lora.LORA_OK
+        for p, (_, _, r) in zip(ps, sizes):
+            if r and bwd:  # su and y are there from the forward before
+                check_full(p)
+            elif r:
+                y, u = oracle.lora_forward(p.f64("x"), p.f64("W"), p.f64("A"), p.f64("B"), p.s)
+                assert G.rel_fro(G.host_f64(p.y), y) <= G.TOL_Y
+                assert G.rel_fro(G.host_f64(p.su), p.s * u) <= G.TOL_SU
+            else:
+                if fwd:
+                    assert G.rel_fro(G.host_f64(p.y), p.f64("x") @ p.f64("W").T) <= G.TOL_Y
+                if bwd:
+                    assert G.rel_fro(G.host_f64(p.dx), p.f64("dy") @ p.f64("W")) <= G.TOL_DX
+
+    for mode in (lora.LORA_FWD, lora.LORA_BWD, lora.LORA_FWD_BWD):
+        for p in ps:
+            for t in (p.dx, p.dA, p.dB) if mode == lora.LORA_BWD else (p.y, p.su, p.dx, p.dA, p.dB):
+                t.fill_(float("nan"))
+        lora.lora_stack_step(projs, mode, ws, ws.numel())
+        check(mode & lora.LORA_FWD, mode & lora.LORA_BWD)
 
 
 def test_few_rows_backward_alone_has_every_sm():
