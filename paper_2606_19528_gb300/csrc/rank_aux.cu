@@ -12,9 +12,15 @@ namespace {
 
 // Second pass: out = sum of a tile's unit partials, in unit order.  One thread
 // per 8 consecutive rank columns (a sector of each partial) of one row of
-// [tile][tile_rows][rpad], lanes along the rows, so that the transposed outputs
-// (su^T, sv^T and dA) are stored in whole lines; the loads of all units are
-// independent and issued together.
+// [tile][tile_rows][rpad]; the loads of all units are independent and issued
+// together.  2 or 4 lanes lie along the columns (64 bytes, or a whole line of
+// a partial), the others along the rows, so that the transposed outputs (su^T, sv^T
+// and dA) are stored in pieces of 16 to 64 bytes.  Launched early, this kernel shares
+// its SMs with the product kernel, whose shared memory leaves little L1 to hold
+// loads in flight: with all lanes along the rows a load touched a line per lane,
+// and su at T = 2048, r = 64 (Qwen-shaped layer) took 43 us with its products where
+// it now takes 32, the forward of a 11008 x 64 projection at T = 8192, r = 64 93 us
+// where it now takes 77.
 template <typename Batch, bool kRow>
 __global__ void __launch_bounds__(256) reduce_partials_kernel(const __grid_constant__ Batch b, int total8) {
   if (b.early_next) griddep_launch_dependents();
@@ -29,7 +35,8 @@ __global__ void __launch_bounds__(256) reduce_partials_kernel(const __grid_const
   const int rpad = P.rpad, upt = P.upt, tr = b.tile_rows;
   const int per = tr * (rpad / 8);  // threads of a tile
   const int tile = e / per, k = e % per;
-  const int j = k / tr * 8, lr = k % tr;
+  const int g = (rpad & 31) == 0 ? 4 : 2;  // lanes along the columns
+  const int j = (k / (tr * g) * g + k % g) * 8, lr = k / g % tr;
   const size_t blk = (size_t)tr * rpad;
   const float* src = b.partials + P.part_off + (size_t)tile * upt * blk + (size_t)lr * rpad + j;
   float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
