@@ -1110,9 +1110,9 @@ int call_cluster_tiles(int n, Q4 q4, const lora_proj* projs, bool bwd, int pairs
 }
 
 // Widths of the side stream in its two phases.  Beside the forward
-// contraction (2TKN FLOPs per projection, compute-bound, 4-bit weights ~1.3x
-// slower per FLOP) it transposes B and su and reads dy once: the fused pass
-// (sv and dB, r <= 16) or the sv pass; the dx contraction waits for sv.
+// contraction (2TKN FLOPs per projection, compute-bound, 4-bit weights as fast)
+// it transposes B and su and reads dy once: the fused pass (sv and dB, r <= 16)
+// or the sv pass; the dx contraction waits for sv.
 // Beside the dx contraction it runs dA = sv^T x (2TK bytes per distinct x) and,
 // where the pass over dy was not fused, dB (dy read again, 0.3 x as costly
 // per byte).  The rank-r kernels are issue-bound, costlier per byte as r
@@ -1123,13 +1123,20 @@ int call_cluster_tiles(int n, Q4 q4, const lora_proj* projs, bool bwd, int pairs
 // partial sums, fp32 gradients).  kappa1 gives the Llama-3.2-3B layer at
 // r = 16 12 SMs, kappa2 8 SMs, the measured best pair at T = 2048; the same
 // constants give 16 / 8 for the Qwen-2.5-3B layer at r = 16 (best measured
-// 16-18 / 8) and 22 / 16 at r = 64 (18-22 / 16: 851 us, 22 / 22: 862 us).  Rounded to even
+// 16-18 / 8) and 22 / 16 at r = 64 (18-22 / 16: 851 us, 22 / 22: 862 us).  In a
+// forward-and-backward call the side's second phase may start before the dx
+// contraction; in a backward alone it starts with it, and the few tokens of a small
+// call do not hide that the unfused pass stores dB, whatever T: there it counts 16
+// bytes per r N more (Llama-shaped layer, backward alone: T = 256, r = 32, 14 -> 22
+// SMs, 93.1 -> 75.2 us; T = 512, r = 64, 16 -> 24, 128.7 -> 99.1; Qwen-shaped T =
+// 4096, r = 64, 16 -> 18, 450 and 451).  Rounded to even
 // counts so the contractions keep whole CTA pairs; LORA_SIDE_SMS and
 // LORA_SIDE_SMS2 override.
 constexpr double kSideKappa1 = 290.0;
 constexpr double kSideKappa2 = 245.0;
 constexpr double kSideAdapter1 = 12.0;  // bytes per r N
 constexpr double kSideAdapter2 = 8.0;   // bytes per r K
+constexpr double kSideStore2 = 16.0;    // bytes per r N where the pass over dy is not fused, backward alone
 constexpr double kSideSecondPass = 0.3;  // the unfused dB pass over dy: its kernel streams faster per byte
 
 int env_int(const char* name) {
@@ -1139,7 +1146,7 @@ int env_int(const char* name) {
 
 bool dy_fusable(int T, int N, int r);
 
-SideWidths side_widths(int num_sms, const lora_proj* projs, int n) {
+SideWidths side_widths(int num_sms, const lora_proj* projs, int n, bool bwd_alone) {
   static const int v1 = env_int("LORA_SIDE_SMS"), v2 = env_int("LORA_SIDE_SMS2");
   double b1 = 0.0, b2 = 0.0, flops = 0.0;
   std::vector<const void*> xs;
@@ -1151,7 +1158,8 @@ SideWidths side_widths(int num_sms, const lora_proj* projs, int n) {
     const double fr = 1.0 + r / 144.0;
     b1 += 2.0 * T * N * fr + kSideAdapter1 * r * N;
     b2 += kSideAdapter2 * r * K;
-    if (!dy_fusable((int)sh.T, (int)sh.d_out, (int)sh.rank)) b2 += kSideSecondPass * 2.0 * T * N * fr;
+    if (!dy_fusable((int)sh.T, (int)sh.d_out, (int)sh.rank))
+      b2 += kSideSecondPass * 2.0 * T * N * fr + (bwd_alone ? kSideStore2 * r * N : 0.0);
     // dA reads each distinct x once (shapes without pointers: once per projection)
     const void* x = projs[i].x;
     if (x == nullptr || std::find(xs.begin(), xs.end(), x) == xs.end()) {
@@ -1255,7 +1263,7 @@ struct Overlap {
   int side_ctas2 = 0;  // beside the dx contraction
   cudaStream_t main = nullptr, side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_sv = nullptr, ev_done = nullptr, ev_fwd = nullptr;
-  int init(const DeviceInfo* d, cudaStream_t st, const lora_proj* projs, int n, const SideWidths& planned) {
+  int init(const DeviceInfo* d, cudaStream_t st, const lora_proj* projs, int n, int mode, const SideWidths& planned) {
     if (!overlap_enabled() || !any_adapter(projs, n)) return LORA_OK;
     SideCtx* ctx = nullptr;
     const int rc = side_ctx(d, &ctx);
@@ -1267,7 +1275,7 @@ struct Overlap {
     ev_sv = c.ev[1];
     ev_done = c.ev[2];
     ev_fwd = c.ev[3];
-    const SideWidths w = d->num_sms == kPlanSms ? planned : side_widths(d->num_sms, projs, n);
+    const SideWidths w = d->num_sms == kPlanSms ? planned : side_widths(d->num_sms, projs, n, mode == LORA_BWD);
     side_ctas = w.w1;
     side_ctas2 = w.w2;
     on = true;
@@ -1331,7 +1339,7 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
   Overlap ov;
   // (a backward alone of few rows stays on the caller's stream: its dA takes a few microseconds after the dx
   // contraction, less than the events of a second stream cost the host)
-  if ((mode & LORA_BWD) && !(mode == LORA_BWD && small_bwd) && (rc = ov.init(d, st, projs, n, pl.side)) != LORA_OK) return rc;
+  if ((mode & LORA_BWD) && !(mode == LORA_BWD && small_bwd) && (rc = ov.init(d, st, projs, n, mode, pl.side)) != LORA_OK) return rc;
   const int gemm_sms = ov.on ? d->num_sms - ov.side_ctas : d->num_sms;      // forward contraction
   const int gemm_sms_b = ov.on ? d->num_sms - ov.side_ctas2 : d->num_sms;  // dx contraction
   // backward rank-r work: B^T, su^T, sv (and sv^T), then dB and dA; on `rs`
@@ -1638,7 +1646,7 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
   // covers a call of either weight kind in any mode
   std::vector<int> pairs_alt[2] = {{kPlanPairs}, {kPlanPairs}};
   if ((mode & LORA_BWD) && overlap_enabled() && any_adapter(projs, n)) {
-    const SideWidths w = pl->side = side_widths(kPlanSms, projs, n);
+    const SideWidths w = pl->side = side_widths(kPlanSms, projs, n, mode == LORA_BWD);
     if (mode == LORA_FWD_BWD) pairs_dir[0] = (kPlanSms - w.w1) / 2;
     const bool few = std::all_of(projs, projs + n, [](const lora_proj& p) { return p.shape.T <= gemm_small_rows(); });
     if (mode == LORA_FWD_BWD || !few) pairs_dir[1] = (kPlanSms - w.w2) / 2;
@@ -1646,10 +1654,13 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
     for (int q4 = 0; q4 < 2; ++q4) {
       std::vector<lora_proj> as(projs, projs + n);
       for (lora_proj& p : as) p.Wq.codes = q4 ? &kAnyCodes : nullptr;
-      const SideWidths wa = side_widths(kPlanSms, as.data(), n);
-      pairs_alt[0].push_back((kPlanSms - wa.w1) / 2);
-      pairs_alt[1].push_back((kPlanSms - wa.w2) / 2);
+      for (bool alone : {false, true}) {
+        const SideWidths wa = side_widths(kPlanSms, as.data(), n, alone);
+        pairs_alt[0].push_back((kPlanSms - wa.w1) / 2);
+        pairs_alt[1].push_back((kPlanSms - wa.w2) / 2);
+      }
     }
+    pairs_alt[1].push_back((kPlanSms - side_widths(kPlanSms, projs, n, true).w2) / 2);
   }
   std::vector<size_t> split_need_dir[2] = {std::vector<size_t>(n, 0), std::vector<size_t>(n, 0)};
   // The splits of direction `dir` on `pairs` pairs with the projections' weights as `kind` says (0 bf16,
@@ -1730,6 +1741,8 @@ int plan_all(const lora_proj* projs, int n, int mode, Plan* pl, bool allow_split
     if (!(mode & (dir == 0 ? LORA_FWD : LORA_BWD))) continue;
     plan_splits(dir, kind, pairs_dir[dir], dir == 0 ? &pl->split_f : &pl->split_b);
     pairs_alt[dir].push_back(pairs_dir[dir]);
+    std::sort(pairs_alt[dir].begin(), pairs_alt[dir].end());
+    pairs_alt[dir].erase(std::unique(pairs_alt[dir].begin(), pairs_alt[dir].end()), pairs_alt[dir].end());
     const bool mixed = std::count(kind.begin(), kind.end(), 1) % n != 0;
     for (int pairs : pairs_alt[dir]) {
       for (int q4 = 0; q4 < 2; ++q4) plan_splits(dir, std::vector<char>(n, (char)q4), pairs, nullptr);
