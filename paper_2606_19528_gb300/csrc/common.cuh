@@ -174,8 +174,10 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
 }
 
 // Arrive on a barrier of either CTA without a cluster-scope fence, for signals that hand over no data one
-// thread wrote and a thread of the other CTA reads: a drained accumulator, a tile id that was read, or an
-// operand tile that the writers' own CTA's tensor core reads (the writers fence it for the async proxy).
+// thread wrote and a thread of the other CTA reads: a drained accumulator (the loads waited for), a tile id
+// whose value the signalling thread holds in a register, or an operand tile that the writers' own CTA's tensor
+// core reads (the writers fence it for the async proxy).  Nothing else orders the thread's earlier reads of
+// shared memory before what the other CTA does next.
 // The cluster-scope release above takes 800 to 1400 cycles beside a running contraction, since the fence
 // waits for the memory traffic in flight.
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {

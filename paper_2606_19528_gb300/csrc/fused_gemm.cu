@@ -229,6 +229,24 @@ __device__ __forceinline__ void dequant_stage(uint32_t slot, uint32_t wdst, int 
   }
 }
 
+// Takes the tile id of a ring slot and lets the slot be refilled (`empty`: the slot's barrier in the even CTA).
+// The refill of the odd CTA's copy is a store by the even CTA, ordered after this read only through the arrival,
+// which carries no cluster-scope release (see mbar_arrive_remote): so the id has to be in a register before the
+// arrival is issued, by the shuffle, or by a branch on it.  (Without, warps of the odd CTA took the id that was
+// written four tiles later: tiles of a contraction of one or two blocks, whose scheduler runs four tiles ahead,
+// were left out.  With a cluster-scope release per warp and tile instead: Llama-shaped layer T = 256 118.4 -> 120.5
+// us, a 3080 x 4104 projection at T = 1000 71.8 -> 73.7.)
+__device__ __forceinline__ int take_tile(volatile int* id, uint32_t empty, int lane) {  // a converged warp
+  const int t = __shfl_sync(0xffffffffu, *id, 0);
+  if (lane == 0) mbar_arrive_remote(empty);
+  return t;
+}
+__device__ __forceinline__ int take_tile(volatile int* id, uint32_t empty) {  // one thread
+  const int t = *id;
+  if (t >= -1) mbar_arrive_remote(empty);  // always
+  return t;
+}
+
 template <bool kBMn, bool kQ, bool kF32 = false, bool kCS = false, bool kN256 = false>
 __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __grid_constant__ GemmBatch b) {
   // fp32 output: 256 x 256 tiles whose accumulator alternates between two TMEM
@@ -358,8 +376,7 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
           mbar_arrive_cluster(mapa_shared(smem_u32(&ctl->tile_full[slot]), pb + 1));
         } else {
           if (!mbar_wait_cluster(smem_u32(&ctl->tile_full[slot]), par, wc, abort_flag)) break;
-          t = *reinterpret_cast<volatile int*>(&ctl->tile_id[slot]);
-          mbar_arrive_remote(tile_empty_root + (uint32_t)slot * 8u);
+          t = take_tile(&ctl->tile_id[slot], tile_empty_root + (uint32_t)slot * 8u);
         }
         if (t < 0) {
           griddep_launch_dependents();  // no tile left for this pair
@@ -449,9 +466,7 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
           bool got = mbar_wait_cluster(smem_u32(&ctl->tile_full[slot]), (uint32_t)((it / kTileRing) & 1), wc, abort_flag);
           got = __all_sync(0xffffffffu, got);
           if (!got) break;
-          t = *reinterpret_cast<volatile int*>(&ctl->tile_id[slot]);
-          t = __shfl_sync(0xffffffffu, t, 0);
-          if (lane == 0) mbar_arrive_remote(tile_empty_root + (uint32_t)slot * 8u);
+          t = take_tile(&ctl->tile_id[slot], tile_empty_root + (uint32_t)slot * 8u, lane);
         }
         if (t < 0) {
           griddep_launch_dependents();  // no tile left for this pair
@@ -626,9 +641,7 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
       bool got = mbar_wait_cluster(smem_u32(&ctl->tile_full[slot]), (uint32_t)((it / kTileRing) & 1), wc, abort_flag);
       got = __all_sync(0xffffffffu, got);
       if (!got) break;
-      const int t = *reinterpret_cast<volatile int*>(&ctl->tile_id[slot]);
-      __syncwarp();
-      if (lane == 0) mbar_arrive_remote(tile_empty_root + (uint32_t)slot * 8u);
+      const int t = take_tile(&ctl->tile_id[slot], tile_empty_root + (uint32_t)slot * 8u, lane);
       if (t < 0) break;
       int p, m0, n0, ks, kb0, kb1;
       decode_tile<kTileN, kTileM>(b, t, p, m0, n0, ks, kb0, kb1);
@@ -890,9 +903,7 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
       bool got = mbar_wait_cluster(smem_u32(&ctl->tile_full[slot]), (uint32_t)((it / kTileRing) & 1), wc, abort_flag);
       got = __all_sync(0xffffffffu, got);
       if (!got) break;
-      const int t = *reinterpret_cast<volatile int*>(&ctl->tile_id[slot]);
-      __syncwarp();
-      if (lane == 0) mbar_arrive_remote(tile_empty_root + (uint32_t)slot * 8u);
+      const int t = take_tile(&ctl->tile_id[slot], tile_empty_root + (uint32_t)slot * 8u, lane);
       if (t < 0) break;
       int p, m0, n0, ks, kb0, kb1;
       decode_tile<kTileN, kTileM>(b, t, p, m0, n0, ks, kb0, kb1);
@@ -973,8 +984,7 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
         const int slot = it % kTileRing;
         if (!mbar_wait_cluster(smem_u32(&ctl->tile_full[slot]), (uint32_t)((it / kTileRing) & 1), wc, abort_flag))
           break;
-        const int t = *reinterpret_cast<volatile int*>(&ctl->tile_id[slot]);
-        mbar_arrive_remote(tile_empty_root + (uint32_t)slot * 8u);
+        const int t = take_tile(&ctl->tile_id[slot], tile_empty_root + (uint32_t)slot * 8u);
         if (t < 0) break;
         int p, m0, n0, ks, kb0, kb1;
         decode_tile<kTileN, kTileM>(b, t, p, m0, n0, ks, kb0, kb1);

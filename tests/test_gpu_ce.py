@@ -98,6 +98,14 @@ def test_ce_full_vocab_parity():
     assert nJ == 4000
 
 
+@pytest.mark.parametrize("T,d,V", [(1562, 8, 21662), (1047, 88, 20570)])
+def test_ce_many_short_tiles(T, d, V):
+    """Logits contractions of one and two blocks over 4 to 8 tiles per CTA pair: the scheduler of a pair runs as far
+    ahead of its epilogue as the ring of tile ids lets it. Every loss, and dh, of several calls on fresh inputs."""
+    for seed in range(4):
+        check(CeCase(T, d, V, frac=1.0, seed=seed))
+
+
 def test_ce_vocabulary_past_2_20():
     """A table of more than 2^20 tokens: the tokens before each of the 128 segments of J are counted in a launch of
     its own. Targets at both ends and the segments' edges, table rows spread over the whole vocabulary."""
