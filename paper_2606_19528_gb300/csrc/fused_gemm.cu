@@ -386,7 +386,11 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
         decode_tile<kTileN, kTileM>(b, t, p, m0, n0, ks, kb0, kb1, cs_half);
         const GemmProblem& Q = b.prob[p];
         const int my_m = m0 + c * kHalf;
-        const bool a_mine = my_m < Q.M;
+        // The odd CTA loads something of every block, if only rows past M (zeros, never stored): its producer
+        // follows the ring by the parity of `empty`, and a block without bytes of its own would not wait for it,
+        // so the ring could pass it twice unseen.
+        const bool odd_any = m0 + kHalf < Q.M || (!kQ && n0 + kHalf < Q.N);
+        const bool a_mine = my_m < Q.M || (c == 1 && !odd_any);
         const bool a_mine2 = kQ && my_m + kBM < Q.M;  // the second row segment
         // weight box (segment h, pair position cc, j): columns n0 + 256 h + 128 cc + 64 j
         auto box_ok = [&](int h, int cc, int j) { return n0 + h * kSeg + cc * kHalf + j * 64 < Q.N; };
@@ -395,7 +399,7 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
           for (int cc = 0; cc < 2; ++cc)
             for (int j = 0; j < 2; ++j) boxes += box_ok(h, cc, j) ? 1u : 0u;
         // bytes landing in this pair per stage (signalled on the even CTA)
-        uint32_t tx_a = (m0 < Q.M ? kAHalf : 0u) + (m0 + kHalf < Q.M ? kAHalf : 0u);
+        uint32_t tx_a = (m0 < Q.M ? kAHalf : 0u) + (m0 + kHalf < Q.M || !odd_any ? kAHalf : 0u);
         if (kQ) tx_a += (m0 + kBM < Q.M ? kAHalf : 0u) + (m0 + kBM + kHalf < Q.M ? kAHalf : 0u);
         const uint32_t tx_pair = tx_a + kBox * boxes;
         bool ok = true;
