@@ -124,12 +124,12 @@ int lora_linear_fwd(const lora_shape* shape, const lora_bf16* x, const lora_bf16
  * overlap on the GPU (for example on two streams at once) race and give
  * wrong results.  Nothing is allocated.  It never stores fp32 partial sums
  * of a contraction: lora_linear_fwd may cut the contraction of a forward
- * with few output tiles (fewer than 76 of 256 x 512) into fp32 partials in
- * its workspace when the two CTA pairs of a cluster cannot share it, and
- * there the two results differ by the bf16 rounding of differently ordered
- * fp32 sums; everywhere else (76 or more tiles, or a contraction shared
- * within clusters, as for 512 tokens x d_out 3072) they are identical bit
- * for bit.  The paper has no counterpart of this entry point.  Returns as
+ * with few output tiles (fewer than 76 of 256 x 512; up to 128 tokens, fewer
+ * than 152 of 128 x 256) into fp32 partials in its workspace, where no
+ * cluster of CTAs can share its tiles, and there the two results differ by
+ * the bf16 rounding of differently ordered fp32 sums; everywhere else (more
+ * tiles, or a contraction shared within clusters, as for 512 tokens x d_out
+ * 3072) they are identical bit for bit.  The paper has no counterpart of this entry point.  Returns as
  * lora_linear_fwd (argument errors first), or LORA_ESCRATCH. */
 int lora_linear_fwd_noalloc(const lora_shape* shape, const lora_bf16* x, const lora_bf16* W,
                             const lora_bf16* A, const lora_bf16* B, lora_bf16* y, lora_bf16* su,
@@ -210,7 +210,9 @@ int lora_stack_step(const lora_proj* projs, int n_proj, int mode, void* workspac
  * stages; no su of any layer outlives its backward.  `projs` holds
  * n_layers x n_per_layer projections, layer-major, each with x, W (or Wq),
  * A, B, dy, y, dA, dB (dx optional); their su fields are ignored.  y is
- * written by both stages (with the same values).  Results equal those of
+ * written by both stages, with the same values but for the bf16 rounding of
+ * differently ordered fp32 sums where a layer's forward contraction is cut
+ * (few output tiles; the second stage's has fewer SMs).  Results equal those of
  * lora_stack_step(LORA_FWD_BWD) layer by layer.  n_per_layer 1..64.
  * Returns as lora_stack_step. */
 int lora_stack_ckpt_workspace_size(const lora_proj* projs, int n_layers, int n_per_layer, size_t* bytes);
@@ -262,8 +264,9 @@ int lora_ce_fwd_bwd(const lora_ce_args* args, void* workspace, size_t workspace_
  * row i of `table` [V, k] int32 lists the k tokens with the largest C[i, :],
  * in descending order, the lower index first on equal similarities (row i
  * starts with i unless another token has the same direction).  The V x V
- * matrix is never formed.  Below V = 32768 similarities are computed some
- * hundreds of rows at a time in fp32 on the tensor cores and each row's top k is selected from
+ * matrix is never formed.  Below V = 32768 similarities are computed in chunks
+ * of rows (up to 64 MB of them to 8192 tokens, up to 96 MB beyond) in fp32 on
+ * the tensor cores and each row's top k is selected from
  * them.  From V = 32768 on, each row first gets a threshold from its
  * similarities to up to 8192 evenly spread tokens, the similarity contraction keeps
  * only the values at or above it (at most 4096 per row, in workspace), and

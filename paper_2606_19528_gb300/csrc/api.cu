@@ -309,18 +309,24 @@ constexpr int kPlanPairs = kPlanSms / 2;  // CTA pairs of a launch on all of the
 // persistent kernel hands out (tile, split) units in order to whichever pair
 // is free, so for each candidate split length L (problem p cut into
 // ceil(kb_p / L) splits, at most 8) the walk is simulated on `pairs` pairs in
-// units of one k-block of a 256 x 512 tile (~0.77 us at the measured rate),
-// with a fixed cost per unit (pipeline fill, epilogue), one more for an fp32
+// units of one k-block of a 256 x 512 tile (0.56 us: 1090 cycles at 1.93 GHz),
+// with a fixed cost per unit (pipeline fill, epilogue), more for an fp32
 // partial epilogue, and the reduce launch plus its traffic; the cheapest
 // candidate wins (fewer splits on ties).  Choices are cached per shape set.
+// The constants are fitted to whole calls (layers of 136 to 1536 tokens, cut and
+// uncut), not measured one by one: the 6 blocks of a partial epilogue hold what the
+// pair that finishes last loses, and partials of up to some tens of MB are read
+// from L2, hence 5 MB per block time (8.9 TB/s).  The known misfit: 104 wide tiles
+// of 17 to 129 blocks on 68 pairs (the Llama-shaped layer's dx contraction at T =
+// 512) are cut where uncut they are some 3 % faster.
 constexpr double kUnitFixBlocks = 3.0;    // per unit: pipeline fill and epilogue
 constexpr double kPartEpiBlocks = 6.0;    // per split unit: fp32 partial tile instead of bf16
 constexpr double kReduceFixBlocks = 6.0;  // the reduce launch
-constexpr double kBytesPerBlock = 5.0e6;  // HBM bytes moved in one block time
+constexpr double kBytesPerBlock = 5.0e6;  // bytes of partials moved in one block time
 
 // A problem's block in those units: a 4-bit problem's 512 x 256 tile holds as many MMAs, half as many when
 // the problem has one 256-row segment only; so does the 256 x 256 tile of fp32 output.
-constexpr double kNarrowBlockCost = 0.75;  // 256 x 256 tiles, bf16: ~820 cycles a block against ~1090 for 256 x 512
+constexpr double kNarrowBlockCost = 0.75;  // 256 x 256 tiles, bf16: 820 cycles a block against 1090 for 256 x 512
 constexpr double kSmallBlockCost = 1.0;  // 128 x 256 tiles of the few-rows kernel, one CTA: the weight stream
 double block_cost(const GemmProblem& g) {
   const bool q4 = g.m_pad == g.num_m_tiles * gemm_tile_m_q4();
@@ -1348,7 +1354,6 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
   // ctas: CTAs of the transposes and the passes over dy, on rs; rs2: the stream bwd_cols runs on
   std::vector<bf*> sut(n), svt(n);
   std::vector<char> fused(n);
-  // early_next: the dx contraction follows on the same stream and may start beside these
   // rank sides as K-major tensor-core operands: B^T for sv = s dy B (bit 0 of `which`) and su^T for dB =
   // dy^T su (bit 1), zero rows past r
   auto transposes = [&](cudaStream_t rs, int which) -> int {
@@ -1380,6 +1385,7 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
   long long bt_elems = 0;
   for (int i = 0; i < n; ++i) bt_elems += projs[i].shape.d_out * rank_pad8((int)projs[i].shape.rank);
   const bool bt_early = bt_elems >= (1 << 17);
+  // early_next: the dx contraction follows on the same stream and may start beside these
   auto bwd_rank = [&](cudaStream_t rs, int ctas, cudaStream_t rs2, bool early_next) -> int {
     int rc;
     std::vector<RowSpec> rows;
@@ -1481,9 +1487,9 @@ int run_step(const lora_proj* projs, int n, int mode, void* ws, const Plan& pl, 
     {
       ProfScope ps(LORA_KERNEL_ROWPROJ, st);
       // Without a side stream the contraction may start beside these products (Llama-shaped layer forward,
-      // T = 32: 56.7 -> 53.5 us).  With one it must not: its CTA pairs would take the free SMs first and its
-      // last pairs then wait for SM pairs that the side stream's CTAs have split up (Llama layer T = 256:
-      // 124 -> 130 us; q projection T = 512: 45.6 -> 47.9 us).
+      // T = 32: 56.7 -> 53.5 us, on the pairs' tiles of that time).  With one it must not: its CTA pairs would
+      // take the free SMs first and its last pairs then wait for SM pairs that the side stream's CTAs have split
+      // up (Llama layer T = 256: 124 -> 130 us; q projection T = 512: 45.6 -> 47.9 us).
       if ((rc = launch_rows(rows, arena(ws, pl, kPhFwdRows), d, d->num_sms, st, !ov.on || small_fwd)) != LORA_OK) return rc;
     }
     if (!rows.empty()) prior_main = true;
@@ -1888,7 +1894,7 @@ int ce_check(const lora_ce_args* a, CePlan* pl) {
     return o;
   };
   pl->tiles = take(16);
-  pl->counts = take(32);  // |T_set|, |J|, error flag, -, two last-block counters
+  pl->counts = take(32);  // |T_set|, |J|, error flag, -, -, positions whose loss is written
   pl->segs = take(128 * 4);
   pl->flags = take((size_t)V);
   pl->J = take((size_t)V * 4);

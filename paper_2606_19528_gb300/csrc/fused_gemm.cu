@@ -293,8 +293,7 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
-      // producer (expect_tx), plus every dequantizing warp of both CTAs
-      mbar_init(smem_u32(&ctl->full[s]), 1);
+      mbar_init(smem_u32(&ctl->full[s]), 1);  // the even CTA's producer (expect_tx)
       mbar_init(smem_u32(&ctl->empty[s]), 1);
     }
     for (int q = 0; q < QS::kStages; ++q) {
@@ -459,7 +458,7 @@ __global__ void __launch_bounds__(Cfg<kQ>::kThreads, 1) fused_lora_gemm(const __
       const uint16_t pair_mask = (uint16_t)(0x3u << pb);
       int stage = 0;
       uint32_t phase = 0;
-      uint32_t wseq = 0;  // 4-bit: contraction blocks so far (weight tile wseq % 2)
+      uint32_t wseq = 0;  // 4-bit: contraction blocks so far (weight tile wseq % kWStages)
       bool ok = true;
       for (int it = 0; ok; ++it) {
         const int slot = it % kTileRing;

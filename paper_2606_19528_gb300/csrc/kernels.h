@@ -328,7 +328,7 @@ struct CeIndex {
   int k;
   uint8_t* flags;
   int32_t *J, *tl, *tpos, *ycol;
-  int32_t* counts;      // [8]: |T_set|, |J|, error flag, -, -, a last-block counter
+  int32_t* counts;      // [8]: |T_set|, |J|, error flag, -, -, positions whose loss is written
   int32_t* seg_counts;  // 128 per-segment counts of the vocabulary compaction
 };
 cudaError_t launch_ce_index(const CeIndex& a, cudaStream_t stream);

@@ -15,7 +15,9 @@
 // Against the pairs, in the same calls: Llama-shaped layer forward at T = 32
 // (201 MB of bf16 weights) 48.6 -> 43.2 us, forward and backward at T = 64 with
 // 4-bit weights 124 -> 91 us, Qwen-shaped layer forward and backward at T = 32,
-// r = 4 117 -> 95 us.  From 129 rows on, a pair's MMAs are as full as a CTA's.
+// r = 4 117 -> 95 us; with what came after (contractions that start beside the
+// rank-r products, clusters, su^T and B^T made earlier) 41.7, 82 and 86 us.  From 129
+// rows on, a pair's MMAs are as full as a CTA's.
 //   warp 0      tile scheduler and TMA producer: 4 stages of [activation 16 KB |
 //               weight 32 KB] (4-bit: 3 stages; the weight part is dequantized)
 //   warp 1      TMEM allocation; tcgen05.mma issuer (one elected lane)

@@ -3,9 +3,9 @@
 // normalised, C = E~ E~^T holds the cosine similarities, and row i of the
 // table lists the k most similar tokens in descending order (lower index
 // first on ties).  The V x V matrix is never formed.
-//   row_norms,          E~_i = bf16(E_i / ||E_i||), the sum of squares
-//                       accumulated in fp32 in index order (squares of bf16
-//                       are exact), correctly rounded sqrt and division
+//   row_norms           ||E_i||, the sum of squares accumulated in fp32 in index
+//                       order (squares of bf16 are exact), correctly rounded sqrt
+//   scale_rows          E~_i = bf16(E_i / ||E_i||), the division correctly rounded
 // Rows shorter than 32768 tokens (the host runs chunks of rows):
 //   topk_short          (up to 8192 tokens) per row of a chunk's fp32 similarities
 //                       (tcgen05 contraction in fused_gemm.cu): the values from
