@@ -132,6 +132,10 @@ int device_info(DeviceInfo** out) {
     d.ready = true;
   }
   if (!d.supported) return LORA_EDEVICE;
+  // A host thread's first CUDA call may be this one: tensor maps are encoded through the driver, which needs the
+  // device's context to be current (a runtime call that takes a stream would make it so, but a call need not have
+  // made one by then).
+  if (cudaSetDevice(dev) != cudaSuccess) return LORA_ECUDA;
   *out = &d;
   return LORA_OK;
 }

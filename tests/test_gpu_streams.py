@@ -97,6 +97,34 @@ def test_two_host_threads_at_once():
         assert same(snapshot(ps), want) is None
 
 
+def test_first_cuda_call_of_a_host_thread():
+    """A forward whose plan needs no counter cleared, as the first CUDA call of a host thread: the same bits as from
+    the thread that made the inputs."""
+    from tests.test_gpu_parity import gen_proj
+    p = G.DevProj(*gen_proj(38, 0, 0, 128, 256, 256, 8, 2.0), 2.0)
+    G.run_single(p, bwd=False)
+    want = p.y.view(torch.int16).clone()
+    p.y.fill_(float("nan"))
+    torch.cuda.synchronize()
+    stream, shape = torch.cuda.Stream().cuda_stream, p.shape
+    ws = G.workspace(lora.lora_workspace_size(shape, lora.LORA_FWD))
+    torch.cuda.synchronize()
+    errors = []
+
+    def work():
+        try:
+            lora.lora_linear_fwd(shape, p.x, p.W, p.A, p.B, p.y, p.su, ws, ws.numel(), stream)
+        except Exception as e:  # reported below
+            errors.append(e)
+
+    t = threading.Thread(target=work)
+    t.start()
+    t.join()
+    assert not errors, errors
+    torch.cuda.synchronize()
+    assert torch.equal(p.y.view(torch.int16), want)
+
+
 def test_graph_capture_of_a_backward_only_call():
     """A backward-only call also forks: sv on the caller's stream, then dA (and
     dB) on the side stream beside the dx contraction.  Captured and replayed,
